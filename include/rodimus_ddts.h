@@ -183,11 +183,14 @@ int rodimus_ddts_step(const rodimus_ddts_step_params *p);
  * `dtype`; d_s0 fp32 [B|N,H,dk,dv] or NULL (not wanted).  No output may overlap an input.
  * Supported widths: dk = 128 and dv = 256 (others: RODIMUS_ERR_UNSUPPORTED); the value gate,
  * the feed-through and the shared-gate layout of the forward call have no backward here.
- * dtype BF16 contracts tf32 operands on the tensor cores with fp32 accumulation; dtype F32
- * splits each operand in two tf32 parts and keeps fp32 accuracy.  The workspace holds the
- * status word, 8 * dk bytes per token and head of scratch, and 6 * dk/2 * dv * 4 bytes per
- * (sequence, head): each sweep may be cut into time segments that run as thread blocks of their
- * own and hand their slice of the state to the next one through that area.  A segment waits
+ * dtype BF16 contracts on the tensor cores with fp32 accumulation: v, d_o and gated operands as
+ * pairs of bf16 (16 bits of mantissa), the carried states as tf32; dtype F32 splits each operand
+ * in two tf32 parts and keeps fp32 accuracy.  The outputs are written more than once: with BF16,
+ * d_q, d_k, d_gate_x and d_temp_y hold the gated operands until the last kernel stores the
+ * gradients there.  The workspace holds the status word, 8 * dk bytes per token and head of
+ * scratch, and 6 * dk/2 * dv * 4 bytes per (sequence, head) (a few per cent more for BF16 where
+ * sequences are long): each sweep may be cut into time segments that run as thread blocks of
+ * their own and hand their slice of the state to the next one through that area.  A segment waits
  * for the one before it under the same limit as every other wait (rodimus_ddts_test_set_wait_limit);
  * if that ran out the status word holds RODIMUS_ERR_TIMEOUT and the outputs are unspecified.
  */

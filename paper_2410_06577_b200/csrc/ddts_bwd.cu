@@ -1,4 +1,5 @@
-// Backward pass of the chunked prefill: gradients with respect to q, k, x, y, v and the initial
+// Backward pass of the chunked prefill for fp32 tokens (the validation build; bf16 tokens run
+// ddts_bwd_tc.cu): gradients with respect to q, k, x, y, v and the initial
 // state, given dL/do and dL/dS_T.  The paper trains the block through the chunkwise form
 // (appendix "Chunkwise Parallel Representation of the Rodimus Block"); this is the adjoint of
 // that form, chunk length 16, with the same notation:
@@ -25,7 +26,7 @@
 // [128 x 128]) slice of the state in REGISTERS as accumulator fragments of mma.sync.m16n8k8
 // (tf32 inputs, fp32 accumulation); the same registers are the A operand of the contraction
 // with dO or V (the k index of that instruction is a free permutation, applied to both
-// operands).  The fp32 build splits every operand into two tf32 parts (three instructions per
+// operands).  Every operand is split into two tf32 parts (three instructions per
 // product), which keeps fp32 accuracy.  A second, small kernel forms the suffix sums and dx, dy.
 #include "ddts_common.cuh"
 
@@ -65,39 +66,13 @@ __device__ __forceinline__ void st_release_s32(int32_t* p, int32_t v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <typename T>
-__device__ __forceinline__ void load8(const T* p, float (&o)[8]);
-template <>
-__device__ __forceinline__ void load8<float>(const float* p, float (&o)[8]) {
-  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+__device__ __forceinline__ void load4(const float* p, float (&o)[4]) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
 }
-template <>
-__device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16* p, float (&o)[8]) {
-  const uint4 a = *reinterpret_cast<const uint4*>(p);
-  const uint32_t w[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    o[2 * i] = __uint_as_float(w[i] << 16);
-    o[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-  }
-}
-template <typename T>
-__device__ __forceinline__ void store8(T* p, const float (&o)[8]);
-template <>
-__device__ __forceinline__ void store8<float>(float* p, const float (&o)[8]) {
+__device__ __forceinline__ void store8(float* p, const float (&o)[8]) {
   *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
   *reinterpret_cast<float4*>(p + 4) = make_float4(o[4], o[5], o[6], o[7]);
-}
-template <>
-__device__ __forceinline__ void store8<__nv_bfloat16>(__nv_bfloat16* p, const float (&o)[8]) {
-  uint32_t w[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(o[2 * i], o[2 * i + 1]);
-    w[i] = *reinterpret_cast<const uint32_t*>(&h);
-  }
-  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 __device__ __forceinline__ float tf32_round(float x) {
@@ -115,69 +90,23 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const float (&a)[4], con
         "r"(__float_as_uint(a[3])), "r"(__float_as_uint(b[0])), "r"(__float_as_uint(b[1])));
 }
 
-// c += a * b for one 16x8x8 tile.  EXACT (fp32 build): operands split as hi + lo (both tf32),
-// the lo*lo term (2^-22 of the product) dropped.  Otherwise the operands go in as they are: what
-// comes from shared memory is bf16 data or was rounded to tf32 when it was stored, and of the
-// fp32 state fragments the instruction reads the tf32 part.
-template <bool EXACT>
+// c += a * b for one 16x8x8 tile: operands split as hi + lo (both tf32), the lo*lo term (2^-22 of
+// the product) dropped.
 __device__ __forceinline__ void mma_tile(float (&c)[4], const float (&a)[4], const float (&b)[2]) {
-  if (EXACT) {
-    float ah[4], bh[2], al[4], bl[2];
+  float ah[4], bh[2], al[4], bl[2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      ah[i] = tf32_round(a[i]);
-      al[i] = tf32_round(a[i] - ah[i]);
-    }
+  for (int i = 0; i < 4; ++i) {
+    ah[i] = tf32_round(a[i]);
+    al[i] = tf32_round(a[i] - ah[i]);
+  }
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      bh[i] = tf32_round(b[i]);
-      bl[i] = tf32_round(b[i] - bh[i]);
-    }
-    mma_tf32(c, al, bh);
-    mma_tf32(c, ah, bl);
-    mma_tf32(c, ah, bh);
-  } else {
-    mma_tf32(c, a, b);
+  for (int i = 0; i < 2; ++i) {
+    bh[i] = tf32_round(b[i]);
+    bl[i] = tf32_round(b[i] - bh[i]);
   }
-}
-
-template <bool FAST>
-__device__ __forceinline__ float exp_f(float x) { return FAST ? __expf(x) : expf(x); }
-
-// log alpha and log ahat of one channel (Eq. "alpha_def").  FAST (bf16 build): hardware
-// exponential / logarithm approximations (relative error about 2^-21, far inside the bf16 bar),
-// with the two places where they would lose everything written out: log(1 + e) for small e, and
-// log(softplus(x)) for very negative x, where softplus(x) = e^x (1 - e^x / 2 + ...).
-template <bool FAST>
-__device__ __forceinline__ void gate_logs(float x, float y, int ingate, float& la, float& lh) {
-  if (!FAST) {
-    gate_logs_f32(x, y, ingate, la, lh);
-    return;
-  }
-  const float e = __expf(-fabsf(x));
-  const float l1p = e < 0.0009765625f ? e * fmaf(-0.5f, e, 1.f) : __logf(1.f + e);
-  const float g = fmaxf(x, 0.f) + l1p;
-  const float tau = __fdividef(1.f, 1.f + __expf(-y));
-  la = -g * tau;
-  if (ingate == RODIMUS_INGATE_POW_G) {
-    lh = tau * (x < -8.f ? fmaf(-0.5f, e, x) : __logf(g));
-  } else {
-    lh = -tau * (fmaxf(-x, 0.f) + l1p);
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void load4(const T* p, float (&o)[4]);
-template <>
-__device__ __forceinline__ void load4<float>(const float* p, float (&o)[4]) {
-  const float4 a = *reinterpret_cast<const float4*>(p);
-  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
-}
-template <>
-__device__ __forceinline__ void load4<__nv_bfloat16>(const __nv_bfloat16* p, float (&o)[4]) {
-  const uint2 a = *reinterpret_cast<const uint2*>(p);
-  o[0] = __uint_as_float(a.x << 16); o[1] = __uint_as_float(a.x & 0xffff0000u);
-  o[2] = __uint_as_float(a.y << 16); o[3] = __uint_as_float(a.y & 0xffff0000u);
+  mma_tf32(c, al, bh);
+  mma_tf32(c, ah, bl);
+  mma_tf32(c, ah, bh);
 }
 
 // MODE 0: forward sweep (dq, u, c); 1: reverse sweep, state [d][j] (dk, w, ds0);
@@ -187,10 +116,9 @@ __device__ __forceinline__ int segment_of_this_cta(const BwdArgs& a) {
   return (int)(blockIdx.x / (gridDim.x / a.nseg));
 }
 
-template <typename T, int MODE>
+template <int MODE>
 __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, const int half,
                           const long long row0, const int len, const int seg) {
-  constexpr bool EXACT = sizeof(T) == 4, FAST = !EXACT;
   constexpr int NCH = MODE == 2 ? DK : DK / 2;      // key channels whose gates this CTA needs
   const int ch0 = MODE == 2 ? 0 : 64 * half;
   float* sQ = smem;                    // [kC][LDK] scale * q
@@ -207,12 +135,12 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
   float* sRed = sRedA + 8 * kC * kC;   // [8][16][LDR] partial contraction of each warp / dv tile
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const T* q = (const T*)a.q + row0 * DK;
-  const T* k = (const T*)a.k + row0 * DK;
-  const T* gx = (const T*)a.gx + row0 * DK;
-  const T* ty = (const T*)a.ty + row0 * DK;
-  const T* v = (const T*)a.v + row0 * DV;
-  const T* dout = (const T*)a.dout + row0 * DV;
+  const float* q = (const float*)a.q + row0 * DK;
+  const float* k = (const float*)a.k + row0 * DK;
+  const float* gx = (const float*)a.gx + row0 * DK;
+  const float* ty = (const float*)a.ty + row0 * DK;
+  const float* v = (const float*)a.v + row0 * DV;
+  const float* dout = (const float*)a.dout + row0 * DV;
   const long long s_off = sh * (long long)DK * DV;
 
   // rows / columns of the state fragments this thread holds
@@ -257,26 +185,28 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
         const int e = tid + it * kThreads, r = e / kGroups, d4 = ch0 + (e % kGroups) * 4;
         if (r < nr) {
           const long long i = (long long)(t0 + r) * DK + d4;
-          load4<T>(q + i, fq[it]);
-          load4<T>(k + i, fk[it]);
-          load4<T>(gx + i, fx[it]);
-          load4<T>(ty + i, fy[it]);
+          load4(q + i, fq[it]);
+          load4(k + i, fk[it]);
+          load4(gx + i, fx[it]);
+          load4(ty + i, fy[it]);
         }
       }
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         const int e = tid + p * kThreads, rr = e >> 5, c8 = (e & 31) * 8;
-        float fv[8], fd[8];
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 v0 = z, v1 = z, d0 = z, d1 = z;
         if (rr < nr) {
           const long long i = (long long)(t0 + rr) * DV + c8;
-          load8<T>(v + i, fv);
-          load8<T>(dout + i, fd);
-        } else {
-#pragma unroll
-          for (int x = 0; x < 8; ++x) fv[x] = fd[x] = 0.f;
+          v0 = *reinterpret_cast<const float4*>(v + i);
+          v1 = *reinterpret_cast<const float4*>(v + i + 4);
+          d0 = *reinterpret_cast<const float4*>(dout + i);
+          d1 = *reinterpret_cast<const float4*>(dout + i + 4);
         }
-        store8<float>(sV + rr * LDV + c8, fv);
-        store8<float>(sDO + rr * LDV + c8, fd);
+        *reinterpret_cast<float4*>(sV + rr * LDV + c8) = v0;
+        *reinterpret_cast<float4*>(sV + rr * LDV + c8 + 4) = v1;
+        *reinterpret_cast<float4*>(sDO + rr * LDV + c8) = d0;
+        *reinterpret_cast<float4*>(sDO + rr * LDV + c8 + 4) = d1;
       }
 #pragma unroll
       for (int it = 0; it < kIter; ++it) {
@@ -286,8 +216,8 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
 #pragma unroll
           for (int x = 0; x < 4; ++x) {
             float lh;
-            gate_logs<FAST>(fx[it][x], fy[it][x], a.ingate, la[x], lh);
-            fa[x] = exp_f<FAST>(lh);
+            gate_logs_f32(fx[it][x], fy[it][x], a.ingate, la[x], lh);
+            fa[x] = expf(lh);
             fk[it][x] *= fa[x];
             fq[it][x] *= a.scale;
           }
@@ -302,8 +232,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
       }
     }
     __syncthreads();
-    // ---- (2) cumulative decay and scaled operands (rounded to tf32 where they only feed the
-    // tensor cores); partial dA on the tensor cores.
+    // ---- (2) cumulative decay and scaled operands; partial dA on the tensor cores.
     // Where no channel decays by more than e^-60 over the chunk, exp(b_r - b_i) is factored as
     // exp(b_r) exp(-b_i) (Ki = kt . exp(-b) stays below e^60 |kt|) and the sums over pairs become
     // plain contractions; otherwise the chunk takes the pair-by-pair form with the difference
@@ -327,8 +256,8 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
           acc += sLa[r * LDK + d];
           if (job == 0) sB[r * LDK + d] = acc;
           if (do_qe) {
-            const float x = sQ[r * LDK + d] * exp_f<FAST>(acc);
-            sQe[r * LDK + d] = FAST ? tf32_round(x) : x;
+            const float x = sQ[r * LDK + d] * expf(acc);
+            sQe[r * LDK + d] = x;
           }
         }
       }
@@ -339,17 +268,17 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
           part += sLa[r * LDK + d];      // same additions in the same order as above
           const float kt = sKt[r * LDK + d];
           if (do_ke) {
-            const float x = kt * exp_f<FAST>(tot - part);
-            sKe[r * LDK + d] = FAST ? tf32_round(x) : x;
+            const float x = kt * expf(tot - part);
+            sKe[r * LDK + d] = x;
           }
-          if (do_ki) sQe[r * LDK + d] = kt * exp_f<FAST>(-part);
+          if (do_ki) sQe[r * LDK + d] = kt * expf(-part);
           if (MODE == 2 && !strong) {    // this thread is the array's only reader in this phase
-            const float x = kt * exp_f<FAST>(-part);
-            sKt[r * LDK + d] = FAST ? tf32_round(x) : x;
+            const float x = kt * expf(-part);
+            sKt[r * LDK + d] = x;
           }
         }
       }
-      if (job == kJobs - 1) sD[d] = exp_f<FAST>(tot);
+      if (job == kJobs - 1) sD[d] = expf(tot);
     }
     if (MODE != 2) {   // dA[r][i] = sum_j dO[r][j] V[i][j], this warp's 32 value columns
       float acc[2][4] = {};
@@ -363,7 +292,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
         for (int nt = 0; nt < 2; ++nt) {
           const float2 y = *reinterpret_cast<const float2*>(sV + (nt * 8 + g) * LDV + j0);
           const float bf[2] = {y.x, y.y};
-          mma_tile<EXACT>(acc[nt], af, bf);
+          mma_tile(acc[nt], af, bf);
         }
       }
       float* red = sRedA + warp * kC * kC;
@@ -395,7 +324,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
 #pragma unroll
         for (int m = 0; m < DK / 32; ++m) {
           const int d = lane + 32 * m;
-          s = fmaf(sQ[r * LDK + d] * sKt[i * LDK + d], exp_f<FAST>(sB[r * LDK + d] - sB[i * LDK + d]), s);
+          s = fmaf(sQ[r * LDK + d] * sKt[i * LDK + d], expf(sB[r * LDK + d] - sB[i * LDK + d]), s);
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -416,7 +345,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
         for (int nt = 0; nt < 2; ++nt) {
           const float2 y = *reinterpret_cast<const float2*>(sKt + (nt * 8 + g) * LDK + d0);
           const float bf[2] = {y.x, y.y};
-          mma_tile<EXACT>(acc[nt], af, bf);
+          mma_tile(acc[nt], af, bf);
         }
       }
       float* red = sRedA + warp * kC * kC;
@@ -441,7 +370,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
         for (int rt = 0; rt < 2; ++rt) {
           const float2 y = *reinterpret_cast<const float2*>(opB + (rt * 8 + g) * ldb + c0);
           const float bf[2] = {y.x, y.y};
-          mma_tile<EXACT>(cacc[rt], af, bf);
+          mma_tile(cacc[rt], af, bf);
         }
         if ((n & 3) == 3) asm volatile("" ::: "memory");   // keep the operand loads near their use
       }
@@ -473,7 +402,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
           for (int n = 0; n < 16; ++n) {
             const int j = nbase + 8 * n + g;
             const float bf[2] = {opV[i0 * LDV + j], opV[(i0 + 4) * LDV + j]};
-            mma_tile<EXACT>(st[n], af, bf);
+            mma_tile(st[n], af, bf);
             if ((n & 3) == 3) asm volatile("" ::: "memory");
           }
         }
@@ -491,7 +420,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
 #pragma unroll
           for (int n = 0; n < 16; ++n) {
             const float bf[2] = {sQe[r0 * LDK + 8 * n + g], sQe[(r0 + 4) * LDK + 8 * n + g]};
-            mma_tile<EXACT>(st[n], af, bf);
+            mma_tile(st[n], af, bf);
             if ((n & 3) == 3) asm volatile("" ::: "memory");
           }
         }
@@ -510,16 +439,16 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
         if (strong) {
 #pragma unroll 2
           for (int i = 0; i <= r; ++i)
-            s = fmaf(sP[r * LDR + i] * sKt[i * LDK + d], exp_f<FAST>(br - sB[i * LDK + d]), s);
-          s = fmaf(exp_f<FAST>(br), r0p[r] + r1p[r], s);
+            s = fmaf(sP[r * LDR + i] * sKt[i * LDK + d], expf(br - sB[i * LDK + d]), s);
+          s = fmaf(expf(br), r0p[r] + r1p[r], s);
         } else {
           s = r0p[r] + r1p[r];
 #pragma unroll 4
           for (int i = 0; i <= r; ++i) s = fmaf(sP[r * LDR + i], sQe[i * LDK + d], s);   // Ki
-          s *= exp_f<FAST>(br);
+          s *= expf(br);
         }
         const long long o = (row0 + t0 + r) * DK + d;   // s = dL/d(scale q)
-        ((T*)a.dq)[o] = from_f32<T>(a.scale * s);
+        ((float*)a.dq)[o] = a.scale * s;
         a.u[o] = sQ[r * LDK + d] * s;                    // q . dq
       }
     } else if (MODE == 1) {
@@ -534,16 +463,16 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
         if (strong) {
 #pragma unroll 2
           for (int r = i; r < nr; ++r)
-            s = fmaf(sP[r * LDR + i] * sQ[r * LDK + d], exp_f<FAST>(sB[r * LDK + d] - bi), s);
-          s = fmaf(exp_f<FAST>(bc - bi), r0p[i] + r1p[i], s);
+            s = fmaf(sP[r * LDR + i] * sQ[r * LDK + d], expf(sB[r * LDK + d] - bi), s);
+          s = fmaf(expf(bc - bi), r0p[i] + r1p[i], s);
         } else {
           s = sD[d] * (r0p[i] + r1p[i]);
 #pragma unroll 4
           for (int r = i; r < nr; ++r) s = fmaf(sP[r * LDR + i], sQe[r * LDK + d], s);
-          s *= exp_f<FAST>(-bi);
+          s *= expf(-bi);
         }
         const long long o = (row0 + t0 + i) * DK + d;   // s = dL/d(ahat k)
-        ((T*)a.dk)[o] = from_f32<T>(s * sKe[i * LDK + d]);
+        ((float*)a.dk)[o] = s * sKe[i * LDK + d];
         a.w[o] = sKt[i * LDK + d] * s;
       }
     } else {
@@ -567,7 +496,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
 #pragma unroll
         for (int rt = 0; rt < 2; ++rt) {
           const float bf[2] = {sP[r0 * LDR + rt * 8 + g], sP[(r0 + 4) * LDR + rt * 8 + g]};
-          mma_tile<true>(cacc[rt], af, bf);   // scores are fp32 values: keep both tf32 parts
+          mma_tile(cacc[rt], af, bf);
         }
       }
       {
@@ -586,7 +515,7 @@ __device__ void bwd_sweep(const BwdArgs& a, float* smem, const long long sh, con
         float o8[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) o8[e] = sRed[i * ldo + c8 + e];
-        store8<T>((T*)a.dv + (row0 + t0 + i) * DV + 128 * half + c8, o8);
+        store8((float*)a.dv + (row0 + t0 + i) * DV + 128 * half + c8, o8);
       }
     }
     __syncthreads();
@@ -651,7 +580,6 @@ constexpr size_t kSweepSmem =
     sizeof(float) * (6 * kC * LDK + 2 * kC * LDV + DK + kC * LDR + 8 * kC * kC + 8 * 16 * LDR);
 static_assert(16 * (128 + 4) <= 8 * 16 * LDR, "the dv tile fits the space of the partials");
 
-template <typename T>
 __global__ void __launch_bounds__(kThreads, 2) ddts_bwd_sweep_kernel(const BwdArgs a) {
   extern __shared__ __align__(16) float smem[];
   // The three sweeps differ in length (on the layer shape: the transposed reverse sweep 1.14 ms,
@@ -705,9 +633,9 @@ __global__ void __launch_bounds__(kThreads, 2) ddts_bwd_sweep_kernel(const BwdAr
       return;
     }
   }
-  if (mode == 0) bwd_sweep<T, 0>(a, smem, sh, half, row0, len, seg);
-  else if (mode == 1) bwd_sweep<T, 1>(a, smem, sh, half, row0, len, seg);
-  else bwd_sweep<T, 2>(a, smem, sh, half, row0, len, seg);
+  if (mode == 0) bwd_sweep<0>(a, smem, sh, half, row0, len, seg);
+  else if (mode == 1) bwd_sweep<1>(a, smem, sh, half, row0, len, seg);
+  else bwd_sweep<2>(a, smem, sh, half, row0, len, seg);
 }
 
 // dL/dlog alpha by suffix sums over the sequence, then dx, dy (Eq. "alpha_def", chain rule):
@@ -716,7 +644,6 @@ __global__ void __launch_bounds__(kThreads, 2) ddts_bwd_sweep_kernel(const BwdAr
 //   dx   = dg sigmoid(x)                dy   = dtau tau (1 - tau)
 // One CTA per (sequence, head, 32 channels): 32 channels x 16 time segments.
 constexpr int kGateCh = 32, kGateSegs = 16;
-template <typename T>
 __global__ void __launch_bounds__(kGateCh * kGateSegs) ddts_bwd_gates_kernel(const BwdArgs a) {
   __shared__ double seg_sum[kGateSegs][kGateCh];
   const long long sh = blockIdx.x / (DK / kGateCh);
@@ -747,14 +674,14 @@ __global__ void __launch_bounds__(kGateCh * kGateSegs) ddts_bwd_gates_kernel(con
   __syncthreads();
   double acc = (double)a.c[sh * DK + d];
   for (int s2 = seg + 1; s2 < kGateSegs; ++s2) acc += seg_sum[s2][dl];
-  const T* gx = (const T*)a.gx;
-  const T* ty = (const T*)a.ty;
+  const float* gx = (const float*)a.gx;
+  const float* ty = (const float*)a.ty;
   for (int r = hi - 1; r >= lo; --r) {
     const long long i = (row0 + r) * DK + d;
     const float w = a.w[i];
     acc += (double)a.u[i] - (double)w;
     const float dla = (float)acc;
-    const float x = to_f32(gx[i]), y = to_f32(ty[i]);
+    const float x = gx[i], y = ty[i];
     const float g = softplus_f32(x);
     const float tau = y >= 0.f ? 1.f / (1.f + expf(-y)) : expf(y) / (1.f + expf(y));
     const float sx = x >= 0.f ? 1.f / (1.f + expf(-x)) : expf(x) / (1.f + expf(x));
@@ -768,18 +695,19 @@ __global__ void __launch_bounds__(kGateCh * kGateSegs) ddts_bwd_gates_kernel(con
     }
     const float dxv = -tau * dla * sx + w * tau * dgx;
     const float dyv = (-g * dla + w * lnu) * tau * (1.f - tau);
-    ((T*)a.dx)[i] = from_f32<T>(dxv);
-    ((T*)a.dy)[i] = from_f32<T>(dyv);
+    ((float*)a.dx)[i] = dxv;
+    ((float*)a.dy)[i] = dyv;
   }
 }
 
-std::atomic<unsigned long long> g_smem_done_bf16{0}, g_smem_done_f32{0};
+std::atomic<unsigned long long> g_smem_done{0};
 
 }  // namespace
 
 bool bwd_supported(const rodimus_ddts_bwd_params& p) { return p.dk == DK && p.dv == DV; }
 
 size_t bwd_scratch_bytes(const rodimus_ddts_bwd_params& p) {
+  if (p.dtype == RODIMUS_BF16) return bwd_tc_scratch_bytes(p);
   const size_t rows = (size_t)p.B * p.H * p.T;
   const size_t nseq = p.cu_seqlens ? (size_t)p.N : (size_t)p.B;
   size_t b = sizeof(float) * (2 * rows * DK + nseq * p.H * DK);
@@ -790,6 +718,7 @@ size_t bwd_scratch_bytes(const rodimus_ddts_bwd_params& p) {
 }
 
 cudaError_t launch_bwd(const rodimus_ddts_bwd_params& p, size_t scratch_offset, int* n_launches) {
+  if (p.dtype == RODIMUS_BF16) return launch_bwd_tc(p, scratch_offset, n_launches);
   *n_launches = 0;
   BwdArgs a;
   a.q = p.q; a.k = p.k; a.gx = p.gate_x; a.ty = p.temp_y; a.v = p.v; a.dout = p.d_o;
@@ -840,17 +769,10 @@ cudaError_t launch_bwd(const rodimus_ddts_bwd_params& p, size_t scratch_offset, 
       if (e != cudaSuccess) return e;
     }
   }
-  if (p.dtype == RODIMUS_BF16) {
-    e = opt_in_shared_memory(ddts_bwd_sweep_kernel<__nv_bfloat16>, (int)kSweepSmem, dev, g_smem_done_bf16);
-    if (e != cudaSuccess) return e;
-    ddts_bwd_sweep_kernel<__nv_bfloat16><<<(unsigned)(items * 6 * a.nseg), kThreads, kSweepSmem, st>>>(a);
-    ddts_bwd_gates_kernel<__nv_bfloat16><<<(unsigned)(items * (DK / kGateCh)), kGateCh * kGateSegs, 0, st>>>(a);
-  } else {
-    e = opt_in_shared_memory(ddts_bwd_sweep_kernel<float>, (int)kSweepSmem, dev, g_smem_done_f32);
-    if (e != cudaSuccess) return e;
-    ddts_bwd_sweep_kernel<float><<<(unsigned)(items * 6 * a.nseg), kThreads, kSweepSmem, st>>>(a);
-    ddts_bwd_gates_kernel<float><<<(unsigned)(items * (DK / kGateCh)), kGateCh * kGateSegs, 0, st>>>(a);
-  }
+  e = opt_in_shared_memory(ddts_bwd_sweep_kernel, (int)kSweepSmem, dev, g_smem_done);
+  if (e != cudaSuccess) return e;
+  ddts_bwd_sweep_kernel<<<(unsigned)(items * 6 * a.nseg), kThreads, kSweepSmem, st>>>(a);
+  ddts_bwd_gates_kernel<<<(unsigned)(items * (DK / kGateCh)), kGateCh * kGateSegs, 0, st>>>(a);
   *n_launches = 2;
   return cudaGetLastError();
 }

@@ -1296,6 +1296,22 @@ cudaError_t launch_pair(const PairMaps& m, const PairArgs& a, int max_pairs, int
 
 }  // namespace
 
+bool encode_bf16_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+  return make_map(m, ptr, rows, cols, box_rows);
+}
+
+bool encode_bf16_slab_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t slabs) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {64, rows, cols / 64};
+  const cuuint64_t strides[2] = {cols * 2, 128};
+  const cuuint32_t box[3] = {64u, (cuuint32_t)kC, slabs};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool fwd_pair_supported(const rodimus_ddts_fwd_params& p) {
   return p.dtype == RODIMUS_BF16 && p.dk == kDK && p.dv % (2 * kDVS) == 0;
 }

@@ -7,6 +7,14 @@
 #include "ddts_common.cuh"
 
 namespace ddts {
+
+// Tensor map of a [rows, cols] bf16 row-major matrix for boxes of box_rows rows x 64 columns (128
+// bytes), 128-byte swizzle; rows past the end of the matrix read as zeros and are not written.
+bool encode_bf16_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);
+// The same matrix seen as [cols / 64][rows][64]: one box of [slabs][64][64] is `slabs` consecutive
+// 64-column tiles of 64 rows, 8 KiB each, brought by ONE copy.
+bool encode_bf16_slab_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t slabs);
+
 namespace {
 
 constexpr long long kWaitCycles = 4000000000LL;   // default limit of a main-loop wait: about two
@@ -128,6 +136,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
 // Ask for a 2-D tile to be brought into L2 (no shared-memory destination, nothing to wait for).
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
@@ -168,6 +183,13 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+// True in one lane of the (converged) warp, always the same one.  Code under it is known to the
+// compiler to run in a single thread, unlike code under a test of the lane number.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.b32 %0, 1, 0, q;\n}" : "=r"(p));
+  return p != 0;
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"

@@ -177,3 +177,22 @@ def test_bwd_packed_sequences_cut_into_time_segments(dtype):
                         name="bwd_packed_segments")
     _check(p, 902, True)
     _check(p, 903, False, host_cu=False, want_d_s0=False)
+
+
+@pytest.mark.parametrize("T", [2, 63, 64, 65, 129, 520])
+@pytest.mark.parametrize("strong", [False, True])
+def test_bwd_bf16_tile_edges_and_cut_tiles(T, strong):
+    """Edges of the 64-row tiles, time segments (520 rows), and tiles that strong decays cut into
+    several chunks: single steps of e^-60 and more among mild ones, in some channels only.  Bar of
+    this file for bf16.
+
+    A strong step's dx is w tau sigmoid(x)/g - dla tau sigmoid(x) where dla, nearly zero, is a
+    difference of sums as large as w; the states are read as tf32 (2^-11), so dx carries an error of up
+    to 2^-11 g of the size of its first term: 4e-2 at g = 80, beyond the bar where such steps are all
+    there is.  Two rows therefore take g = 20 (1e-2); longer sequences have mild rows, whose dx is
+    larger and sets the scale."""
+    p = wl.make_prefill(1000 + T, 1, 2, T, 128, 256, "bf16", s0_std=0.1, name=f"bwd_tile_{T}")
+    if strong:
+        p.x[:, :, T // 3:T // 3 + 7, ::5] = 80.0 if T > 2 else 20.0     # softplus(80) sigmoid(4) = 78.6 per step
+        p.y[:, :, T // 3:T // 3 + 7, ::5] = 4.0
+    _check(p, 1100 + T, True, scale=0.5)
