@@ -192,7 +192,7 @@ ddts_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 
   if (warp == 0) {
     // ===================================== TMA producer =====================================
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t f = 0;         // fills issued
       int j = 0, tpos = 0;    // speculative position: item index and token
       int seen = 0;           // last redirect taken
@@ -255,7 +255,7 @@ ddts_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     }
   } else if (warp == 1) {
     // ====================================== MMA issuer ======================================
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t kIdescP = make_idesc(64, 64, 0, 0);
       constexpr uint32_t kIdescO = make_idesc(64, kDVS, 0, 1);
       constexpr uint32_t kIdescS = make_idesc(128, kDVS, 1, 1);
@@ -622,7 +622,7 @@ ddts_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   tc_fence_before();
   __syncthreads();
   if (ctl->wait.abort_flag && warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       umma_commit(bar(BAR_DRAIN));
       mbar_drain(bar(BAR_DRAIN), 0);
     }

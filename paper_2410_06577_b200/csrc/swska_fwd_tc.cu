@@ -17,8 +17,9 @@
 //                    packed bf16 (tcgen05.st)
 //   O += P V         tcgen05.mma, A = P from tensor memory, B = the V tile (token-major, i.e.
 //                    N-major) from shared memory
-// Issuing a tcgen05.mma or a TMA load costs its thread about a hundred cycles here, which is why
-// two threads of two warps share that work and the softmax warps do none of it.  Tensor memory: 256 columns
+// One warp issues every contraction and one every load, under elect_one(): with a test of the lane
+// number instead an instruction cost its thread about a hundred cycles (layer shape 84.1 us, now 79.6).
+// Tensor memory: 256 columns
 // (S twice 64, O 128); shared memory 96 KiB (Q 32, two K tiles, two V tiles; a tile is requested
 // two tiles ahead, as soon as the contraction that read its slot is complete): two CTAs per SM.  Only key tiles that
 // touch the 128 queries' windows are visited.  Every wait is bounded; a wait that runs out ends
@@ -160,7 +161,7 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
   if (warp == kProducerWarp) {
     // =========================== producer warp: every TMA load ================================
-    if (lane == 0) {
+    if (elect_one()) {
       int k_sent = 0, v_sent = 0;
       auto load = [&](const CUtensorMap* map, uint32_t dst, uint32_t slab, int row, int which, uint32_t bytes) {
         mbar_expect_tx(bar(which), bytes);
@@ -194,51 +195,62 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     __syncwarp();
   } else if (warp == kIssuerWarp) {
     // =========================== issuing warp: every contraction ==============================
-    if (lane == 0) {
+    // Every lane walks the tiles; what is issued sits in elect_one() blocks.
+    {
       constexpr uint32_t kIdescS = make_idesc(kBM, kBN, 0, 0);   // S = Q K^T, both K-major
       constexpr uint32_t kIdescO = make_idesc(kBM, kD, 0, 1);    // O += P V: A in tensor memory, B N-major
       int k_seen = 0, v_seen = 0;
+      auto wait = [&](int b, uint32_t parity) -> bool {
+        return __all_sync(0xffffffffu, sw_wait(bar(b), parity, ctl, a.status)) != 0;
+      };
+      const uint32_t dq0 = desc_lo_kmajor(base + kOffQ), dq1 = desc_lo_kmajor(base + kOffQ + kQSlabBytes);
       auto issue_s = [&](int j) {   // scores of tile j into buffer j & 1
-        const uint32_t dq0 = desc_lo_kmajor(base + kOffQ), dq1 = desc_lo_kmajor(base + kOffQ + kQSlabBytes);
         const uint32_t ks = base + kOffK + (j & 1) * kTileBytes;
         const uint32_t dk0 = desc_lo_kmajor(ks), dk1 = desc_lo_kmajor(ks + kSlabBytes);
         const uint32_t d = tmem + kColS + (j & 1) * kBN;
-        umma_bf16_lo<false>(d, dq0, dk0, kIdescS);
+        if (elect_one()) {
+          umma_bf16_lo<false>(d, dq0, dk0, kIdescS);
 #pragma unroll
-        for (int kk = 1; kk < 4; ++kk) umma_bf16_lo<true>(d, dq0 + 2 * kk, dk0 + 2 * kk, kIdescS);
+          for (int kk = 1; kk < 4; ++kk) umma_bf16_lo<true>(d, dq0 + 2 * kk, dk0 + 2 * kk, kIdescS);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) umma_bf16_lo<true>(d, dq1 + 2 * kk, dk1 + 2 * kk, kIdescS);
-        umma_commit(bar(BAR_S0 + (j & 1)));
+          for (int kk = 0; kk < 4; ++kk) umma_bf16_lo<true>(d, dq1 + 2 * kk, dk1 + 2 * kk, kIdescS);
+          umma_commit(bar(BAR_S0 + (j & 1)));
+        }
+        __syncwarp();
       };
-      bool ok = sw_wait(bar(BAR_Q), 0, ctl, a.status);
-      if (ok) { ok = sw_wait(bar(BAR_K0), 0, ctl, a.status); k_seen += ok; }
+      bool ok = wait(BAR_Q, 0);
+      if (ok) { ok = wait(BAR_K0, 0); k_seen += ok; }
       if (ok) { tc_fence_after(); issue_s(0); }
       for (int it = 0; ok && it < n_tiles; ++it) {
         const int sb = it & 1;
         const uint32_t ph = (it >> 1) & 1;
         if (it + 1 < n_tiles) {            // the next tile's scores, while this tile's softmax runs
-          ok = sw_wait(bar(BAR_K0 + (sb ^ 1)), ((it + 1) >> 1) & 1, ctl, a.status);
+          ok = wait(BAR_K0 + (sb ^ 1), ((it + 1) >> 1) & 1);
           k_seen += ok;
           if (!ok) break;
           tc_fence_after();
           issue_s(it + 1);
         }
-        if (!(ok = sw_wait(bar(BAR_P0 + sb), ph, ctl, a.status))) break;   // probabilities in place
-        ok = sw_wait(bar(BAR_V0 + sb), ph, ctl, a.status);
+        if (!(ok = wait(BAR_P0 + sb, ph))) break;   // probabilities in place
+        ok = wait(BAR_V0 + sb, ph);
         v_seen += ok;
         if (!ok) break;
         tc_fence_after();
         const uint32_t dv = desc_lo_mnmajor(base + kOffV + sb * kTileBytes, kSlabBytes);
         const uint32_t pa = tmem + kColS + sb * kBN;
+        if (elect_one()) {
+          if (it == 0) umma_bf16_atmem<false>(tmem + kColO, pa, dv, kIdescO);
+          else umma_bf16_atmem<true>(tmem + kColO, pa, dv, kIdescO);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          if (kk == 0 && it == 0) umma_bf16_atmem<false>(tmem + kColO, pa, dv, kIdescO);
-          else umma_bf16_atmem<true>(tmem + kColO, pa + 8 * kk, dv + 128 * kk, kIdescO);
+          for (int kk = 1; kk < 4; ++kk) umma_bf16_atmem<true>(tmem + kColO, pa + 8 * kk, dv + 128 * kk, kIdescO);
+          umma_commit(bar(BAR_O0 + sb));   // (two barriers, by tile parity: a waiter is never two phases behind)
         }
-        umma_commit(bar(BAR_O0 + sb));   // (two barriers, by tile parity: a waiter is never two phases behind)
+        __syncwarp();
       }
-      ctl->k_seen = k_seen;
-      ctl->v_seen = v_seen;
+      if (lane == 0) {
+        ctl->k_seen = k_seen;
+        ctl->v_seen = v_seen;
+      }
     }
     __syncwarp();
   } else {
@@ -413,7 +425,7 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       for (int j = ctl->k_seen; j < ctl->k_sent; ++j) mbar_drain(bar(BAR_K0 + (j & 1)), (j >> 1) & 1);
       for (int j = ctl->v_seen; j < ctl->v_sent; ++j) mbar_drain(bar(BAR_V0 + (j & 1)), (j >> 1) & 1);
     }
-    if (warp == kIssuerWarp && lane == 0) {   // (a commit follows the contractions of the thread that makes it)
+    if (warp == kIssuerWarp && elect_one()) {   // (a commit follows the contractions of the thread that makes it)
       umma_commit(bar(BAR_DRAIN));            // completes when every contraction issued so far has
       mbar_drain(bar(BAR_DRAIN), 0);
     }
