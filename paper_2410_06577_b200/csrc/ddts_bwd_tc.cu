@@ -36,15 +36,12 @@
 
 #include "ddts_common.cuh"
 #include "ddts_tc_ptx.cuh"
+#include "ddts_tiles.cuh"
 
 namespace ddts {
 namespace {
 
-constexpr int kTile = 64;               // rows of a tile, and of a chunk unless decays are strong
 constexpr int DK = 128, DV = 256;       // the widths these kernels are built for
-constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kLg2Ln2 = -0.5287663729448977f;   // log2(ln 2)
-constexpr float kRange2 = 60.f * kLog2e;          // largest decay range of a chunk, log2 units
 
 struct BwdTcArgs {
   const __nv_bfloat16 *q, *k, *gx, *ty;
@@ -72,92 +69,7 @@ struct BwdTcArgs {
   int ingate;
   long long limit;
 };
-
-// The tile of one (head, slot): packed sequences take slots floor(start / 64) + n ... , which are
-// disjoint for consecutive sequences; a slot may belong to none.
-struct TileRef {
-  int n, t, nr;            // sequence, tile of the sequence, live rows (0: no such tile)
-  int len;                 // rows of the sequence
-  long long row0;          // first row of the tile
-  long long sh;            // sequence * H + head
-};
-
-__device__ __forceinline__ void seq_range(const int32_t* cu, int n, int T, int& lo, int& hi) {
-  lo = cu[n];
-  hi = cu[n + 1];
-  lo = lo < 0 ? 0 : (lo > T ? T : lo);
-  hi = hi < lo ? lo : (hi > T ? T : hi);
-}
-
-// Block-wide (every thread takes part; s_n is one shared int).
-__device__ __forceinline__ TileRef find_tile(const BwdTcArgs& a, int head, int local, int* s_n) {
-  TileRef r;
-  if (!a.cu) {
-    r.n = head / a.H;
-    r.t = local;
-    r.len = a.T;
-    r.nr = min(kTile, a.T - r.t * kTile);
-    r.row0 = (long long)head * a.T + (long long)r.t * kTile;
-    r.sh = head;
-    return r;
-  }
-  if (threadIdx.x == 0) *s_n = -1;
-  __syncthreads();
-  int best = -1;   // the last sequence whose first slot is not beyond this one
-  for (int n = threadIdx.x; n < a.n_seq; n += blockDim.x) {
-    int lo, hi;
-    seq_range(a.cu, n, a.T, lo, hi);
-    if (lo / kTile + n <= local) best = n;
-  }
-  if (best >= 0) atomicMax(s_n, best);
-  __syncthreads();
-  r.n = *s_n;
-  r.nr = 0;
-  if (r.n < 0) return r;
-  int lo, hi;
-  seq_range(a.cu, r.n, a.T, lo, hi);
-  r.t = local - (lo / kTile + r.n);
-  r.len = hi - lo;
-  r.nr = min(kTile, r.len - r.t * kTile);
-  r.row0 = (long long)head * a.T + lo + (long long)r.t * kTile;
-  r.sh = (long long)r.n * a.H + head;
-  return r;
-}
-
-__device__ __forceinline__ float2 unpack_bf16(uint32_t w) {
-  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-// hi + lo = x to 16 bits of mantissa, both bf16; packed for two values.
-__device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
-  hi = pack_bf16(x, y);
-  const float2 h = unpack_bf16(hi);
-  lo = pack_bf16(x - h.x, y - h.y);
-}
-
-// Everything the gates need of one channel (Eq. "alpha_def"), hardware exponential / logarithm
-// approximations (relative error about 2^-21, far inside the rounding of bf16 results) with the
-// places where they would lose digits written out.
-struct Gate {
-  float g2;        // softplus(x) * log2(e)
-  float e, r;      // e^-|x|, 1 / (1 + e)
-  float tau;
-  float la2, lh2;  // log2 alpha (not below -kRange2), log2 ahat
-};
-__device__ __forceinline__ Gate gate_of(float x, float y, int ingate) {
-  Gate o;
-  o.e = ex2f(-fabsf(x) * kLog2e);
-  const float l1p2 = o.e < 9.765625e-4f ? o.e * fmaf(-0.72134752f, o.e, kLog2e) : lg2f(1.f + o.e);
-  o.g2 = fmaf(fmaxf(x, 0.f), kLog2e, l1p2);
-  o.tau = rcpf(1.f + ex2f(-y * kLog2e));
-  o.la2 = fmaxf(-o.g2 * o.tau, -kRange2);
-  if (ingate == RODIMUS_INGATE_POW_G) {
-    const float lg = x < -8.f ? fmaf(-0.5f, o.e, x) * kLog2e : lg2f(o.g2) + kLg2Ln2;
-    o.lh2 = o.tau * lg;
-  } else {
-    o.lh2 = -o.tau * fmaf(fmaxf(-x, 0.f), kLog2e, l1p2);
-  }
-  return o;
-}
+__device__ __forceinline__ TileGeometry geometry(const BwdTcArgs& a) { return {a.cu, a.n_seq, a.T, a.cu ? 1 : a.H}; }
 
 __device__ __forceinline__ int32_t ld_acquire_s32(const int32_t* p) {
   int32_t v;
@@ -169,87 +81,6 @@ __device__ __forceinline__ void st_release_s32(int32_t* p, int32_t v) {
 }
 __device__ __forceinline__ void red_release_add(int32_t* p, int32_t v) {
   asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Row r's chunk: the last set bit of the mask at or before r.
-__device__ __forceinline__ int chunk_start(unsigned long long mask, int r) {
-  return 63 - __clzll((long long)(mask & (~0ull >> (63 - r))));
-}
-// one past the chunk's last row
-__device__ __forceinline__ int chunk_end(unsigned long long mask, int r, int nr) {
-  const unsigned long long later = r == 63 ? 0ull : mask & (~0ull << (r + 1));
-  return later ? __ffsll((long long)later) - 1 : nr;
-}
-
-// Cumulative decay (log2) since the chunk's start, in place, for ROWS rows of two of the CTA's CH
-// channels; v holds the rows' own log2 decays on entry.  `part` is a [kTile / ROWS][CH] float tile,
-// `la` a [kTile][CH] one that is used only where a tile has several chunks; la_of(i) then gives row i's
-// own decays again.  Returns the tile's chunk mask: the given one or, when MAKE_MASK, the one it
-// determines (dyadic blocks whose decay exceeds the range in some channel are cut in the middle).
-template <int ROWS, int CH, bool MAKE_MASK, typename LaOf>
-__device__ __forceinline__ unsigned long long tile_scan(float2 (&v)[ROWS], int cp, int rg, int nr, float* la, float* part,
-                                                        unsigned long long* s_mask, unsigned long long mask, LaOf la_of) {
-  constexpr int kGroups = kTile / ROWS;
-#pragma unroll
-  for (int i = 1; i < ROWS; ++i) v[i] = __fadd2_rn(v[i], v[i - 1]);
-  *reinterpret_cast<float2*>(part + rg * CH + 2 * cp) = v[ROWS - 1];
-  __syncthreads();
-  float2 pre = make_float2(0.f, 0.f), all = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int w = 0; w < kGroups; ++w) {
-    if (w == rg) pre = all;
-    all = __fadd2_rn(all, *reinterpret_cast<const float2*>(part + w * CH + 2 * cp));
-  }
-  bool whole;
-  if (MAKE_MASK) {
-    whole = __syncthreads_or(all.x < -kRange2 || all.y < -kRange2) == 0;
-    mask = 1ull;
-  } else {
-    whole = mask == 1ull;
-  }
-  if (whole) {
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) v[i] = __fadd2_rn(v[i], pre);
-    return mask;
-  }
-  // ---- rare: several chunks in the tile
-#pragma unroll 1
-  for (int i = 0; i < ROWS; ++i) *reinterpret_cast<float2*>(la + (rg * ROWS + i) * CH + 2 * cp) = la_of(i);
-  if (MAKE_MASK) {
-    if (threadIdx.x == 0) *s_mask = 1ull;
-    __syncthreads();
-    for (int d = threadIdx.x; d < CH; d += blockDim.x) {
-      unsigned long long m = 0ull;
-#pragma unroll 1
-      for (int len = kTile; len >= 2; len >>= 1)
-#pragma unroll 1
-        for (int r0 = 0; r0 < nr; r0 += len) {
-          float s = 0.f;
-          for (int r = r0; r < min(r0 + len, nr); ++r) s += la[r * CH + d];
-          if (s < -kRange2 && r0 + len / 2 < nr) m |= 1ull << (r0 + len / 2);
-        }
-      if (m) atomicOr(s_mask, m);
-    }
-    __syncthreads();
-    mask = *s_mask;
-  } else {
-    __syncthreads();
-  }
-#pragma unroll 1
-  for (int i = 0; i < ROWS; ++i) {
-    const int r = rg * ROWS + i;
-    float2 acc = make_float2(0.f, 0.f);
-    if (r < nr) {
-      for (int j = chunk_start(mask, r); j <= r; ++j) {
-        acc.x += la[j * CH + 2 * cp];
-        acc.y += la[j * CH + 2 * cp + 1];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < ROWS; ++u)
-      if (u == i) v[u] = acc;
-  }
-  return mask;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -267,7 +98,7 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
   for (long long i = (long long)blockIdx.x * kPreThreads + tid; i < a.n_flags; i += (long long)gridDim.x * kPreThreads)
     a.seg_flag[i] = 0;
   const int head = (int)(blockIdx.x / (unsigned)a.slots_per_head), local = (int)(blockIdx.x % (unsigned)a.slots_per_head);
-  const TileRef tr = find_tile(a, head, local, &s_n);
+  const TileRef tr = find_tile(geometry(a), head, local, &s_n);
   const long long slot = (long long)head * a.slots_per_head + local;
   if (tid < 4) a.tile_flag[slot * 4 + tid] = 0;
   if (tr.nr <= 0) return;
@@ -411,10 +242,6 @@ __device__ __forceinline__ void umma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, u
       "mov.b64 db, {%2, %5};\n"
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], db, %3, p;\n}"
       ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(acc), "r"(kDescHi) : "memory");
-}
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 __device__ __forceinline__ float tf32_rna(float x) {
   uint32_t r;
@@ -1122,7 +949,7 @@ __global__ void __launch_bounds__(kPostThreads, 3) ddts_bwd_post_kernel(const Bw
   const int tid = threadIdx.x;
   const int quarter = (int)(blockIdx.x & 3u), hs = (int)(blockIdx.x >> 2);
   const int head = hs % a.heads, local = a.slots_per_head - 1 - hs / a.heads;
-  const TileRef tr = find_tile(a, head, local, &s_n);
+  const TileRef tr = find_tile(geometry(a), head, local, &s_n);
   if (tr.nr <= 0) return;
   const long long slot = (long long)head * a.slots_per_head + local;
   const int cp = tid & 15, rg = tid >> 4, ch = quarter * kPostCh + 2 * cp;
@@ -1243,8 +1070,8 @@ __global__ void __launch_bounds__(kPostThreads, 3) ddts_bwd_post_kernel(const Bw
     acc0 = v.x;
     acc1 = v.y;
   } else {
-    acc0 = a.dsT ? (double)a.c[tr.sh * DK + ch] : 0.0;
-    acc1 = a.dsT ? (double)a.c[tr.sh * DK + ch + 1] : 0.0;
+    acc0 = a.dsT ? (double)a.c[(long long)(tr.n * a.H + (a.cu ? head : head % a.H)) * DK + ch] : 0.0;
+    acc1 = a.dsT ? (double)a.c[(long long)(tr.n * a.H + (a.cu ? head : head % a.H)) * DK + ch + 1] : 0.0;
   }
 #pragma unroll 1
   for (int g = kTile / kPostRows - 1; g > rg; --g) {

@@ -52,6 +52,9 @@ size_t bwd_tc_scratch_bytes(const rodimus_ddts_bwd_params& p);
 cudaError_t launch_swska(const rodimus_swska_fwd_params& p, int* n_launches);
 cudaError_t launch_swska_tc(const rodimus_swska_fwd_params& p, int* n_launches);   // bf16, tcgen05
 bool swska_supported(const rodimus_swska_fwd_params& p);
+cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches);
+// Workspace with which the two-launch prefill (operands, scan) takes this request; 0: it does not.
+size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p);
 bool fwd_tc_supported(const rodimus_ddts_fwd_params& p);
 bool fwd_pair_supported(const rodimus_ddts_fwd_params& p);
 // Workspace a dense call needs if its sequences are to be split along time (0: no split).

@@ -1,0 +1,927 @@
+// Chunked DDTS prefill in two launches, for calls whose gates serve several CTAs or whose items are
+// too few to fill the device: operands first, then the scan.
+//
+// Chunk algebra (appendix "Chunkwise Parallel Representation of the Rodimus Block"; chunk length 64,
+// log2 domain, decays anchored at the chunk start, b_r = sum_{j<=r} log2 alpha_j <= 0):
+//   Qt_r = scale q_r 2^{b_r}      Kt_i = k_i ahat_i 2^{-b_i}      D = 2^{b_C}
+//   P = mask(Qt Kt^T)             O = P V + Qt S_in               S_out = D . (S_in + Kt^T V)
+// Everything that depends on the gates - Qt, Kt, D and also P - is the same for all value columns.
+//
+//   ddts_operands_kernel   a CTA per 64-row tile of every set of gates: Kt, Qt, P and D of the tile as
+//                          ONE block of global memory, laid out as the tensor core reads it from
+//                          shared memory (128-byte swizzle), so that a single bulk copy brings it in
+//   ddts_scan_kernel       a CTA per (sequence, head, 128 value columns): no gate arithmetic, per
+//                          chunk two bulk copies, a tensor copy of the v tile and three contractions
+// In the layout with one set of gates for all heads the first kernel does 1/H of the work that every
+// head's own gates would be, and its blocks are read from L2 by all H dv / 128 CTAs of a sequence.
+// Figures (layer shape, B=4 H=16 T=2048 dv=256): one set of gates, dk = 64: 9.6 us + 36 us, the scan
+// bound by the issue of its contractions (1670 cycles per chunk of 28 instructions, 1216 cycles of tensor
+// work) with 11 TB/s out of L2; gates per head, dk = 128: operands 55 us (issue-bound), scan 36 us (218 MB,
+// 6 TB/s).
+//
+// dk = 128: operands in bf16, the precision of the kernel with the gates inside.  dk = 64 (the paper's
+// own key width): Kt as three bf16 parts (24 bits), Qt, P and the state's copy for the readout as two
+// (16 bits), gates with accurate functions: fp32 accuracy in the state, 2^-16 before the rounding of o.
+//
+// Where a tile decays by more than e^-60 in some channel it is cut in halves until every chunk fits
+// (down to single rows, which always fit because a step's decay is applied as at least e^-60): P
+// then keeps pairs of the same chunk only, and the scan takes the tile once per chunk, with the other
+// rows of Kt set to zero.
+#include <cuda.h>
+
+#include <cstring>
+
+#include "ddts_common.cuh"
+#include "ddts_tc_ptx.cuh"
+#include "ddts_tiles.cuh"
+
+namespace ddts {
+namespace {
+
+constexpr int kSlab = kTile * 128;          // [64 rows][128 bytes], 128-byte swizzled
+
+// The block of a tile: slabs of Kt and P, then of Qt, then D and the header.
+template <int DK>
+struct Block {
+  static constexpr bool kExact = DK == 64;
+  static constexpr int kSlabs = DK / 64;                    // slabs of one part of Kt or Qt
+  static constexpr int kKp = kExact ? 3 : 1, kQp = kExact ? 2 : 1;   // parts of Kt; of Qt and P
+  static constexpr int kK = 0, kP = kKp * kSlabs * kSlab, kQ = kP + kQp * kSlab, kD = kQ + kQp * kSlabs * kSlab;
+  static constexpr int kHead = kD + 512;                    // chunk mask of the tile
+  static constexpr int kBytes = kD + 1024;
+};
+
+struct ScanArgs {
+  const __nv_bfloat16 *q, *k, *gx, *ty;
+  const float *s0;
+  float* sT;
+  const float* feed_d;
+  unsigned char* blocks;
+  const int32_t *cu, *order;
+  WorkspaceHeader* hdr;
+  int H, T, dv, n_seq;
+  int gate_heads;       // sets of gates per sequence: H, or 1 when all heads share one
+  int slots_per_head;   // tiles of one (batch, set) of a dense call, of one set of a packed one
+  int cols;             // slices of 128 value columns
+  int has_beta;
+  float scale;
+  int ingate;
+  long long limit;
+};
+
+template <bool EXACT>
+__device__ __forceinline__ void gate_pair(float x, float y, int ingate, float& la2, float& lh2) {
+  if (EXACT) {
+    gate_logs_f32(x, y, ingate, la2, lh2);
+    la2 = fmaxf(la2 * kLog2e, -kRange2);
+    lh2 *= kLog2e;
+  } else {
+    const Gate g = gate_of(x, y, ingate);
+    la2 = g.la2;
+    lh2 = g.lh2;
+  }
+}
+
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// ---------------------------------------------------------------------------------------------
+// Operands of one tile
+// ---------------------------------------------------------------------------------------------
+constexpr int kOpThreads = 512;
+template <int DK>
+constexpr int kOpRowsOf = DK / 16;          // 4 or 8 rows x 2 channels a thread
+template <int DK>
+constexpr int kOpSmem = Block<DK>::kBytes + (kTile / kOpRowsOf<DK>) * DK * 4 + 1024;
+
+template <int DK>
+__global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const ScanArgs a) {
+  using B = Block<DK>;
+  constexpr int kOpRows = kOpRowsOf<DK>;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ unsigned long long s_mask;
+  __shared__ int s_n;
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
+  float* s_part = reinterpret_cast<float*>(gbase + B::kBytes);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (!a.cu && blockIdx.x == 0 && tid == 0) a.hdr->status = RODIMUS_OK;
+  const int head = (int)(blockIdx.x / (unsigned)a.slots_per_head), local = (int)(blockIdx.x % (unsigned)a.slots_per_head);
+  const TileRef tr = find_tile({a.cu, a.n_seq, a.T, a.cu ? 1 : a.gate_heads}, head, local, &s_n);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tr.nr <= 0) return;
+  const int cp = tid & (DK / 2 - 1), rg = tid / (DK / 2);
+  const int live = tr.nr - rg * kOpRows;
+  const long long e0 = (tr.row0 + rg * kOpRows) * (DK / 2) + cp;
+  const uint32_t* gx = reinterpret_cast<const uint32_t*>(a.gx) + e0;
+  const uint32_t* ty = reinterpret_cast<const uint32_t*>(a.ty) + e0;
+  const uint32_t* q = reinterpret_cast<const uint32_t*>(a.q) + e0;
+  const uint32_t* k = reinterpret_cast<const uint32_t*>(a.k) + e0;
+  uint32_t wx[kOpRows], wy[kOpRows], wq[kOpRows], wk[kOpRows];
+#pragma unroll
+  for (int i = 0; i < kOpRows; ++i) {
+    wx[i] = wy[i] = wq[i] = wk[i] = 0u;       // rows past the end: q = k = 0
+    if (i < live) {
+      wx[i] = __ldg(gx + i * (DK / 2));
+      wy[i] = __ldg(ty + i * (DK / 2));
+      wq[i] = __ldg(q + i * (DK / 2));
+      wk[i] = __ldg(k + i * (DK / 2));
+    }
+  }
+  float2 b[kOpRows], lh2[kOpRows];
+#pragma unroll
+  for (int i = 0; i < kOpRows; ++i) {
+    const float2 x = unpack_bf16(wx[i]), y = unpack_bf16(wy[i]);
+    gate_pair<B::kExact>(x.x, y.x, a.ingate, b[i].x, lh2[i].x);
+    gate_pair<B::kExact>(x.y, y.y, a.ingate, b[i].y, lh2[i].y);
+    if (i >= live) b[i] = make_float2(0.f, 0.f);
+  }
+  auto la_of = [&](int i) {
+    float2 la = make_float2(0.f, 0.f);
+    if (i >= live) return la;
+    const float2 x = unpack_bf16(__ldg(gx + i * (DK / 2))), y = unpack_bf16(__ldg(ty + i * (DK / 2)));
+    float lh;
+    gate_pair<B::kExact>(x.x, y.x, a.ingate, la.x, lh);
+    gate_pair<B::kExact>(x.y, y.y, a.ingate, la.y, lh);
+    return la;
+  };
+  const unsigned long long mask = tile_scan<kOpRows, DK, true>(b, cp, rg, tr.nr, reinterpret_cast<float*>(gbase), s_part,
+                                                               &s_mask, 0ull, la_of);
+  if (mask != 1ull) __syncthreads();          // the scan's scratch becomes operands
+  {
+    const uint32_t w = base + (cp >> 5) * kSlab + ((cp & 3) << 2), c16 = (uint32_t)(cp & 31) >> 2;
+#pragma unroll
+    for (int i = 0; i < kOpRows; ++i) {
+      const int r = rg * kOpRows + i;
+      const uint32_t at = w + r * 128 + ((c16 ^ (uint32_t)(r & 7)) << 4);
+      const float2 qv = unpack_bf16(wq[i]), kv = unpack_bf16(wk[i]);
+      const float ex = ex2f(b[i].x), ey = ex2f(b[i].y);
+      float qx = qv.x * a.scale * ex, qy = qv.y * a.scale * ey;
+#pragma unroll
+      for (int p = 0; p < B::kQp; ++p) {
+        const uint32_t h = pack_bf16(qx, qy);
+        sts32(at + B::kQ + p * B::kSlabs * kSlab, h);
+        const float2 f = unpack_bf16(h);
+        qx -= f.x;
+        qy -= f.y;
+      }
+      float kx = kv.x * ex2f(lh2[i].x - b[i].x), ky = kv.y * ex2f(lh2[i].y - b[i].y);
+#pragma unroll
+      for (int p = 0; p < B::kKp; ++p) {
+        const uint32_t h = pack_bf16(kx, ky);
+        sts32(at + B::kK + p * B::kSlabs * kSlab, h);
+        const float2 f = unpack_bf16(h);
+        kx -= f.x;
+        ky -= f.y;
+      }
+      if (r + 1 == tr.nr) *reinterpret_cast<float2*>(gbase + B::kD + 8 * cp) = make_float2(ex, ey);
+    }
+    if (tid == 0) *reinterpret_cast<unsigned long long*>(gbase + B::kHead) = mask;
+  }
+  __syncthreads();
+  // P = mask(Qt Kt^T): 16 x 16 blocks, those right of the diagonal are zero
+  {
+#pragma unroll 1
+    for (int blk = warp; blk < 16; blk += kOpThreads / 32) {
+      const int wr = blk >> 2, wc = blk & 3;
+      float acc[2][4] = {};
+      if (wc <= wr) {
+        const int ra = 16 * wr + (lane & 15), rb = 16 * wc + (lane & 7) + ((lane >> 4) << 3);
+#pragma unroll
+        for (int kk = 0; kk < DK / 16; ++kk) {
+          const uint32_t ca = (uint32_t)(2 * kk + (lane >> 4)), cb = (uint32_t)(2 * kk + ((lane >> 3) & 1));
+          const uint32_t aa = base + B::kQ + (ca >> 3) * kSlab + ra * 128 + (((ca & 7) ^ (uint32_t)(ra & 7)) << 4);
+          const uint32_t ab = base + B::kK + (cb >> 3) * kSlab + rb * 128 + (((cb & 7) ^ (uint32_t)(rb & 7)) << 4);
+          uint32_t fa[4], fb[4];
+          ldmatrix_x4(aa, fa);
+          ldmatrix_x4(ab, fb);
+          mma_bf16_16816(acc[0], fa, fb[0], fb[1]);
+          mma_bf16_16816(acc[1], fa, fb[2], fb[3]);
+          if (B::kExact) {                    // high x low, low x high
+            uint32_t la[4], lb[4];
+            ldmatrix_x4(aa + kSlab, la);
+            ldmatrix_x4(ab + kSlab, lb);
+            mma_bf16_16816(acc[0], fa, lb[0], lb[1]);
+            mma_bf16_16816(acc[1], fa, lb[2], lb[3]);
+            mma_bf16_16816(acc[0], la, fb[0], fb[1]);
+            mma_bf16_16816(acc[1], la, fb[2], fb[3]);
+          }
+        }
+      }
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int r = 16 * wr + 8 * hf + (lane >> 2);
+        const int lo = mask == 1ull ? 0 : chunk_start(mask, r);
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          const int i = 16 * wc + 8 * nt + 2 * (lane & 3);
+          const float v0 = i <= r && i >= lo ? acc[nt][2 * hf] : 0.f;
+          const float v1 = i + 1 <= r && i + 1 >= lo ? acc[nt][2 * hf + 1] : 0.f;
+          const uint32_t at = base + B::kP + r * 128 + (((uint32_t)(2 * wc + nt) ^ (uint32_t)(r & 7)) << 4) + ((lane & 3) << 2);
+          const uint32_t h = pack_bf16(v0, v1);
+          sts32(at, h);
+          if (B::kExact) {
+            const float2 f = unpack_bf16(h);
+            sts32(at + kSlab, pack_bf16(v0 - f.x, v1 - f.y));
+          }
+        }
+      }
+    }
+  }
+  fence_proxy_async();
+  __syncthreads();
+  if (tid == 0) {
+    bulk_store(a.blocks + ((long long)head * a.slots_per_head + local) * B::kBytes, base, B::kBytes);
+    bulk_commit();
+    bulk_wait_read<0>();
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The scan
+// ---------------------------------------------------------------------------------------------
+// Everything is computed with the value column as the M extent (tensor-memory lane = value column):
+//   dS^T = V^T Kt              [128 value columns x dk]    A = V^T, B = Kt (shared memory)
+//   O^T  = V^T P^T + Sb Qt^T   [128 x 64 rows]             A = V^T / Sb (tensor memory), B = P, Qt
+// The fp32 state lives in the REGISTERS of the state group: per chunk it takes dS of the chunk before
+// out of tensor memory, S <- D . (S + dS), and writes the copy Sb that the readout contracts with.  So
+// no contraction but the readout depends on the state's trip, and dS, O and Sb each have two buffers:
+// the tensor core works on dS and P V of a chunk while the state that enters it is being formed.  (With
+// the state accumulated in tensor memory instead, the chain update -> scaling -> update took 2270
+// cycles per chunk of dk = 64.)
+// Roles: warp 0 loads, 1 issues the contractions, 2 sends the output tiles (and fetches the feed-
+// through's), 3 prepares chunks of cut tiles, 4-11 state group (tensor-memory quarter = warp % 4, half
+// of the key channels each), 12-15 outputs, 16-19 (BLOCK) apply the value gate to the v tile.
+// Two rings: A (Kt, P and the v tile, free once P V is done) and Q (Qt and D).
+template <int DK, bool BLOCK>
+struct Scan {
+  using B = Block<DK>;
+  static constexpr int kABytes = B::kQ, kQBytes = B::kBytes - B::kQ;
+  static constexpr int kAStages = DK == 128 && !BLOCK ? 3 : 2, kQStages = 3;
+  static constexpr int kOffV = kABytes, kOffBeta = kOffV + 2 * kSlab;
+  static constexpr int kAStage = kOffBeta + (BLOCK ? 2 * kSlab : 0);
+  static constexpr int kOffQ = kAStages * kAStage;
+  static constexpr int kOffOt = kOffQ + kQStages * kQBytes;  // two output tiles of two slabs
+  static constexpr int kOffDc = kOffOt + 4 * kSlab;          // float [4][DK]: decays of chunks of cut tiles
+  static constexpr int kOffBar = kOffDc + 4 * DK * 4;
+  static constexpr int kOffCtl = kOffBar + 40 * 8;
+  static constexpr int kSmem = kOffCtl + 512 + 1024;         // + slack for 1024-byte alignment
+  static constexpr int kThreads = BLOCK ? 640 : 512;
+  // dk = 64: the high and middle parts of Kt lie one behind the other in shared memory and are taken as
+  // one operand with N = 128 (64 cycles instead of 2 x 48, and half the instructions); dS is then a pair
+  // of accumulators, added when it is read.  (P and Qt the same way would leave room for one O buffer
+  // only: 2080 cycles per chunk instead of 1740.)
+  static constexpr uint32_t kColS = 0, kDsCols = 128, kColO = 256, kColSb = 384, kSbCols = 64;
+  static_assert(kSmem <= 232448, "shared memory budget");
+};
+
+enum { FB_AFULL0 = 0,                   // [3] Kt, P, v landed                          (1 + bytes)
+       FB_AEMPTY0 = 3,                  // [3] their contractions are done              (1 + warp 3)
+       FB_QFULL0 = 6,                   // [3] Qt, D landed                             (1 + bytes)
+       FB_QEMPTY0 = 9,                  // [3] readout done, D read                     (outputs' warp 12 + 8 warps)
+       FB_VREADY0 = 12,                 // [3] value gate applied                       (4 warps)
+       FB_SREADY0 = 15, FB_SREADY1,     // state entering the chunk is in tensor memory, Qt landed (8 warps)
+       FB_SFULL0, FB_SFULL1,            // dS complete                                  (1)
+       FB_OFULL0, FB_OFULL1,            // outputs complete                             (1)
+       FB_OFREE0, FB_OFREE1,            // outputs read from tensor memory              (4 warps)
+       FB_OTFULL0, FB_OTFULL1,          // output tile written                          (4 warps)
+       FB_OTFREE0, FB_OTFREE1,          // output tile's copies have read it            (1)
+       FB_XFULL0, FB_XFULL1,            // feed-through tile landed in the output tile  (1 + bytes)
+       FB_CUT0,                         // [4] a chunk of a cut tile is prepared        (1)
+       FB_DRAIN = FB_CUT0 + 4, FB_COUNT };
+static_assert(FB_COUNT <= 40, "barrier count");
+
+struct PassDesc {
+  long long row;       // first row of the tile in v, o
+  long long rowq;      // the same in q, k, x, y
+  int lo, hi;          // rows of the chunk within the tile
+  int flags;           // kLastPass, kCutTile
+  int pad;
+};
+constexpr int kLastPass = 1, kCutTile = 2;
+struct ScanCtl {
+  uint32_t tmem_base;
+  int pad;
+  WaitCtl wait;
+  int n_a, n_q, n_x;   // loads issued (for the clean exit)
+  int pad2;
+  PassDesc desc[8];    // pass & 7: the outputs may be a few passes behind the loads
+};
+static_assert(sizeof(ScanCtl) <= 512, "control block");
+
+struct ScanMaps {
+  CUtensorMap v, beta, fx, o, o8, o1;
+};
+
+template <int DK, bool BLOCK>
+__global__ void __launch_bounds__(Scan<DK, BLOCK>::kThreads, 1)
+ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
+  using B = Block<DK>;
+  using C = Scan<DK, BLOCK>;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
+  auto bar = [&](int i) { return base + C::kOffBar + 8u * (uint32_t)i; };
+  volatile ScanCtl* ctl = reinterpret_cast<volatile ScanCtl*>(gbase + C::kOffCtl);
+  volatile WaitCtl* wc = &ctl->wait;
+  WorkspaceHeader* hdr = a.hdr;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q4 = warp & 3;
+
+  // ---- the item
+  const int slice = (int)(blockIdx.x % (unsigned)a.cols);
+  const int sh = (int)(blockIdx.x / (unsigned)a.cols), h = sh % a.H;
+  int n = sh / a.H;
+  const int hq = a.gate_heads == 1 ? 0 : h;
+  long long row0, rowq0;
+  int len;
+  long long slot0;
+  if (a.cu) {
+    n = a.order[n];
+    int lo, hi;
+    seq_range(a.cu, n, a.T, lo, hi);
+    len = hi - lo;
+    row0 = (long long)h * a.T + lo;
+    rowq0 = (long long)hq * a.T + lo;
+    slot0 = (long long)hq * a.slots_per_head + lo / kTile + n;
+  } else {
+    len = a.T;
+    row0 = ((long long)n * a.H + h) * a.T;
+    rowq0 = ((long long)n * a.gate_heads + hq) * a.T;
+    slot0 = ((long long)n * a.gate_heads + hq) * a.slots_per_head;
+  }
+  const int col0 = slice * 128;
+  const int ntiles = (len + kTile - 1) / kTile;
+  const long long state_off = ((long long)n * a.H + h) * DK * (long long)a.dv + col0;
+
+  if (tid == 0) {
+    if (!a.cu && a.T == 0 && blockIdx.x == 0) hdr->status = RODIMUS_OK;   // (no operand kernel then)
+    ctl->wait.abort_flag = 0;
+    ctl->wait.limit = a.limit;
+    ctl->n_a = ctl->n_q = ctl->n_x = 0;
+    for (int i = 0; i < FB_COUNT; ++i) {
+      int cnt = 1;
+      if (i >= FB_QEMPTY0 && i < FB_QEMPTY0 + 3) cnt = 9;
+      if (i >= FB_AEMPTY0 && i < FB_AEMPTY0 + 3) cnt = 2;
+      if (i == FB_SREADY0 || i == FB_SREADY1) cnt = 8;
+      if ((i >= FB_VREADY0 && i < FB_VREADY0 + 3) || i == FB_OFREE0 || i == FB_OFREE1 || i == FB_OTFULL0 || i == FB_OTFULL1)
+        cnt = 4;
+      mbar_init(bar(i), cnt);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(base + C::kOffCtl), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = ctl->tmem_base;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the operand kernel is done, its writes visible
+  auto wait_all = [&](int b, uint32_t parity) -> bool {   // whole warps: tensor-memory accesses need them
+    return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, wc, hdr)) != 0;
+  };
+
+  if (warp == 0) {
+    // ======================================= loads =========================================
+    if (ntiles > 0 && elect_one()) {
+      const unsigned char* blk = a.blocks + slot0 * B::kBytes;
+      auto mask_of = [&](int t) {
+        return __ldcg(reinterpret_cast<const unsigned long long*>(blk + (long long)t * B::kBytes + B::kHead));
+      };
+      unsigned long long next_mask = mask_of(0);
+      uint32_t s = 0, ph = 1, qs = 0, qph = 1;
+      int pass = 0;
+      bool ok = true;
+      for (int t = 0; ok && t < ntiles; ++t) {
+        const unsigned long long mask = next_mask;
+        if (t + 1 < ntiles) next_mask = mask_of(t + 1);
+        const int nr = min(kTile, len - t * kTile);
+        for (int lo = 0; lo < nr; ++pass) {
+          if (!(ok = mbar_wait(bar(FB_AEMPTY0 + s), ph, wc, hdr))) break;
+          const int hi = chunk_end(mask, lo, nr);
+          volatile PassDesc* d = &ctl->desc[pass & 7];
+          const long long row = row0 + (long long)t * kTile;
+          d->row = row;
+          d->rowq = rowq0 + (long long)t * kTile;
+          d->lo = lo;
+          d->hi = hi;
+          d->flags = (t + 1 == ntiles && hi == nr ? kLastPass : 0) | (mask != 1ull ? kCutTile : 0);
+          const uint32_t st = base + s * C::kAStage, fb = bar(FB_AFULL0 + s);
+          const bool beta = BLOCK && a.has_beta;
+          mbar_expect_tx(fb, C::kABytes + 2 * kSlab + (beta ? 2 * kSlab : 0));
+          tma_load_3d(st + C::kOffV, &maps.v, 0, (int)row, col0 >> 6, fb);
+          if (beta) tma_load_3d(st + C::kOffBeta, &maps.beta, 0, (int)row, col0 >> 6, fb);
+          bulk_load(st, blk + (long long)t * B::kBytes, C::kABytes, fb);
+          ctl->n_a = pass + 1;
+          if (lo == 0 && t + C::kAStages < ntiles) {   // asked into L2 before its stage is free
+            tma_prefetch_3d(&maps.v, 0, (int)row + C::kAStages * kTile, col0 >> 6);
+            if (beta) tma_prefetch_3d(&maps.beta, 0, (int)row + C::kAStages * kTile, col0 >> 6);
+          }
+          if (++s == C::kAStages) { s = 0; ph ^= 1; }
+          if (!(ok = mbar_wait(bar(FB_QEMPTY0 + qs), qph, wc, hdr))) break;
+          mbar_expect_tx(bar(FB_QFULL0 + qs), C::kQBytes);
+          bulk_load(base + C::kOffQ + qs * C::kQBytes, blk + (long long)t * B::kBytes + B::kQ, C::kQBytes, bar(FB_QFULL0 + qs));
+          ctl->n_q = pass + 1;
+          if (++qs == C::kQStages) { qs = 0; qph ^= 1; }
+          lo = hi;
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ==================================== contractions =====================================
+    if (ntiles > 0 && elect_one()) {
+      constexpr uint32_t kIs = make_idesc(128, 128, 1, 1);   // dS^T = V^T Kt
+      constexpr uint32_t kIv = make_idesc(128, 64, 1, 0);   // O^T  = V^T P^T
+      constexpr uint32_t kIq = make_idesc(128, 64, 0, 0);   // O^T += Sb Qt^T, A in tensor memory
+      uint32_t s = 0, ph = 0, qs = 0;
+      int n_cut = 0;
+      for (int c = 0;; ++c) {
+        if (!mbar_wait(bar(FB_AFULL0 + s), ph, wc, hdr)) break;
+        if (BLOCK && a.has_beta && !mbar_wait(bar(FB_VREADY0 + s), ph, wc, hdr)) break;
+        const int flags = ctl->desc[c & 7].flags;
+        if (flags & kCutTile) {
+          if (!mbar_wait(bar(FB_CUT0 + (n_cut & 3)), (n_cut >> 2) & 1, wc, hdr)) break;
+          ++n_cut;
+        }
+        const uint32_t st = base + s * C::kAStage, sq = base + C::kOffQ + qs * C::kQBytes;
+        const uint32_t dv = desc_lo_mnmajor(st + C::kOffV, kSlab);
+        tc_fence_after();
+        // dS (buffer c & 1: the state group has taken dS of two chunks before, or the readout of the
+        // chunk before could not have been issued)
+        {
+          const uint32_t d = tmem + C::kColS + (c & 1) * C::kDsCols;
+          const uint32_t dk = desc_lo_mnmajor(st + B::kK, kSlab);       // 128 channels, or high and middle parts
+          umma_bf16_lo<false>(d, dv, dk, kIs);
+#pragma unroll
+          for (int kk = 1; kk < 4; ++kk) umma_bf16_lo<true>(d, dv + 128 * kk, dk + 128 * kk, kIs);
+          if (B::kExact) {
+            const uint32_t dl = desc_lo_mnmajor(st + B::kK + 2 * kSlab, kSlab);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) umma_bf16_lo<true>(d + 64, dv + 128 * kk, dl + 128 * kk, make_idesc(128, 64, 1, 1));
+          }
+        }
+        umma_commit(bar(FB_SFULL0 + (c & 1)));
+        if (!mbar_wait(bar(FB_OFREE0 + (c & 1)), ((c >> 1) & 1) ^ 1, wc, hdr)) break;
+        tc_fence_after();
+        const uint32_t o = tmem + C::kColO + (c & 1) * 64, sb = tmem + C::kColSb + (c & 1) * C::kSbCols;
+#pragma unroll
+        for (int p = 0; p < B::kQp; ++p) {
+          const uint32_t dp = desc_lo_kmajor(st + B::kP + p * kSlab);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            if (p == 0 && kk == 0) umma_bf16_lo<false>(o, dv, dp, kIv);
+            else umma_bf16_lo<true>(o, dv + 128 * kk, dp + 2 * kk, kIv);
+          }
+        }
+        umma_commit(bar(FB_AEMPTY0 + s));
+        if (!mbar_wait(bar(FB_SREADY0 + (c & 1)), (c >> 1) & 1, wc, hdr)) break;
+        tc_fence_after();
+#pragma unroll
+        for (int kk = 0; kk < DK / 16; ++kk)
+          umma_bf16_atmem<true>(o, sb + 8 * kk, desc_lo_kmajor(sq + (kk >> 2) * kSlab) + 2 * (kk & 3), kIq);
+        if (B::kExact) {
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)                     // high part of the state x low part of Qt
+            umma_bf16_atmem<true>(o, sb + 8 * kk, desc_lo_kmajor(sq + kSlab) + 2 * kk, kIq);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)                     // low x high
+            umma_bf16_atmem<true>(o, sb + 32 + 8 * kk, desc_lo_kmajor(sq) + 2 * kk, kIq);
+        }
+        umma_commit(bar(FB_OFULL0 + (c & 1)));
+        if (flags & kLastPass) break;
+        if (++s == C::kAStages) { s = 0; ph ^= 1; }
+        if (++qs == C::kQStages) qs = 0;
+      }
+    }
+    __syncwarp();
+  } else if (warp == 2) {
+    // ================================= output tiles to global ==============================
+    // Feed-through: the x' tile of a pass is fetched INTO its output tile, to be combined with the
+    // accumulators in place.
+    const bool feed = BLOCK && a.feed_d != nullptr;
+    auto fetch_x = [&](int c, long long row) {
+      if (elect_one()) {
+        mbar_expect_tx(bar(FB_XFULL0 + (c & 1)), 2 * kSlab);
+        tma_load_3d(base + C::kOffOt + (c & 1) * 2 * kSlab, &maps.fx, 0, (int)row, col0 >> 6, bar(FB_XFULL0 + (c & 1)));
+        ctl->n_x = c + 1;
+      }
+      __syncwarp();
+    };
+    if (feed && ntiles > 0) fetch_x(0, row0);
+    for (int c = 0; ntiles > 0; ++c) {
+      const uint32_t pr = c & 1;
+      const uint32_t ot = base + C::kOffOt + pr * 2 * kSlab;
+      if (!wait_all(FB_OTFULL0 + pr, (c >> 1) & 1)) break;
+      const volatile PassDesc* d = &ctl->desc[c & 7];
+      const long long row = d->row;
+      const int lo = d->lo, hi = d->hi;
+      const bool last = (d->flags & kLastPass) != 0;
+      if (lo == 0 && hi == kTile) {
+        if (elect_one()) {
+          tma_store_3d(&maps.o, 0, (int)row, col0 >> 6, ot);
+          bulk_commit();
+          bulk_wait_read<0>();
+        }
+      } else {
+        // part of a tile: boxes of 8 rows and of 1 row, so that no other row is touched
+        const int n8 = (hi - lo) >> 3, n1 = (hi - lo) & 7;    // at most 7 + 7 boxes per slab
+        const int slab = lane & 1, v = lane >> 1;
+        const int r = v < n8 ? lo + 8 * v : lo + 8 * n8 + (v - n8);
+        if (v < n8) tma_store_2d(&maps.o8, col0 + 64 * slab, (int)row + r, ot + slab * kSlab + r * 128);
+        else if (v < n8 + n1) tma_store_2d(&maps.o1, col0 + 64 * slab, (int)row + r, ot + slab * kSlab + r * 128);
+        bulk_commit();
+        bulk_wait_read<0>();
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(FB_OTFREE0 + pr));
+      if (last) break;
+      if (feed) fetch_x(c + 1, hi == kTile ? row + kTile : row);
+    }
+  } else if (warp == 3) {
+    // ================================= chunks of cut tiles =================================
+    // rows of other chunks contribute nothing to a chunk's update; the chunk's decays come from the
+    // same additions as its operands'
+    uint32_t s = 0, ph = 0;
+    int n_cut = 0;
+    for (int c = 0; ntiles > 0; ++c) {
+      if (!wait_all(FB_AFULL0 + s, ph)) break;
+      const volatile PassDesc* d = &ctl->desc[c & 7];
+      const int lo = d->lo, hi = d->hi, flags = d->flags;
+      if (flags & kCutTile) {
+        const uint32_t k = base + s * C::kAStage + B::kK;
+        for (int e = lane; e < B::kKp * B::kSlabs * kTile * 8; e += 32) {
+          const int r = (e >> 3) & (kTile - 1);
+          if (r < lo || r >= hi) sts128(k + e * 16, 0u, 0u, 0u, 0u);
+        }
+        fence_proxy_async();
+        // (four buffers: this one's last reader, the state's trip two passes on, precedes the
+        // contractions whose end let the tile of this pass in)
+        float* dc = reinterpret_cast<float*>(gbase + C::kOffDc) + (n_cut & 3) * DK;
+        for (int ch = lane; ch < DK; ch += 32) {
+          const long long e = d->rowq * DK + ch;
+          float acc = 0.f, lh, la;
+          for (int r = lo; r < hi; ++r) {
+            gate_pair<B::kExact>(__bfloat162float(a.gx[e + r * DK]), __bfloat162float(a.ty[e + r * DK]), a.ingate, la, lh);
+            acc += la;
+          }
+          dc[ch] = ex2f(acc);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(FB_CUT0 + (n_cut & 3)));
+        ++n_cut;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(FB_AEMPTY0 + s));
+      if (flags & kLastPass) break;
+      if (++s == C::kAStages) { s = 0; ph ^= 1; }
+    }
+  } else if (warp >= 4 && warp < 12) {
+    // ======================================= state =========================================
+    constexpr int kHalf = DK / 2;
+    const int ch0 = ((warp - 4) >> 2) * kHalf;
+    const uint32_t t_lane = tmem + ((uint32_t)(q4 * 32) << 16);
+    // element (channel d, own value column) of the state: off + d * dv
+    const long long off = state_off + q4 * 32 + lane + (long long)ch0 * a.dv;
+    float2 S[kHalf / 2];
+#pragma unroll
+    for (int e = 0; e < kHalf / 2; ++e) {
+      S[e] = make_float2(0.f, 0.f);
+      if (a.s0) S[e] = make_float2(__ldg(a.s0 + off + (long long)(2 * e) * a.dv), __ldg(a.s0 + off + (long long)(2 * e + 1) * a.dv));
+    }
+    uint32_t qs = 0, qph = 0;
+    int n_cut = 0;
+    bool ok = true;
+    // S <- D . (S + dS) with dS and D of pass c
+    auto advance = [&](int c, const float* D) {
+      constexpr int kLd = BLOCK ? 16 : 32;              // (fewer registers a thread with 20 warps)
+#pragma unroll
+      for (int piece = 0; piece < kHalf / kLd; ++piece) {
+        uint32_t r[kLd];
+        const uint32_t ds = t_lane + C::kColS + (c & 1) * C::kDsCols + ch0 + kLd * piece;
+        if constexpr (kLd == 16) tmem_ld16(ds, r);
+        else tmem_ld32(ds, r);
+        if constexpr (B::kExact) {
+          uint32_t r2[32];
+          tmem_ld32(ds + 64, r2);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(r2[e]));
+        } else {
+          tmem_ld_wait();
+        }
+#pragma unroll
+        for (int e = 0; e < kLd / 4; ++e) {
+          const float4 d = *reinterpret_cast<const float4*>(D + ch0 + kLd * piece + 4 * e);   // broadcast
+          float2* x = S + kLd / 2 * piece + 2 * e;
+          x[0] = __fmul2_rn(__fadd2_rn(x[0], make_float2(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]))), make_float2(d.x, d.y));
+          x[1] = __fmul2_rn(__fadd2_rn(x[1], make_float2(__uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3]))), make_float2(d.z, d.w));
+        }
+      }
+    };
+    if (ntiles > 0) {
+      for (int c = 0;; ++c) {
+        // the state entering pass c, as bf16 parts (the readout of pass c - 2, the buffer's last reader,
+        // precedes dS of pass c - 1 in the tensor pipe)
+        const uint32_t t_sb = t_lane + C::kColSb + (c & 1) * C::kSbCols + ch0 / 2;
+#pragma unroll
+        for (int piece = 0; piece < kHalf / 32; ++piece) {
+          uint32_t w[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) w[e] = pack_bf16(S[16 * piece + e].x, S[16 * piece + e].y);
+          tmem_st16(t_sb + 16 * piece, w);
+          if (B::kExact) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              const float2 f = unpack_bf16(w[e]);
+              w[e] = pack_bf16(S[16 * piece + e].x - f.x, S[16 * piece + e].y - f.y);
+            }
+            tmem_st16(t_sb + DK / 2 + 16 * piece, w);
+          }
+        }
+        if (!(ok = wait_all(FB_QFULL0 + qs, qph))) break;   // (for the readout as well)
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(FB_SREADY0 + (c & 1)));
+        const int flags = ctl->desc[c & 7].flags;
+        const float* D = reinterpret_cast<const float*>(gbase + C::kOffQ + qs * C::kQBytes + (B::kD - B::kQ));
+        if (flags & kCutTile) {
+          if (!(ok = wait_all(FB_CUT0 + (n_cut & 3), (n_cut >> 2) & 1))) break;
+          D = reinterpret_cast<const float*>(gbase + C::kOffDc) + (n_cut & 3) * DK;
+          ++n_cut;
+        }
+        if ((flags & kLastPass) && !a.sT) break;
+        if (!(ok = wait_all(FB_SFULL0 + (c & 1), (c >> 1) & 1))) break;
+        tc_fence_after();
+        advance(c, D);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(FB_QEMPTY0 + qs));
+        if (flags & kLastPass) break;
+        if (++qs == C::kQStages) { qs = 0; qph ^= 1; }
+      }
+    }
+    if (ok && a.sT) {
+#pragma unroll
+      for (int e = 0; e < kHalf / 2; ++e) {
+        a.sT[off + (long long)(2 * e) * a.dv] = S[e].x;
+        a.sT[off + (long long)(2 * e + 1) * a.dv] = S[e].y;
+      }
+    }
+  } else if (warp >= 12 && warp < 16) {
+    // ====================================== outputs ========================================
+    // O^T has the value columns in the tensor-memory lanes.  The 16x256b load hands out 8x8 fragments
+    // [value column][row]; stmatrix.trans writes them transposed into a tile of two swizzled 64-column
+    // slabs, which leaves through a tensor copy.  Two tiles alternate.
+    const int mat_k = lane & 7, mat_h = (lane >> 3) & 1, mat_j = lane >> 4;
+    const uint32_t t_lane = tmem + ((uint32_t)(q4 * 32) << 16);
+    const bool feed = BLOCK && a.feed_d != nullptr;
+    uint32_t qs = 0;
+    for (int c = 0; ntiles > 0; ++c) {
+      const uint32_t pr = c & 1, ph = (c >> 1) & 1;
+      if (!wait_all(FB_OFULL0 + pr, ph)) break;
+      if (warp == 12 && lane == 0) mbar_arrive(bar(FB_QEMPTY0 + qs));
+      if (++qs == C::kQStages) qs = 0;
+      tc_fence_after();
+      const bool last = (ctl->desc[c & 7].flags & kLastPass) != 0;
+      if (feed) {   // (asked for once the tile was free)
+        if (!wait_all(FB_XFULL0 + pr, ph)) break;
+      } else {
+        if (!wait_all(FB_OTFREE0 + pr, ph ^ 1)) break;
+      }
+      // this thread addresses output row 8 * (2 jp + mat_j) + mat_k of column block mat_h
+      const uint32_t ot_mat = base + C::kOffOt + pr * 2 * kSlab + (q4 >> 1) * kSlab + (mat_j * 8 + mat_k) * 128;
+#pragma unroll 1
+      for (int hv = 0; hv < 2; ++hv) {                  // lanes 0..15 / 16..31 of the quarter
+        uint32_t r[32];
+        tmem_ld_16x256b_x8(t_lane + ((uint32_t)(16 * hv) << 16) + C::kColO + pr * 64, r);
+        tmem_ld_wait();
+        if (hv == 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(FB_OFREE0 + pr));
+        }
+        const uint32_t chunk = (uint32_t)(4 * (q4 & 1) + 2 * hv + mat_h);
+        const uint32_t dst = ot_mat + ((chunk ^ (uint32_t)mat_k) << 4);
+        if (feed) {
+          const float* dh = a.feed_d + h * (long long)a.dv + col0 + q4 * 32 + 16 * hv + (lane >> 2);
+          const float d_lo = __ldg(dh), d_hi = __ldg(dh + 8);
+#pragma unroll
+          for (int jp = 0; jp < 4; ++jp) {
+            uint32_t xf[4];
+            ldmatrix_x4_trans(dst + jp * 16 * 128, xf);
+#pragma unroll
+            for (int mi = 0; mi < 4; ++mi) {            // (lo, j0) (hi, j0) (lo, j1) (hi, j1)
+              const int ri = 4 * (2 * jp + (mi >> 1)) + 2 * (mi & 1);
+              const float dd = (mi & 1) ? d_hi : d_lo;
+              const float2 xv = unpack_bf16(xf[mi]);
+              r[ri] = __float_as_uint(fmaf(dd, xv.x, __uint_as_float(r[ri])));
+              r[ri + 1] = __float_as_uint(fmaf(dd, xv.y, __uint_as_float(r[ri + 1])));
+            }
+          }
+        }
+#pragma unroll
+        for (int jp = 0; jp < 4; ++jp) {                // output rows 16 jp .. 16 jp + 15
+          const int j0 = 2 * jp, j1 = 2 * jp + 1;
+          stmatrix_x4_trans(dst + jp * 16 * 128,
+                            pack_bf16(__uint_as_float(r[4 * j0]), __uint_as_float(r[4 * j0 + 1])),
+                            pack_bf16(__uint_as_float(r[4 * j0 + 2]), __uint_as_float(r[4 * j0 + 3])),
+                            pack_bf16(__uint_as_float(r[4 * j1]), __uint_as_float(r[4 * j1 + 1])),
+                            pack_bf16(__uint_as_float(r[4 * j1 + 2]), __uint_as_float(r[4 * j1 + 3])));
+        }
+      }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(FB_OTFULL0 + pr));
+      if (last) break;
+    }
+  } else if (BLOCK && warp >= 16) {
+    // ===================================== value gate ======================================
+    // v becomes beta_hat . v in place (the exact product of two bf16 rounded once)
+    uint32_t s = 0, ph = 0;
+    for (int c = 0; a.has_beta && ntiles > 0; ++c) {
+      if (!wait_all(FB_AFULL0 + s, ph)) break;
+      const bool last = (ctl->desc[c & 7].flags & kLastPass) != 0;
+      const uint32_t st = base + s * C::kAStage + C::kOffV + (tid - 512) * 16;
+#pragma unroll 4
+      for (int u = 0; u < 2 * kSlab / (128 * 16); ++u) {
+        const uint32_t at = st + u * 128 * 16;
+        const uint4 v = lds128(at), g = lds128(at + (C::kOffBeta - C::kOffV));
+        sts128(at, hmul2_bf16(v.x, g.x), hmul2_bf16(v.y, g.y), hmul2_bf16(v.z, g.z), hmul2_bf16(v.w, g.w));
+      }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(FB_VREADY0 + s));
+      if (last) break;
+      if (++s == C::kAStages) { s = 0; ph ^= 1; }
+    }
+  }
+
+  // ------------------------------------------ teardown ------------------------------------------
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (ctl->wait.abort_flag) {   // nothing may still be writing this CTA's shared or tensor memory
+    if (tid == 0) {
+      for (int back = 1; back <= C::kAStages && back <= ctl->n_a; ++back) {
+        const int f = ctl->n_a - back;
+        mbar_drain(bar(FB_AFULL0 + f % C::kAStages), (f / C::kAStages) & 1);
+      }
+      for (int back = 1; back <= C::kQStages && back <= ctl->n_q; ++back) {
+        const int f = ctl->n_q - back;
+        mbar_drain(bar(FB_QFULL0 + f % C::kQStages), (f / C::kQStages) & 1);
+      }
+      for (int back = 1; back <= 2 && back <= ctl->n_x; ++back) {
+        const int f = ctl->n_x - back;
+        mbar_drain(bar(FB_XFULL0 + (f & 1)), (f >> 1) & 1);
+      }
+    }
+    if (warp == 1 && elect_one()) {   // a commit follows the contractions of the thread that makes it
+      umma_commit(bar(FB_DRAIN));
+      mbar_drain(bar(FB_DRAIN), 0);
+    }
+  }
+  __syncthreads();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+}
+
+template <int DK>
+size_t blocks_bytes(long long slots) { return (size_t)slots * Block<DK>::kBytes; }
+
+struct ScanPlan {
+  long long slots;        // tiles, over all sets of gates
+  int slots_per_head, gate_heads;
+  size_t blocks, bytes;   // workspace: offset of the blocks, total
+};
+
+ScanPlan scan_plan(const rodimus_ddts_fwd_params& p) {
+  ScanPlan s;
+  const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
+  s.gate_heads = p.shared_gates ? 1 : p.H;
+  s.slots_per_head = varlen ? p.T / kTile + p.N : (p.T + kTile - 1) / kTile;
+  s.slots = (long long)s.slots_per_head * s.gate_heads * (varlen ? 1 : p.B);
+  size_t order = (size_t)(varlen ? p.N : 0) * sizeof(int32_t);
+  s.blocks = sizeof(WorkspaceHeader) + ((order + 1023) & ~(size_t)1023);
+  s.bytes = s.blocks + (p.dk == 64 ? blocks_bytes<64>(s.slots) : blocks_bytes<128>(s.slots));
+  return s;
+}
+
+template <int DK, bool BLOCK>
+cudaError_t launch_scan(const ScanMaps& m, const ScanArgs& a, long long slots, long long items, int dev, cudaStream_t st) {
+  static std::atomic<unsigned long long> opted_ops{0}, opted{0};   // per instantiation
+  using C = Scan<DK, BLOCK>;
+  cudaError_t e = opt_in_shared_memory(ddts_operands_kernel<DK>, kOpSmem<DK>, dev, opted_ops);
+  if (e == cudaSuccess) e = opt_in_shared_memory(ddts_scan_kernel<DK, BLOCK>, Scan<DK, BLOCK>::kSmem, dev, opted);
+  if (e != cudaSuccess) return e;
+  if (slots > 0) ddts_operands_kernel<DK><<<(unsigned)slots, kOpThreads, kOpSmem<DK>, st>>>(a);
+  // The scan may start while the operand kernel's last CTAs run: it sets up (barriers, tensor memory)
+  // and waits for that kernel before it reads a block.
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)items);
+  cfg.blockDim = dim3(C::kThreads);
+  cfg.dynamicSmemBytes = C::kSmem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = slots > 0 ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, ddts_scan_kernel<DK, BLOCK>, m, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+// Which requests this file's kernels compute, given room for the tiles' blocks; bytes of that room
+// (0: not this path).  All timings are one call, the other kernel against this path.
+//   dk = 64            always (B=4 H=16 T=2048, one set of gates: fp32 CUDA-core kernel 3.9 ms, here
+//                      47 us); not with block terms, whose products the fp32 kernel does not round.
+//   one set of gates   always where the pair kernel would be the other choice (same precision; layer
+//                      shape 82 -> 40 us).
+//   gates per head     the gates cost the same in both, here their operands travel through memory, and
+//                      here they are formed by all SMs however few the heads are:
+//       dv % 256 == 0  against the pair kernel, when a dense call has at most a quarter as many items of
+//                      256 columns as there are SMs (16 items x 2048 rows 77 -> 47 us, 32 items 79 ->
+//                      67, 37 x 1024 45 -> 39, but 48 x 1024 47 -> 47 and 64 x 2048 82 -> 101), a packed
+//                      one, whose longest sequence keeps the other pairs waiting, half as many (64 items
+//                      of 100..1500 rows 59 -> 47 us); sequences of four tiles or more on average.
+//       odd multiples  against the single-CTA kernel: dense calls (B=4 H=16 T=2048 dv=128 146 -> 96 us,
+//       of 128         1 x 16 x 1000 76 -> 27) and packed ones with no more items than SMs (640 items
+//                      307 -> 329 us).
+size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
+  if (p.dtype != RODIMUS_BF16 || p.value_decay || p.dv % 128 || (p.dk != 64 && p.dk != 128)) return 0;
+  const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
+  const bool block = p.beta_hat || p.feed_d, whole = p.dv % 256 == 0;
+  const long long n_seq = varlen ? p.N : p.B, items = n_seq * p.H * (p.dv / 128);
+  if (p.dk == 64) {
+    if (block) return 0;
+  } else if (p.shared_gates) {
+    if (!whole) return 0;
+  } else {
+    int dev = 0, sms = 0;
+    if (current_device(&dev, &sms) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    if (n_seq == 0 || p.T / (varlen ? n_seq : 1) < 4 * kTile) return 0;
+    if (whole ? items > (varlen ? sms : sms / 2) : (block || (varlen && items > sms))) return 0;
+  }
+  const ScanPlan s = scan_plan(p);
+  if (s.slots > 0x7fffffffLL || items > 0x7fffffffLL) return 0;
+  return s.bytes;
+}
+
+cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
+  *n_launches = 0;
+  const ScanPlan s = scan_plan(p);
+  const long long n_seq = p.cu_seqlens ? p.N : p.B, items = n_seq * p.H * (p.dv / 128);
+  if (items == 0) return cudaSuccess;
+  char* ws = reinterpret_cast<char*>(p.workspace);
+  ScanArgs a;
+  a.q = (const __nv_bfloat16*)p.q; a.k = (const __nv_bfloat16*)p.k;
+  a.gx = (const __nv_bfloat16*)p.gate_x; a.ty = (const __nv_bfloat16*)p.temp_y;
+  a.s0 = p.s0; a.sT = p.sT; a.feed_d = p.feed_d;
+  a.blocks = reinterpret_cast<unsigned char*>(ws + s.blocks);
+  a.cu = p.cu_seqlens;
+  a.order = reinterpret_cast<const int32_t*>(ws + sizeof(WorkspaceHeader));
+  a.hdr = reinterpret_cast<WorkspaceHeader*>(ws);
+  a.H = p.H; a.T = p.T; a.dv = p.dv; a.n_seq = (int)n_seq;
+  a.gate_heads = s.gate_heads;
+  a.slots_per_head = s.slots_per_head;
+  a.cols = p.dv / 128;
+  a.has_beta = p.beta_hat != nullptr;
+  a.scale = p.scale; a.ingate = p.ingate;
+  a.limit = main_loop_wait_cycles();
+  int dev = 0, sms = 0;
+  cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
+  ScanMaps m;
+  const uint64_t rows = (uint64_t)p.B * p.H * p.T, dv = (uint64_t)p.dv;
+  if (rows > 0) {
+    if (!encode_bf16_slab_map(&m.v, p.v, rows, dv, 2) || !encode_bf16_slab_map(&m.o, p.o, rows, dv, 2) ||
+        !encode_bf16_map(&m.o8, p.o, rows, dv, 8) || !encode_bf16_map(&m.o1, p.o, rows, dv, 1))
+      return cudaErrorInvalidValue;
+    m.beta = m.fx = m.v;
+    if (p.beta_hat && !encode_bf16_slab_map(&m.beta, p.beta_hat, rows, dv, 2)) return cudaErrorInvalidValue;
+    if (p.feed_x && !encode_bf16_slab_map(&m.fx, p.feed_x, rows, dv, 2)) return cudaErrorInvalidValue;
+  } else {
+    memset(&m, 0, sizeof(m));   // never used: no tiles
+  }
+  const long long slots = rows > 0 ? s.slots : 0;
+  if (p.dk == 64) e = launch_scan<64, false>(m, a, slots, items, dev, st);
+  else if (p.beta_hat || p.feed_d) e = launch_scan<128, true>(m, a, slots, items, dev, st);
+  else e = launch_scan<128, false>(m, a, slots, items, dev, st);
+  *n_launches = slots > 0 ? 2 : 1;
+  return e;
+}
+
+}  // namespace ddts

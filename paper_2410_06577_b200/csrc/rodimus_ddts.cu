@@ -69,9 +69,18 @@ bool fwd_pair_selected(const rodimus_ddts_fwd_params& p) { return fwd_pair_suppo
 
 bool has_block_terms(const rodimus_ddts_fwd_params& p) { return p.beta_hat || p.feed_d; }
 
+// Workspace of the two-launch prefill where it is to be used; dense calls that the pair kernel splits
+// along time stay there (their few heads fill the device only that way).
+size_t scan_path_bytes(const rodimus_ddts_fwd_params& p) {
+  if (fwd_pair_selected(p) && fwd_pair_split_workspace_bytes(p) > 0) return 0;
+  return fwd_scan_workspace_bytes(p);
+}
+
 // 0: cluster-pair tensor-core kernel, 1: single-CTA tensor-core kernel (the recurrence alone),
-// 2: fp32 CUDA-core kernel
+// 2: fp32 CUDA-core kernel, 3: operands and scan in two launches (if the workspace has room for it)
 int fwd_kernel_choice(const rodimus_ddts_fwd_params& p) {
+  const size_t scan = scan_path_bytes(p);
+  if (scan > 0 && p.workspace_bytes >= scan) return 3;
   if (fwd_pair_selected(p)) return 0;
   if (fwd_tc_supported(p) && !has_block_terms(p) && !p.shared_gates && !p.value_decay) return 1;
   return 2;
@@ -89,13 +98,14 @@ size_t rodimus_ddts_fwd_workspace_bytes(const rodimus_ddts_fwd_params* p) {
   // long dense sequences with few heads run faster split along time, given room for the
   // segments' states; a caller that passes only the base size still gets the unsplit path
   const size_t split = ddts::fwd_pair_selected(*p) ? ddts::fwd_pair_split_workspace_bytes(*p) : 0;
-  return split > base ? split : base;
+  const size_t more = split > 0 ? split : ddts::scan_path_bytes(*p);
+  return more > base ? more : base;
 }
 
 const char* rodimus_ddts_fwd_kernel_name(const rodimus_ddts_fwd_params* p) {
   if (!p) return "invalid";
   if (check_fwd_sizes(p, p->cu_seqlens != nullptr) != RODIMUS_OK) return "invalid";
-  return ddts::fwd_kernel_choice(*p) < 2 ? "tcgen05" : "simt";
+  return ddts::fwd_kernel_choice(*p) != 2 ? "tcgen05" : "simt";
 }
 
 int rodimus_ddts_fwd(const rodimus_ddts_fwd_params* p) {
@@ -138,6 +148,8 @@ int rodimus_ddts_fwd(const rodimus_ddts_fwd_params* p) {
     e = ddts::launch_fwd_pair(*p, &n);
   else if (choice == 1)
     e = ddts::launch_fwd_tc(*p, &n);
+  else if (choice == 3)
+    e = ddts::launch_fwd_scan(*p, &n);
   else
     e = ddts::launch_fwd_simt(*p, &n);
   launches += n;

@@ -829,3 +829,71 @@ def test_shared_gates_decode_steps():
         ro = orc.ref_step(wq.q[s], wq.k[s], wq.x[s], wq.y[s], wv.v[s], ref_state, shared_gates=True)
         assert o.shape == (Nseq, H, dv) and rel_err(host(o), ro) <= TOL_BF16
     assert rel_err(host(state), ref_state) <= TOL_F32
+
+
+# ------------------------------------------------------------------------------------------
+# operands and scan in two launches
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("dk,H,shared,dv", [(64, 3, True, 256), (64, 2, False, 384), (128, 3, True, 256)])
+@pytest.mark.parametrize("lens", [[1], [63], [64], [65], [200], [5, 0, 64, 130, 1, 77]])
+@pytest.mark.parametrize("strong", [False, True])
+def test_two_launch_prefill_tile_edges_and_cut_tiles(dk, H, shared, dv, lens, strong):
+    """Edges of the 64-row tiles, packed sequences with an empty one, and tiles that strong decays (steps
+    of e^-60 and more in some channels) cut into several chunks.  dk = 64 carries its state at fp32
+    accuracy: bar 1e-4 on the final state, whatever the token dtype."""
+    import torch
+    T, Hq = sum(lens), 1 if shared else H
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32) if len(lens) > 1 else None
+    pq = wl.make_prefill(900 + T, 1, Hq, T, dk, dv, "bf16")
+    pv = wl.make_prefill(901 + T, 1, H, T, dk, dv, "bf16", s0_std=0.2, cu_seqlens=cu)
+    if strong:
+        pq.x[:, :, T // 3:T // 3 + 7, ::5] = 80.0
+        pq.y[:, :, T // 3:T // 3 + 7, ::5] = 4.0
+    q, k, x, y, v = (dev(a, "bf16") for a in (pq.q, pq.k, pq.x, pq.y, pv.v))
+    s0 = torch.from_numpy(pv.s0).cuda()
+    cu_d = None if cu is None else torch.from_numpy(cu).cuda()
+    o = torch.full((1, H, T, dv), float("nan"), dtype=q.dtype, device="cuda")
+    sT = torch.full((len(lens), H, dk, dv), float("nan"), dtype=torch.float32, device="cuda")
+    prm = rd.fwd_params(q, k, x, y, v, o, s0, sT, cu_d, None, None, 0.5)
+    ws = rd.new_workspace(prm, "cuda")
+    prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
+    assert rd.fwd_kernel_name(prm) == "tcgen05"
+    assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
+    assert rd.last_launch_count() == (2 if cu is None else 3)
+    ro, rs = orc.ref_fwd(pq.q, pq.k, pq.x, pq.y, pv.v, s0=pv.s0, cu_seqlens=cu, scale=0.5, shared_gates=shared)
+    eo, es = _worst_err(host(o), host(sT), ro, rs, cu)
+    assert eo <= TOL_BF16 and es <= (TOL_F32 if dk == 64 else TOL_BF16), (eo, es)
+
+
+def test_two_launch_prefill_wait_that_runs_out_is_reported():
+    import torch
+    pq, pv = _shared_inputs(950, 1, 4, 300, 64, 256, "bf16")
+    q, k, x, y, v = (dev(a, "bf16") for a in (pq.q, pq.k, pq.x, pq.y, pv.v))
+    o = torch.empty((1, 4, 300, 256), dtype=q.dtype, device="cuda")
+    prm = rd.fwd_params(q, k, x, y, v, o)
+    ws = rd.new_workspace(prm, "cuda")
+    prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
+    rd.test_set_wait_limit(0)
+    try:
+        assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.ERR_TIMEOUT
+    finally:
+        rd.test_set_wait_limit(-1)
+    assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
+    ro, _ = orc.ref_fwd(pq.q, pq.k, pq.x, pq.y, pv.v, shared_gates=True)
+    assert rel_err(host(o), ro) <= TOL_BF16
+
+
+@pytest.mark.parametrize("block,dv", [("none", 256), ("both", 256), ("gate", 512), ("feed", 256), ("none", 128), ("none", 384)])
+@pytest.mark.parametrize("lens", [[256], [300, 511, 257]])
+def test_two_launch_prefill_gates_per_head(block, dv, lens):
+    """The rule that sends few heads with their own gates here starts at four tiles per sequence."""
+    T = sum(lens)
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32) if len(lens) > 1 else None
+    p = wl.make_prefill(960 + T, 1, 2, T, 128, dv, "bf16", s0_std=0.2, cu_seqlens=cu)
+    if block != "none":
+        assert _check_block(p, block) == (2 if cu is None else 3)
+        return
+    assert rd.fwd_workspace_bytes(rd.fwd_params(*(dev(a, "bf16") for a in (p.q, p.k, p.x, p.y, p.v)), None,
+                                                cu_seqlens=prefill_to_device(p)["cu"])) > 4096
+    _check_prefill(p, rd.INGATE_POW_SIGMOID, 0.5)
