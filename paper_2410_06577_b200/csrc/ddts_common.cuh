@@ -34,6 +34,26 @@ inline cudaError_t opt_in_shared_memory(Kernel kernel, int bytes, int dev, std::
   return e;
 }
 
+// Launch of a kernel that may start while the one before it on the stream still runs: it sets up, then
+// calls wait_for_previous_kernel() before it touches what that one wrote.  The one before says with
+// let_next_kernel_start() from when on that is allowed (once every CTA of it has said so or ended).
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, int threads, int smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Limit, in clock cycles, that the tensor-core prefill kernels give each of their main-loop
 // waits (see rodimus_ddts_test_set_wait_limit).
 long long main_loop_wait_cycles();
@@ -42,6 +62,7 @@ long long main_loop_wait_cycles();
 cudaError_t launch_step(const rodimus_ddts_step_params& p, int* n_launches);
 cudaError_t launch_plan(const rodimus_ddts_fwd_params& p, int* n_launches);
 cudaError_t launch_fwd_simt(const rodimus_ddts_fwd_params& p, int* n_launches);
+size_t fwd_simt_chunks_workspace_bytes(const rodimus_ddts_fwd_params& p);   // 0: not the parallel form
 cudaError_t launch_fwd_tc(const rodimus_ddts_fwd_params& p, int* n_launches);
 cudaError_t launch_fwd_pair(const rodimus_ddts_fwd_params& p, int* n_launches);
 cudaError_t launch_bwd(const rodimus_ddts_bwd_params& p, size_t scratch_offset, int* n_launches);

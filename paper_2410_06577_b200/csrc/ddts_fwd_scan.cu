@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
   if (!a.cu && blockIdx.x == 0 && tid == 0) a.hdr->status = RODIMUS_OK;
   const int head = (int)(blockIdx.x / (unsigned)a.slots_per_head), local = (int)(blockIdx.x % (unsigned)a.slots_per_head);
   const TileRef tr = find_tile({a.cu, a.n_seq, a.T, a.cu ? 1 : a.gate_heads}, head, local, &s_n);
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_kernel_start();
   if (tr.nr <= 0) return;
   const int cp = tid & (DK / 2 - 1), rg = tid / (DK / 2);
   const int live = tr.nr - rg * kOpRows;
@@ -382,7 +382,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // the operand kernel is done, its writes visible
+  wait_for_previous_kernel();   // the operands are there
   auto wait_all = [&](int b, uint32_t parity) -> bool {   // whole warps: tensor-memory accesses need them
     return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, wc, hdr)) != 0;
   };
@@ -824,17 +824,7 @@ cudaError_t launch_scan(const ScanMaps& m, const ScanArgs& a, long long slots, l
   if (slots > 0) ddts_operands_kernel<DK><<<(unsigned)slots, kOpThreads, kOpSmem<DK>, st>>>(a);
   // The scan may start while the operand kernel's last CTAs run: it sets up (barriers, tensor memory)
   // and waits for that kernel before it reads a block.
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)items);
-  cfg.blockDim = dim3(C::kThreads);
-  cfg.dynamicSmemBytes = C::kSmem;
-  cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = slots > 0 ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, ddts_scan_kernel<DK, BLOCK>, m, a);
+  e = launch_overlapped(ddts_scan_kernel<DK, BLOCK>, (unsigned)items, C::kThreads, C::kSmem, st, m, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

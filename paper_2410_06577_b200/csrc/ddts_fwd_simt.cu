@@ -15,8 +15,11 @@
 //   O_r   = sum_{i<=r} P_ri (v_i . exp(c_r - c_i)) + exp(c_r) . ((q_r . exp(b_r)) S_in)
 //   S_out = (exp(b_C)^T exp(c_C)) . S_in + sum_i (k_i . ahat_i . exp(b_C - b_i))^T (v_i . exp(c_C - c_i))
 //
-// Work item = (sequence, head, tile of kTileV state columns); one CTA per item keeps its
-// [dk, kTileV] slice of the state in shared memory for the whole sequence.
+// Two forms.  Where the states of all 16-row chunks stay in L2, the chunks are computed side by side:
+// per chunk the operands, the scores and its own contribution to the state; an elementwise pass that
+// turns contributions into the states entering the chunks, S <- D . S + dS; per chunk the outputs.
+// Elsewhere (and where the caller's workspace has no room, and with the value-side decay) one CTA per
+// (sequence, head, kTileV state columns) walks the sequence with its slice of the state in shared memory.
 #include "ddts_common.cuh"
 
 namespace ddts {
@@ -208,7 +211,295 @@ size_t simt_smem_bytes(int dk) {
   return sizeof(float) * ((size_t)dk * kTileV + 3 * (size_t)kC * ld + 2 * kC * kTileV + kC * kC + dk);
 }
 
+// ---------------------------------------------------------------------------------------------
+// Chunks side by side
+// ---------------------------------------------------------------------------------------------
+struct ChunkArgs {
+  SimtArgs s;
+  float *states;          // [chunk slots of all heads][dk][dv]: dS of the chunk, then the state entering it
+  float *qe, *scores, *decay;   // [slots][kC][dk], [slots][kC][kC], [slots][dk]
+  int slots_per_head, heads;    // dense: (batch, head) pairs; packed: heads
+  long long slots;
+};
+
+// A sequence's chunks have consecutive slots: packed sequence n of a head starts at floor(start / 16) + n.
+struct ChunkRef {
+  int n, h, t, nr, len;         // sequence, head, chunk of the sequence, live rows (0: no such chunk)
+  long long row0, slot0;        // first row and first slot of the sequence
+};
+__device__ __forceinline__ void sequence_of(const ChunkArgs& a, int n, int h, ChunkRef& r) {
+  r.n = n;
+  r.h = h;
+  if (a.s.cu) {
+    int lo = a.s.cu[n], hi = a.s.cu[n + 1];
+    lo = lo < 0 ? 0 : (lo > a.s.T ? a.s.T : lo);
+    hi = hi < lo ? lo : (hi > a.s.T ? a.s.T : hi);
+    r.len = hi - lo;
+    r.row0 = (long long)h * a.s.T + lo;
+    r.slot0 = (long long)h * a.slots_per_head + lo / kC + n;
+  } else {
+    r.len = a.s.T;
+    r.row0 = ((long long)n * a.s.H + h) * a.s.T;
+    r.slot0 = ((long long)n * a.s.H + h) * a.slots_per_head;
+  }
+}
+// Block-wide.
+__device__ __forceinline__ ChunkRef chunk_of(const ChunkArgs& a, long long slot, int* s_n) {
+  ChunkRef r;
+  const int head = (int)(slot / a.slots_per_head), local = (int)(slot % a.slots_per_head);
+  if (!a.s.cu) {
+    sequence_of(a, head / a.s.H, head % a.s.H, r);
+  } else {
+    if (threadIdx.x == 0) *s_n = -1;
+    __syncthreads();
+    int best = -1;   // the last sequence whose first slot is not beyond this one
+    for (int n = threadIdx.x; n < a.s.n_seq; n += blockDim.x) {
+      ChunkRef c;
+      sequence_of(a, n, 0, c);
+      if (c.slot0 <= local) best = n;
+    }
+    if (best >= 0) atomicMax(s_n, best);
+    __syncthreads();
+    r.nr = 0;
+    if (*s_n < 0) return r;
+    sequence_of(a, *s_n, head, r);
+  }
+  r.t = (int)(slot - r.slot0);
+  r.nr = min(kC, r.len - r.t * kC);
+  return r;
+}
+
+// Operands, scores and state contribution of one chunk.  Bound by the latency of its phases.
+constexpr int kOpsThreads = 1024;
+template <typename T>
+__global__ void __launch_bounds__(kOpsThreads, 1) ddts_chunk_ops_kernel(const ChunkArgs a) {
+  extern __shared__ float smem[];
+  __shared__ int s_n;
+  const int dk = a.s.dk, dv = a.s.dv, ld = dk + 1, tid = threadIdx.x;
+  float* sQ = smem;                 // [kC][ld] q
+  float* sW = sQ + kC * ld;         // [kC][ld] ahat k
+  float* sB = sW + kC * ld;         // [kC][ld] log decay, then cumulative
+  float* sV = sB + kC * ld;         // [kC][kTileV]
+  if (!a.s.cu && blockIdx.x == 0 && tid == 0) a.s.hdr->status = RODIMUS_OK;
+  const long long slot = blockIdx.x;
+  let_next_kernel_start();
+  const ChunkRef r = chunk_of(a, slot, &s_n);
+  if (r.nr <= 0) return;
+  const long long row = r.row0 + (long long)r.t * kC;
+  // rows of q,k,gx,ty: the head's own, or the sequence's single shared set
+  const long long rq = a.s.shared ? row - ((long long)r.h + (a.s.cu ? 0 : (long long)r.n * (a.s.H - 1))) * a.s.T : row;
+  for (int e = tid; e < kC * dk; e += kOpsThreads) {
+    const int rr = e / dk, d = e % dk;
+    float la = 0.f, lh = 0.f, qv = 0.f, kv = 0.f;
+    if (rr < r.nr) {
+      const long long i = rq * dk + e;
+      qv = to_f32(((const T*)a.s.q)[i]);
+      kv = to_f32(((const T*)a.s.k)[i]);
+      gate_logs_f32(to_f32(((const T*)a.s.gx)[i]), to_f32(((const T*)a.s.ty)[i]), a.s.ingate, la, lh);
+    }
+    sB[rr * ld + d] = la;
+    sW[rr * ld + d] = expf(lh) * kv;
+    sQ[rr * ld + d] = qv;
+  }
+  __syncthreads();
+  for (int d = tid; d < dk; d += kOpsThreads) {
+    float b = 0.f;
+#pragma unroll
+    for (int rr = 0; rr < kC; ++rr) {
+      b += sB[rr * ld + d];
+      sB[rr * ld + d] = b;
+    }
+    a.decay[slot * dk + d] = expf(b);
+  }
+  __syncthreads();
+  // scores, the difference of the exponents formed before the exponential; four threads a pair
+  constexpr int kPairs = kC * (kC + 1) / 2;
+  if (tid < 4 * kPairs) {                                     // (whole warps: 544 threads)
+    const int p = tid >> 2;
+    int rr = 0, i = p;
+    while (i > rr) i -= ++rr;
+    float v = 0.f;
+#pragma unroll 4
+    for (int d = tid & 3; d < dk; d += 4)
+      v = fmaf(sQ[rr * ld + d] * sW[i * ld + d], expf(sB[rr * ld + d] - sB[i * ld + d]), v);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if ((tid & 3) == 0) a.scores[slot * (kC * kC) + rr * kC + i] = v;
+  }
+  __syncthreads();
+  for (int e = tid; e < kC * dk; e += kOpsThreads) {
+    const int rr = e / dk, d = e % dk;
+    const float b = sB[rr * ld + d];
+    a.qe[slot * (kC * dk) + e] = sQ[rr * ld + d] * expf(b);
+    sW[rr * ld + d] *= expf(sB[(kC - 1) * ld + d] - b);       // (rows past the end: decay 0, operand 0)
+  }
+  const T* v = (const T*)a.s.v + row * dv;
+  const T* bh = a.s.beta_hat ? (const T*)a.s.beta_hat + row * dv : nullptr;
+  float* ds = a.states + slot * (long long)dk * dv;
+  const int c = tid & (kTileV - 1), dg = tid / kTileV, per = dk / (kOpsThreads / kTileV);
+  for (int col0 = 0; col0 < dv; col0 += kTileV) {
+    __syncthreads();
+    for (int e = tid; e < kC * kTileV; e += kOpsThreads) {
+      const int rr = e / kTileV, cc = col0 + e % kTileV;
+      float vv = 0.f;
+      if (rr < r.nr && cc < dv) {
+        vv = to_f32(v[(long long)rr * dv + cc]);
+        if (bh) vv *= to_f32(bh[(long long)rr * dv + cc]);
+      }
+      sV[e] = vv;
+    }
+    __syncthreads();
+    if (col0 + c < dv) {
+      float vr[kC];
+#pragma unroll
+      for (int rr = 0; rr < kC; ++rr) vr[rr] = sV[rr * kTileV + c];
+      for (int j = 0; j < per; ++j) {
+        const int d = dg * per + j;
+        float acc = 0.f;
+#pragma unroll
+        for (int rr = 0; rr < kC; ++rr) acc = fmaf(sW[rr * ld + d], vr[rr], acc);
+        ds[(long long)d * dv + col0 + c] = acc;
+      }
+    }
+  }
+}
+
+// States entering the chunks and the final state; a thread per four state columns of a key channel.
+__global__ void __launch_bounds__(128) ddts_chunk_states_kernel(const ChunkArgs a) {
+  let_next_kernel_start();
+  const int v4 = a.s.dv / 4;
+  const long long per = (long long)a.s.dk * v4;
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long sh = idx / per;
+  if (sh >= (long long)a.s.n_seq * a.s.H) return;
+  const int d = (int)(idx % per / v4), c = (int)(idx % v4) * 4;
+  ChunkRef r;
+  sequence_of(a, (int)(sh / a.s.H), (int)(sh % a.s.H), r);
+  const long long size = (long long)a.s.dk * a.s.dv, e = (long long)d * a.s.dv + c;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (a.s.s0) s = *reinterpret_cast<const float4*>(a.s.s0 + sh * size + e);
+  wait_for_previous_kernel();
+  const int chunks = (r.len + kC - 1) / kC;
+  float* st = a.states + r.slot0 * size + e;
+  const float* dec = a.decay + r.slot0 * a.s.dk + d;
+  constexpr int kAhead = 8;
+  for (int c0 = 0; c0 < chunks; c0 += kAhead) {
+    float4 ds[kAhead];
+    float f[kAhead];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      if (c0 + j < chunks) {
+        ds[j] = *reinterpret_cast<const float4*>(st + (c0 + j) * size);
+        f[j] = dec[(long long)(c0 + j) * a.s.dk];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      if (c0 + j < chunks) {
+        *reinterpret_cast<float4*>(st + (c0 + j) * size) = s;
+        s = make_float4(fmaf(f[j], s.x, ds[j].x), fmaf(f[j], s.y, ds[j].y), fmaf(f[j], s.z, ds[j].z), fmaf(f[j], s.w, ds[j].w));
+      }
+    }
+  }
+  if (a.s.sT) *reinterpret_cast<float4*>(a.s.sT + sh * size + e) = s;
+}
+
+// Outputs of one chunk and kTileV value columns: a thread per column and row.
+constexpr int kOutThreads = kC * kTileV;
+template <typename T>
+__global__ void __launch_bounds__(kOutThreads) ddts_chunk_out_kernel(const ChunkArgs a) {
+  extern __shared__ float smem[];
+  __shared__ int s_n;
+  const int dk = a.s.dk, dv = a.s.dv, tid = threadIdx.x;
+  float* sS = smem;                    // [dk][kTileV]
+  float* sQ = sS + dk * kTileV;        // [kC][dk]
+  float* sV = sQ + kC * dk;            // [kC][kTileV]
+  float* sP = sV + kC * kTileV;        // [kC][kC]
+  const long long slot = blockIdx.x / (unsigned)a.s.tiles;
+  const int col0 = (int)(blockIdx.x % (unsigned)a.s.tiles) * kTileV;
+  const ChunkRef r = chunk_of(a, slot, &s_n);
+  if (r.nr <= 0) return;
+  const long long row = r.row0 + (long long)r.t * kC;
+  const int c = tid & (kTileV - 1), rr = tid / kTileV;
+  const bool live = rr < r.nr && col0 + c < dv;
+  const long long at = (row + rr) * dv + col0 + c;
+  float vv = 0.f, fx = 0.f;
+  if (live) {
+    vv = to_f32(((const T*)a.s.v)[at]);
+    if (a.s.beta_hat) vv *= to_f32(((const T*)a.s.beta_hat)[at]);
+    if (a.s.feed_d) fx = a.s.feed_d[(long long)r.h * dv + col0 + c] * to_f32(((const T*)a.s.feed_x)[at]);
+  }
+  wait_for_previous_kernel();
+  const float* S = a.states + slot * (long long)dk * dv + col0;
+  for (int e = tid; e < dk * (kTileV / 4); e += kOutThreads) {
+    const int d = e / (kTileV / 4), c4 = e % (kTileV / 4) * 4;
+    if (col0 + c4 < dv) *reinterpret_cast<float4*>(sS + d * kTileV + c4) = *reinterpret_cast<const float4*>(S + (long long)d * dv + c4);
+  }
+  for (int e = tid; e < kC * dk; e += kOutThreads) sQ[e] = a.qe[slot * (kC * dk) + e];
+  if (tid < kC * kC) sP[tid] = a.scores[slot * (kC * kC) + tid];
+  sV[tid] = vv;
+  __syncthreads();
+  if (!live) return;
+  float acc = 0.f, acc2 = 0.f;
+  for (int i = 0; i <= rr; ++i) acc = fmaf(sP[rr * kC + i], sV[i * kTileV + c], acc);
+#pragma unroll 8
+  for (int d = 0; d < dk; d += 2) {
+    acc = fmaf(sQ[rr * dk + d], sS[d * kTileV + c], acc);
+    acc2 = fmaf(sQ[rr * dk + d + 1], sS[(d + 1) * kTileV + c], acc2);
+  }
+  ((T*)a.s.o)[at] = from_f32<T>(fmaf(acc + acc2, a.s.scale, fx));
+}
+
+struct ChunkPlan {
+  long long slots;
+  int slots_per_head, heads;
+  size_t states, qe, scores, decay, bytes;   // workspace offsets, total
+};
+ChunkPlan chunk_plan(const rodimus_ddts_fwd_params& p) {
+  ChunkPlan c;
+  const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
+  c.heads = varlen ? p.H : p.B * p.H;
+  c.slots_per_head = varlen ? p.T / kC + p.N : (p.T + kC - 1) / kC;
+  c.slots = (long long)c.heads * c.slots_per_head;
+  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  c.states = sizeof(WorkspaceHeader) + up((size_t)(varlen ? p.N : 0) * sizeof(int32_t));
+  c.qe = c.states + up((size_t)c.slots * p.dk * p.dv * 4);
+  c.scores = c.qe + up((size_t)c.slots * kC * p.dk * 4);
+  c.decay = c.scores + up((size_t)c.slots * kC * kC * 4);
+  c.bytes = c.decay + up((size_t)c.slots * p.dk * 4);
+  return c;
+}
+
+template <typename T>
+cudaError_t launch_chunks(const ChunkArgs& a, cudaStream_t st) {
+  const int smem_ops = (int)sizeof(float) * (3 * kC * (a.s.dk + 1) + kC * kTileV);
+  const int smem_out = (int)sizeof(float) * (a.s.dk * kTileV + kC * a.s.dk + kC * kTileV + kC * kC);
+  cudaError_t e = cudaSuccess;
+  if (smem_ops > 48 * 1024)
+    e = cudaFuncSetAttribute(ddts_chunk_ops_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_ops);
+  if (e == cudaSuccess && smem_out > 48 * 1024)
+    e = cudaFuncSetAttribute(ddts_chunk_out_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_out);
+  if (e != cudaSuccess) return e;
+  const long long threads = (long long)a.s.n_seq * a.s.H * a.s.dk * (a.s.dv / 4);
+  ddts_chunk_ops_kernel<T><<<(unsigned)a.slots, kOpsThreads, smem_ops, st>>>(a);
+  e = launch_overlapped(ddts_chunk_states_kernel, (unsigned)((threads + 127) / 128), 128, 0, st, a);
+  if (e == cudaSuccess)
+    e = launch_overlapped(ddts_chunk_out_kernel<T>, (unsigned)(a.slots * a.s.tiles), kOutThreads, smem_out, st, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 }  // namespace
+
+// Workspace with which this kernel's chunks are computed side by side; 0: they are not.  The states of
+// the chunks cross memory four times, which pays while they stay in L2 (126 MB): up to 64 MiB of them.
+// B=1 H=1 T=256 dk=dv=64 fp32: one CTA walking the 16 chunks 318 us, side by side 28 us.
+size_t fwd_simt_chunks_workspace_bytes(const rodimus_ddts_fwd_params& p) {
+  if (p.value_decay || (long long)p.B * p.H * p.T == 0 || p.T <= kC) return 0;
+  if ((p.cu_seqlens || p.cu_seqlens_host) && p.N == 0) return 0;
+  const ChunkPlan c = chunk_plan(p);
+  if (c.slots * ((p.dv + kTileV - 1) / kTileV) > 0x7fffffffLL) return 0;
+  return c.qe - c.states <= (size_t)64 << 20 ? c.bytes : 0;
+}
 
 cudaError_t launch_fwd_simt(const rodimus_ddts_fwd_params& p, int* n_launches) {
   *n_launches = 0;
@@ -227,6 +518,23 @@ cudaError_t launch_fwd_simt(const rodimus_ddts_fwd_params& p, int* n_launches) {
   const size_t smem = simt_smem_bytes(p.dk);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
   cudaError_t e;
+  const size_t chunks = fwd_simt_chunks_workspace_bytes(p);
+  if (chunks > 0 && p.workspace_bytes >= chunks) {
+    const ChunkPlan c = chunk_plan(p);
+    char* ws = reinterpret_cast<char*>(p.workspace);
+    ChunkArgs ca;
+    ca.s = a;
+    ca.states = reinterpret_cast<float*>(ws + c.states);
+    ca.qe = reinterpret_cast<float*>(ws + c.qe);
+    ca.scores = reinterpret_cast<float*>(ws + c.scores);
+    ca.decay = reinterpret_cast<float*>(ws + c.decay);
+    ca.slots_per_head = c.slots_per_head;
+    ca.heads = c.heads;
+    ca.slots = c.slots;
+    e = p.dtype == RODIMUS_BF16 ? launch_chunks<__nv_bfloat16>(ca, st) : launch_chunks<float>(ca, st);
+    *n_launches = 3;
+    return e;
+  }
   if (p.dtype == RODIMUS_BF16) {
     e = cudaFuncSetAttribute(ddts_fwd_simt_kernel<__nv_bfloat16>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

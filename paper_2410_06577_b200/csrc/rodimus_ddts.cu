@@ -98,7 +98,8 @@ size_t rodimus_ddts_fwd_workspace_bytes(const rodimus_ddts_fwd_params* p) {
   // long dense sequences with few heads run faster split along time, given room for the
   // segments' states; a caller that passes only the base size still gets the unsplit path
   const size_t split = ddts::fwd_pair_selected(*p) ? ddts::fwd_pair_split_workspace_bytes(*p) : 0;
-  const size_t more = split > 0 ? split : ddts::scan_path_bytes(*p);
+  size_t more = split > 0 ? split : ddts::scan_path_bytes(*p);
+  if (more == 0 && ddts::fwd_kernel_choice(*p) == 2) more = ddts::fwd_simt_chunks_workspace_bytes(*p);
   return more > base ? more : base;
 }
 
