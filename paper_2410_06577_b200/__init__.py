@@ -2,7 +2,8 @@
 
 Every step of the path runs in the kernels behind the C ABI of ``include/rodimus_ddts.h``;
 PyTorch is used for device memory and streams.  There is no CPU fallback: if the shared
-library has not been built, or no CUDA device is present, calls raise.
+library has not been built, or no CUDA device is present, calls raise.  The tensor functions marshal
+through a small CPython module (``csrc/binding.cpp``), the raw ones through ctypes.
 """
 from __future__ import annotations
 
@@ -143,6 +144,23 @@ def load_library() -> ctypes.CDLL:
     return _lib
 
 
+_module = None     # the CPython module that marshals the arguments of the four tensor functions
+_bound = None      # the library handle whose functions it calls
+
+
+def _native():
+    global _module, _bound
+    if _bound is None or _bound is not _lib:
+        from . import _binding
+        lib = load_library()
+        addr = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+        _binding.bind(addr(lib.rodimus_ddts_fwd), addr(lib.rodimus_ddts_fwd_workspace_bytes),
+                      addr(lib.rodimus_ddts_step), addr(lib.rodimus_ddts_bwd),
+                      addr(lib.rodimus_ddts_bwd_workspace_bytes), addr(lib.rodimus_swska_fwd))
+        _module, _bound = _binding, lib
+    return _module
+
+
 def status_str(status: int) -> str:
     return load_library().rodimus_status_str(int(status)).decode()
 
@@ -166,12 +184,6 @@ def _dtype_code(t) -> int:
 
 def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
-
-
-def _check_cuda(*tensors):
-    for t in tensors:
-        if t is not None and not (t.is_cuda and t.is_contiguous()):
-            raise ValueError("tensors must be contiguous CUDA tensors")
 
 
 def fwd_params(q, k, gate_x, temp_y, v, o, s0=None, sT=None, cu_seqlens=None,
@@ -313,27 +325,11 @@ def ddts_bwd(q, k, gate_x, temp_y, v, d_o, s0=None, d_sT=None, cu_seqlens=None,
     None).  Returns a dict with d_q, d_k, d_gate_x, d_temp_y [B,H,T,dk], d_v [B,H,T,dv] (dtype of
     the inputs) and d_s0 (fp32, None unless wanted).  Asynchronous on the current stream.
     """
-    import torch
-    _check_cuda(q, k, gate_x, temp_y, v, d_o, s0, d_sT, cu_seqlens)
-    B, H, T, dk = q.shape
-    dv = v.shape[-1]
-    nseq = B if cu_seqlens is None else cu_seqlens.numel() - 1
-    out = {n: torch.empty_like(q) for n in ("d_q", "d_k", "d_gate_x", "d_temp_y")}
-    out["d_v"] = torch.empty_like(v)
-    out["d_s0"] = (torch.empty((nseq, H, dk, dv), dtype=torch.float32, device=q.device)
-                   if want_d_s0 else None)
-    p = bwd_params(q, k, gate_x, temp_y, v, d_o, out["d_q"], out["d_k"], out["d_gate_x"],
-                   out["d_temp_y"], out["d_v"], s0, d_sT, out["d_s0"], cu_seqlens,
-                   cu_seqlens_host, None, scale, ingate)
-    ws = workspace
-    if ws is None:
-        ws = torch.empty(max(bwd_workspace_bytes(p), 256), dtype=torch.uint8, device=q.device)
-    p.workspace = ws.data_ptr()
-    p.workspace_bytes = ws.numel() * ws.element_size()
-    rc = bwd_raw(p)
-    if rc != OK:
-        raise RodimusError(rc, "rodimus_ddts_bwd")
-    return out
+    r = _native().ddts_bwd(q, k, gate_x, temp_y, v, d_o, s0, d_sT, cu_seqlens, cu_seqlens_host, scale, ingate,
+                           want_d_s0, workspace)
+    if type(r) is int:
+        raise RodimusError(r, "rodimus_ddts_bwd")
+    return dict(zip(("d_q", "d_k", "d_gate_x", "d_temp_y", "d_v", "d_s0"), r))
 
 
 def swska_params(q, k, v, o, window: int, scale: float, stream: Optional[int] = None,
@@ -362,16 +358,10 @@ def swska_fwd(q, k, v, window: int, scale: Optional[float] = None, out=None):
     """Sliding-window shared-key attention (``rodimus_swska_fwd``): q, v [B,H,T,d], k [B,T,d]
     (one key per token for all heads); token t attends to tokens t-window+1 .. t.  ``scale``
     defaults to 1/sqrt(d).  Returns o [B,H,T,d].  Asynchronous on the current stream."""
-    import torch
-    _check_cuda(q, k, v)
-    if k.shape != (q.shape[0], q.shape[2], q.shape[3]) or v.shape != q.shape:
-        raise ValueError("q, v must be [B,H,T,d] and k [B,T,d]")
-    o = out if out is not None else torch.empty_like(q)
-    p = swska_params(q, k, v, o, window, q.shape[-1] ** -0.5 if scale is None else scale)
-    rc = swska_raw(p)
-    if rc != OK:
-        raise RodimusError(rc, "rodimus_swska_fwd")
-    return o
+    r = _native().swska_fwd(q, k, v, int(window), scale, out)
+    if type(r) is int:
+        raise RodimusError(r, "rodimus_swska_fwd")
+    return r
 
 
 def ddts_fwd(q, k, gate_x, temp_y, v, s0=None, cu_seqlens=None, cu_seqlens_host=None,
@@ -388,25 +378,11 @@ def ddts_fwd(q, k, gate_x, temp_y, v, s0=None, cu_seqlens=None, cu_seqlens_host=
     paper ablates and drops; fp32 CUDA-core kernel).
     Returns (o, sT) with sT None unless ``want_final_state``.  Asynchronous on the current stream.
     """
-    import torch
-    _check_cuda(q, k, gate_x, temp_y, v, s0, cu_seqlens, beta_hat, feed_d, feed_x, value_decay)
-    B, _, T, dk = q.shape
-    H = v.shape[1]            # q,k,gate_x,temp_y may have a single head shared by all H of v
-    dv = v.shape[-1]
-    nseq = B if cu_seqlens is None else cu_seqlens.numel() - 1
-    o = out if out is not None else torch.empty((B, H, T, dv), dtype=q.dtype, device=q.device)
-    sT = final_state
-    if sT is None and want_final_state:
-        sT = torch.empty((nseq, H, dk, dv), dtype=torch.float32, device=q.device)
-    p = fwd_params(q, k, gate_x, temp_y, v, o, s0, sT, cu_seqlens, cu_seqlens_host, None, scale,
-                   ingate, beta_hat=beta_hat, feed_d=feed_d, feed_x=feed_x, value_decay=value_decay)
-    ws = workspace if workspace is not None else new_workspace(p, q.device)
-    p.workspace = ws.data_ptr()
-    p.workspace_bytes = ws.numel() * ws.element_size()
-    rc = fwd_raw(p)
-    if rc != OK:
-        raise RodimusError(rc, "rodimus_ddts_fwd")
-    return o, sT
+    r = _native().ddts_fwd(q, k, gate_x, temp_y, v, s0, cu_seqlens, cu_seqlens_host, scale, ingate,
+                           want_final_state, out, final_state, workspace, beta_hat, feed_d, feed_x, value_decay)
+    if type(r) is int:
+        raise RodimusError(r, "rodimus_ddts_fwd")
+    return r
 
 
 def ddts_step(q, k, gate_x, temp_y, v, state, scale: float = 1.0, ingate: int = INGATE_POW_G,
@@ -415,28 +391,11 @@ def ddts_step(q, k, gate_x, temp_y, v, state, scale: float = 1.0, ingate: int = 
 
     q,k,gate_x,temp_y: [Nseq,H,dk]; v: [Nseq,H,dv].  Returns o [Nseq,H,dv].
     """
-    import torch
-    _check_cuda(q, k, gate_x, temp_y, v, state, beta_hat, feed_d, feed_x, value_decay)
-    Nseq, Hq, dk = q.shape
-    H = v.shape[1]
-    dv = v.shape[-1]
-    o = out if out is not None else torch.empty((Nseq, H, dv), dtype=q.dtype, device=q.device)
-    p = StepParams()
-    p.struct_size = ctypes.sizeof(StepParams)
-    p.dtype = _dtype_code(q)
-    p.ingate = ingate
-    p.Nseq, p.H, p.dk, p.dv = Nseq, H, dk, dv
-    p.scale = scale
-    p.q, p.k, p.gate_x, p.temp_y, p.v, p.o = (_ptr(t) for t in (q, k, gate_x, temp_y, v, o))
-    p.state = _ptr(state)
-    p.stream = torch.cuda.current_stream().cuda_stream
-    p.beta_hat, p.feed_d, p.feed_x = _ptr(beta_hat), _ptr(feed_d), _ptr(feed_x)
-    p.shared_gates = 1 if (Hq == 1 and H > 1) else 0
-    p.value_decay = _ptr(value_decay)
-    rc = step_raw(p)
-    if rc != OK:
-        raise RodimusError(rc, "rodimus_ddts_step")
-    return o
+    r = _native().ddts_step(q, k, gate_x, temp_y, v, state, scale, ingate, out, beta_hat, feed_d, feed_x,
+                            value_decay)
+    if type(r) is int:
+        raise RodimusError(r, "rodimus_ddts_step")
+    return r
 
 
 def ddts_fwd_host(q, k, gate_x, temp_y, v, s0=None, cu_seqlens=None, scale: float = 1.0,
