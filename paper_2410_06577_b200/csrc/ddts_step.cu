@@ -2,11 +2,14 @@
 // (Eq. "rodimus_recurrent_form" applied once).  Pure HBM streaming: every fp32 state element
 // is read once and written once with 16-byte accesses; nothing else is comparable in size.
 //
-// Work item = (sequence, head, tile of 128 state columns).  A CTA of 4 warps walks the dk rows
-// of its tile: warp w owns rows w, w+4, ..., lane l owns columns 4l..4l+3, so each warp-wide
-// access is one 512-byte row segment.  Rows are processed in batches of kBatch per warp with
-// all loads of a batch in flight at once; the first batch is issued before the gate math so
-// that its latency hides the token loads and the transcendental work.
+// Work item = (sequence, head, tile of 4 LC state columns).  A CTA of W warps walks the dk rows of its
+// tile, 32 / LC rows per warp-wide access; a lane owns four columns.  Rows are processed in batches of
+// BATCH accesses per warp with all loads of a batch in flight at once; the first batch is issued before
+// the gate math so that its latency hides the token loads and the transcendental work.
+//   W = 4, LC = 32, BATCH = 16   128 columns, every access one 512-byte row segment: the shape for
+//                                streaming many states (256 x 16 states 168 us, 0.99 of the copy rate)
+//   W = 8, LC = 8,  BATCH = 8    32 columns, up to 256 rows in flight at once: calls too small to fill
+//                                the device are latency, and this spreads them over 4 times the CTAs
 #include <type_traits>
 
 #include "ddts_common.cuh"
@@ -14,10 +17,6 @@
 namespace ddts {
 namespace {
 
-constexpr int kStepThreads = 128;
-constexpr int kStepWarps = kStepThreads / 32;
-constexpr int kTileCols = 128;
-constexpr int kBatch = 16;
 constexpr int kMaxDk = 256;
 
 __device__ __forceinline__ float4 ld_stream(const float4* p) { return __ldcs(p); }
@@ -25,39 +24,41 @@ __device__ __forceinline__ void st_stream(float4* p, const float4& v) { __stcs(p
 
 // VDECAY: the value-side decay beta_t of the general transition is given (the paper's ablation
 // arm); a separate instantiation, so that the plain path carries none of it.
-template <typename T, bool VDECAY>
-__global__ void __launch_bounds__(kStepThreads, 4)
+template <typename T, bool VDECAY, int W, int LC, int BATCH>
+__global__ void __launch_bounds__(32 * W, W == 4 ? 4 : 2)
 ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ gx,
                  const T* __restrict__ ty, const T* __restrict__ v, T* __restrict__ o,
                  float* __restrict__ state, int n_seq_heads, int dk, int dv, float scale,
                  int ingate, const T* __restrict__ beta_hat, const float* __restrict__ feed_d,
                  const T* __restrict__ feed_x, int H, int shared, const T* __restrict__ vdecay) {
+  constexpr int kThreads = 32 * W, kTileCols = 4 * LC, kSub = 32 / LC, kStride = W * kSub;
   __shared__ float s_alpha[kMaxDk];
   __shared__ float s_w[kMaxDk];   // ahat * k
   __shared__ float s_q[kMaxDk];   // scale * q
-  __shared__ float4 s_red[kStepWarps][32];
+  __shared__ float4 s_red[W][LC];
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
+  const int row0 = warp * kSub + lane / LC, cl = lane % LC;   // this thread's rows: row0 + kStride j
   const int tiles = (dv + kTileCols - 1) / kTileCols;
   const long long n_items = (long long)n_seq_heads * tiles;
 
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
     const long long nh = item / tiles;
-    const int col = (int)(item % tiles) * kTileCols + lane * 4;
+    const int col = (int)(item % tiles) * kTileCols + cl * 4;
     const bool col_ok = col < dv;
     float* S = state + nh * (long long)dk * dv + col;
 
     // First batch of state rows: issued before anything else of this item.
-    float4 buf[kBatch];
+    float4 buf[BATCH];
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) {
-      const int r = warp + kStepWarps * j;
+    for (int j = 0; j < BATCH; ++j) {
+      const int r = row0 + kStride * j;
       if (col_ok && r < dk) buf[j] = ld_stream(reinterpret_cast<const float4*>(S + (long long)r * dv));
     }
 
     // Gates of this token (fp32 throughout).
-    for (int d = tid; d < dk; d += kStepThreads) {
+    for (int d = tid; d < dk; d += kThreads) {
       const long long i = (shared ? nh / H : nh) * dk + d;   // shared: q,k,gx,ty are [Nseq,1,dk]
       float la, lh;
       gate_logs_f32(to_f32(gx[i]), to_f32(ty[i]), ingate, la, lh);
@@ -82,10 +83,10 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     __syncthreads();
 
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int base = 0; base < dk; base += kStepWarps * kBatch) {
+    for (int base = 0; base < dk; base += kStride * BATCH) {
 #pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int r = base + warp + kStepWarps * j;
+      for (int j = 0; j < BATCH; ++j) {
+        const int r = base + row0 + kStride * j;
         if (col_ok && r < dk) {
           const float a = s_alpha[r], w = s_w[r], qq = s_q[r];
           float4 s = buf[j];
@@ -107,24 +108,31 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
           st_stream(reinterpret_cast<float4*>(S + (long long)r * dv), s);
         }
       }
-      const int next = base + kStepWarps * kBatch;
+      const int next = base + kStride * BATCH;
       if (next < dk) {
 #pragma unroll
-        for (int j = 0; j < kBatch; ++j) {
-          const int r = next + warp + kStepWarps * j;
+        for (int j = 0; j < BATCH; ++j) {
+          const int r = next + row0 + kStride * j;
           if (col_ok && r < dk)
             buf[j] = ld_stream(reinterpret_cast<const float4*>(S + (long long)r * dv));
         }
       }
     }
 
-    // o = sum over the four warps' row subsets.
-    s_red[warp][lane] = acc;
+    // o = sum over the row subsets of the warp's lane groups, then of the warps.
+#pragma unroll
+    for (int m = LC; m < 32; m <<= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, m);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, m);
+      acc.z += __shfl_xor_sync(0xffffffffu, acc.z, m);
+      acc.w += __shfl_xor_sync(0xffffffffu, acc.w, m);
+    }
+    if (lane < LC) s_red[warp][lane] = acc;
     __syncthreads();
-    if (warp == 0 && col_ok) {
+    if (tid < LC && col_ok) {
       float4 t = s_red[0][lane];
 #pragma unroll
-      for (int w = 1; w < kStepWarps; ++w) {
+      for (int w = 1; w < W; ++w) {
         const float4 u = s_red[w][lane];
         t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
       }
@@ -150,22 +158,25 @@ cudaError_t launch_step(const rodimus_ddts_step_params& p, int* n_launches) {
   *n_launches = 0;
   const long long nh = (long long)p.Nseq * p.H;
   if (nh == 0) return cudaSuccess;
-  const int tiles = (p.dv + kTileCols - 1) / kTileCols;
-  const long long items = nh * tiles;
   int dev = 0, sms = 0;
   cudaError_t e = current_device(&dev, &sms);
   if (e != cudaSuccess) return e;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
   // One CTA per item: measured 6 % faster than a persistent grid of 8 CTAs per SM (the hardware
   // block scheduler balances the tail better than a fixed stride does).  The in-kernel loop only
   // matters beyond the grid-size limit.
-  const long long max_grid = items < 0x7fffffffLL ? items : 0x7fffffffLL;
-  (void)sms;
-  const int grid = (int)(items < max_grid ? items : max_grid);
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
+  auto grid = [&](int cols) {
+    const long long items = nh * ((p.dv + cols - 1) / cols);
+    return (unsigned)(items < 0x7fffffffLL ? items : 0x7fffffffLL);
+  };
+  // The narrow tile while its CTAs are all resident at once, two per SM (16 states 5.3 us against 7.5,
+  // 32 states 5.1 against 6.2; 64 states 8.2 against 6.2).
+  const bool small = grid(32) <= 2u * (unsigned)sms;
   auto launch = [&](auto tag, auto decay) {
     using T = decltype(tag);
     constexpr bool VD = decltype(decay)::value;
-    ddts_step_kernel<T, VD><<<grid, kStepThreads, 0, st>>>(
+    auto kernel = small ? ddts_step_kernel<T, VD, 8, 8, 8> : ddts_step_kernel<T, VD, 4, 32, 16>;
+    kernel<<<grid(small ? 32 : 128), small ? 256 : 128, 0, st>>>(
         (const T*)p.q, (const T*)p.k, (const T*)p.gate_x, (const T*)p.temp_y, (const T*)p.v,
         (T*)p.o, p.state, (int)nh, p.dk, p.dv, p.scale, p.ingate, (const T*)p.beta_hat, p.feed_d,
         (const T*)p.feed_x, p.H, p.shared_gates, (const T*)p.value_decay);

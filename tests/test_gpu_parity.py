@@ -897,3 +897,17 @@ def test_two_launch_prefill_gates_per_head(block, dv, lens):
     assert rd.fwd_workspace_bytes(rd.fwd_params(*(dev(a, "bf16") for a in (p.q, p.k, p.x, p.y, p.v)), None,
                                                 cu_seqlens=prefill_to_device(p)["cu"])) > 4096
     _check_prefill(p, rd.INGATE_POW_SIGMOID, 0.5)
+
+
+@pytest.mark.parametrize("Nseq,H,dk,dv", [(37, 1, 128, 256), (38, 1, 128, 256),    # last call of the narrow tile, first of the wide
+                                          (50, 3, 48, 80), (160, 1, 256, 80)])     # wide tile: ragged columns, two batches of rows
+def test_decode_tile_widths(Nseq, H, dk, dv):
+    import torch
+    w = wl.make_decode(970, Nseq, H, dk, dv, ring=2)
+    state = torch.from_numpy(w.state).cuda()
+    ref_state = w.state.astype(np.float64)
+    for s in range(2):
+        o = rd.ddts_step(*(dev(a[s], "bf16") for a in (w.q, w.k, w.x, w.y, w.v)), state)
+        ro = orc.ref_step(w.q[s], w.k[s], w.x[s], w.y[s], w.v[s], ref_state)
+        assert rel_err(host(o), ro) <= TOL_BF16
+    assert rel_err(host(state), ref_state) <= TOL_F32
