@@ -56,13 +56,13 @@ struct BwdTcArgs {
   unsigned long long* mask;   // [slots]: bit r = row r of the tile starts a chunk
   float *raw_q, *raw_k;       // [rows][DK]; within a tile [groups of 8 rows][DK][rows of the group]
   int32_t* tile_flag;         // [slots][4]: suffix sums of this tile and 32 channels are there
-  float* c;                   // [n_seq * H][DK]
-  float* seg_state;           // [n_seq * H * 3][DK][DV]
-  int32_t* seg_flag;          // [n_seq * H * 3]: 8 per segment that has handed its state on
+  float *c, *c2;              // [n_seq * H][DK]: the constant of the suffix sums, in two halves
+  float* seg_state;           // [n_seq * H * 3][DK][DV]: state of a sweep cut in two, at the cut
+  int32_t* seg_flag;          // [n_seq * H * 3]: 8 when that state is there
   const int32_t *cu, *order;
   WorkspaceHeader* hdr;
   long long n_flags;          // entries of seg_flag
-  int H, T, n_seq, nseg;
+  int H, T, n_seq;
   int heads;                  // tile grids: (batch, head) pairs of a dense call, heads of a packed one
   int slots_per_head;
   float scale;
@@ -156,7 +156,9 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
 // ---------------------------------------------------------------------------------------------
 // The sweeps
 // ---------------------------------------------------------------------------------------------
-// One CTA per (time segment, sweep, sequence, head), 20 warps.  The three sweeps share one skeleton:
+// A persistent CTA per SM, 20 warps, takes pieces of sweeps one after another (see get_piece); barriers
+// and chunk counters run on from piece to piece, so that the next piece's tiles are on their way while
+// the last one ends.  The three sweeps share one skeleton:
 // with operand tiles X, Y, P (64 rows of 512 bytes each) and a state of 256 tensor-memory columns,
 //               X      Y      P        state                       results
 //   raw_q       V      dO     Ki       S  [lane = key channel]     raw_q^T  [channel][row]
@@ -180,8 +182,7 @@ constexpr int kOffX = 0, kOffY = 2 * kOpBytes, kOffP = 3 * kOpBytes, kOffY32 = 4
 constexpr int kOffT = kOffY32 + 2 * kOpBytes;      // T: high and low parts, 8 KiB each
 constexpr int kOffOut = kOffY32 + kOpBytes;        // dv only (its Y32 is half as large): output tile
 constexpr int kOffD = kOffT + 2 * kSlab;           // float [4][DK]: chunk decays, per chunk (c & 3)
-constexpr int kOffRed = kOffD + 4 * DK * 4;        // float [2][DK]
-constexpr int kOffBar = kOffRed + 2 * DK * 4;
+constexpr int kOffBar = kOffD + 4 * DK * 4;
 constexpr int kSwBars = 32;
 constexpr int kOffCtl = kOffBar + kSwBars * 8;
 constexpr int kSwSmemUsed = kOffCtl + 256;
@@ -211,7 +212,7 @@ struct ChunkDesc {
   int nr_tile;       // rows of the tile
   int flags;         // kLast, kWhole
 };
-constexpr int kLast = 1, kWhole = 2;   // last chunk of the CTA's segment; the tile is one chunk
+constexpr int kLast = 1, kWhole = 2;   // last chunk of the piece; the tile is one chunk
 struct SwCtl {
   uint32_t tmem_base;
   int pad;
@@ -253,62 +254,106 @@ struct SweepMaps {
   CUtensorMap v, dout, qe_hi, qe_lo, ki_hi, ki_lo, dv, dv8, dv1;
 };
 
+// A piece of a sweep: its tiles i_lo .. i_hi-1, counted in the order of the sweep.
+struct Piece {
+  int kind, n, h;
+  int i_lo, i_hi;
+  bool wait, hand;   // the state comes from the piece before / goes to the piece after
+};
+
+// The k-th piece of CTA `cta` of `ctas`.  Sweeps are numbered from the longest kind to the shortest.
+// Dense calls have sweeps of equal length: laid end to end, each CTA takes an equal share of the tiles,
+// so a sweep may be cut in two (never in three: there are no more CTAs than sweeps).  A CTA takes the
+// beginning of its last sweep first, so that the CTA after it has the state it needs, then its whole
+// sweeps, then the end of the sweep that the CTA before it (lower index: running or done) has begun.
+// Layer shape, 192 sweeps of 32 tiles on 148 SMs: 42 tiles each; as 576 CTAs of a third of a sweep, four
+// rounds of set-up and state hand-over, the launch took 215 us.
+// Packed calls: whole sweeps of sequences ordered from the longest, dealt back and forth.
+__device__ __forceinline__ bool get_piece(const BwdTcArgs& a, int cta, int ctas, int k, Piece& p) {
+  const int items = a.n_seq * a.H, sweeps = 3 * items, nt = a.cu ? 0 : (a.T + kTile - 1) / kTile;
+  p.wait = p.hand = false;
+  int s;
+  if (nt == 0) {
+    const long long at = (long long)k * ctas + (k & 1 ? ctas - 1 - cta : cta);
+    if (at >= sweeps) return false;
+    const int of = 3 * a.H, rem = (int)(at % of);
+    p.kind = 2 - rem / a.H;
+    p.h = rem % a.H;
+    p.n = (int)(at / of);
+    if (a.cu) {
+      p.n = a.order[p.n];
+      int lo, hi;
+      seq_range(a.cu, p.n, a.T, lo, hi);
+      p.i_hi = (hi - lo + kTile - 1) / kTile;
+    } else {
+      p.i_hi = 0;
+    }
+    p.i_lo = 0;
+    return true;
+  }
+  const long long total = (long long)sweeps * nt, lo = total * cta / ctas, hi = total * (cta + 1) / ctas;
+  const int s_lo = (int)(lo / nt), r_lo = (int)(lo % nt), s_hi = (int)(hi / nt), r_hi = (int)(hi % nt);
+  const int first = s_lo + (r_lo > 0), n_head = r_hi > 0 ? 1 : 0;
+  if (k < n_head) {                                   // beginning of the last sweep
+    s = s_hi;
+    p.i_lo = 0;
+    p.i_hi = r_hi;
+    p.hand = true;
+  } else if (k - n_head < s_hi - first) {             // a whole one
+    s = first + k - n_head;
+    p.i_lo = 0;
+    p.i_hi = nt;
+  } else if (k - n_head == s_hi - first && r_lo > 0) {   // end of the first one
+    s = s_lo;
+    p.i_lo = r_lo;
+    p.i_hi = nt;
+    p.wait = true;
+  } else {
+    return false;
+  }
+  p.kind = 2 - s / items;
+  p.n = s % items / a.H;
+  p.h = s % items % a.H;
+  return true;
+}
+
+// What a thread carries from piece to piece: the number of the next chunk, chunks of cut tiles and dv
+// output tiles so far, and whether every wait has been satisfied.
+struct Carry {
+  int c, n_cut, n_ot;
+  bool ok;
+};
+
 // KIND 0: raw_q (forward), 1: raw_k, 2: dv (both reverse)
 template <int KIND>
-__device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& maps, const long long sh, const int h,
-                                          const int n, const int seg) {
+__device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps& maps, const Piece& pc, const uint32_t base,
+                                            uint8_t* gbase, const uint32_t tmem, Carry& k) {
   constexpr bool REV = KIND != 0, DVK = KIND == 2;
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
   auto bar = [&](int i) { return base + kOffBar + 8u * (uint32_t)i; };
   volatile SwCtl* ctl = reinterpret_cast<volatile SwCtl*>(gbase + kOffCtl);
   volatile WaitCtl* wc = &ctl->wait;
   float* sD = reinterpret_cast<float*>(gbase + kOffD);
-  float* sRed = reinterpret_cast<float*>(gbase + kOffRed);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q4 = warp & 3;
   WorkspaceHeader* hdr = a.hdr;
+  const long long sh = (long long)pc.n * a.H + pc.h;
 
   long long row0;
   int len, slot_base;
   if (a.cu) {
     int lo, hi;
-    seq_range(a.cu, n, a.T, lo, hi);
-    row0 = (long long)h * a.T + lo;
+    seq_range(a.cu, pc.n, a.T, lo, hi);
+    row0 = (long long)pc.h * a.T + lo;
     len = hi - lo;
-    slot_base = h * a.slots_per_head + lo / kTile + n;   // of masks and decays
+    slot_base = pc.h * a.slots_per_head + lo / kTile + pc.n;   // of masks and decays
   } else {
     row0 = sh * a.T;
     len = a.T;
     slot_base = (int)(sh * a.slots_per_head);
   }
   const int ntiles = (len + kTile - 1) / kTile;
-  // this segment's tiles, in the order of the sweep
-  const int i_lo = (int)((long long)ntiles * seg / a.nseg), i_hi = (int)((long long)ntiles * (seg + 1) / a.nseg);
+  const int i_lo = pc.i_lo, i_hi = pc.i_hi;
   const bool any = i_hi > i_lo;
-
-  if (tid == 0) {
-    ctl->wait.abort_flag = 0;
-    ctl->wait.limit = a.limit;
-    ctl->n_x = ctl->n_y = ctl->n_p = ctl->n_d = 0;
-    for (int i = 0; i < SB_COUNT; ++i) {
-      int cnt = 1;
-      if (i == SB_EY) cnt = 9;
-      if (i == SB_SREADY) cnt = 8;
-      if (i == SB_TREADY || i == SB_OFREE0 || i == SB_OFREE1 || i == SB_OTFULL || i == SB_DRDY) cnt = 4;
-      mbar_init(bar(i), cnt);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(base + kOffCtl), "r"(kSwTmemCols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = ctl->tmem_base;
+  const int first = k.c;               // number of the piece's first chunk
   // warp-uniform bounded wait (the tensor-memory accesses need whole warps)
   auto wait_all = [&](uint32_t b, uint32_t parity) -> bool {
     return __all_sync(0xffffffffu, mbar_wait(b, parity, wc, hdr)) != 0;
@@ -316,7 +361,7 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
 
   if (warp == 0) {
     // ===================================== producer ========================================
-    if (any && elect_one()) {
+    if (any && elect_one() && k.ok) {
       // a tile of four 64-column slabs: one copy, or (high and low parts) two
       struct Src { const CUtensorMap *m0, *m1; };
       const Src v = {&maps.v, nullptr}, dout = {&maps.dout, nullptr};
@@ -324,7 +369,6 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
       const Src mx = KIND == 0 ? v : (KIND == 1 ? dout : qe);
       const Src my = KIND == 0 ? dout : (KIND == 1 ? v : ki);
       const Src mp = KIND == 0 ? ki : (KIND == 1 ? qe : dout);
-      int n_x = 0, n_y = 0, n_p = 0, n_d = 0;
       // chunk iterator
       int i = i_lo, t = REV ? ntiles - 1 - i : i;
       unsigned long long mask = __ldcg(a.mask + slot_base + t), mask_next = 0ull;
@@ -377,35 +421,33 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
         } else {
           mbar_arrive(db);   // the state group computes them
         }
-        ++n_d;
+        ctl->n_d = c + 1;
         load4(base + kOffX + (c & 1) * kOpBytes, mx, cur.row, bar(SB_FX0 + (c & 1)));
-        ++n_x;
+        ctl->n_x = c + 1;
         return true;
       };
       auto load_y = [&](int c) -> bool {
         if (!mbar_wait(bar(SB_EY), (c & 1) ^ 1, wc, hdr)) return false;
         load4(base + kOffY, my, cur.row, bar(SB_FY));
-        ++n_y;
+        ctl->n_y = c + 1;
         return true;
       };
       // Tiles are asked for in the order in which their buffers come free: X(c+1) with M2(c-1), P(c)
       // with M3(c-1), Y(c+1) with M0(c).
-      bool ok = start_chunk(0) && load_y(0);
+      bool ok = start_chunk(first) && load_y(first);
       int prow = cur.row;
-      for (int c = 0; ok; ++c) {
+      for (int c = first; ok; ++c) {
+        k.c = c + 1;
         const bool next = more;
         if (next && !(ok = start_chunk(c + 1))) break;
         if (!(ok = mbar_wait(bar(SB_EP), (c & 1) ^ 1, wc, hdr))) break;
         load4(base + kOffP, mp, prow, bar(SB_FP));
-        ++n_p;
+        ctl->n_p = c + 1;
         if (!next) break;
         if (!(ok = load_y(c + 1))) break;
         prow = cur.row;
       }
-      ctl->n_x = n_x;
-      ctl->n_y = n_y;
-      ctl->n_p = n_p;
-      ctl->n_d = n_d;
+      k.ok = ok;
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -414,7 +456,7 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
     // with a branch on the lane number instead an instruction costs its thread 80 to 110 cycles, here
     // 32 to 48, which is what the tensor core needs for it.)  The loops are rolled: this code runs once
     // per chunk, and what does not stay in the instruction cache is fetched anew each time.
-    if (any) {
+    if (any && k.ok) {
       constexpr uint32_t kI0 = make_idesc(64, 64, 0, 0), kI1 = idesc_tf32(128, 64);
       constexpr uint32_t kI2 = DVK ? make_idesc(128, 128, 1, 1) : make_idesc(128, 256, 1, 1);
       constexpr uint32_t kI3 = make_idesc(128, 64, 1, 0);
@@ -439,18 +481,20 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
         }
         __syncwarp();
       };
-      bool ok = wait_all(bar(SB_FX0), 0) && wait_all(bar(SB_FY), 0);
+      bool ok = wait_all(bar(SB_FX0 + (first & 1)), (first >> 1) & 1) && wait_all(bar(SB_FY), first & 1);
       if (ok) {
         tc_fence_after();
-        m0(0);
+        m0(first);
       }
-      for (int c = 0; ok; ++c) {
+      for (int c = first; ok; ++c) {
+        k.c = c + 1;
         const uint32_t ph = c & 1;
         if (!(ok = wait_all(bar(SB_DESC0 + (c & 3)), (c >> 2) & 1))) break;
         const bool last = (ctl->desc[c & 3].flags & kLast) != 0;
         if (!(ok = wait_all(bar(SB_SREADY), ph))) break;
-        // the results' columns must have been read: two buffers in turn, or (dv) one
-        if (!DVK) {
+        // the results' columns must have been read: two buffers in turn, or (dv, and a piece's first
+        // chunk, which may follow a dv piece) one
+        if (!DVK && c > first) {
           if (!(ok = wait_all(bar(SB_OFREE0 + (c & 1)), ((c >> 1) & 1) ^ 1))) break;
         } else if (c > 0) {
           if (!(ok = wait_all(bar(SB_OFREE0 + ((c - 1) & 1)), ((c - 1) >> 1) & 1))) break;
@@ -507,6 +551,7 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
         tc_fence_after();
         m0(c + 1);
       }
+      k.ok = ok;
     }
   } else if (warp >= 4 && warp < 8) {
     // ==================================== mask group =======================================
@@ -519,8 +564,9 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
     const uint32_t diag = (keep0 ? 0x0000FFFFu : 0u) | (keep1 ? 0xFFFF0000u : 0u);
     const uint32_t t_lane = tmem + ((uint32_t)(q4 * 32) << 16);
     const uint32_t dst = base + kOffT + (q4 * 16 + mat_h * 8 + mat_k) * 128;
-    bool ok = any;
-    for (int c = 0; ok; ++c) {
+    bool ok = k.ok;
+    for (int c = first; ok && any; ++c) {
+      k.c = c + 1;
       if (!(ok = wait_all(bar(SB_TFULL), c & 1))) break;
       if (c > 0 && !(ok = wait_all(bar(SB_OFULL0 + ((c - 1) & 1)), ((c - 1) >> 1) & 1))) break;   // T's last reader
       if (!(ok = wait_all(bar(SB_DESC0 + (c & 3)), (c >> 2) & 1))) break;
@@ -553,11 +599,13 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
       if (lane == 0) mbar_arrive(bar(SB_TREADY));
       if (last) break;
     }
+    k.ok = ok;
   } else if (warp >= 8 && warp < 12) {
     // =================================== output group ======================================
     const uint32_t t_lane = tmem + ((uint32_t)(q4 * 32) << 16);
-    bool ok = any;
-    for (int c = 0; ok; ++c) {
+    bool ok = k.ok;
+    for (int c = first; ok && any; ++c) {
+      k.c = c + 1;
       if (!(ok = wait_all(bar(SB_DESC0 + (c & 3)), (c >> 2) & 1))) break;
       if (!(ok = wait_all(bar(SB_OFULL0 + (c & 1)), (c >> 1) & 1))) break;
       const volatile ChunkDesc* d = &ctl->desc[c & 3];
@@ -602,7 +650,7 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
         // dv^T fragments [value column][row] are transposed by stmatrix.trans into four swizzled
         // 64-column slabs and leave by tensor copies
         const int mat_k = lane & 7, mat_h = (lane >> 3) & 1, mat_j = lane >> 4;
-        if (c > 0 && !(ok = wait_all(bar(SB_OTFREE), (c - 1) & 1))) break;
+        if (k.n_ot > 0 && !(ok = wait_all(bar(SB_OTFREE), (k.n_ot - 1) & 1))) break;
 #pragma unroll
         for (int bl = 0; bl < 2; ++bl) {
           const uint32_t mat = base + kOffOut + (2 * bl + (q4 >> 1)) * kSlab + (mat_j * 8 + mat_k) * 128;
@@ -633,7 +681,7 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(SB_OTFULL));
         if (q4 == 0) {
-          if (!(ok = wait_all(bar(SB_OTFULL), c & 1))) break;
+          if (!(ok = wait_all(bar(SB_OTFULL), k.n_ot & 1))) break;
           if (nr == kTile) {
             if (lane < 4) tma_store_2d(&maps.dv, 64 * lane, (int)row, base + kOffOut + lane * kSlab);
           } else {   // boxes of 8 rows and of 1 row, so that no row of another chunk is touched
@@ -652,9 +700,11 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(SB_OTFREE));
         }
+        ++k.n_ot;
       }
       if (last) break;
     }
+    k.ok = ok;
   } else if (warp >= 12) {
     // ==================================== state group ======================================
     // 8 warps: tensor-memory quarter q4, columns 128 half .. 128 half + 127 of the state.
@@ -667,17 +717,17 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
     };
     const float* init = KIND == 0 ? a.s0 : a.dsT;
     if (init) init += sh * (long long)DK * DV;
-    bool ok = true;
-    if (seg > 0) {
-      // The segment before this one belongs to a CTA with a lower index, and CTAs start in the order
-      // of their index: it is running or done.  The wait is bounded all the same.
+    bool ok = k.ok;
+    if (ok && pc.wait) {
+      // The piece before this one is the first one of a CTA with a lower index, and CTAs start in the
+      // order of their index: it is running or done.  The wait is bounded all the same.
       const int32_t* flag = a.seg_flag + sh * 3 + KIND;
       if (lane == 0) {
         const long long t0 = clock64();
-        while (ld_acquire_s32(flag) < 8 * seg) {
+        while (ld_acquire_s32(flag) < 8) {
           if (wc->abort_flag) { ok = false; break; }
           if (clock64() - t0 >= a.limit) {
-            ok = ld_acquire_s32(flag) >= 8 * seg;
+            ok = ld_acquire_s32(flag) >= 8;
             if (!ok) {
               wc->abort_flag = 1;
               atomicMax(&hdr->status, (int)RODIMUS_ERR_TIMEOUT);
@@ -772,7 +822,7 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
         }
       }
     };
-    int c = 0;
+    int c = first;
     if (ok && !any) {   // nothing to sweep: the state is only passed on
 #pragma unroll 1
       for (int piece = 0; piece < 4; ++piece) {
@@ -783,7 +833,8 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
       tmem_st_wait();
     }
     bool last = !any;
-    int n_cut = 0;
+    // the dv output tile lies where the other kinds keep half of their expanded Y: its copies are done
+    if (ok && !DVK && k.n_ot > 0) ok = wait_all(bar(SB_OTFREE), (k.n_ot - 1) & 1);
     while (ok && !last) {
       if (!(ok = wait_all(bar(SB_FY), c & 1))) break;
       if (c > 0 && !(ok = wait_all(bar(SB_M1), (c - 1) & 1))) break;    // Y32's last reader
@@ -805,24 +856,24 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(SB_DRDY));
         }
-        if (!(ok = wait_all(bar(SB_DRDY), n_cut & 1))) break;
-        ++n_cut;
+        if (!(ok = wait_all(bar(SB_DRDY), k.n_cut & 1))) break;
+        ++k.n_cut;
       }
       const float* dvec = sD + ((REV ? c : c - 1) & 3) * DK;   // forward: of the chunk before
-      if (c > 0) {
+      if (c > first) {
         if (!(ok = wait_all(bar(SB_UFULL), (c - 1) & 1))) break;
         tc_fence_after();
       }
 #pragma unroll 1
       for (int piece = 0; piece < 4; ++piece) {
         uint32_t r[32];
-        if (c > 0) {
+        if (c > first) {
           tmem_ld32(t_st + 32 * piece, r);
           tmem_ld_wait();
         } else {
           load_init(r, piece);
         }
-        if (REV || c > 0) scale_by(r, dvec, piece);
+        if (REV || c > first) scale_by(r, dvec, piece);
         tmem_st32(t_st + 32 * piece, r);
       }
       if (nr < kTile) {
@@ -838,11 +889,13 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
       if (lane == 0) mbar_arrive(bar(SB_SREADY));
       ++c;
     }
+    k.c = c;
+    if (DVK) k.n_ot += c - first;
     // ---- after the last chunk
     if (ok && any) ok = wait_all(bar(SB_UFULL), (c - 1) & 1);
     if (ok) {
       tc_fence_after();
-      const bool hand_on = seg + 1 < a.nseg;
+      const bool hand_on = pc.hand;
       float* dst = nullptr;
       if (hand_on) dst = a.seg_state + (sh * 3 + KIND) * (long long)DK * DV;
       else if (KIND == 1 && a.ds0) dst = a.ds0 + sh * (long long)DK * DV;
@@ -877,7 +930,7 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
             }
           }
         }
-        if (dot) sRed[half * DK + ln] = acc;
+        if (dot) (half ? a.c2 : a.c)[sh * DK + ln] = acc;
         if (hand_on) {
           __threadfence();
           __syncwarp();
@@ -886,15 +939,57 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
       }
       tc_fence_before();
     }
+    k.ok = ok;
+  }
+}
+
+__global__ void __launch_bounds__(kSwThreads, 1)
+ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
+  auto bar = [&](int i) { return base + kOffBar + 8u * (uint32_t)i; };
+  volatile SwCtl* ctl = reinterpret_cast<volatile SwCtl*>(gbase + kOffCtl);
+  const int tid = threadIdx.x, warp = tid >> 5;
+  if (tid == 0) {
+    ctl->wait.abort_flag = 0;
+    ctl->wait.limit = a.limit;
+    ctl->n_x = ctl->n_y = ctl->n_p = ctl->n_d = 0;
+    for (int i = 0; i < SB_COUNT; ++i) {
+      int cnt = 1;
+      if (i == SB_EY) cnt = 9;
+      if (i == SB_SREADY) cnt = 8;
+      if (i == SB_TREADY || i == SB_OFREE0 || i == SB_OFREE1 || i == SB_OTFULL || i == SB_DRDY) cnt = 4;
+      mbar_init(bar(i), cnt);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(base + kOffCtl), "r"(kSwTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = ctl->tmem_base;
+
+  // (bad cu_seqlens have been reported: nothing to compute)
+  if (!a.cu || *(volatile int32_t*)&a.hdr->status != RODIMUS_ERR_SEQLENS) {
+    Carry k = {0, 0, 0, true};
+    Piece pc;
+    for (int i = 0; get_piece(a, (int)blockIdx.x, (int)gridDim.x, i, pc); ++i) {
+      if (pc.kind == 0) sweep_piece<0>(a, maps, pc, base, gbase, tmem, k);
+      else if (pc.kind == 1) sweep_piece<1>(a, maps, pc, base, gbase, tmem, k);
+      else sweep_piece<2>(a, maps, pc, base, gbase, tmem, k);
+    }
   }
 
   // ------------------------------------------ teardown ------------------------------------------
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const bool aborted = ctl->wait.abort_flag != 0;
-  if (KIND == 0 && !aborted && a.dsT && seg + 1 == a.nseg && tid < DK) a.c[sh * DK + tid] = sRed[tid] + sRed[DK + tid];
-  if (aborted) {   // nothing may still be writing this CTA's shared or tensor memory
+  if (ctl->wait.abort_flag != 0) {   // nothing may still be writing this CTA's shared or tensor memory
     if (tid == 0) {
       for (int back = 1; back <= 2; ++back)
         if (ctl->n_x >= back) mbar_drain(bar(SB_FX0 + ((ctl->n_x - back) & 1)), ((ctl->n_x - back) >> 1) & 1);
@@ -911,22 +1006,6 @@ __device__ __forceinline__ void sweep_cta(const BwdTcArgs& a, const SweepMaps& m
   __syncthreads();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSwTmemCols) : "memory");
-}
-
-__global__ void __launch_bounds__(kSwThreads, 1)
-ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs a) {
-  if (a.cu && *(volatile int32_t*)&a.hdr->status == RODIMUS_ERR_SEQLENS) return;   // reported; nothing to compute
-  // index = (segment, sweep from the longest kind to the shortest, (sequence, head))
-  const unsigned n_items = gridDim.x / (3 * a.nseg);
-  const int item = (int)(blockIdx.x % n_items), part = (int)(blockIdx.x / n_items);
-  const int seg = part / 3, kind = 2 - part % 3;
-  const int h = item % a.H;
-  int n = item / a.H;
-  if (a.cu) n = a.order[n];
-  const long long sh = (long long)n * a.H + h;
-  if (kind == 0) sweep_cta<0>(a, maps, sh, h, n, seg);
-  else if (kind == 1) sweep_cta<1>(a, maps, sh, h, n, seg);
-  else sweep_cta<2>(a, maps, sh, h, n, seg);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1070,8 +1149,9 @@ __global__ void __launch_bounds__(kPostThreads, 3) ddts_bwd_post_kernel(const Bw
     acc0 = v.x;
     acc1 = v.y;
   } else {
-    acc0 = a.dsT ? (double)a.c[(long long)(tr.n * a.H + (a.cu ? head : head % a.H)) * DK + ch] : 0.0;
-    acc1 = a.dsT ? (double)a.c[(long long)(tr.n * a.H + (a.cu ? head : head % a.H)) * DK + ch + 1] : 0.0;
+    const long long e = (long long)(tr.n * a.H + (a.cu ? head : head % a.H)) * DK + ch;
+    acc0 = a.dsT ? (double)(a.c[e] + a.c2[e]) : 0.0;
+    acc1 = a.dsT ? (double)(a.c[e + 1] + a.c2[e + 1]) : 0.0;
   }
 #pragma unroll 1
   for (int g = kTile / kPostRows - 1; g > rg; --g) {
@@ -1101,16 +1181,13 @@ __global__ void __launch_bounds__(kPostThreads, 3) ddts_bwd_post_kernel(const Bw
 std::atomic<unsigned long long> g_sweep_smem_done{0};
 
 // Workspace beyond header and order: raw_q and raw_k (1 KiB per row), c, and an area that holds the
-// states handed from segment to segment (384 KiB per (sequence, head), only where a call may be
-// segmented) and the few words per tile; where those fit into the 384 KiB the size does not change.
+// states of sweeps cut in two (384 KiB per (sequence, head), dense calls of more than one tile) and the
+// few words per tile; where those fit into the 384 KiB the size does not change.
 struct Scratch {
-  size_t raw_q, raw_k, c, dtile, mask, tile_flag, seg_flag, seg_state, bytes;
+  size_t raw_q, raw_k, c, c2, dtile, mask, tile_flag, seg_flag, seg_state, bytes;
   long long slots;
   int slots_per_head, heads;
-  bool may_segment;
 };
-
-constexpr int kSegTiles = 4;             // a segment has at least this many tiles (on average, if packed)
 
 Scratch scratch_layout(const rodimus_ddts_bwd_params& p) {
   Scratch s;
@@ -1120,14 +1197,13 @@ Scratch scratch_layout(const rodimus_ddts_bwd_params& p) {
   s.heads = varlen ? p.H : p.B * p.H;
   s.slots_per_head = varlen ? p.T / kTile + p.N : (p.T + kTile - 1) / kTile;
   s.slots = (long long)s.heads * s.slots_per_head;
-  s.may_segment = nseq > 0 && (size_t)p.T / (varlen ? nseq : 1) >= (size_t)2 * kSegTiles * kTile;
   auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
   s.raw_q = 0;
   s.raw_k = rows * DK * 4;
   s.c = 2 * rows * DK * 4;
   const size_t area = up(s.c + items * DK * 4), states = items * 3 * (size_t)DK * DV * 4;
   s.seg_state = area;
-  size_t at = area + (s.may_segment ? states : 0);
+  size_t at = area + (!varlen && p.T > kTile ? states : 0);
   auto take = [&](size_t bytes) {
     const size_t o = at;
     at += up(bytes);
@@ -1137,6 +1213,7 @@ Scratch scratch_layout(const rodimus_ddts_bwd_params& p) {
   s.mask = take((size_t)s.slots * 8);
   s.tile_flag = take((size_t)s.slots * 16);
   s.seg_flag = take(items * 3 * 4);
+  s.c2 = take(items * DK * 4);
   const size_t least = area + states + up(items * 6 * 4);
   s.bytes = at > least ? at : least;
   return s;
@@ -1164,6 +1241,7 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
   a.raw_q = (float*)(ws + s.raw_q); a.raw_k = (float*)(ws + s.raw_k);
   a.tile_flag = (int32_t*)(ws + s.tile_flag);
   a.c = (float*)(ws + s.c);
+  a.c2 = (float*)(ws + s.c2);
   a.seg_state = (float*)(ws + s.seg_state);
   a.seg_flag = (int32_t*)(ws + s.seg_flag);
   a.cu = p.cu_seqlens;
@@ -1182,21 +1260,7 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
   if (e != cudaSuccess) return e;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
 
-  // Time segments per sweep: 3 sweeps per (sequence, head) seldom fill the SMs (one CTA each) evenly.
-  // n segments cost ceil(3 items n / SMs) rounds of 1/n of a sweep each plus kSegCost tiles' worth of
-  // set-up and state hand-over per round.
-  {
-    constexpr double kSegCost = 2.0;
-    const double tiles = (double)(((long long)p.T / (p.cu_seqlens ? a.n_seq : 1) + kTile - 1) / kTile);
-    double best = 1e30;
-    a.nseg = 1;
-    for (int n = 1; n <= 16; ++n) {
-      if (n > 1 && (!s.may_segment || tiles < (double)kSegTiles * n)) break;
-      const double cost = (double)((items * 3 * n + sms - 1) / sms) * (tiles / n + kSegCost);
-      if (cost < best * 0.999) { best = cost; a.nseg = n; }
-    }
-    if (items * 3 * a.nseg > 0x7fffffffLL || s.slots > 0x1fffffffLL) return cudaErrorInvalidValue;
-  }
+  if (items * 3 > 0x7fffffffLL || s.slots > 0x1fffffffLL) return cudaErrorInvalidValue;
   SweepMaps m;
   const uint64_t rows = (uint64_t)p.B * p.H * p.T;
   if (rows > 0) {
@@ -1218,7 +1282,7 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
     ddts_bwd_pre_kernel<<<(unsigned)s.slots, kPreThreads, 0, st>>>(a);
     ++*n_launches;
   }
-  ddts_bwd_sweep_tc_kernel<<<(unsigned)(items * 3 * a.nseg), kSwThreads, kSwSmem, st>>>(m, a);
+  ddts_bwd_sweep_tc_kernel<<<(unsigned)(items * 3 < sms ? items * 3 : sms), kSwThreads, kSwSmem, st>>>(m, a);
   ++*n_launches;
   if (rows > 0) {
     ddts_bwd_post_kernel<<<(unsigned)(s.slots * 4), kPostThreads, 0, st>>>(a);
