@@ -56,6 +56,7 @@ struct BwdTcArgs {
   unsigned long long* mask;   // [slots]: bit r = row r of the tile starts a chunk
   float *raw_q, *raw_k;       // [rows][DK]; within a tile [groups of 8 rows][DK][rows of the group]
   int32_t* tile_flag;         // [slots][4]: suffix sums of this tile and 32 channels are there
+  int2* tile_order;           // packed: (sequence, tile) of every head's tiles as the last kernel takes them
   float *c, *c2;              // [n_seq * H][DK]: the constant of the suffix sums, in two halves
   float* seg_state;           // [n_seq * H * 3][DK][DV]: state of a sweep cut in two, at the cut
   int32_t* seg_flag;          // [n_seq * H * 3]: 8 when that state is there
@@ -88,6 +89,59 @@ __device__ __forceinline__ void red_release_add(int32_t* p, int32_t v) {
 // ---------------------------------------------------------------------------------------------
 constexpr int kPreThreads = 512, kPreRows = kTile / (kPreThreads / 64);   // 8 rows x 2 channels a thread
 
+// Packed sequences: the order in which the last kernel takes a head's tiles.  The tiles of a sequence are
+// chained from its end, a hop being about 2 us; with the sequences one after another the chain runs through
+// all of them, so the order is: the last tile of every sequence, then the last but one of all that have
+// one, and so on (sequences longest first, so those are a prefix of the list).  Block-wide.
+__device__ void order_tiles(const BwdTcArgs& a, int* s_nt, int* s_scan) {
+  const int tid = threadIdx.x, N = a.n_seq;
+  auto tiles_of = [&](int n) {
+    int lo, hi;
+    seq_range(a.cu, n, a.T, lo, hi);
+    return (hi - lo + kTile - 1) / kTile;
+  };
+  if (N > kMaxSortedSeqs) {   // not sorted: sequence after sequence, from the last one's end
+    for (int pos = tid; pos < a.slots_per_head; pos += kPreThreads) a.tile_order[pos] = make_int2(-1, 0);
+    __syncthreads();
+    for (int n = tid; n < N; n += kPreThreads) {
+      int lo, hi;
+      seq_range(a.cu, n, a.T, lo, hi);
+      for (int t = 0, nt = tiles_of(n); t < nt; ++t)
+        a.tile_order[a.slots_per_head - 1 - (lo / kTile + n + t)] = make_int2(n, t);
+    }
+    return;
+  }
+  for (int j = tid; j < N; j += kPreThreads) s_nt[j] = tiles_of(a.order[j]);
+  __syncthreads();
+  const int most = s_nt[0];
+  int at = 0;                 // tiles before this batch of kPreThreads ranks
+  for (int r0 = 0; r0 < most; r0 += kPreThreads) {
+    int cnt = 0;              // sequences with more than r tiles
+    const int r = r0 + tid;
+    if (r < most) {
+      int hi = N;
+      while (cnt < hi) {
+        const int mid = (cnt + hi) >> 1;
+        if (s_nt[mid] > r) cnt = mid + 1;
+        else hi = mid;
+      }
+    }
+    s_scan[tid] = cnt;
+    __syncthreads();
+    for (int d = 1; d < kPreThreads; d <<= 1) {
+      const int v = tid >= d ? s_scan[tid - d] : 0;
+      __syncthreads();
+      s_scan[tid] += v;
+      __syncthreads();
+    }
+    const int base = at + s_scan[tid] - cnt;
+    for (int j = 0; j < cnt; ++j) a.tile_order[base + j] = make_int2(a.order[j], s_nt[j] - 1 - r);
+    at += s_scan[kPreThreads - 1];
+    __syncthreads();
+  }
+  for (int pos = at + tid; pos < a.slots_per_head; pos += kPreThreads) a.tile_order[pos] = make_int2(-1, 0);
+}
+
 __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdTcArgs a) {
   __shared__ __align__(16) float s_la[kTile * DK];
   __shared__ __align__(16) float s_part[(kTile / kPreRows) * DK];
@@ -97,6 +151,10 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
   if (blockIdx.x == 0 && tid == 0 && !a.cu) a.hdr->status = RODIMUS_OK;
   for (long long i = (long long)blockIdx.x * kPreThreads + tid; i < a.n_flags; i += (long long)gridDim.x * kPreThreads)
     a.seg_flag[i] = 0;
+  if (a.cu && blockIdx.x == gridDim.x - 1) {   // one block more than there are slots
+    order_tiles(a, reinterpret_cast<int*>(s_la), reinterpret_cast<int*>(s_part));
+    return;
+  }
   const int head = (int)(blockIdx.x / (unsigned)a.slots_per_head), local = (int)(blockIdx.x % (unsigned)a.slots_per_head);
   const TileRef tr = find_tile(geometry(a), head, local, &s_n);
   const long long slot = (long long)head * a.slots_per_head + local;
@@ -1014,8 +1072,8 @@ ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs
 //   dg   = -tau dla + w tau u'/u        dtau = -g dla + w ln u         (u = g, or 1 - e^-g = sigmoid(x))
 //   dx   = dg sigmoid(x)  =  w tau sigmoid(x) u'/u  -  dla tau sigmoid(x)
 //   dy   = dtau tau (1 - tau)  =  (1 - tau) (dla log alpha + w log ahat)
-// One CTA per (tile, 32 channels).  Tiles run from the end of the sequences to their start: a CTA waits
-// (bounded) for the suffix sums of the tile after it, whose CTA has a lower index.
+// One CTA per (tile, 32 channels).  Tiles run from the end of the sequences to their start (see
+// order_tiles): a CTA waits (bounded) for the suffix sums of the tile after it, whose CTA has a lower index.
 constexpr int kPostThreads = 256, kPostCh = 32, kPostRows = 4;   // 4 rows x 2 channels a thread
 static_assert(kPostThreads == kPostCh / 2 * (kTile / kPostRows), "one thread per 4 rows x 2 channels");
 
@@ -1023,14 +1081,31 @@ __global__ void __launch_bounds__(kPostThreads, 3) ddts_bwd_post_kernel(const Bw
   __shared__ __align__(16) float s_la[kTile * kPostCh];
   __shared__ __align__(16) float s_part[(kTile / kPostRows) * kPostCh];
   __shared__ __align__(16) double s_sum[(kTile / kPostRows) * kPostCh];
-  __shared__ int s_n, s_late;
+  __shared__ int s_late;
   if (a.cu && *(volatile int32_t*)&a.hdr->status == RODIMUS_ERR_SEQLENS) return;
   const int tid = threadIdx.x;
   const int quarter = (int)(blockIdx.x & 3u), hs = (int)(blockIdx.x >> 2);
-  const int head = hs % a.heads, local = a.slots_per_head - 1 - hs / a.heads;
-  const TileRef tr = find_tile(geometry(a), head, local, &s_n);
-  if (tr.nr <= 0) return;
-  const long long slot = (long long)head * a.slots_per_head + local;
+  const int head = hs % a.heads, pos = hs / a.heads;
+  TileRef tr;
+  long long slot;
+  if (a.cu) {
+    const int2 e = __ldg(a.tile_order + pos);
+    if (e.x < 0) return;
+    int lo, hi;
+    seq_range(a.cu, e.x, a.T, lo, hi);
+    tr.n = e.x;
+    tr.t = e.y;
+    tr.len = hi - lo;
+    tr.row0 = (long long)head * a.T + lo + (long long)e.y * kTile;
+    slot = (long long)head * a.slots_per_head + lo / kTile + e.x + e.y;
+  } else {
+    tr.n = head / a.H;
+    tr.t = a.slots_per_head - 1 - pos;
+    tr.len = a.T;
+    tr.row0 = (long long)head * a.T + (long long)tr.t * kTile;
+    slot = (long long)head * a.slots_per_head + tr.t;
+  }
+  tr.nr = min(kTile, tr.len - tr.t * kTile);
   const int cp = tid & 15, rg = tid >> 4, ch = quarter * kPostCh + 2 * cp;
   const int live = tr.nr - rg * kPostRows;
   const long long e0 = (tr.row0 + rg * kPostRows) * 64 + ch / 2;
@@ -1184,7 +1259,7 @@ std::atomic<unsigned long long> g_sweep_smem_done{0};
 // states of sweeps cut in two (384 KiB per (sequence, head), dense calls of more than one tile) and the
 // few words per tile; where those fit into the 384 KiB the size does not change.
 struct Scratch {
-  size_t raw_q, raw_k, c, c2, dtile, mask, tile_flag, seg_flag, seg_state, bytes;
+  size_t raw_q, raw_k, c, c2, dtile, mask, tile_flag, tile_order, seg_flag, seg_state, bytes;
   long long slots;
   int slots_per_head, heads;
 };
@@ -1214,6 +1289,7 @@ Scratch scratch_layout(const rodimus_ddts_bwd_params& p) {
   s.tile_flag = take((size_t)s.slots * 16);
   s.seg_flag = take(items * 3 * 4);
   s.c2 = take(items * DK * 4);
+  s.tile_order = take(varlen ? (size_t)s.slots_per_head * 8 : 0);
   const size_t least = area + states + up(items * 6 * 4);
   s.bytes = at > least ? at : least;
   return s;
@@ -1242,6 +1318,7 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
   a.tile_flag = (int32_t*)(ws + s.tile_flag);
   a.c = (float*)(ws + s.c);
   a.c2 = (float*)(ws + s.c2);
+  a.tile_order = (int2*)(ws + s.tile_order);
   a.seg_state = (float*)(ws + s.seg_state);
   a.seg_flag = (int32_t*)(ws + s.seg_flag);
   a.cu = p.cu_seqlens;
@@ -1279,7 +1356,7 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
   e = opt_in_shared_memory(ddts_bwd_sweep_tc_kernel, kSwSmem, dev, g_sweep_smem_done);
   if (e != cudaSuccess) return e;
   if (rows > 0) {
-    ddts_bwd_pre_kernel<<<(unsigned)s.slots, kPreThreads, 0, st>>>(a);
+    ddts_bwd_pre_kernel<<<(unsigned)s.slots + (p.cu_seqlens ? 1u : 0u), kPreThreads, 0, st>>>(a);
     ++*n_launches;
   }
   ddts_bwd_sweep_tc_kernel<<<(unsigned)(items * 3 < sms ? items * 3 : sms), kSwThreads, kSwSmem, st>>>(m, a);
