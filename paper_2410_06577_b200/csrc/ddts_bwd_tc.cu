@@ -58,7 +58,8 @@ struct BwdTcArgs {
   int32_t* tile_flag;         // [slots][4]: suffix sums of this tile and 32 channels are there
   int2* tile_order;           // packed: (sequence, tile) of every head's tiles as the last kernel takes them
   float *c, *c2;              // [n_seq * H][DK]: the constant of the suffix sums, in two halves
-  float* seg_state;           // [n_seq * H * 3][DK][DV]: state of a sweep cut in two, at the cut
+  float* seg_state;           // [n_seq * H * 3][32][256] of 16 bytes: state of a sweep cut in two, at the
+                              // cut, as the 256 threads of the state group hold it
   int32_t* seg_flag;          // [n_seq * H * 3]: 8 when that state is there
   const int32_t *cu, *order;
   WorkspaceHeader* hdr;
@@ -232,11 +233,15 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
 // to be scaled by the chunk decay D (forward: after the update; reverse: before the use).
 // Precision: V and dO are exact; Qe, Ki and T are bf16 pairs (products of two pairs drop low x low,
 // 2^-16); the state is read as tf32 by M1 and kept in fp32.
-// The issue order M1(c) M2(c) M3(c) M0(c+1) gives the tensor pipe M3 and M0 to work on while the
-// state makes its trip, and the mask warps all of M1 and M2.
+// The issue order is M1 M0 M2 M3: the chain of the state is M1, M0, M2, then its trip, during which M3
+// runs and Y of the next chunk, which has two buffers, is expanded.  (With M0 of the next chunk at the
+// end, X in two buffers and Y in one, the layer shape took 361 us a call, so 354.)
+// What bounds it: about 500 KiB go through shared memory per chunk (M0 64, M1 64, M2 96, M3 72, expanding
+// Y 96, tiles in 96, T 16), 3900 cycles at 128 bytes a clock; a chunk takes 6000, a 32 KiB tile 3000 to
+// 4000 cycles to arrive although it comes from L2 (prefetching it there changes nothing).
 constexpr int kSlab = kTile * 128;                 // [64 rows][128 bytes], 128-byte swizzled
-constexpr int kOpBytes = 4 * kSlab;                // X, Y, P: 32 KiB
-constexpr int kOffX = 0, kOffY = 2 * kOpBytes, kOffP = 3 * kOpBytes, kOffY32 = 4 * kOpBytes;
+constexpr int kOpBytes = 4 * kSlab;                // X, Y (two buffers), P: 32 KiB each
+constexpr int kOffX = 0, kOffY = kOpBytes, kOffP = 3 * kOpBytes, kOffY32 = 4 * kOpBytes;
 constexpr int kOffT = kOffY32 + 2 * kOpBytes;      // T: high and low parts, 8 KiB each
 constexpr int kOffOut = kOffY32 + kOpBytes;        // dv only (its Y32 is half as large): output tile
 constexpr int kOffD = kOffT + 2 * kSlab;           // float [4][DK]: chunk decays, per chunk (c & 3)
@@ -250,9 +255,9 @@ constexpr int kSwThreads = 640;
 constexpr uint32_t kColS = 0, kColO = 256, kColT = 384, kSwTmemCols = 512;
 
 enum { SB_DESC0 = 0,                       // [4] descriptor and decays of a chunk      (1 + bytes)
-       SB_FX0 = 4, SB_FX1, SB_FY, SB_FP,   // tiles landed                              (1 + bytes)
-       SB_EX0, SB_EX1, SB_EP,              // tile reusable: its contractions are done  (1)
-       SB_EY,                              // Y reusable: M0 done, expanded             (1 + 8 warps)
+       SB_FX = 4, SB_FY0, SB_FY1, SB_FP,   // tiles landed                              (1 + bytes)
+       SB_EX, SB_EP,                       // tile reusable: its contractions are done  (1)
+       SB_EY0, SB_EY1,                     // Y reusable: M0 done, expanded             (1 + 8 warps)
        SB_TFULL, SB_TREADY,                // T computed (1), masked into shared memory (4 warps)
        SB_M1, SB_UFULL,                    // M1 / M2 complete                          (1)
        SB_SREADY,                          // state scaled, Y32 written                 (8 warps)
@@ -437,15 +442,15 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
       peek();
       int r = REV ? chunk_start(mask, nr_tile - 1) : 0;   // first row of the chunk within the tile
       bool more = true;
-      struct { int row, nr; } cur = {0, 0};
       auto load4 = [&](uint32_t dst, const Src& m, int row, uint32_t b) {
         mbar_expect_tx(b, kOpBytes);
         tma_load_3d(dst, m.m0, 0, row, 0, b);
         if (m.m1) tma_load_3d(dst + 2 * kSlab, m.m1, 0, row, 0, b);
       };
-      // descriptor, decays and X tile of chunk number c; leaves its row in `cur`
+      auto row_of = [&](int c) { return (int)ctl->desc[c & 3].row; };
+      // descriptor, decays and Y tile of chunk number c
       auto start_chunk = [&](int c) -> bool {
-        if (!mbar_wait(bar(SB_EX0 + (c & 1)), ((c >> 1) & 1) ^ 1, wc, hdr)) return false;
+        if (!mbar_wait(bar(SB_EY0 + (c & 1)), ((c >> 1) & 1) ^ 1, wc, hdr)) return false;
         const int end = chunk_end(mask, r, nr_tile);
         volatile ChunkDesc* d = &ctl->desc[c & 3];
         const long long row = row0 + (long long)t * kTile + r;
@@ -454,7 +459,6 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
         d->roff = r;
         d->nr_tile = nr_tile;
         const bool whole = mask == 1ull;
-        cur.row = (int)row;
         const float* decays = a.dtile + (long long)(slot_base + t) * DK;
         // step to the chunk after this one
         bool last = false;
@@ -480,30 +484,24 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
           mbar_arrive(db);   // the state group computes them
         }
         ctl->n_d = c + 1;
-        load4(base + kOffX + (c & 1) * kOpBytes, mx, cur.row, bar(SB_FX0 + (c & 1)));
-        ctl->n_x = c + 1;
-        return true;
-      };
-      auto load_y = [&](int c) -> bool {
-        if (!mbar_wait(bar(SB_EY), (c & 1) ^ 1, wc, hdr)) return false;
-        load4(base + kOffY, my, cur.row, bar(SB_FY));
+        load4(base + kOffY + (c & 1) * kOpBytes, my, (int)row, bar(SB_FY0 + (c & 1)));
         ctl->n_y = c + 1;
         return true;
       };
-      // Tiles are asked for in the order in which their buffers come free: X(c+1) with M2(c-1), P(c)
-      // with M3(c-1), Y(c+1) with M0(c).
-      bool ok = start_chunk(first) && load_y(first);
-      int prow = cur.row;
+      // Tiles are asked for in the order in which their buffers come free: X(c) with M2(c-1), Y(c+1) with
+      // M0 and the expansion of c-1, P(c) with M3(c-1).
+      bool ok = start_chunk(first);
       for (int c = first; ok; ++c) {
         k.c = c + 1;
+        if (!(ok = mbar_wait(bar(SB_EX), (c & 1) ^ 1, wc, hdr))) break;
+        load4(base + kOffX, mx, row_of(c), bar(SB_FX));
+        ctl->n_x = c + 1;
         const bool next = more;
         if (next && !(ok = start_chunk(c + 1))) break;
         if (!(ok = mbar_wait(bar(SB_EP), (c & 1) ^ 1, wc, hdr))) break;
-        load4(base + kOffP, mp, prow, bar(SB_FP));
+        load4(base + kOffP, mp, row_of(c), bar(SB_FP));
         ctl->n_p = c + 1;
         if (!next) break;
-        if (!(ok = load_y(c + 1))) break;
-        prow = cur.row;
       }
       k.ok = ok;
     }
@@ -518,32 +516,12 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
       constexpr uint32_t kI0 = make_idesc(64, 64, 0, 0), kI1 = idesc_tf32(128, 64);
       constexpr uint32_t kI2 = DVK ? make_idesc(128, 128, 1, 1) : make_idesc(128, 256, 1, 1);
       constexpr uint32_t kI3 = make_idesc(128, 64, 1, 0);
-      const uint32_t dy = desc_lo_kmajor(base + kOffY), dx0 = desc_lo_kmajor(base + kOffX);
+      const uint32_t dy0 = desc_lo_kmajor(base + kOffY), dx = desc_lo_kmajor(base + kOffX);
       const uint32_t dy32 = desc_lo_kmajor(base + kOffY32), dt = desc_lo_kmajor(base + kOffT);
-      const uint32_t dxm0 = desc_lo_mnmajor(base + kOffX, kSlab), dp = desc_lo_mnmajor(base + kOffP, kSlab);
+      const uint32_t dxm = desc_lo_mnmajor(base + kOffX, kSlab), dp = desc_lo_mnmajor(base + kOffP, kSlab);
       constexpr uint32_t kS = kSlab >> 4;              // one slab, in descriptor units
       const uint32_t t_s = tmem + kColS, t_t = tmem + kColT;
-      auto m0 = [&](int c) {
-        const uint32_t dx = dx0 + (c & 1) * 4 * kS;
-        if (elect_one()) {
-#pragma unroll 1
-          for (uint32_t i = 0; i < (DVK ? 6u : 4u); ++i) {
-            // dv: slab pairs (high, high), (high, low), (low, high) of the 128 channels' two slabs
-            const uint32_t ya = dy + (DVK ? (i & 1) + (i >= 4 ? 2u : 0u) : i) * kS;
-            const uint32_t xa = dx + (DVK ? (i & 1) + ((i >> 1) == 1 ? 2u : 0u) : i) * kS;
-#pragma unroll
-            for (uint32_t kk = 0; kk < 4; ++kk) umma_ss(t_t, ya + 2 * kk, xa + 2 * kk, kI0, i | kk);
-          }
-          umma_commit(bar(SB_TFULL));
-          umma_commit(bar(SB_EY));
-        }
-        __syncwarp();
-      };
-      bool ok = wait_all(bar(SB_FX0 + (first & 1)), (first >> 1) & 1) && wait_all(bar(SB_FY), first & 1);
-      if (ok) {
-        tc_fence_after();
-        m0(first);
-      }
+      bool ok = true;
       for (int c = first; ok; ++c) {
         k.c = c + 1;
         const uint32_t ph = c & 1;
@@ -571,10 +549,26 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
           umma_commit(bar(SB_M1));
         }
         __syncwarp();
+        if (!(ok = wait_all(bar(SB_FX), ph))) break;
+        tc_fence_after();
+        // M0 (Y has landed: the state group has expanded it)
+        const uint32_t dy = dy0 + ph * 4 * kS;
+        if (elect_one()) {
+#pragma unroll 1
+          for (uint32_t i = 0; i < (DVK ? 6u : 4u); ++i) {
+            // dv: slab pairs (high, high), (high, low), (low, high) of the 128 channels' two slabs
+            const uint32_t ya = dy + (DVK ? (i & 1) + (i >= 4 ? 2u : 0u) : i) * kS;
+            const uint32_t xa = dx + (DVK ? (i & 1) + ((i >> 1) == 1 ? 2u : 0u) : i) * kS;
+#pragma unroll
+            for (uint32_t kk = 0; kk < 4; ++kk) umma_ss(t_t, ya + 2 * kk, xa + 2 * kk, kI0, i | kk);
+          }
+          umma_commit(bar(SB_TFULL));
+          umma_commit(bar(SB_EY0 + ph));
+        }
+        __syncwarp();
         if (!(ok = wait_all(bar(SB_FP), ph))) break;
         tc_fence_after();
         // M2
-        const uint32_t dxm = dxm0 + ph * 4 * kS;
         if (elect_one()) {
 #pragma unroll 1
           for (uint32_t i = 0; i < (DVK ? 4u : 2u); ++i) {
@@ -584,7 +578,7 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
             for (uint32_t kk = 0; kk < 4; ++kk) umma_ss(d, pa + 128 * kk, xa + 128 * kk, kI2, 1u);
           }
           umma_commit(bar(SB_UFULL));
-          umma_commit(bar(SB_EX0 + ph));
+          umma_commit(bar(SB_EX));
         }
         __syncwarp();
         if (!(ok = wait_all(bar(SB_TREADY), ph))) break;
@@ -604,10 +598,6 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
         }
         __syncwarp();
         if (last) break;
-        if (!(ok = wait_all(bar(SB_FX0 + (ph ^ 1)), ((c + 1) >> 1) & 1))) break;
-        if (!(ok = wait_all(bar(SB_FY), ph ^ 1))) break;
-        tc_fence_after();
-        m0(c + 1);
       }
       k.ok = ok;
     }
@@ -798,9 +788,11 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
       ok = __all_sync(0xffffffffu, ok) != 0;
       init = a.seg_state + (sh * 3 + KIND) * (long long)DK * DV;
     }
-    auto expand = [&]() {
+    // (a state handed over is read and written 16 bytes per thread, 512 contiguous bytes per warp)
+    auto handed = [&](const float* p, int piece, int e) { return p + ((8 * piece + e / 4) * 256 + rt) * 4; };
+    auto expand = [&](int c) {
       const int r = rt & 63;
-      const uint32_t src = base + kOffY + r * 128, dst = base + kOffY32 + r * 128, sw = (uint32_t)(r & 7);
+      const uint32_t src = base + kOffY + (c & 1) * kOpBytes + r * 128, dst = base + kOffY32 + r * 128, sw = (uint32_t)(r & 7);
       // (loads are issued ahead of the stores, four at a time)
       if (!DVK) {
 #pragma unroll
@@ -866,13 +858,13 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
       if (!init) {
 #pragma unroll
         for (int e = 0; e < 32; ++e) r[e] = 0u;
-      } else if (DVK) {
+      } else if (DVK && !pc.wait) {
 #pragma unroll
         for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__ldcg(init + elem(32 * piece + e)));
       } else {
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
-          const float4 v = __ldcg(reinterpret_cast<const float4*>(init + elem(32 * piece + e)));
+          const float4 v = __ldcg(reinterpret_cast<const float4*>(pc.wait ? handed(init, piece, e) : init + elem(32 * piece + e)));
           r[e] = __float_as_uint(v.x);
           r[e + 1] = __float_as_uint(v.y);
           r[e + 2] = __float_as_uint(v.z);
@@ -894,12 +886,12 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
     // the dv output tile lies where the other kinds keep half of their expanded Y: its copies are done
     if (ok && !DVK && k.n_ot > 0) ok = wait_all(bar(SB_OTFREE), (k.n_ot - 1) & 1);
     while (ok && !last) {
-      if (!(ok = wait_all(bar(SB_FY), c & 1))) break;
+      if (!(ok = wait_all(bar(SB_FY0 + (c & 1)), (c >> 1) & 1))) break;
       if (c > 0 && !(ok = wait_all(bar(SB_M1), (c - 1) & 1))) break;    // Y32's last reader
-      expand();
+      expand(c);
       fence_proxy_async();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(SB_EY));
+      if (lane == 0) mbar_arrive(bar(SB_EY0 + (c & 1)));
       if (!(ok = wait_all(bar(SB_DESC0 + (c & 3)), (c >> 2) & 1))) break;
       const int nr = ctl->desc[c & 3].nr, flags = ctl->desc[c & 3].flags;
       last = (flags & kLast) != 0;
@@ -967,17 +959,12 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
           tmem_ld32(t_st + 32 * piece, r);
           tmem_ld_wait();
           if (!REV && any) scale_by(r, sD + ((c - 1) & 3) * DK, piece);
-          if (dst) {
-            if (!DVK) {
+          if (dst) {   // (of the dv sweep only the handed-over state is ever wanted)
 #pragma unroll
-              for (int e = 0; e < 32; e += 4)
-                __stcg(reinterpret_cast<float4*>(dst + elem(32 * piece + e)),
-                       make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
-                                   __uint_as_float(r[e + 3])));
-            } else {
-#pragma unroll
-              for (int e = 0; e < 32; ++e) __stcg(dst + elem(32 * piece + e), __uint_as_float(r[e]));
-            }
+            for (int e = 0; e < 32; e += 4)
+              __stcg(reinterpret_cast<float4*>(const_cast<float*>(hand_on ? handed(dst, piece, e) : dst + elem(32 * piece + e))),
+                     make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
+                                 __uint_as_float(r[e + 3])));
           }
           if (dot) {
 #pragma unroll
@@ -1015,7 +1002,7 @@ ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs
     ctl->n_x = ctl->n_y = ctl->n_p = ctl->n_d = 0;
     for (int i = 0; i < SB_COUNT; ++i) {
       int cnt = 1;
-      if (i == SB_EY) cnt = 9;
+      if (i == SB_EY0 || i == SB_EY1) cnt = 9;
       if (i == SB_SREADY) cnt = 8;
       if (i == SB_TREADY || i == SB_OFREE0 || i == SB_OFREE1 || i == SB_OTFULL || i == SB_DRDY) cnt = 4;
       mbar_init(bar(i), cnt);
@@ -1050,8 +1037,8 @@ ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs
   if (ctl->wait.abort_flag != 0) {   // nothing may still be writing this CTA's shared or tensor memory
     if (tid == 0) {
       for (int back = 1; back <= 2; ++back)
-        if (ctl->n_x >= back) mbar_drain(bar(SB_FX0 + ((ctl->n_x - back) & 1)), ((ctl->n_x - back) >> 1) & 1);
-      if (ctl->n_y > 0) mbar_drain(bar(SB_FY), (ctl->n_y - 1) & 1);
+        if (ctl->n_y >= back) mbar_drain(bar(SB_FY0 + ((ctl->n_y - back) & 1)), ((ctl->n_y - back) >> 1) & 1);
+      if (ctl->n_x > 0) mbar_drain(bar(SB_FX), (ctl->n_x - 1) & 1);
       if (ctl->n_p > 0) mbar_drain(bar(SB_FP), (ctl->n_p - 1) & 1);
       for (int back = 1; back <= 4; ++back)
         if (ctl->n_d >= back) mbar_drain(bar(SB_DESC0 + ((ctl->n_d - back) & 3)), ((ctl->n_d - back) >> 2) & 1);
