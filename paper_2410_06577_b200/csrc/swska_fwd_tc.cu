@@ -31,20 +31,19 @@
 namespace ddts {
 namespace {
 
-constexpr int kD = 128, kBM = 128, kBN = 64, kHalf = kBN / 2;
-constexpr int kSoftmaxWarps = 8, kIssuerWarp = 8, kProducerWarp = 9, kThreads = 32 * (kSoftmaxWarps + 2);
+constexpr int kD = 128, kBM = 128, kBN = 64;
+constexpr int kSoftmaxWarps = 4, kIssuerWarp = 4, kProducerWarp = 5, kThreads = 32 * (kSoftmaxWarps + 2);
 constexpr uint32_t kQSlabBytes = kBM * 128;           // [128 rows][64 columns] bf16
 constexpr uint32_t kSlabBytes = kBN * 128;            // [64 rows][64 columns] bf16
 constexpr uint32_t kTileBytes = 2 * kSlabBytes;       // 64 x 128 bf16
 constexpr uint32_t kOffQ = 0, kOffK = 2 * kQSlabBytes, kOffV = kOffK + 2 * kTileBytes;
 constexpr uint32_t kOffCtl = kOffV + 2 * kTileBytes;
-constexpr uint32_t kOffMax = kOffCtl + 256;            // [2][2][128] floats: the halves' row maxima (by buffer) / sums
-constexpr uint32_t kSmemBytes = kOffMax + 2048 + 1024; // + slack for 1024-byte alignment
+constexpr uint32_t kSmemBytes = kOffCtl + 256 + 1024;  // + slack for 1024-byte alignment
 constexpr uint32_t kTmemCols = 256, kColS = 0, kColO = 128;
 constexpr float kLog2e = 1.4426950408889634f;
 
-enum { BAR_Q = 0, BAR_K0, BAR_K1, BAR_V0, BAR_V1, BAR_S0, BAR_S1, BAR_P0, BAR_P1, BAR_O0, BAR_O1, BAR_PAIR0,
-       BAR_DRAIN = BAR_PAIR0 + 4, kNumBars };
+enum { BAR_Q = 0, BAR_K0, BAR_K1, BAR_V0, BAR_V1, BAR_S0, BAR_S1, BAR_P0, BAR_P1, BAR_O0, BAR_O1,
+       BAR_DRAIN, kNumBars };
 
 struct SwCtl {
   uint64_t bar[kNumBars];
@@ -119,7 +118,6 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   unsigned char* gen = smem_raw + (base - smem_u32(smem_raw));
   volatile SwCtl* ctl = reinterpret_cast<volatile SwCtl*>(gen + kOffCtl);
   auto bar = [&](int i) { return base + kOffCtl + 8u * (uint32_t)i; };
-  float* sMax = reinterpret_cast<float*>(gen + kOffMax);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // Query tiles late in the sequence see the most keys.  CTAs are handed out in the order of
@@ -143,9 +141,7 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     ctl->limit = a.limit;
     ctl->k_sent = ctl->v_sent = ctl->k_seen = ctl->v_seen = 0;
     for (int i = 0; i < kNumBars; ++i) {
-      const bool per_warp = i == BAR_P0 || i == BAR_P1;
-      const bool pair = i >= BAR_PAIR0 && i < BAR_PAIR0 + 4;
-      mbar_init(bar(i), per_warp ? kSoftmaxWarps : (pair ? 2 : 1));
+      mbar_init(bar(i), i == BAR_P0 || i == BAR_P1 ? kSoftmaxWarps : 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -255,153 +251,126 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     __syncwarp();
   } else {
     // =========================== softmax warps =================================================
-    // thread = (query row, half of a tile's 64 key columns): warps 0-3 the first half, warps 4-7
-    // the second; a warp reaches the 32 tensor-memory lanes of its number mod 4
-    const int rowl = tid & (kBM - 1), half = tid >> 7, col0 = half * kHalf;
-    const int row = m0 + rowl;
-    const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t pair_bar = bar(BAR_PAIR0 + (warp & 3));   // this warp and the one with the other half
+    // thread = query row = tensor-memory lane
+    const int row = m0 + tid;
+    const uint32_t t_row = tmem + ((uint32_t)(warp * 32) << 16);
     const float sc = a.scale * kLog2e;        // > 0 (checked by the host)
     // Reference exponent of the row (log2 domain).  It follows the running maximum lazily: it
     // moves only when a tile's maximum exceeds it by more than 8, so probabilities stay below 2^8
     // and O, l are rescaled rarely; the final division by l makes the result independent of it.
     float m_ref = -INFINITY, l_run = 0.f;
     bool ok = true;
-    int it = 0;
-    // the two threads of a row exchange their maxima of a tile (both have then read S, which the
-    // probabilities overwrite); the reference exponent follows; returns the factor for O and l
-    auto exchange = [&](int sb, int it, float mx, float& alpha) -> bool {
-      sMax[(sb * 2 + half) * kBM + rowl] = mx * sc;   // (-inf stays -inf: sc > 0)
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(pair_bar);
-      bool good = sw_wait(pair_bar, it & 1, ctl, a.status);
-      good = __all_sync(0xffffffffu, good);
-      if (!good) return false;
-      tc_fence_after();
-      const float m_tile = fmaxf(sMax[(sb * 2) * kBM + rowl], sMax[(sb * 2 + 1) * kBM + rowl]);
-      alpha = 1.f;
-      if (m_tile > m_ref + 8.f) {               // also the first tile with a visible key
-        alpha = ex2f(m_ref - m_tile);           // 0 when nothing had been seen
-        m_ref = m_tile;
-      }
-      return true;
+    auto wait = [&](int b, uint32_t parity) -> bool {   // whole warps: tensor-memory accesses need them
+      return __all_sync(0xffffffffu, sw_wait(bar(b), parity, ctl, a.status)) != 0;
     };
-    // rescaling O (rare) needs the previous O += P V complete; writing P does not
-    auto rescale = [&](int it, float alpha) -> bool {
-      if (it > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
-        bool good = sw_wait(bar(BAR_O0 + ((it - 1) & 1)), ((it - 1) >> 1) & 1, ctl, a.status);
-        good = __all_sync(0xffffffffu, good);
-        if (!good) return false;
-        tc_fence_after();
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          uint32_t r[32];
-          tmem_ld32(t_row + kColO + 64 * half + 32 * c, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-          tmem_st32(t_row + kColO + 64 * half + 32 * c, r);
-        }
-      }
-      return true;
-    };
-    auto publish = [&](int sb, const uint32_t (&pk)[kHalf / 2]) {
-      tmem_st16(t_row + kColS + sb * kBN + 16 * half, pk);     // keys col0 .. col0+31, two per column
+    auto publish = [&](int sb) {
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(BAR_P0 + sb));
     };
-    for (; it < n_tiles; ++it) {
+    for (int it = 0; it < n_tiles; ++it) {
       const int sb = it & 1;
-      const uint32_t ph = (it >> 1) & 1;
       const int n0 = (nt_lo + it) * kBN;
-      ok = sw_wait(bar(BAR_S0 + sb), ph, ctl, a.status);
-      ok = __all_sync(0xffffffffu, ok);     // the tensor-memory accesses below need the whole warp
-      if (!ok) break;
+      const uint32_t t_s = t_row + kColS + sb * kBN;
+      if (!(ok = wait(BAR_S0 + sb, (it >> 1) & 1))) break;
       tc_fence_after();
-      // the visible keys of this thread's 32 are e_lo .. e_hi (none when e_lo > e_hi)
-      const int k0 = n0 + col0;
-      const int e_lo = max(0, row - W + 1 - k0), e_hi = min(kHalf - 1, row - k0);
+      // the visible keys of the row are e_lo .. e_hi (none when e_lo > e_hi)
+      const int e_lo = max(0, row - W + 1 - n0), e_hi = min(kBN - 1, row - n0);
       if (__all_sync(0xffffffffu, e_lo > e_hi)) {
         // on the diagonal and at the window's far edge whole warps see no key of a tile: they
-        // take part in the hand-offs and write zeros, without the arithmetic
-        float alpha;
-        if (!(ok = exchange(sb, it, -INFINITY, alpha))) break;
-        l_run *= alpha;
-        if (!(ok = rescale(it, alpha))) break;
-        uint32_t pk[kHalf / 2];
+        // write zeros, without the arithmetic
+        uint32_t z[32];
 #pragma unroll
-        for (int e = 0; e < kHalf / 2; ++e) pk[e] = 0u;
-        publish(sb, pk);
+        for (int e = 0; e < 32; ++e) z[e] = 0u;
+        tmem_st32(t_s, z);
+        publish(sb);
         continue;
       }
-      // ---- this thread's 32 columns of its row of S: mask, maximum
-      float sv[kHalf];
-      float mx;
+      // ---- the row of S: mask, maximum (four independent chains of three-input steps)
+      float sv[kBN];
       {
-        uint32_t r[32];
-        tmem_ld32(t_row + kColS + sb * kBN + col0, r);
+        uint32_t r0[32], r1[32];
+        tmem_ld32(t_s, r0);
+        tmem_ld32(t_s + 32, r1);
         tmem_ld_wait();
-        if (e_lo == 0 && e_hi == kHalf - 1) {
 #pragma unroll
-          for (int e = 0; e < kHalf; ++e) sv[e] = __uint_as_float(r[e]);
-        } else {
-          const uint32_t bits = e_lo > e_hi ? 0u : ((0xffffffffu >> (kHalf - 1 - e_hi)) & (0xffffffffu << e_lo));
-#pragma unroll
-          for (int e = 0; e < kHalf; ++e) sv[e] = ((bits >> e) & 1u) ? __uint_as_float(r[e]) : -INFINITY;
+        for (int e = 0; e < 32; ++e) {
+          sv[e] = __uint_as_float(r0[e]);
+          sv[32 + e] = __uint_as_float(r1[e]);
         }
-        // maximum as a tree: four independent chains of three-input steps over eight values each
-        float m4[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float* s8 = sv + 8 * c;
-          m4[c] = fmaxf(max3(max3(max3(s8[0], s8[1], s8[2]), s8[3], s8[4]), s8[5], s8[6]), s8[7]);
-        }
-        mx = fmaxf(max3(m4[0], m4[1], m4[2]), m4[3]);
       }
-      float alpha;
-      if (!(ok = exchange(sb, it, mx, alpha))) break;
+      if (!__all_sync(0xffffffffu, e_lo == 0 && e_hi == kBN - 1)) {
+        const unsigned long long bits = e_lo > e_hi ? 0ull : ((~0ull >> (kBN - 1 - e_hi)) & (~0ull << e_lo));
+        const uint32_t b0 = (uint32_t)bits, b1 = (uint32_t)(bits >> 32);
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+          sv[e] = ((b0 >> e) & 1u) ? sv[e] : -INFINITY;
+          sv[32 + e] = ((b1 >> e) & 1u) ? sv[32 + e] : -INFINITY;
+        }
+      }
+      float m4[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float* s16 = sv + 16 * c;
+        float m = max3(s16[0], s16[1], s16[2]);
+#pragma unroll
+        for (int e = 3; e < 15; e += 2) m = max3(m, s16[e], s16[e + 1]);
+        m4[c] = fmaxf(m, s16[15]);
+      }
+      const float m_tile = fmaxf(max3(m4[0], m4[1], m4[2]), m4[3]) * sc;   // (-inf stays -inf: sc > 0)
+      if (__any_sync(0xffffffffu, m_tile > m_ref + 8.f)) {     // rare but for the first tile
+        float alpha = 1.f;
+        if (m_tile > m_ref + 8.f) {
+          alpha = ex2f(m_ref - m_tile);           // 0 when nothing had been seen
+          m_ref = m_tile;
+        }
+        l_run *= alpha;
+        if (it > 0) {                             // O += P V of the tile before is complete
+          if (!(ok = wait(BAR_O0 + ((it - 1) & 1), ((it - 1) >> 1) & 1))) break;
+          tc_fence_after();
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {
+            uint32_t r[32];
+            tmem_ld32(t_row + kColO + 32 * c, r);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
+            tmem_st32(t_row + kColO + 32 * c, r);
+          }
+        }
+      }
       const float m_use = m_ref == -INFINITY ? 0.f : m_ref;
       uint64_t ps[4] = {0ull, 0ull, 0ull, 0ull};     // four pairs of partial sums: short dependent chains
-      uint32_t pk[kHalf / 2];
       const uint64_t sc2 = pair_f32(sc, sc), nm2 = pair_f32(-m_use, -m_use);
 #pragma unroll
-      for (int e = 0; e < kHalf; e += 2) {
-        float x0, x1;
-        unpair_f32(fma2(pair_f32(sv[e], sv[e + 1]), sc2, nm2), x0, x1);
-        const float p0 = ex2f(x0), p1 = ex2f(x1);
-        ps[(e >> 1) & 3] = add2(ps[(e >> 1) & 3], pair_f32(p0, p1));
-        pk[e >> 1] = pack_bf16(p0, p1);
+      for (int hf = 0; hf < 2; ++hf) {
+        uint32_t pk[16];
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) {
+          float x0, x1;
+          unpair_f32(fma2(pair_f32(sv[32 * hf + e], sv[32 * hf + e + 1]), sc2, nm2), x0, x1);
+          const float p0 = ex2f(x0), p1 = ex2f(x1);
+          ps[(e >> 1) & 3] = add2(ps[(e >> 1) & 3], pair_f32(p0, p1));
+          pk[e >> 1] = pack_bf16(p0, p1);
+        }
+        tmem_st16(t_s + 16 * hf, pk);                // over S, two keys per column
       }
-      {
-        float s0, s1;
-        unpair_f32(add2(add2(ps[0], ps[1]), add2(ps[2], ps[3])), s0, s1);
-        l_run = l_run * alpha + (s0 + s1);
-      }
-      if (!(ok = rescale(it, alpha))) break;
-      publish(sb, pk);
+      publish(sb);
+      float s0, s1;
+      unpair_f32(add2(add2(ps[0], ps[1]), add2(ps[2], ps[3])), s0, s1);
+      l_run += s0 + s1;
     }
-    // ---- the last O += P V, then normalise and store this thread's 64 columns of its row
-    if (ok) ok = sw_wait(bar(BAR_O0 + ((n_tiles - 1) & 1)), ((n_tiles - 1) >> 1) & 1, ctl, a.status);
-    ok = __all_sync(0xffffffffu, ok);
+    // ---- the last O += P V, then normalise and store the row
+    if (ok) ok = wait(BAR_O0 + ((n_tiles - 1) & 1), ((n_tiles - 1) >> 1) & 1);
     if (ok) {
       tc_fence_after();
-      sMax[half * kBM + rowl] = l_run;
-      __syncwarp();
-      if (lane == 0) mbar_arrive(pair_bar);
-      ok = sw_wait(pair_bar, n_tiles & 1, ctl, a.status);
-      ok = __all_sync(0xffffffffu, ok);
-    }
-    if (ok) {
-      const float l = sMax[rowl] + sMax[kBM + rowl];
-      const float inv = l > 0.f ? 1.f / l : 0.f;
-      __nv_bfloat16* orow = (__nv_bfloat16*)a.o + (qrow0 + rowl) * kD + 64 * half;
+      const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+      __nv_bfloat16* orow = (__nv_bfloat16*)a.o + (qrow0 + tid) * kD;
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
+      for (int c = 0; c < 4; ++c) {
         uint32_t r[32];
-        tmem_ld32(t_row + kColO + 64 * half + 32 * c, r);
+        tmem_ld32(t_row + kColO + 32 * c, r);
         tmem_ld_wait();
         if (row < T) {
 #pragma unroll
