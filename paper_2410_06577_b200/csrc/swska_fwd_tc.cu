@@ -2,23 +2,27 @@
 //   s_ti = scale <q^h_t, k_i>,  t - W < i <= t      p_ti = softmax_i(s_ti)      o^h_t = sum_i p_ti v^h_i
 // (Sec. "Shared-Key Attention for Lossless Head Compression": one key per token for all heads.)
 //
-// One CTA per (batch, head, 128 queries): 8 softmax warps, one warp that issues the contractions
-// and one that issues the TMA loads.  Query row =
-// tensor-memory lane; two softmax threads per row (32 of a tile's 64 key columns each; they
-// exchange one maximum per tile and one sum at the end through shared memory).  Per key tile of
-// 64 tokens:
+// One CTA per (batch, head, 128 queries): 4 softmax warps, one warp that issues the contractions and
+// one that issues the TMA loads.  Query row = tensor-memory lane = softmax thread: a row's maximum and
+// sum need no exchange (two threads per row, which exchanged both through shared memory: 78.7 us at
+// the layer shape, one: 68.1).  Per key tile of 64 tokens:
 //   S = Q K^T        tcgen05.mma, Q tile and K tile K-major in shared memory (TMA, 128-byte
 //                    swizzle), accumulator [128 x 64] fp32 in tensor memory, TWO buffers: the
 //                    scores of tile i+1 are computed while the softmax of tile i runs
-//   softmax          each thread reads its part of a row of S (tcgen05.ld), keeps a reference
-//                    exponent and a sum in the log2 domain, rescales its part of the row of O in
-//                    tensor memory when the reference moved (lazily: only when a tile's maximum
-//                    exceeds it by more than 2^8), and writes the probabilities back over S as
-//                    packed bf16 (tcgen05.st)
+//   softmax          each thread reads its row of S (tcgen05.ld), keeps a reference exponent and a
+//                    sum in the log2 domain, rescales its row of O in tensor memory when the
+//                    reference moved (lazily: only when a tile's maximum exceeds it by more than
+//                    2^8), and writes the probabilities back over S as packed bf16 (tcgen05.st)
 //   O += P V         tcgen05.mma, A = P from tensor memory, B = the V tile (token-major, i.e.
 //                    N-major) from shared memory
+// What bounds it: two CTAs on an SM take 825 cycles per key tile, in which the tensor cores are busy
+// for 640 (S 384: from shared memory at N = 64 the operand reads, not the arithmetic, set the rate;
+// O 256) and the special-function units for 512.
 // One warp issues every contraction and one every load, under elect_one(): with a test of the lane
 // number instead an instruction cost its thread about a hundred cycles (layer shape 84.1 us, now 79.6).
+// The first loads leave before the block has met, and a whole tile of O leaves through shared memory
+// by tensor copies instead of 16-byte pieces 256 bytes apart: 3.3 us less at the layer shape
+// (4 x 16 x 2048, window 1024: 64.5 us), 4 us of 41 with a window of 128.
 // Tensor memory: 256 columns
 // (S twice 64, O 128); shared memory 96 KiB (Q 32, two K tiles, two V tiles; a tile is requested
 // two tiles ahead, as soon as the contraction that read its slot is complete): two CTAs per SM.  Only key tiles that
@@ -43,7 +47,7 @@ constexpr uint32_t kTmemCols = 256, kColS = 0, kColO = 128;
 constexpr float kLog2e = 1.4426950408889634f;
 
 enum { BAR_Q = 0, BAR_K0, BAR_K1, BAR_V0, BAR_V1, BAR_S0, BAR_S1, BAR_P0, BAR_P1, BAR_O0, BAR_O1,
-       BAR_DRAIN, kNumBars };
+       BAR_OUT, BAR_DRAIN, kNumBars };
 
 struct SwCtl {
   uint64_t bar[kNumBars];
@@ -112,7 +116,8 @@ __device__ __forceinline__ bool sw_wait(uint32_t bar, uint32_t parity, volatile 
 
 __global__ void __launch_bounds__(kThreads, 2)
 swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                    const __grid_constant__ CUtensorMap map_v, const SwTcArgs a) {
+                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
+                    const SwTcArgs a) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* gen = smem_raw + (base - smem_u32(smem_raw));
@@ -136,15 +141,35 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   const int nt_lo = first_key / kBN, nt_hi = min(m0 + kBM - 1, T - 1) / kBN;
   const int n_tiles = nt_hi - nt_lo + 1;
 
-  if (tid == 0) {
+  auto load = [&](const CUtensorMap* map, uint32_t dst, uint32_t slab, int row, int which, uint32_t bytes) {
+    mbar_expect_tx(bar(which), bytes);
+    tma_load_2d(base + dst, map, 0, row, bar(which));
+    tma_load_2d(base + dst + slab, map, 64, row, bar(which));
+  };
+  auto fill_k = [&](int j) {
+    load(&map_k, kOffK + (j & 1) * kTileBytes, kSlabBytes, krow0 + (nt_lo + j) * kBN, BAR_K0 + (j & 1), kTileBytes);
+  };
+  auto fill_v = [&](int j) {
+    load(&map_v, kOffV + (j & 1) * kTileBytes, kSlabBytes, vrow0 + (nt_lo + j) * kBN, BAR_V0 + (j & 1), kTileBytes);
+  };
+  // The thread that sets the barriers up asks for the first tiles at once: their way is as long as the
+  // allocation of tensor memory and the block's first meeting together.
+  if (warp == kProducerWarp && elect_one()) {
     ctl->abort = 0;
     ctl->limit = a.limit;
-    ctl->k_sent = ctl->v_sent = ctl->k_seen = ctl->v_seen = 0;
+    ctl->k_seen = ctl->v_seen = 0;
     for (int i = 0; i < kNumBars; ++i) {
-      mbar_init(bar(i), i == BAR_P0 || i == BAR_P1 ? kSoftmaxWarps : 1);
+      mbar_init(bar(i), i == BAR_P0 || i == BAR_P1 || i == BAR_OUT ? kSoftmaxWarps : 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_proxy_async();
+    fill_k(0);
+    load(&map_q, kOffQ, kQSlabBytes, (int)qrow0, BAR_Q, 2 * kQSlabBytes);
+    fill_v(0);
+    if (n_tiles > 1) { fill_k(1); fill_v(1); }
+    ctl->k_sent = ctl->v_sent = min(2, n_tiles);
   }
+  __syncwarp();
   if (warp == kIssuerWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  ::"r"(base + kOffCtl + (uint32_t)offsetof(SwCtl, tmem_base)), "r"(kTmemCols) : "memory");
@@ -158,32 +183,17 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   if (warp == kProducerWarp) {
     // =========================== producer warp: every TMA load ================================
     if (elect_one()) {
-      int k_sent = 0, v_sent = 0;
-      auto load = [&](const CUtensorMap* map, uint32_t dst, uint32_t slab, int row, int which, uint32_t bytes) {
-        mbar_expect_tx(bar(which), bytes);
-        tma_load_2d(base + dst, map, 0, row, bar(which));
-        tma_load_2d(base + dst + slab, map, 64, row, bar(which));
-      };
-      auto fill_k = [&](int j) {
-        load(&map_k, kOffK + (j & 1) * kTileBytes, kSlabBytes, krow0 + (nt_lo + j) * kBN, BAR_K0 + (j & 1), kTileBytes);
-        ++k_sent;
-      };
-      auto fill_v = [&](int j) {
-        load(&map_v, kOffV + (j & 1) * kTileBytes, kSlabBytes, vrow0 + (nt_lo + j) * kBN, BAR_V0 + (j & 1), kTileBytes);
-        ++v_sent;
-      };
-      load(&map_q, kOffQ, kQSlabBytes, (int)qrow0, BAR_Q, 2 * kQSlabBytes);
-      fill_k(0);
-      fill_v(0);
-      if (n_tiles > 1) { fill_k(1); fill_v(1); }
+      int k_sent = min(2, n_tiles), v_sent = k_sent;
       bool ok = true;
       // a slot is refilled as soon as the contraction that read it is complete: K two tiles ahead
       // of the scores that will read it, V two tiles ahead of its O += P V
       for (int it = 0; ok && it + 2 < n_tiles; ++it) {
         if (!(ok = sw_wait(bar(BAR_S0 + (it & 1)), (it >> 1) & 1, ctl, a.status))) break;
         fill_k(it + 2);
+        ++k_sent;
         if (!(ok = sw_wait(bar(BAR_O0 + (it & 1)), (it >> 1) & 1, ctl, a.status))) break;
         fill_v(it + 2);
+        ++v_sent;
       }
       ctl->k_sent = k_sent;
       ctl->v_sent = v_sent;
@@ -366,6 +376,11 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     if (ok) {
       tc_fence_after();
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+      // A whole tile goes through shared memory (where Q was: its last reader is done) and leaves by two
+      // tensor copies; in the last tile of a sequence every thread stores its own row, 256 bytes apart
+      // from its neighbour's, so that no row of the next head is touched.
+      const bool whole = m0 + kBM <= T;
+      const uint32_t orow_s = base + kOffQ + tid * 128;
       __nv_bfloat16* orow = (__nv_bfloat16*)a.o + (qrow0 + tid) * kD;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -375,13 +390,29 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         if (row < T) {
 #pragma unroll
           for (int e = 0; e < 32; e += 8) {
+            const uint32_t c16 = (uint32_t)(4 * c + e / 8);        // 16-byte piece of the row
             uint4 w;
             w.x = pack_bf16(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv);
             w.y = pack_bf16(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
             w.z = pack_bf16(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv);
             w.w = pack_bf16(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv);
-            *reinterpret_cast<uint4*>(orow + 32 * c + e) = w;
+            if (whole) sts128(orow_s + (c16 >> 3) * kQSlabBytes + (((c16 & 7) ^ (uint32_t)(tid & 7)) << 4), w.x, w.y, w.z, w.w);
+            else *reinterpret_cast<uint4*>(orow + 32 * c + e) = w;
           }
+        }
+      }
+      if (whole) {
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_OUT));
+        if (warp == 0) {
+          if (wait(BAR_OUT, 0) && elect_one()) {
+            tma_store_2d(&map_o, 0, (int)qrow0, base + kOffQ);
+            tma_store_2d(&map_o, 64, (int)qrow0, base + kOffQ + kQSlabBytes);
+            bulk_commit();
+            bulk_wait_read<0>();
+          }
+          __syncwarp();
         }
       }
     }
@@ -436,10 +467,10 @@ bool sw_make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint32_t box_ro
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-struct SwMapCache {     // the three maps of the last call on this host thread
-  const void *q = nullptr, *k = nullptr, *v = nullptr;
+struct SwMapCache {     // the four maps of the last call on this host thread
+  const void *q = nullptr, *k = nullptr, *v = nullptr, *o = nullptr;
   uint64_t rows_q = 0, rows_k = 0;
-  CUtensorMap mq, mk, mv;
+  CUtensorMap mq, mk, mv, mo;
 };
 thread_local SwMapCache t_sw_maps;
 std::atomic<unsigned long long> g_sw_tc_smem_done{0};
@@ -450,13 +481,13 @@ cudaError_t launch_swska_tc(const rodimus_swska_fwd_params& p, int* n_launches) 
   *n_launches = 0;
   const uint64_t rows_q = (uint64_t)p.B * p.H * p.T, rows_k = (uint64_t)p.B * p.T;
   SwMapCache& c = t_sw_maps;
-  if (c.q != p.q || c.k != p.k || c.v != p.v || c.rows_q != rows_q || c.rows_k != rows_k) {
+  if (c.q != p.q || c.k != p.k || c.v != p.v || c.o != p.o || c.rows_q != rows_q || c.rows_k != rows_k) {
     if (!sw_make_map(&c.mq, p.q, rows_q, kBM) || !sw_make_map(&c.mk, p.k, rows_k, kBN) ||
-        !sw_make_map(&c.mv, p.v, rows_q, kBN)) {
+        !sw_make_map(&c.mv, p.v, rows_q, kBN) || !sw_make_map(&c.mo, p.o, rows_q, kBM)) {
       c.q = nullptr;
       return cudaErrorInvalidValue;
     }
-    c.q = p.q; c.k = p.k; c.v = p.v; c.rows_q = rows_q; c.rows_k = rows_k;
+    c.q = p.q; c.k = p.k; c.v = p.v; c.o = p.o; c.rows_q = rows_q; c.rows_k = rows_k;
   }
   int dev = 0, sms = 0;
   cudaError_t e = current_device(&dev, &sms);
@@ -477,7 +508,7 @@ cudaError_t launch_swska_tc(const rodimus_swska_fwd_params& p, int* n_launches) 
     if (e != cudaSuccess) return e;
   }
   const dim3 grid((unsigned)n_ctas);
-  swska_fwd_tc_kernel<<<grid, kThreads, kSmemBytes, st>>>(c.mq, c.mk, c.mv, a);
+  swska_fwd_tc_kernel<<<grid, kThreads, kSmemBytes, st>>>(c.mq, c.mk, c.mv, c.mo, a);
   *n_launches = 1;
   return cudaGetLastError();
 }
