@@ -36,14 +36,19 @@
 // scheduler w % 4, and a scheduler's first-level instruction cache holds about 8 KiB, less than
 // the loops of all roles together: the single-warp roles, long straight-line code run once per
 // pass, share scheduler 0, so that the loops of schedulers 1-3 (gate, state, score) stay cached.
-//   warp 0          TMA producer (own channel slab of q,k,x,y and both slabs of the v slice)
+//   warps 0, 24     TMA producers: own channel slab of q,k and both slabs of the v slice; own slab of x,y
 //   warp 4          tcgen05.mma issuer, owns the TMEM allocation
-//   warp 8          control: which fill is an attempt, scan of the row groups' sums, chunk decays,
-//                   verdict exchange and slab copies to the partner, publishing, orders
+//   warp 8          control: which fills are an attempt, chunk decays, verdict exchange and slab
+//                   copies to the partner, publishing, orders
 //   warps 1-3, 12   state group (TMEM quarter = warp % 4): TMEM <-> registers trip of S^T, state I/O
 //   warps 5-7, 16   score / output group
 //   the other 16    gate workers (one on scheduler 0, five on each other): 4 rows x 2 channels
 //                   per thread, packed fp32x2 arithmetic, on orders of the control warp
+//
+// What bounds it: instruction issue.  A pass (64 rows, 3500 cycles) issues about 2300 instructions on
+// each of schedulers 1-3, and their special-function units are busy for 1920 cycles; the tensor cores
+// for 960.  B=4 H=16 T=2048 dv=256: 76.0 us (82.3 before x, y got a ring of their own, the workers
+// their own scan and orders the stage of q, k, v ahead; floor by bytes 42.9).
 //
 // The loop-carried chain is  state update of pass g -> rescaling of S -> state update of pass
 // g+1 , so the issuer puts the state update of a pass BEFORE its output contractions, and the
@@ -66,17 +71,23 @@ constexpr int kDK = 128;                      // key channels
 constexpr int kCH = 64;                       // key channels whose gates one CTA computes
 constexpr int kDVS = 128;                     // value columns per CTA
 constexpr int kSlabBytes = kC * 128;          // [64 rows][64 bf16] = 8 KiB, 128-byte swizzled
-// one stage of the TMA ring: own-channel slabs of q,k,x,y and the two slabs of v
-constexpr int kStQ = 0, kStK = kSlabBytes, kStX = 2 * kSlabBytes, kStY = 3 * kSlabBytes,
-              kStV = 4 * kSlabBytes;
-constexpr int kStageBytes = 6 * kSlabBytes;   // 48 KiB
+// one stage of the TMA ring: own-channel slabs of q,k and the two slabs of v
+constexpr int kStQ = 0, kStK = kSlabBytes, kStV = 2 * kSlabBytes;
+constexpr int kStageBytes = 4 * kSlabBytes;   // 32 KiB
+// The gate logits have a ring of their own: they are done with after phase 1, long before the
+// contractions have read the rest of the tile.  With x and y in the stages of q,k,v the ring of three
+// set the pace (a tile's way from its request to its last contraction, 10500 cycles, over three
+// stages).
+constexpr int kXYStages = 2, kXYBytes = 2 * kSlabBytes;   // x, y
 // one receive buffer: the partner's Qt, Kt slabs
 constexpr int kRxQ = 0, kRxK = kSlabBytes;
 constexpr int kRxBytes = 2 * kSlabBytes;      // 16 KiB
 constexpr int kStages = 3, kRxBufs = 2;
-constexpr int kOperandBytes = kStages * kStageBytes + kRxBufs * kRxBytes;  // 176 KiB
+constexpr int kOperandBytes = kStages * kStageBytes + kRxBufs * kRxBytes;  // 128 KiB
 constexpr int kOtBytes = 2 * kSlabBytes;                  // output tile: two [64 rows][64 bf16] slabs
-constexpr int kOffOt = kOperandBytes;                     // two output tiles (pass parity)
+constexpr int kOffXY = kOperandBytes;                     // ring of x, y
+constexpr int kOffP = kOffXY + kXYStages * kXYBytes;      // masked scores of the pass, [64 rows][64] bf16
+constexpr int kOffOt = kOffP + kSlabBytes;                // two output tiles (pass parity)
 constexpr int kOffDp = kOffOt + 2 * kOtBytes;             // float [4][128]: chunk decays of all
                                                           // channels, per published pass (g & 3)
 constexpr int kBlkFloats = 68;                            // 64 decays, verdict, stage, 2 pad
@@ -86,8 +97,9 @@ constexpr int kOffRx = kOffTx + kRxBufs * kBlkBytes;      // float [2][68]: bloc
 constexpr int kGateWarp0 = 12, kGateWarps = 16;
 constexpr int kGR = kC / kGateWarps;                       // rows per gate thread
 constexpr int kOffTot = kOffRx + kRxBufs * kBlkBytes;     // float [2][8][64]: scan partials
-constexpr int kOffBar = kOffTot + 2 * kGateWarps * kCH * 4;
-constexpr int kNumBars = 40;
+constexpr int kOffAll = kOffTot + 2 * kGateWarps * kCH * 4;   // float [2][64]: decay totals of a tile
+constexpr int kOffBar = kOffAll + 2 * kCH * 4;
+constexpr int kNumBars = 44;
 constexpr int kOffMisc = kOffBar + kNumBars * 8;          // control block
 constexpr int kSmemUsed = kOffMisc + 320;
 constexpr int kSmemBytes = kSmemUsed + 1024;              // slack for manual 1024-byte alignment
@@ -114,9 +126,13 @@ enum { BAR_FULL0 = 0,                 // [3] TMA fill landed                    
        BAR_OTFULL0, BAR_OTFULL1,      // output tile written by the whole score group        (128)
        BAR_OTFREE0, BAR_OTFREE1,      // output tile's copies to global have read it            (1)
        BAR_GO0, BAR_GO1,              // an order for the gate warps is in its slot              (1)
-       BAR_PRE,                       // the row groups' prefixes are in place                   (1)
-       BAR_ROWS,                      // every gate warp has rewritten its rows of the pass
+       BAR_PRE0, BAR_PRE1,            // the order's q, k, v are known and have landed           (1)
+       BAR_TOT,                       // the tile's decay totals are in place                    (1)
+       BAR_ROWS0, BAR_ROWS1,          // every gate warp has rewritten its rows (by parity of the order: the
+                                      // workers may be done with the next one before anybody looks)
        BAR_DRAIN,                     // teardown after a timeout: issued contractions are done  (1)
+       BAR_XYFULL0, BAR_XYFULL1,      // a fill of x, y landed                         (1 + bytes)
+       BAR_XYEMPTY0, BAR_XYEMPTY1,    // phase 1 has read it                                   (1)
        BAR_XFULL0, BAR_XFULL1 };      // feed-through tile x' landed in the output tile (1 + bytes)
 static_assert(BAR_XFULL1 < kNumBars, "barrier count");
 
@@ -206,11 +222,13 @@ struct Control {            // lives in shared memory
   int redir_seq;            // bumped by the gate group after writing redir_j / redir_tpos
   int redir_j, redir_tpos;  // where the producer must continue (CTA-local item index, token)
   int tag[kStages][2];      // per stage: (item index, token position) of the fill it holds
+  int tag_xy[kXYStages][2]; // the same for the ring of x, y
   int pad[2];
   PassDesc pd[4];
-  // orders of the control warp to the gate warps (stage < 0: leave); row and col0 locate the
-  // tile in global memory for the value gate
-  struct { int stage, nr, col0, pad; long long row; } ord[2];
+  // orders of the control warp to the gate warps: stage of x, y (< 0: leave) and, written before
+  // its BAR_PRE, the stage of q, k, v (< 0: the order is dropped); row and col0 locate the tile in
+  // global memory for the value gate
+  struct { int xy, nr, col0, stage; long long row; } ord[2];
 };
 static_assert(sizeof(Control) <= 320, "control block");
 
@@ -256,9 +274,15 @@ __device__ __forceinline__ float2 gate_phase1(uint32_t xs, uint32_t ys, const ui
     } else {                                                            // tau * log2(sigmoid(x))
       eh[i] = __fmul2_rn(ntau, __ffma2_rn(xl, splat(-1.f), sp2));
     }
-    if (row0 + i >= nr) l2a = splat(0.f);                               // rows past the pass
     run = __fadd2_rn(run, l2a);
     b[i] = run;
+  }
+  // rows past the pass count for nothing (phase 2 overwrites what it makes of them)
+  if (row0 + kGR > nr) {
+    run = splat(0.f);
+#pragma unroll
+    for (int i = 0; i < kGR; ++i)
+      if (row0 + i < nr) run = b[i];
   }
   return run;
 }
@@ -275,15 +299,22 @@ __device__ __forceinline__ void gate_phase2(uint32_t qs, uint32_t ks, const uint
     const float2 bb = __fadd2_rn(b[i], pre);
     const float2 hb = __ffma2_rn(bb, splat(-1.f), eh[i]);
     const float2 ek = make_float2(ex2f(hb.x), ex2f(hb.y));
-    if (row0 + i >= nr) k = splat(0.f);
     const float2 kt = __fmul2_rn(k, ek);
     sts32(ks + off[i], pack_bf16(kt.x, kt.y));
     if (!STATE_ONLY) {
       float2 q = bf16x2_to_f2(lds32(qs + off[i]));
       const float2 eq = make_float2(ex2f(bb.x), ex2f(bb.y));
-      if (row0 + i >= nr) q = splat(0.f);
       const float2 qt = __fmul2_rn(q, eq);
       sts32(qs + off[i], pack_bf16(qt.x, qt.y));
+    }
+  }
+  if (row0 + kGR > nr) {   // rows past the pass
+#pragma unroll
+    for (int i = 0; i < kGR; ++i) {
+      if (row0 + i >= nr) {
+        sts32(ks + off[i], 0u);
+        if (!STATE_ONLY) sts32(qs + off[i], 0u);
+      }
     }
   }
 }
@@ -312,18 +343,19 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   volatile float* sTx = reinterpret_cast<volatile float*>(gbase + kOffTx);
   volatile float* sRx = reinterpret_cast<volatile float*>(gbase + kOffRx);
   float* sTot = reinterpret_cast<float*>(gbase + kOffTot);
+  float* sAll = reinterpret_cast<float*>(gbase + kOffAll);
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   // Warp w runs on scheduler w % 4.  The single-warp roles (long straight-line code once per pass)
   // all sit on scheduler 0 together with one gate worker; schedulers 1-3 run five gate workers,
   // a state warp and a score warp each, whose loops fit the scheduler's instruction cache.
-  // role: 0 producer, 1 issuer, 2 control, 3 state, 4 score, 5 gate worker, 6 none
+  // role: 0 producers, 1 issuer, 2 control, 3 state, 4 score, 5 gate worker
   int role, gw_of_warp = 0;
   if (warp == 0) role = 0;
   else if (warp == 4) role = 1;
   else if (warp == 8) role = 2;
-  else if (warp == 24) role = 6;
+  else if (warp == 24) role = 0;
   else if (warp == 12 || warp < 4) role = 3;
   else if (warp == 16 || warp < 8) role = 4;
   else {
@@ -372,37 +404,53 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     mbar_init(bar(BAR_GSCAN), kGateWarps);
     mbar_init(bar(BAR_GO0), 1);
     mbar_init(bar(BAR_GO1), 1);
-    mbar_init(bar(BAR_PRE), 1);
+    mbar_init(bar(BAR_PRE0), 1);
+    mbar_init(bar(BAR_PRE1), 1);
+    mbar_init(bar(BAR_TOT), 1);
     mbar_init(bar(BAR_DRAIN), 1);
     mbar_init(bar(BAR_XFULL0), 1);
     mbar_init(bar(BAR_XFULL1), 1);
-    mbar_init(bar(BAR_ROWS), kGateWarps);
+    mbar_init(bar(BAR_ROWS0), kGateWarps);
+    mbar_init(bar(BAR_ROWS1), kGateWarps);
+    for (int i = 0; i < kXYStages; ++i) {
+      mbar_init(bar(BAR_XYFULL0 + i), 1);
+      mbar_init(bar(BAR_XYEMPTY0 + i), 1);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // One 64-row tile of this CTA's operands into stage s (this thread is the producer).
+  // One 64-row tile of this CTA's operands into stage s of the ring of q,k,v, or of that of x,y (this
+  // thread is the ring's producer).  Rows beyond the tensor read as zeros; rows of the next sequence are
+  // masked later.  The tile that will go into this stage NEXT time is asked into L2 now: a stage is
+  // refilled only when its pass has been consumed, so the fill's latency is on the critical cycle of
+  // the ring, and from L2 it is less than half of what it is from HBM.
+  const int xc = rank * kCH;
+  auto issue_xy = [&](uint32_t s, const Item& it, int j, int tpos) {
+    ctl->tag_xy[s][0] = j;
+    ctl->tag_xy[s][1] = tpos;
+    const uint32_t st = base + kOffXY + s * kXYBytes, fb = bar(BAR_XYFULL0 + s);
+    const int yq = (int)(it.rowq + tpos);
+    mbar_expect_tx(fb, kXYBytes);
+    tma_load_2d(st, &map_x, xc, yq, fb);
+    tma_load_2d(st + kSlabBytes, &map_y, xc, yq, fb);
+    if (tpos + kXYStages * kC < it.len) {
+      tma_prefetch_2d(&map_x, xc, yq + kXYStages * kC);
+      tma_prefetch_2d(&map_y, xc, yq + kXYStages * kC);
+    }
+  };
   auto issue_fill = [&](uint32_t s, const Item& it, int j, int tpos) {
     ctl->tag[s][0] = j;
     ctl->tag[s][1] = tpos;
     const uint32_t st = stage_base + s * kStageBytes;
     const uint32_t fb = bar(BAR_FULL0 + s);
     mbar_expect_tx(fb, STATE_ONLY ? kStageBytes - kSlabBytes : kStageBytes);
-    // rows beyond the tensor read as zeros; rows of the next sequence are masked later
     const int y = (int)(it.row0 + tpos);
     const int yq = (int)(it.rowq + tpos);
-    const int xc = rank * kCH;
-    tma_load_2d(st + kStX, &map_x, xc, yq, fb);
-    tma_load_2d(st + kStY, &map_y, xc, yq, fb);
-    if (!STATE_ONLY) tma_load_2d(st + kStQ, &map_q, xc, yq, fb);
     tma_load_2d(st + kStK, &map_k, xc, yq, fb);
+    if (!STATE_ONLY) tma_load_2d(st + kStQ, &map_q, xc, yq, fb);
     tma_load_2d(st + kStV, &map_v, it.col0, y, fb);
     tma_load_2d(st + kStV + kSlabBytes, &map_v, it.col0 + 64, y, fb);
-    // The tile that will go into this stage NEXT time is asked into L2 now: a stage is refilled
-    // only when its pass has been consumed, so the fill's latency is on the critical cycle of
-    // the ring, and from L2 it is less than half of what it is from HBM.
     const int yp = y + kStages * kC, yqp = yq + kStages * kC;
     if (tpos + kStages * kC < it.len) {
-      tma_prefetch_2d(&map_x, xc, yqp);
-      tma_prefetch_2d(&map_y, xc, yqp);
       if (!STATE_ONLY) tma_prefetch_2d(&map_q, xc, yqp);
       tma_prefetch_2d(&map_k, xc, yqp);
       tma_prefetch_2d(&map_v, it.col0, yp);
@@ -417,15 +465,18 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
     }
   };
-  // The first fill touches only this CTA's own barriers and shared memory, so it goes out
+  // The first fills touch only this CTA's own barriers and shared memory, so they go out
   // before the tensor-memory allocation and the cluster handshake instead of after them.
   uint32_t early_fills = 0;
-  if (tid == 0) {
+  if (role == 0) {
     const long long item0 = (long long)(blockIdx.x >> 1);
     if (item0 < a.n_items) {
       const Item it = decode_item(a, item0, rank);
       if (it.len > 0) {
-        issue_fill(0, it, 0, 0);
+        if (tid == 0) {
+          issue_xy(0, it, 0, 0);
+          issue_fill(0, it, 0, 0);
+        }
         early_fills = 1;
       }
     }
@@ -447,16 +498,20 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   auto item_of = [&](int j) { return pair_id + (long long)j * n_pairs_grid; };
 
   if (role == 0) {
-    // ===================================== TMA producer =====================================
+    // ============================ TMA producers, one warp per ring ============================
+    const bool xy = warp != 0;
+    const uint32_t stages = xy ? kXYStages : kStages;
+    const int full0 = xy ? BAR_XYFULL0 : BAR_FULL0, empty0 = xy ? BAR_XYEMPTY0 : BAR_EMPTY0;
     if (elect_one()) {
       uint32_t f = early_fills;            // fills issued
       uint32_t s = early_fills, ph = 0;    // stage and phase of fill f
       int j = 0, tpos = early_fills * kC;  // speculative position: item index and token
       int seen = 0;           // last redirect taken
+      int jd = -1;            // item that `it` describes
+      Item it;
       bool ok = true;
       while (ok) {
-        if (!(ok = mbar_wait_cluster(bar(BAR_EMPTY0 + s), ph ^ 1, abort_flag, a.hdr))) break;
-        Item it;
+        if (!(ok = mbar_wait_cluster(bar(empty0 + s), ph ^ 1, abort_flag, a.hdr))) break;
         bool have = false;
         const long long t0 = clock64();
         while (true) {
@@ -468,7 +523,10 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             seen = sq;
           }
           while (item_of(j) < a.n_items) {   // next position that has tokens left
-            it = decode_item(a, item_of(j), rank);
+            if (j != jd) {
+              it = decode_item(a, item_of(j), rank);
+              jd = j;
+            }
             if (tpos < it.len) { have = true; break; }
             ++j;
             tpos = 0;
@@ -482,16 +540,17 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           __nanosleep(100);
         }
         if (!have) break;
-        issue_fill(s, it, j, tpos);
+        if (xy) issue_xy(s, it, j, tpos);
+        else issue_fill(s, it, j, tpos);
         ++f;
-        if (++s == kStages) { s = 0; ph ^= 1; }
+        if (++s == stages) { s = 0; ph ^= 1; }
         tpos += kC;
       }
       // Leave no bulk copy in flight when the CTA exits: the last fills' barriers complete by
       // byte count, whoever consumed them.
-      for (uint32_t back = 1; back <= (uint32_t)kStages && back <= f; ++back) {
+      for (uint32_t back = 1; back <= stages && back <= f; ++back) {
         const uint32_t ff = f - back;
-        mbar_drain(bar(BAR_FULL0 + ff % kStages), (ff / kStages) & 1);
+        mbar_drain(bar(full0 + ff % stages), (ff / stages) & 1);
       }
     }
   } else if (role == 1) {
@@ -531,7 +590,7 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           const uint32_t dkt = desc_lo_mnmajor(k_lo_addr, k_hi_addr - k_lo_addr);
           // V as [rows][128 value columns], two 64-column slabs
           const uint32_t dv = desc_lo_mnmajor(st + kStV, kSlabBytes);
-          const uint32_t dp = desc_lo_kmajor(st + kStY);
+          const uint32_t dp = desc_lo_kmajor(base + kOffP);
           const uint32_t t_sb = tmem + kColSb + (g & 1) * 64;
           tc_fence_after();
           // P = Qt Kt^T : M = 64 (rows r), N = 64 (rows i), K = 128 channels
@@ -557,7 +616,7 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           if (!(ok = mbar_wait(bar(BAR_OFREE), ph1 ^ 1, abort_flag, a.hdr))) break;
           tc_fence_after();
           // O^T = V^T P^T : M = 128 value columns, N = 64 rows r, K = 64 rows i (the masked
-          // scores P[r][i] live in the consumed y slab)
+          // scores P[r][i])
           umma_bf16_lo<false>(tmem + kColO, dv, dp, kIdescOv);
 #pragma unroll
           for (int kk = 1; kk < 4; ++kk) umma_bf16_lo<true>(tmem + kColO, dv + 128 * kk, dp + 2 * kk, kIdescOv);
@@ -731,13 +790,12 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           continue;
         }
         if (!(ok = mbar_wait(bar(BAR_PFULL), ph1, abort_flag, a.hdr))) break;
-        const int s = ctl->pd[g & 3].stage;
         const int nr = ctl->pd[g & 3].nr;
         const long long row = ctl->pd[g & 3].row;
         last = (ctl->pd[g & 3].flags & kPassLast) != 0;
         // row of the P tile ([r][i], 128-byte rows, 16-byte chunks swizzled by r & 7) whose
         // address this thread supplies to stmatrix: row block mat_h, row mat_k within it
-        const uint32_t ps_mat = stage_base + s * kStageBytes + kStY + (q4 * 16 + mat_h * 8 + mat_k) * 128;
+        const uint32_t ps_mat = base + kOffP + (q4 * 16 + mat_h * 8 + mat_k) * 128;
         tc_fence_after();
         const bool feed = BLOCK && a.feed_d != nullptr;
         if (feed && q4 == 0) {
@@ -888,10 +946,11 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   } else if (role == 5 || role == 2) {
     // ============================== gate group and its control warp ==============================
     // The gate warps are workers: for every order of the control warp (a stage and a row count)
-    // they run phase 1 on their rows, hand in the column sums, wait for their prefix, run phase
-    // 2 and report.  Everything serial or rare lives in the control warp: which fill is an
-    // attempt, the scan over the 16 row groups, decays, verdict exchange, the copies to the
-    // partner, refusals and redirects, publishing the pass.
+    // they run phase 1 on their rows, hand in the column sums, add up those of the row groups
+    // before their own, run phase 2 and report.  (With the scan in the control warp every worker
+    // waited about 1000 cycles of a pass for it.)  Everything serial or rare lives in the control
+    // warp: which fill is an attempt, decays, verdict exchange, the copies to the partner, refusals
+    // and redirects, publishing the pass.
     const int gw = gw_of_warp;                            // rows kGR*gw .. kGR*gw+kGR-1 of the tile
     const bool is_ctl = role == 2;
     bool ok = true;
@@ -904,53 +963,72 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
       for (uint32_t oc = 0;; ++oc) {                      // order counter
         if (!mbar_wait(bar(BAR_GO0 + (oc & 1)), (oc >> 1) & 1, abort_flag, a.hdr)) break;
-        const int s = ctl->ord[oc & 1].stage;
+        const int xs = ctl->ord[oc & 1].xy;
         const int nr = ctl->ord[oc & 1].nr;
-        if (s < 0) break;                                 // no more work
-        const uint32_t st = stage_base + (uint32_t)s * kStageBytes;
-        float* tot = sTot + (oc & 1) * (kGateWarps * kCH) + gw * kCH + 2 * lane;
-        float2 b[kGR], eh[kGR];
-        const float2 run = gate_phase1<INGATE>(st + kStX, st + kStY, off, gw * kGR, nr, b, eh);
-        *reinterpret_cast<float2*>(tot) = run;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(BAR_GSCAN));
-        if (BLOCK && a.beta_hat) {
-          // Value gate (Eq. "beta_def"): the v tile becomes beta_hat . v in place, while the
-          // control warp scans.  Every gate thread takes its share of 16-byte chunks (8 value columns); the
-          // gate comes straight from global memory (asked into L2 when the stage was filled).
+        if (xs < 0) break;                                // no more work
+        const uint32_t xt = base + kOffXY + (uint32_t)xs * kXYBytes;
+        float* tot0 = sTot + (oc & 1) * (kGateWarps * kCH) + 2 * lane;
+        // Value gate (Eq. "beta_def"): the v tile becomes beta_hat . v in place.  Every gate thread takes
+        // its share of 16-byte chunks (8 value columns) of the [64 rows][16 chunks] tile; the gate comes
+        // straight from global memory (asked into L2 when the stage was filled), and phase 1 covers its way.
+        constexpr int kGateChunks = BLOCK ? kC * 16 / (kGateWarps * 32) : 1;
+        uint4 g4[kGateChunks];
+        const bool gate_v = BLOCK && a.beta_hat;
+        if (gate_v) {
           const long long row = ctl->ord[oc & 1].row;
           const int col0 = ctl->ord[oc & 1].col0;
 #pragma unroll
-          for (int u = 0; u < kC * 16 / (kGateWarps * 32); ++u) {
-            const int ci = gw * 32 + lane + kGateWarps * 32 * u;   // chunk of the [64 rows][16 chunks] tile
-            const int r = ci >> 4, c16 = ci & 15;
-            if (r < nr) {
-              const uint4 g4 = __ldg(reinterpret_cast<const uint4*>(
-                  a.beta_hat + (row + r) * a.dv + col0 + c16 * 8));
-              const uint32_t va = st + kStV + (c16 >> 3) * kSlabBytes + r * 128 +
-                                  ((((uint32_t)c16 & 7u) ^ ((uint32_t)r & 7u)) << 4);
-              uint4 v4 = lds128(va);
-              v4.x = hmul2_bf16(v4.x, g4.x);
-              v4.y = hmul2_bf16(v4.y, g4.y);
-              v4.z = hmul2_bf16(v4.z, g4.z);
-              v4.w = hmul2_bf16(v4.w, g4.w);
-              sts128(va, v4.x, v4.y, v4.z, v4.w);
-            }
+          for (int u = 0; u < kGateChunks; ++u) {
+            const int ci = gw * 32 + lane + kGateWarps * 32 * u, r = ci >> 4, c16 = ci & 15;
+            if (r < nr) g4[u] = __ldg(reinterpret_cast<const uint4*>(a.beta_hat + (row + r) * a.dv + col0 + c16 * 8));
           }
         }
-        // the control warp replaces each row group's sum by the sum of the groups before it
-        if (!mbar_wait(bar(BAR_PRE), oc & 1, abort_flag, a.hdr)) break;
-        const float2 pre = *reinterpret_cast<const float2*>(tot);
-        gate_phase2<STATE_ONLY>(st + kStQ, st + kStK, off, gw * kGR, nr, pre, b, eh);
+        float2 b[kGR], eh[kGR];
+        const float2 run = gate_phase1<INGATE>(xt, xt + kSlabBytes, off, gw * kGR, nr, b, eh);
+        *reinterpret_cast<float2*>(tot0 + gw * kCH) = run;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_GSCAN));
+        // sum of the row groups before this one; the last group's warp hands the tile's totals to
+        // the control warp
+        if (!mbar_wait(bar(BAR_GSCAN), oc & 1, abort_flag, a.hdr)) break;
+        float2 pre = splat(0.f);
+#pragma unroll 4
+        for (int w = 0; w < gw; ++w) pre = __fadd2_rn(pre, *reinterpret_cast<const float2*>(tot0 + w * kCH));
+        if (gw == kGateWarps - 1) {
+          *reinterpret_cast<float2*>(sAll + (oc & 1) * kCH + 2 * lane) = __fadd2_rn(pre, run);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(BAR_TOT));
+        }
+        // the order's stage of q, k, v; negative: the order is dropped
+        if (!mbar_wait(bar(BAR_PRE0 + (oc & 1)), (oc >> 1) & 1, abort_flag, a.hdr)) break;
+        const int s = ctl->ord[oc & 1].stage;
+        if (s >= 0) {
+          const uint32_t st = stage_base + (uint32_t)s * kStageBytes;
+          if (gate_v) {
+#pragma unroll
+            for (int u = 0; u < kGateChunks; ++u) {
+              const int ci = gw * 32 + lane + kGateWarps * 32 * u, r = ci >> 4, c16 = ci & 15;
+              if (r < nr) {
+                const uint32_t va = st + kStV + (c16 >> 3) * kSlabBytes + r * 128 +
+                                    ((((uint32_t)c16 & 7u) ^ ((uint32_t)r & 7u)) << 4);
+                const uint4 v4 = lds128(va);
+                sts128(va, hmul2_bf16(v4.x, g4[u].x), hmul2_bf16(v4.y, g4[u].y), hmul2_bf16(v4.z, g4[u].z),
+                       hmul2_bf16(v4.w, g4[u].w));
+              }
+            }
+          }
+          gate_phase2<STATE_ONLY>(st + kStQ, st + kStK, off, gw * kGR, nr, pre, b, eh);
+        }
         // the rewritten rows are visible to the bulk-copy engine and to the tensor core; the
         // control warp sends the whole slabs to the partner once every gate warp has said so
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(BAR_ROWS));
+        if (lane == 0) mbar_arrive(bar(BAR_ROWS0 + (oc & 1)));
       }
     } else {
       const bool leader = lane == 0;
-      uint32_t fs = 0, fph = 0;                           // stage and phase of the next fill
+      uint32_t fs = 0, fph = 0;                           // stage and phase of the next fill of q, k, v
+      uint32_t xs = 0, xph = 0;                           // the same of x, y
       uint32_t g = 0, m = 0, oc = 0;                      // passes, exchanged attempts, orders given
       bool armed = false;                                 // attempt m's receive barriers expect bytes
       uint32_t sent_blk = 0, sent_slab = 0;               // leader: copies issued to the partner
@@ -962,9 +1040,9 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       };
       // Order number oc goes into slot oc & 1.  The workers read order oc-2 before they reported
       // on it, and at most two orders are outstanding.
-      auto give_order = [&](int stage, int nr, long long row = 0, int col0 = 0) {
+      auto give_order = [&](int xy, int nr, long long row = 0, int col0 = 0) {
         if (leader) {
-          ctl->ord[oc & 1].stage = stage;
+          ctl->ord[oc & 1].xy = xy;
           ctl->ord[oc & 1].nr = nr;
           if (BLOCK) {
             ctl->ord[oc & 1].row = row;
@@ -991,65 +1069,85 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // fill - if it has landed and is the tile that follows when the attempt is accepted - is
       // ordered at once, so that the workers never wait for the control warp's serial tail
       // (copies to the partner, verdict, publishing).  If the attempt is then refused, the
-      // order ahead is carried through (the workers are on it) and its stage handed back unused.
-      bool ahead = false;
-      uint32_t ahead_s = 0;
+      // order ahead is carried through (the workers are on it) and dropped after phase 1.
+      bool ahead = false, ahead_q = false;
+      uint32_t ahead_x = 0, ahead_s = 0, cur_s = 0;
       int ahead_nr = 0;
+      // the workers learn which stage holds the q, k, v of order o (or that the order is dropped)
+      auto tell_stage = [&](uint32_t o, int stage) {
+        if (leader) {
+          ctl->ord[o & 1].stage = stage;
+          mbar_arrive(bar(BAR_PRE0 + (o & 1)));
+        }
+      };
+      // q, k, v of order o, which is for position (jj, tt): the next fill that is for this position;
+      // fills for others (speculation that did not hold) go back unused
+      auto take_q = [&](int jj, int tt, uint32_t o) -> bool {
+        while (true) {
+          cur_s = fs;
+          if (!mbar_wait(bar(BAR_FULL0 + cur_s), fph, abort_flag, a.hdr)) return false;
+          if (++fs == kStages) { fs = 0; fph ^= 1; }
+          if (ctl->tag[cur_s][0] == jj && ctl->tag[cur_s][1] == tt) break;
+          __syncwarp();
+          if (leader) mbar_arrive_cnt(bar(BAR_EMPTY0 + cur_s), 2);   // nothing was sent from it
+        }
+        tell_stage(o, (int)cur_s);
+        return true;
+      };
       while (ok && have) {
-        uint32_t s;
+        uint32_t x;                                       // stage of the attempt's x, y
         int nr;
+        bool have_q = false;
         const int left = it.len - tpos;
         if (ahead) {
-          s = ahead_s;
+          x = ahead_x;
           nr = ahead_nr;
-          ahead = false;
+          have_q = ahead_q;
+          cur_s = ahead_s;
+          ahead = ahead_q = false;
         } else {
-          s = fs;
-          if (!(ok = mbar_wait(bar(BAR_FULL0 + s), fph, abort_flag, a.hdr))) break;
-          if (++fs == kStages) { fs = 0; fph ^= 1; }
-          if (ctl->tag[s][0] != j || ctl->tag[s][1] != tpos) {
+          x = xs;
+          if (!(ok = mbar_wait(bar(BAR_XYFULL0 + x), xph, abort_flag, a.hdr))) break;
+          if (++xs == kXYStages) { xs = 0; xph ^= 1; }
+          if (ctl->tag_xy[x][0] != j || ctl->tag_xy[x][1] != tpos) {
             // speculative fill for a position we are not at: hand the stage back unused
-            if (leader) mbar_arrive_cnt(bar(BAR_EMPTY0 + s), 2);   // nothing was sent from it
+            if (leader) mbar_arrive(bar(BAR_XYEMPTY0 + x));
             continue;
           }
           nr = min(min(kC, left), lcap);
-          give_order((int)s, nr, it.row0 + tpos, it.col0);
+          give_order((int)x, nr, it.row0 + tpos, it.col0);
         }
-        const uint32_t st = stage_base + s * kStageBytes;
         const uint32_t ocur = oc - 1;                     // the order of this attempt
         // ---- the position that follows if this attempt is accepted, and the order ahead
         int nj = j, ntpos = tpos + nr, nlcap = lcap < kC ? min(kC, lcap * 2) : kC;
         Item nit = it;
         const bool nhave = ntpos < it.len ? true : seek(nj, nit, ntpos);
         auto try_ahead = [&]() {
-          if (ahead || !nhave || !mbar_test(bar(BAR_FULL0 + fs), fph)) return;
-          if (ctl->tag[fs][0] != nj || ctl->tag[fs][1] != ntpos) return;
+          if (!nhave || !__all_sync(0xffffffffu, mbar_test(bar(BAR_XYFULL0 + xs), xph))) return;
+          if (ctl->tag_xy[xs][0] != nj || ctl->tag_xy[xs][1] != ntpos) return;
           ahead = true;
-          ahead_s = fs;
+          ahead_x = xs;
           ahead_nr = min(min(kC, nit.len - ntpos), nlcap);
+          if (++xs == kXYStages) { xs = 0; xph ^= 1; }
+          give_order((int)ahead_x, ahead_nr, nit.row0 + ntpos, nit.col0);
+          // its q, k, v as well, if they are there already
+          if (!__all_sync(0xffffffffu, mbar_test(bar(BAR_FULL0 + fs), fph)) || ctl->tag[fs][0] != nj || ctl->tag[fs][1] != ntpos) return;
+          ahead_q = true;
+          ahead_s = fs;
           if (++fs == kStages) { fs = 0; fph ^= 1; }
-          give_order((int)ahead_s, ahead_nr, nit.row0 + ntpos, nit.col0);
+          tell_stage(oc - 1, (int)ahead_s);
         };
         // ---- attempt m
         const uint32_t rxi = m & 1, rxph = (m >> 1) & 1;
-        float* tot = sTot + (ocur & 1) * (kGateWarps * kCH) + 2 * lane;
-        if (!(ok = mbar_wait(bar(BAR_GSCAN), ocur & 1, abort_flag, a.hdr))) break;
-        // scan over the row groups (this lane: two channels): each group's sum becomes the sum
-        // of the groups before it; the total gives the chunk decays and the verdict
-        float2 all = splat(0.f);
-        {
-          float2 t[kGateWarps];
-#pragma unroll
-          for (int w = 0; w < kGateWarps; ++w) t[w] = *reinterpret_cast<const float2*>(tot + w * kCH);
-#pragma unroll
-          for (int w = 0; w < kGateWarps; ++w) {
-            *reinterpret_cast<float2*>(tot + w * kCH) = all;
-            all = __fadd2_rn(all, t[w]);
-          }
+        if (!have_q) {
+          if (!(ok = take_q(j, tpos, ocur))) break;
         }
-        __syncwarp();
-        if (leader) mbar_arrive(bar(BAR_PRE));
-        try_ahead();                                      // if the next fill had not landed before
+        const uint32_t s = cur_s, st = stage_base + s * kStageBytes;
+        if (!(ok = mbar_wait(bar(BAR_TOT), ocur & 1, abort_flag, a.hdr))) break;
+        if (leader) mbar_arrive(bar(BAR_XYEMPTY0 + x));   // phase 1 has read x, y
+        // the decay totals (this lane: two channels) give the chunk decays and the verdict
+        const float2 all = *reinterpret_cast<const float2*>(sAll + (ocur & 1) * kCH + 2 * lane);
+        try_ahead();                                      // while the workers are in phase 2
         const bool viol_own = __any_sync(0xffffffffu, all.x < -kRange || all.y < -kRange) && nr > 1;
         const float2 D = make_float2(ex2f(all.x), ex2f(all.y));
         // the send block m&1 (like the partner's receive buffer m&1) must be free again
@@ -1085,8 +1183,7 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // both operand slabs of the attempt go to the partner in one copy each (also when the
         // attempt turns out to be abandoned: the byte count the partner's barrier expects is
         // fixed); the partner's receive buffer m&1 is free, see above
-        try_ahead();                                      // second chance: the fill may have landed by now
-        if (!(ok = mbar_wait(bar(BAR_ROWS), ocur & 1, abort_flag, a.hdr))) break;
+        if (!(ok = mbar_wait(bar(BAR_ROWS0 + (ocur & 1)), (ocur >> 1) & 1, abort_flag, a.hdr))) break;
         if (leader) {
           const uint32_t dst = peer_rx_base + rxi * kRxBytes;
           const uint32_t pb = map_to_cta(bar(BAR_PEER0 + rxi), peer);
@@ -1105,11 +1202,12 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           if (ahead) {
             // carry the order ahead through with the workers, then drop it
             const uint32_t oa = oc - 1;
-            if (!(ok = mbar_wait(bar(BAR_GSCAN), oa & 1, abort_flag, a.hdr))) break;
-            if (leader) mbar_arrive(bar(BAR_PRE));
-            if (!(ok = mbar_wait(bar(BAR_ROWS), oa & 1, abort_flag, a.hdr))) break;
-            if (leader) mbar_arrive_cnt(bar(BAR_EMPTY0 + ahead_s), 2);
-            ahead = false;
+            if (!(ok = mbar_wait(bar(BAR_TOT), oa & 1, abort_flag, a.hdr))) break;
+            if (leader) mbar_arrive(bar(BAR_XYEMPTY0 + ahead_x));
+            if (!ahead_q) tell_stage(oa, -1);
+            if (!(ok = mbar_wait(bar(BAR_ROWS0 + (oa & 1)), (oa >> 1) & 1, abort_flag, a.hdr))) break;
+            if (ahead_q && leader) mbar_arrive_cnt(bar(BAR_EMPTY0 + ahead_s), 2);   // nothing was sent from it
+            ahead = ahead_q = false;
           }
           // whatever the partner sent for this attempt must have landed before its buffer
           // and its stage are declared reusable
