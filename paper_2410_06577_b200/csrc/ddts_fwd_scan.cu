@@ -422,6 +422,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
           if (lo == 0 && t + C::kAStages < ntiles) {   // asked into L2 before its stage is free
             tma_prefetch_3d(&maps.v, 0, (int)row + C::kAStages * kTile, col0 >> 6);
             if (beta) tma_prefetch_3d(&maps.beta, 0, (int)row + C::kAStages * kTile, col0 >> 6);
+            if (BLOCK && a.feed_d) tma_prefetch_3d(&maps.fx, 0, (int)row + C::kAStages * kTile, col0 >> 6);
           }
           if (++s == C::kAStages) { s = 0; ph ^= 1; }
           if (!(ok = mbar_wait(bar(FB_QEMPTY0 + qs), qph, wc, hdr))) break;
@@ -504,17 +505,34 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   } else if (warp == 2) {
     // ================================= output tiles to global ==============================
     // Feed-through: the x' tile of a pass is fetched INTO its output tile, to be combined with the
-    // accumulators in place.
+    // accumulators in place; two passes ahead, as soon as the copies have read that tile (one pass ahead
+    // a fetch and a store were on the way of every pass: 2.7 us a tile instead of 1.2).
     const bool feed = BLOCK && a.feed_d != nullptr;
-    auto fetch_x = [&](int c, long long row) {
+    int xt = 0, xlo = 0;                               // tile and first row of the next chunk to fetch for
+    auto mask_of = [&](int t) {
+      return __ldcg(reinterpret_cast<const unsigned long long*>(a.blocks + (slot0 + t) * B::kBytes + B::kHead));
+    };
+    unsigned long long xmask = feed && ntiles > 0 ? mask_of(0) : 0ull;
+    auto fetch_x = [&](int c) {
+      if (xt >= ntiles) return;
       if (elect_one()) {
         mbar_expect_tx(bar(FB_XFULL0 + (c & 1)), 2 * kSlab);
-        tma_load_3d(base + C::kOffOt + (c & 1) * 2 * kSlab, &maps.fx, 0, (int)row, col0 >> 6, bar(FB_XFULL0 + (c & 1)));
+        tma_load_3d(base + C::kOffOt + (c & 1) * 2 * kSlab, &maps.fx, 0, (int)(row0 + (long long)xt * kTile), col0 >> 6,
+                    bar(FB_XFULL0 + (c & 1)));
         ctl->n_x = c + 1;
       }
       __syncwarp();
+      const int nr = min(kTile, len - xt * kTile);
+      xlo = chunk_end(xmask, xlo, nr);
+      if (xlo == nr) {
+        xlo = 0;
+        if (++xt < ntiles) xmask = mask_of(xt);
+      }
     };
-    if (feed && ntiles > 0) fetch_x(0, row0);
+    if (feed) {
+      fetch_x(0);
+      fetch_x(1);
+    }
     for (int c = 0; ntiles > 0; ++c) {
       const uint32_t pr = c & 1;
       const uint32_t ot = base + C::kOffOt + pr * 2 * kSlab;
@@ -542,7 +560,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(FB_OTFREE0 + pr));
       if (last) break;
-      if (feed) fetch_x(c + 1, hi == kTile ? row + kTile : row);
+      if (feed) fetch_x(c + 2);
     }
   } else if (warp == 3) {
     // ================================= chunks of cut tiles =================================
