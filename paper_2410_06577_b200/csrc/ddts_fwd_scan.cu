@@ -253,6 +253,10 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
 // the tensor core works on dS and P V of a chunk while the state that enters it is being formed.  (With
 // the state accumulated in tensor memory instead, the chain update -> scaling -> update took 2270
 // cycles per chunk of dk = 64.)
+// What bounds it at dk = 128: shared memory.  About 160 KiB go through it per pass (57 in by TMA, 72 read
+// by the contractions, 32 for the output tile), 1300 of the pass's 1500 cycles at 128 bytes a clock; the
+// value gate and the feed-through add 96 KiB (2500 cycles a pass).  Twice as many state warps, or dS of
+// the next pass issued before the readout of this one, change nothing or cost 2 to 4 %.
 // Roles: warp 0 loads, 1 issues the contractions, 2 sends the output tiles (and fetches the feed-
 // through's), 3 prepares chunks of cut tiles, 4-11 state group (tensor-memory quarter = warp % 4, half
 // of the key channels each), 12-15 outputs, 16-19 (BLOCK) apply the value gate to the v tile.
@@ -266,9 +270,9 @@ struct Scan {
   static constexpr int kAStage = kOffBeta + (BLOCK ? 2 * kSlab : 0);
   static constexpr int kOffQ = kAStages * kAStage;
   static constexpr int kOffOt = kOffQ + kQStages * kQBytes;  // two output tiles of two slabs
-  static constexpr int kOffDc = kOffOt + 4 * kSlab;          // float [4][DK]: decays of chunks of cut tiles
-  static constexpr int kOffBar = kOffDc + 4 * DK * 4;
-  static constexpr int kOffCtl = kOffBar + 40 * 8;
+  static constexpr int kOffDc = kOffOt + 4 * kSlab;          // float [8][DK]: decays of chunks of cut tiles
+  static constexpr int kOffBar = kOffDc + 8 * DK * 4;
+  static constexpr int kOffCtl = kOffBar + 48 * 8;
   static constexpr int kSmem = kOffCtl + 512 + 1024;         // + slack for 1024-byte alignment
   static constexpr int kThreads = BLOCK ? 640 : 512;
   // dk = 64: the high and middle parts of Kt lie one behind the other in shared memory and are taken as
@@ -291,9 +295,9 @@ enum { FB_AFULL0 = 0,                   // [3] Kt, P, v landed                  
        FB_OTFULL0, FB_OTFULL1,          // output tile written                          (4 warps)
        FB_OTFREE0, FB_OTFREE1,          // output tile's copies have read it            (1)
        FB_XFULL0, FB_XFULL1,            // feed-through tile landed in the output tile  (1 + bytes)
-       FB_CUT0,                         // [4] a chunk of a cut tile is prepared        (1)
-       FB_DRAIN = FB_CUT0 + 4, FB_COUNT };
-static_assert(FB_COUNT <= 40, "barrier count");
+       FB_CUT0,                         // [8] a chunk of a cut tile is prepared        (1)
+       FB_DRAIN = FB_CUT0 + 8, FB_COUNT };
+static_assert(FB_COUNT <= 48, "barrier count");
 
 struct PassDesc {
   long long row;       // first row of the tile in v, o
@@ -448,7 +452,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         if (BLOCK && a.has_beta && !mbar_wait(bar(FB_VREADY0 + s), ph, wc, hdr)) break;
         const int flags = ctl->desc[c & 7].flags;
         if (flags & kCutTile) {
-          if (!mbar_wait(bar(FB_CUT0 + (n_cut & 3)), (n_cut >> 2) & 1, wc, hdr)) break;
+          if (!mbar_wait(bar(FB_CUT0 + (n_cut & 7)), (n_cut >> 3) & 1, wc, hdr)) break;
           ++n_cut;
         }
         const uint32_t st = base + s * C::kAStage, sq = base + C::kOffQ + qs * C::kQBytes;
@@ -579,9 +583,9 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
           if (r < lo || r >= hi) sts128(k + e * 16, 0u, 0u, 0u, 0u);
         }
         fence_proxy_async();
-        // (four buffers: this one's last reader, the state's trip two passes on, precedes the
+        // (eight buffers: this one's last reader, the state's trip eight passes back, precedes the
         // contractions whose end let the tile of this pass in)
-        float* dc = reinterpret_cast<float*>(gbase + C::kOffDc) + (n_cut & 3) * DK;
+        float* dc = reinterpret_cast<float*>(gbase + C::kOffDc) + (n_cut & 7) * DK;
         for (int ch = lane; ch < DK; ch += 32) {
           const long long e = d->rowq * DK + ch;
           float acc = 0.f, lh, la;
@@ -592,7 +596,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
           dc[ch] = ex2f(acc);
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(FB_CUT0 + (n_cut & 3)));
+        if (lane == 0) mbar_arrive(bar(FB_CUT0 + (n_cut & 7)));
         ++n_cut;
       }
       __syncwarp();
@@ -671,8 +675,8 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         const int flags = ctl->desc[c & 7].flags;
         const float* D = reinterpret_cast<const float*>(gbase + C::kOffQ + qs * C::kQBytes + (B::kD - B::kQ));
         if (flags & kCutTile) {
-          if (!(ok = wait_all(FB_CUT0 + (n_cut & 3), (n_cut >> 2) & 1))) break;
-          D = reinterpret_cast<const float*>(gbase + C::kOffDc) + (n_cut & 3) * DK;
+          if (!(ok = wait_all(FB_CUT0 + (n_cut & 7), (n_cut >> 3) & 1))) break;
+          D = reinterpret_cast<const float*>(gbase + C::kOffDc) + (n_cut & 7) * DK;
           ++n_cut;
         }
         if ((flags & kLastPass) && !a.sT) break;
