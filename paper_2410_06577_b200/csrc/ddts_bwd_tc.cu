@@ -27,9 +27,9 @@
 //                          sums chained from tile to tile (fp64), dq, dk, dx, dy.
 // What this replaces for bf16 - one launch of 16-row chunks on mma.sync with the gates computed in
 // each of six CTAs per (sequence, head), bound by instruction issue - took 1.79 ms on the layer
-// shape (B=4 H=16 T=2048); this takes 0.39 ms there: 52 us (4.1 TB/s; issue slots 70 % busy) + 215 us
-// (3.6 TB/s of DRAM, shared memory about two thirds busy: per chunk 96 KiB in by TMA, 296 KiB read by
-// the contractions, 96 KiB of expanding Y) + 118 us (issue slots 49 %, latency between its barriers).
+// shape (B=4 H=16 T=2048); this takes 0.35 ms there: 52 us (5.1 TB/s; issue slots 70 % busy) + 180 us
+// (shared memory, see the sweeps) + 120 us (3.3 TB/s; issue slots 50 %, special-function units 41 %, the
+// rest latency: 18 warps on an SM on average, a third of their stalls waiting for loads).
 #include <cuda.h>
 
 #include <cstring>
@@ -60,10 +60,10 @@ struct BwdTcArgs {
   float *c, *c2;              // [n_seq * H][DK]: the constant of the suffix sums, in two halves
   float* seg_state;           // [n_seq * H * 3][32][256] of 16 bytes: state of a sweep cut in two, at the
                               // cut, as the 256 threads of the state group hold it
-  int32_t* seg_flag;          // [n_seq * H * 3]: 8 when that state is there
+  int32_t* seg_flag;          // [n_seq * H * 3]: 8 when that state is there; then the ticket counter
   const int32_t *cu, *order;
   WorkspaceHeader* hdr;
-  long long n_flags;          // entries of seg_flag
+  long long n_flags;          // entries of seg_flag with the counter
   int H, T, n_seq;
   int heads;                  // tile grids: (batch, head) pairs of a dense call, heads of a packed one
   int slots_per_head;
@@ -265,6 +265,8 @@ enum { SB_DESC0 = 0,                       // [4] descriptor and decays of a chu
        SB_OFREE0, SB_OFREE1,               // results read                              (4 warps)
        SB_DRDY,                            // decays of a chunk of a cut tile computed           (4 warps)
        SB_OTFULL, SB_OTFREE,               // dv output tile written (4 warps) / read by its copies (1)
+       SB_TICKET0, SB_TICKET1,             // a ticket is in its slot                   (1)
+       SB_TKFREE0, SB_TKFREE1,             // every warp has read it                    (20 warps)
        SB_DRAIN, SB_COUNT };
 static_assert(SB_COUNT <= kSwBars, "barrier count");
 
@@ -281,6 +283,7 @@ struct SwCtl {
   int pad;
   WaitCtl wait;
   int n_x, n_y, n_p, n_d;    // loads issued (for the clean exit)
+  uint32_t ticket[2];        // of the next piece (packed calls)
   ChunkDesc desc[4];
 };
 static_assert(sizeof(SwCtl) <= 256, "control block");
@@ -331,27 +334,29 @@ struct Piece {
 // sweeps, then the end of the sweep that the CTA before it (lower index: running or done) has begun.
 // Layer shape, 192 sweeps of 32 tiles on 148 SMs: 42 tiles each; as 576 CTAs of a third of a sweep, four
 // rounds of set-up and state hand-over, the launch took 215 us.
-// Packed calls: whole sweeps of sequences ordered from the longest, dealt back and forth.
-__device__ __forceinline__ bool get_piece(const BwdTcArgs& a, int cta, int ctas, int k, Piece& p) {
-  const int items = a.n_seq * a.H, sweeps = 3 * items, nt = a.cu ? 0 : (a.T + kTile - 1) / kTile;
+// Packed calls: whole sweeps, drawn as tickets from the longest sequence to the shortest, the costlier
+// kinds first; the first ticket is the CTA's index.  (Dealt back and forth instead, 7 sequences of 50 to
+// 600 tokens, 16 heads: the CTAs end after 143 us, 100 on average; a raw_q or raw_k sweep takes 5 us a
+// tile there, a dv sweep 3.)
+template <bool VARLEN>
+__device__ __forceinline__ bool get_piece(const BwdTcArgs& a, int cta, int ctas, int k, uint32_t ticket, Piece& p) {
+  const int items = a.n_seq * a.H, sweeps = 3 * items, nt = VARLEN ? 0 : (a.T + kTile - 1) / kTile;
   p.wait = p.hand = false;
   int s;
   if (nt == 0) {
-    const long long at = (long long)k * ctas + (k & 1 ? ctas - 1 - cta : cta);
+    const long long at = VARLEN ? (long long)ticket : (long long)k * ctas + cta;
     if (at >= sweeps) return false;
     const int of = 3 * a.H, rem = (int)(at % of);
-    p.kind = 2 - rem / a.H;
+    p.kind = rem / a.H;
     p.h = rem % a.H;
     p.n = (int)(at / of);
-    if (a.cu) {
+    p.i_lo = p.i_hi = 0;
+    if (VARLEN) {
       p.n = a.order[p.n];
       int lo, hi;
       seq_range(a.cu, p.n, a.T, lo, hi);
       p.i_hi = (hi - lo + kTile - 1) / kTile;
-    } else {
-      p.i_hi = 0;
     }
-    p.i_lo = 0;
     return true;
   }
   const long long total = (long long)sweeps * nt, lo = total * cta / ctas, hi = total * (cta + 1) / ctas;
@@ -388,7 +393,7 @@ struct Carry {
 };
 
 // KIND 0: raw_q (forward), 1: raw_k, 2: dv (both reverse)
-template <int KIND>
+template <int KIND, bool VARLEN>
 __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps& maps, const Piece& pc, const uint32_t base,
                                             uint8_t* gbase, const uint32_t tmem, Carry& k) {
   constexpr bool REV = KIND != 0, DVK = KIND == 2;
@@ -402,7 +407,7 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
 
   long long row0;
   int len, slot_base;
-  if (a.cu) {
+  if (VARLEN) {
     int lo, hi;
     seq_range(a.cu, pc.n, a.T, lo, hi);
     row0 = (long long)pc.h * a.T + lo;
@@ -854,6 +859,8 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
         }
       }
     };
+    // (a caller's state is read through L1: 16 bytes a thread are half a sector, the other half is the next
+    // load's.  Past L1 the packed shape of get_piece took 8 us more.)
     auto load_init = [&](uint32_t (&r)[32], int piece) {
       if (!init) {
 #pragma unroll
@@ -864,7 +871,8 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
       } else {
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
-          const float4 v = __ldcg(reinterpret_cast<const float4*>(pc.wait ? handed(init, piece, e) : init + elem(32 * piece + e)));
+          const float4 v = pc.wait ? __ldcg(reinterpret_cast<const float4*>(handed(init, piece, e)))
+                                   : __ldg(reinterpret_cast<const float4*>(init + elem(32 * piece + e)));
           r[e] = __float_as_uint(v.x);
           r[e + 1] = __float_as_uint(v.y);
           r[e + 2] = __float_as_uint(v.z);
@@ -988,6 +996,7 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
   }
 }
 
+template <bool VARLEN>
 __global__ void __launch_bounds__(kSwThreads, 1)
 ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -1004,6 +1013,7 @@ ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs
       int cnt = 1;
       if (i == SB_EY0 || i == SB_EY1) cnt = 9;
       if (i == SB_SREADY) cnt = 8;
+      if (i == SB_TKFREE0 || i == SB_TKFREE1) cnt = kSwThreads / 32;
       if (i == SB_TREADY || i == SB_OFREE0 || i == SB_OFREE1 || i == SB_OTFULL || i == SB_DRDY) cnt = 4;
       mbar_init(bar(i), cnt);
     }
@@ -1020,13 +1030,33 @@ ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs
   const uint32_t tmem = ctl->tmem_base;
 
   // (bad cu_seqlens have been reported: nothing to compute)
-  if (!a.cu || *(volatile int32_t*)&a.hdr->status != RODIMUS_ERR_SEQLENS) {
+  if (!VARLEN || *(volatile int32_t*)&a.hdr->status != RODIMUS_ERR_SEQLENS) {
     Carry k = {0, 0, 0, true};
     Piece pc;
-    for (int i = 0; get_piece(a, (int)blockIdx.x, (int)gridDim.x, i, pc); ++i) {
-      if (pc.kind == 0) sweep_piece<0>(a, maps, pc, base, gbase, tmem, k);
-      else if (pc.kind == 1) sweep_piece<1>(a, maps, pc, base, gbase, tmem, k);
-      else sweep_piece<2>(a, maps, pc, base, gbase, tmem, k);
+    for (int i = 0;; ++i) {
+      uint32_t ticket = blockIdx.x;
+      if (VARLEN && i > 0) {
+        // The producer's warp draws the next ticket when it has asked for the last tile of a piece; two
+        // slots, so that a slow warp can still read the one before.
+        const int slot = i & 1;
+        const uint32_t ph = (uint32_t)((i - 1) >> 1) & 1;   // slot 1 is first used for i = 1, slot 0 for i = 2
+        if (warp == 0) {
+          if (!__all_sync(0xffffffffu, mbar_wait(bar(SB_TKFREE0 + slot), ph ^ 1, &ctl->wait, a.hdr))) break;
+          if (elect_one()) {
+            ctl->ticket[slot] = gridDim.x + atomicAdd(reinterpret_cast<unsigned int*>(a.seg_flag + a.n_flags - 1), 1u);
+            mbar_arrive(bar(SB_TICKET0 + slot));
+          }
+          __syncwarp();
+        }
+        if (!__all_sync(0xffffffffu, mbar_wait(bar(SB_TICKET0 + slot), ph, &ctl->wait, a.hdr))) break;
+        ticket = ctl->ticket[slot];
+        __syncwarp();
+        if ((tid & 31) == 0) mbar_arrive(bar(SB_TKFREE0 + slot));
+      }
+      if (!get_piece<VARLEN>(a, (int)blockIdx.x, (int)gridDim.x, i, ticket, pc)) break;
+      if (pc.kind == 0) sweep_piece<0, VARLEN>(a, maps, pc, base, gbase, tmem, k);
+      else if (pc.kind == 1) sweep_piece<1, VARLEN>(a, maps, pc, base, gbase, tmem, k);
+      else sweep_piece<2, VARLEN>(a, maps, pc, base, gbase, tmem, k);
     }
   }
 
@@ -1240,7 +1270,7 @@ __global__ void __launch_bounds__(kPostThreads, 3) ddts_bwd_post_kernel(const Bw
   }
 }
 
-std::atomic<unsigned long long> g_sweep_smem_done{0};
+std::atomic<unsigned long long> g_sweep_smem_done[2];   // dense, packed
 
 // Workspace beyond header and order: raw_q and raw_k (1 KiB per row), c, and an area that holds the
 // states of sweeps cut in two (384 KiB per (sequence, head), dense calls of more than one tile) and the
@@ -1274,7 +1304,7 @@ Scratch scratch_layout(const rodimus_ddts_bwd_params& p) {
   s.dtile = take((size_t)s.slots * DK * 4);
   s.mask = take((size_t)s.slots * 8);
   s.tile_flag = take((size_t)s.slots * 16);
-  s.seg_flag = take(items * 3 * 4);
+  s.seg_flag = take((items * 3 + 1) * 4);
   s.c2 = take(items * DK * 4);
   s.tile_order = take(varlen ? (size_t)s.slots_per_head * 8 : 0);
   const size_t least = area + states + up(items * 6 * 4);
@@ -1318,7 +1348,7 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
   a.limit = main_loop_wait_cycles();
   const long long items = (long long)a.n_seq * p.H;
   if (items == 0) return cudaSuccess;
-  a.n_flags = items * 3;
+  a.n_flags = items * 3 + 1;
   int dev = 0, sms = 0;
   cudaError_t e = current_device(&dev, &sms);
   if (e != cudaSuccess) return e;
@@ -1340,13 +1370,14 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
     if (e == cudaSuccess && !p.cu_seqlens) e = cudaMemsetAsync(a.hdr, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
   }
-  e = opt_in_shared_memory(ddts_bwd_sweep_tc_kernel, kSwSmem, dev, g_sweep_smem_done);
+  auto* const sweep = p.cu_seqlens ? ddts_bwd_sweep_tc_kernel<true> : ddts_bwd_sweep_tc_kernel<false>;
+  e = opt_in_shared_memory(sweep, kSwSmem, dev, g_sweep_smem_done[p.cu_seqlens != nullptr]);
   if (e != cudaSuccess) return e;
   if (rows > 0) {
     ddts_bwd_pre_kernel<<<(unsigned)s.slots + (p.cu_seqlens ? 1u : 0u), kPreThreads, 0, st>>>(a);
     ++*n_launches;
   }
-  ddts_bwd_sweep_tc_kernel<<<(unsigned)(items * 3 < sms ? items * 3 : sms), kSwThreads, kSwSmem, st>>>(m, a);
+  sweep<<<(unsigned)(items * 3 < sms ? items * 3 : sms), kSwThreads, kSwSmem, st>>>(m, a);
   ++*n_launches;
   if (rows > 0) {
     ddts_bwd_post_kernel<<<(unsigned)(s.slots * 4), kPostThreads, 0, st>>>(a);
