@@ -495,7 +495,11 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const uint32_t tmem = ctl->tmem_base;
   const long long n_pairs_grid = gridDim.x >> 1;
   const long long pair_id = blockIdx.x >> 1;
-  auto item_of = [&](int j) { return pair_id + (long long)j * n_pairs_grid; };
+  // Items are dealt back and forth: those of a packed call are ordered from the longest sequence to the
+  // shortest, and a pair that took the longer one of a round takes the shorter one of the next.
+  auto item_of = [&](int j) {
+    return (long long)j * n_pairs_grid + (j & 1 ? n_pairs_grid - 1 - pair_id : pair_id);
+  };
 
   if (role == 0) {
     // ============================ TMA producers, one warp per ring ============================

@@ -21,7 +21,7 @@
 //   warps 8-11    score/output group: P -> masked bf16 operand, O -> global memory
 //   warps 12-19   gate group: softplus/sigmoid/log/exp2 math, in-chunk scan, operand tiles
 //                 written IN PLACE over the raw q,k,x tiles (same swizzled layout)
-// Work item = (sequence, head, 128-column slice of dv), dealt round-robin to a persistent grid.
+// Work item = (sequence, head, 128-column slice of dv), dealt back and forth to a persistent grid.
 #include <cuda.h>
 
 #include <cstring>
@@ -188,7 +188,10 @@ ddts_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
-  auto item_of = [&](int j) { return (long long)blockIdx.x + (long long)j * gridDim.x; };
+  // back and forth: a CTA that took the longer item of a round takes the shorter one of the next
+  auto item_of = [&](int j) {
+    return (long long)j * gridDim.x + (j & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+  };
 
   if (warp == 0) {
     // ===================================== TMA producer =====================================
