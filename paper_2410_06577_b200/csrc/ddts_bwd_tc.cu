@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
   for (long long i = (long long)blockIdx.x * kPreThreads + tid; i < a.n_flags; i += (long long)gridDim.x * kPreThreads)
     a.seg_flag[i] = 0;
   if (a.cu && blockIdx.x == gridDim.x - 1) {   // one block more than there are slots
+    wait_for_previous_kernel();
     order_tiles(a, reinterpret_cast<int*>(s_la), reinterpret_cast<int*>(s_part));
     return;
   }
@@ -1029,6 +1030,7 @@ ddts_bwd_sweep_tc_kernel(const __grid_constant__ SweepMaps maps, const BwdTcArgs
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
 
+  wait_for_previous_kernel();   // the operands are there
   // (bad cu_seqlens have been reported: nothing to compute)
   if (!VARLEN || *(volatile int32_t*)&a.hdr->status != RODIMUS_ERR_SEQLENS) {
     Carry k = {0, 0, 0, true};
@@ -1099,6 +1101,7 @@ __global__ void __launch_bounds__(kPostThreads, 3) ddts_bwd_post_kernel(const Bw
   __shared__ __align__(16) float s_part[(kTile / kPostRows) * kPostCh];
   __shared__ __align__(16) double s_sum[(kTile / kPostRows) * kPostCh];
   __shared__ int s_late;
+  wait_for_previous_kernel();
   if (a.cu && *(volatile int32_t*)&a.hdr->status == RODIMUS_ERR_SEQLENS) return;
   const int tid = threadIdx.x;
   const int quarter = (int)(blockIdx.x & 3u), hs = (int)(blockIdx.x >> 2);
@@ -1374,13 +1377,21 @@ cudaError_t launch_bwd_tc(const rodimus_ddts_bwd_params& p, size_t scratch_offse
   e = opt_in_shared_memory(sweep, kSwSmem, dev, g_sweep_smem_done[p.cu_seqlens != nullptr]);
   if (e != cudaSuccess) return e;
   if (rows > 0) {
-    ddts_bwd_pre_kernel<<<(unsigned)s.slots + (p.cu_seqlens ? 1u : 0u), kPreThreads, 0, st>>>(a);
+    // (packed: beside the plan of the sequences, which only its last block reads)
+    if (p.cu_seqlens) e = launch_overlapped(ddts_bwd_pre_kernel, (unsigned)s.slots + 1u, kPreThreads, 0, st, a);
+    else ddts_bwd_pre_kernel<<<(unsigned)s.slots, kPreThreads, 0, st>>>(a);
+    if (e != cudaSuccess) return e;
     ++*n_launches;
   }
-  sweep<<<(unsigned)(items * 3 < sms ? items * 3 : sms), kSwThreads, kSwSmem, st>>>(m, a);
+  // (each of these is launched while the one before it ends, and waits for it before it reads anything of
+  // its; allowed to start when that one STARTS, their CTAs took room from it: layer shape 352 -> 440 us,
+  // with the launches overlapped only 347)
+  e = launch_overlapped(sweep, (unsigned)(items * 3 < sms ? items * 3 : sms), kSwThreads, kSwSmem, st, m, a);
+  if (e != cudaSuccess) return e;
   ++*n_launches;
   if (rows > 0) {
-    ddts_bwd_post_kernel<<<(unsigned)(s.slots * 4), kPostThreads, 0, st>>>(a);
+    e = launch_overlapped(ddts_bwd_post_kernel, (unsigned)(s.slots * 4), kPostThreads, 0, st, a);
+    if (e != cudaSuccess) return e;
     ++*n_launches;
   }
   return cudaGetLastError();

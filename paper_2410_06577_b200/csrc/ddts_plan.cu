@@ -15,6 +15,7 @@ ddts_plan_kernel(const int32_t* __restrict__ cu, int N, int T, WorkspaceHeader* 
   __shared__ int s_bad;
   __shared__ int s_len[kMaxSortedSeqs];
   const int tid = threadIdx.x;
+  let_next_kernel_start();
   if (tid == 0) s_bad = 0;
   __syncthreads();
   int bad = 0;
