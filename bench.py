@@ -357,7 +357,7 @@ def measure(workload, p, steps, warmup, world, rank, local, peaks, peak_kind, sf
                                  s0=s0, d_sT=g_s, d_s0=d_s0, cu_seqlens=cu, cu_seqlens_host=cu_host)
             ws = torch.empty(rd.bwd_workspace_bytes(bprm), dtype=torch.uint8, device=device)
             bprm.workspace, bprm.workspace_bytes = ws.data_ptr(), ws.numel()
-            kernel = "ddts_bwd_sweep_kernel"
+            kernel = "ddts_bwd_sweep_tc_kernel"
             alg_bytes = token_heads * (8 * dk + 3 * dv) * el + nseq * H * dk * dv * 4 * (2 + (s0 is not None))
 
             def step(i):
@@ -461,7 +461,7 @@ def measure(workload, p, steps, warmup, world, rank, local, peaks, peak_kind, sf
         rec["config"] = dict(rec["config"], variant={
             "block": "value gate beta_hat and feed-through d*x' fused (Eq. beta_def, Eq. rodimus_recurrent_form)",
             "shared": "one q,k,x,y per token for all 16 heads ([B,1,T,dk])",
-            "backward": "backward pass (dq, dk, dx, dy, dv, ds0 from dL/do and dL/dS_T), two launches",
+            "backward": "backward pass (dq, dk, dx, dy, dv, ds0 from dL/do and dL/dS_T), three launches",
             "vdecay": "value-side decay beta_t of the general transition (the paper's ablation arm), fp32 CUDA-core kernel"}[variant])
         if variant == "backward":
             rec["metric"] = "DDTS prefill backward tokens/s"

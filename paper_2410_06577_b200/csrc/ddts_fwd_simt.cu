@@ -492,7 +492,7 @@ cudaError_t launch_chunks(const ChunkArgs& a, cudaStream_t st) {
 
 // Workspace with which this kernel's chunks are computed side by side; 0: they are not.  The states of
 // the chunks cross memory four times, which pays while they stay in L2 (126 MB): up to 64 MiB of them.
-// B=1 H=1 T=256 dk=dv=64 fp32: one CTA walking the 16 chunks 318 us, side by side 28 us.
+// B=1 H=1 T=256 dk=dv=64 fp32: one CTA walking the 16 chunks 318 us, side by side 16.4 us a call.
 size_t fwd_simt_chunks_workspace_bytes(const rodimus_ddts_fwd_params& p) {
   if (p.value_decay || (long long)p.B * p.H * p.T == 0 || p.T <= kC) return 0;
   if ((p.cu_seqlens || p.cu_seqlens_host) && p.N == 0) return 0;
