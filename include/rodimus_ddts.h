@@ -156,9 +156,12 @@ typedef struct {
  * the sequences into time segments that run side by side (the state recurrence is linear in
  * the state, so segments are joined exactly up to rounding) and part of the work is enqueued
  * on the library's own second stream, forked from and joined back into `stream` with events, so
- * the call still behaves as one piece of work on `stream`.  A caller that passes less (never
- * less than 256 bytes plus 4 bytes per packed sequence, rounded up to 256) gets the same
- * result from a single launch. */
+ * the call still behaves as one piece of work on `stream`.  For bf16 requests with dk = 64, with
+ * one set of gates for all heads or with few heads it includes a block of gated operands per 64
+ * tokens and set of gates, and for small fp32 requests the states of 16-token chunks, so that all
+ * SMs can form them ahead of the scan.  A caller that passes less (never less than 256 bytes plus
+ * 4 bytes per packed sequence, rounded up to 256) gets the same result, to the same accuracy, from
+ * a kernel that needs no more. */
 size_t rodimus_ddts_fwd_workspace_bytes(const rodimus_ddts_fwd_params *p);
 
 /* Chunked prefill; see rodimus_ddts_fwd_params. */
@@ -307,7 +310,7 @@ int rodimus_ddts_device_status(const void *workspace, void *stream);
 int rodimus_ddts_last_launch_count(void);
 
 /* Name of the kernel family the given prefill request would run: "tcgen05", "simt" or
- * "invalid".  Pointers are not read. */
+ * "invalid"; with the workspace_bytes it gives.  Pointers are not read. */
 const char *rodimus_ddts_fwd_kernel_name(const rodimus_ddts_fwd_params *p);
 
 /* Diagnostic for benchmarks (the paper has no counterpart): enqueues on `stream` one launch that
