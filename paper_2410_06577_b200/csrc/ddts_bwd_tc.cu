@@ -265,7 +265,9 @@ enum { SB_DESC0 = 0,                       // [4] descriptor and decays of a chu
        SB_OFULL0, SB_OFULL1,               // results complete                          (1)
        SB_OFREE0, SB_OFREE1,               // results read                              (4 warps)
        SB_DRDY,                            // decays of a chunk of a cut tile computed           (4 warps)
-       SB_OTFULL, SB_OTFREE,               // dv output tile written (4 warps) / read by its copies (1)
+       SB_OTFULL,                          // dv output tile written                    (4 warps)
+       SB_OTFREE0, SB_OTFREE1,             // dv output tile read by its copies         (1); two barriers in turn:
+                                           // the state group may ask for a tile while the one before is out
        SB_TICKET0, SB_TICKET1,             // a ticket is in its slot                   (1)
        SB_TKFREE0, SB_TKFREE1,             // every warp has read it                    (20 warps)
        SB_DRAIN, SB_COUNT };
@@ -704,7 +706,7 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
         // dv^T fragments [value column][row] are transposed by stmatrix.trans into four swizzled
         // 64-column slabs and leave by tensor copies
         const int mat_k = lane & 7, mat_h = (lane >> 3) & 1, mat_j = lane >> 4;
-        if (k.n_ot > 0 && !(ok = wait_all(bar(SB_OTFREE), (k.n_ot - 1) & 1))) break;
+        if (k.n_ot > 0 && !(ok = wait_all(bar(SB_OTFREE0 + ((k.n_ot - 1) & 1)), ((k.n_ot - 1) >> 1) & 1))) break;
 #pragma unroll
         for (int bl = 0; bl < 2; ++bl) {
           const uint32_t mat = base + kOffOut + (2 * bl + (q4 >> 1)) * kSlab + (mat_j * 8 + mat_k) * 128;
@@ -752,7 +754,7 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
           bulk_commit();
           bulk_wait_read<0>();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar(SB_OTFREE));
+          if (lane == 0) mbar_arrive(bar(SB_OTFREE0 + (k.n_ot & 1)));
         }
         ++k.n_ot;
       }
@@ -893,7 +895,7 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
     }
     bool last = !any;
     // the dv output tile lies where the other kinds keep half of their expanded Y: its copies are done
-    if (ok && !DVK && k.n_ot > 0) ok = wait_all(bar(SB_OTFREE), (k.n_ot - 1) & 1);
+    if (ok && !DVK && k.n_ot > 0) ok = wait_all(bar(SB_OTFREE0 + ((k.n_ot - 1) & 1)), ((k.n_ot - 1) >> 1) & 1);
     while (ok && !last) {
       if (!(ok = wait_all(bar(SB_FY0 + (c & 1)), (c >> 1) & 1))) break;
       if (c > 0 && !(ok = wait_all(bar(SB_M1), (c - 1) & 1))) break;    // Y32's last reader

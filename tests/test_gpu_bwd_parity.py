@@ -196,3 +196,19 @@ def test_bwd_bf16_tile_edges_and_cut_tiles(T, strong):
         p.x[:, :, T // 3:T // 3 + 7, ::5] = 80.0 if T > 2 else 20.0     # softplus(80) sigmoid(4) = 78.6 per step
         p.y[:, :, T // 3:T // 3 + 7, ::5] = 4.0
     _check(p, 1100 + T, True, scale=0.5)
+
+
+@pytest.mark.parametrize("n_seq,shortest,longest", [(30, 62, 148), (7, 50, 600)])
+def test_bwd_packed_pieces_that_follow_one_another_on_a_block(n_seq, shortest, longest):
+    """More sweeps than thread blocks, of one to a few tiles and of every kind in turn: what a block's
+    roles hand over from the end of one sweep to the beginning of the next.  Nothing depends on which
+    block runs which sweep, so repeated calls agree bit for bit; the first against the oracle."""
+    lens = np.random.default_rng(n_seq).integers(shortest, longest + 1, n_seq)
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    p = wl.make_prefill(1200 + n_seq, 1, 16, int(cu[-1]), 128, 256, "bf16", cu_seqlens=cu, s0_std=0.1, name=f"bwd_pieces_{n_seq}")
+    _check(p, 1201, True)
+    d_o, d_sT = wl.make_grads(1201, p, True)
+    first = _run_bwd(p, d_o, d_sT, rd.INGATE_POW_G, 1.0)
+    for _ in range(12):
+        again = _run_bwd(p, d_o, d_sT, rd.INGATE_POW_G, 1.0)
+        assert all(np.array_equal(first[n], again[n]) for n in first)
