@@ -771,6 +771,7 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                                (2 * (lane & 3) + 1 <= (lane >> 2) ? 0xFFFF0000u : 0u);
     const uint32_t t_lane = tmem + ((uint32_t)(q4 * 32) << 16);
     const bool unit_scale = a.scale == 1.0f;
+    uint32_t n_x = 0;   // feed-through tiles asked for (warp of quarter 0)
     uint32_t g = 0;
     bool ok = true;
     for (int j = 0; ok && item_of(j) < a.n_items; ++j) {
@@ -814,6 +815,7 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             tma_load_2d(xt, &map_fx, it.col0, (int)row, xb);
             tma_load_2d(xt + kSlabBytes, &map_fx, it.col0 + 64, (int)row, xb);
           }
+          n_x = g + 1;
         }
         if (q4 == 0 && lane == 0) {
           // P exists, so the partner's copies out of ITS stage have all landed here (the issuer
@@ -945,6 +947,10 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         ++g;
       }
     }
+    // (after a wait that ran out a feed-through tile may still be on its way)
+    if (BLOCK && !ok && lane == 0)
+      for (uint32_t back = 1; back <= 2 && back <= n_x; ++back)
+        mbar_drain(bar(BAR_XFULL0 + ((n_x - back) & 1)), ((n_x - back) >> 1) & 1);
     bulk_wait_read<0>();   // this thread's output copies have read their tile before the CTA may exit
                            // (their writes complete with the kernel)
   } else if (role == 5 || role == 2) {
