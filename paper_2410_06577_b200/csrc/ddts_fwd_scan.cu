@@ -843,10 +843,16 @@ cudaError_t launch_scan(const ScanMaps& m, const ScanArgs& a, long long slots, l
   cudaError_t e = opt_in_shared_memory(ddts_operands_kernel<DK>, kOpSmem<DK>, dev, opted_ops);
   if (e == cudaSuccess) e = opt_in_shared_memory(ddts_scan_kernel<DK, BLOCK>, Scan<DK, BLOCK>::kSmem, dev, opted);
   if (e != cudaSuccess) return e;
-  if (slots > 0) ddts_operands_kernel<DK><<<(unsigned)slots, kOpThreads, kOpSmem<DK>, st>>>(a);
-  // The scan may start while the operand kernel's last CTAs run: it sets up (barriers, tensor memory)
-  // and waits for that kernel before it reads a block.
-  e = launch_overlapped(ddts_scan_kernel<DK, BLOCK>, (unsigned)items, C::kThreads, C::kSmem, st, m, a);
+  if (slots > 0) {
+    ddts_operands_kernel<DK><<<(unsigned)slots, kOpThreads, kOpSmem<DK>, st>>>(a);
+    // The scan may start while the operand kernel's last CTAs run: it sets up (barriers, tensor memory)
+    // and waits for that kernel before it reads a block.
+    e = launch_overlapped(ddts_scan_kernel<DK, BLOCK>, (unsigned)items, C::kThreads, C::kSmem, st, m, a);
+  } else {
+    // No tokens: what is in front now is the plan of the sequences, whose order the scan reads before it
+    // waits for anything.  So it starts when that has ended.
+    ddts_scan_kernel<DK, BLOCK><<<(unsigned)items, C::kThreads, C::kSmem, st>>>(m, a);
+  }
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -911,3 +911,20 @@ def test_decode_tile_widths(Nseq, H, dk, dv):
         ro = orc.ref_step(w.q[s], w.k[s], w.x[s], w.y[s], w.v[s], ref_state)
         assert rel_err(host(o), ro) <= TOL_BF16
     assert rel_err(host(state), ref_state) <= TOL_F32
+
+
+@pytest.mark.parametrize("dk,H,shared", [(64, 3, True), (64, 2, False), (128, 3, True)])
+def test_two_launch_prefill_packed_sequences_without_tokens(dk, H, shared):
+    """Nothing but empty sequences: no operands are formed, and the scan follows the plan of the sequences
+    directly.  Every state passes through unchanged."""
+    import torch
+    N, dv = 37, 256
+    q, k, x, y = (torch.empty((1, 1 if shared else H, 0, dk), dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    v = torch.empty((1, H, 0, dv), dtype=torch.bfloat16, device="cuda")
+    cu = torch.zeros(N + 1, dtype=torch.int32, device="cuda")
+    s0 = torch.randn((N, H, dk, dv), device="cuda")
+    for _ in range(20):
+        o, sT = rd.ddts_fwd(q, k, x, y, v, s0, cu_seqlens=cu)
+        assert o.shape == v.shape and torch.equal(sT, s0)
+    _, sT = rd.ddts_fwd(q, k, x, y, v, None, cu_seqlens=cu)
+    assert torch.equal(sT, torch.zeros_like(s0))
