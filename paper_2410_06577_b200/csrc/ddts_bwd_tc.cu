@@ -154,6 +154,8 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
     a.seg_flag[i] = 0;
   if (a.cu && blockIdx.x == gridDim.x - 1) {   // one block more than there are slots
     wait_for_previous_kernel();
+    // (ranges of a refused cu_seqlens may overlap: there is no bound on their tiles, and nobody reads the order)
+    if (*(volatile int32_t*)&a.hdr->status == RODIMUS_ERR_SEQLENS) return;
     order_tiles(a, reinterpret_cast<int*>(s_la), reinterpret_cast<int*>(s_part));
     return;
   }

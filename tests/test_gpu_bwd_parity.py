@@ -212,3 +212,21 @@ def test_bwd_packed_pieces_that_follow_one_another_on_a_block(n_seq, shortest, l
     for _ in range(12):
         again = _run_bwd(p, d_o, d_sT, rd.INGATE_POW_G, 1.0)
         assert all(np.array_equal(first[n], again[n]) for n in first)
+
+
+def test_bwd_bad_cu_seqlens_with_overlapping_ranges_stays_in_the_workspace():
+    """Ranges that overlap have more tiles than the workspace has places for.  At this length the list of
+    tiles ends the workspace (its few words per tile outgrow the room for states), so that entries beyond
+    the list would land in the guard behind it."""
+    import torch
+    T, N, guard = 160000, 3, 1 << 20
+    q, k, x, y = (torch.zeros((1, 1, T, 128), dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    v, d_o = (torch.zeros((1, 1, T, 256), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    out = [torch.empty_like(t) for t in (q, k, x, y, v)]
+    cu = torch.tensor([0, T, 0, T], dtype=torch.int32, device="cuda")
+    prm = rd.bwd_params(q, k, x, y, v, d_o, *out, cu_seqlens=cu)
+    need = rd.bwd_workspace_bytes(prm)
+    ws = torch.full((need + guard,), 0xA5, dtype=torch.uint8, device="cuda")
+    prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
+    assert rd.bwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.ERR_SEQLENS
+    assert bool((ws[need:] == 0xA5).all())
