@@ -358,7 +358,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     slot0 = ((long long)n * a.gate_heads + hq) * a.slots_per_head;
   }
   const int col0 = slice * 128;
-  const int ntiles = (len + kTile - 1) / kTile;
+  int ntiles = (len + kTile - 1) / kTile;
   const long long state_off = ((long long)n * a.H + h) * DK * (long long)a.dv + col0;
 
   if (tid == 0) {
@@ -387,6 +387,8 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
   wait_for_previous_kernel();   // the operands are there
+  // A cu_seqlens that the plan has refused may leave blocks unwritten: no tile of it is looked at.
+  if (a.cu && *(volatile int32_t*)&hdr->status == RODIMUS_ERR_SEQLENS) ntiles = 0;
   auto wait_all = [&](int b, uint32_t parity) -> bool {   // whole warps: tensor-memory accesses need them
     return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, wc, hdr)) != 0;
   };

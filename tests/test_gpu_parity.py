@@ -928,3 +928,25 @@ def test_two_launch_prefill_packed_sequences_without_tokens(dk, H, shared):
         assert o.shape == v.shape and torch.equal(sT, s0)
     _, sT = rd.ddts_fwd(q, k, x, y, v, None, cu_seqlens=cu)
     assert torch.equal(sT, torch.zeros_like(s0))
+
+
+@pytest.mark.parametrize("dk,shared", [(64, True), (64, False), (128, True), (128, False)])
+@pytest.mark.parametrize("ends", [(1, 0, 0), (1, 0, 1), (0, 1, 0, 1)])
+def test_two_launch_prefill_bad_seqlens_reported_by_device(dk, shared, ends):
+    """Ranges that decrease or overlap leave blocks of operands that nobody has written.  The scan does not
+    look at them: no wait runs out (that would replace the report), and the blocks' places hold garbage."""
+    import torch
+    H, T, dv = 2, 1100, 256                                   # (T per sequence large enough for the per-head rule)
+    q, k, x, y = (torch.zeros((1, 1 if shared else H, T, dk), dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    v = torch.zeros((1, H, T, dv), dtype=torch.bfloat16, device="cuda")
+    o, cu = torch.zeros_like(v), torch.tensor([0] + [T * e for e in ends], dtype=torch.int32, device="cuda")
+    prm = rd.fwd_params(q, k, x, y, v, o, None, None, cu)
+    need = rd.fwd_workspace_bytes(prm)
+    assert need > 100000                                      # the two-launch form
+    ws = torch.full((need,), 0xEE, dtype=torch.uint8, device="cuda")
+    prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
+    assert rd.fwd_raw(prm) == rd.OK
+    assert rd.device_status(ws) == rd.ERR_SEQLENS
+    good = torch.tensor([0] + [T] * len(ends), dtype=torch.int32, device="cuda")
+    prm.cu_seqlens = good.data_ptr()
+    assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
