@@ -149,9 +149,9 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
     gate_pair<B::kExact>(x.y, y.y, a.ingate, la.y, lh);
     return la;
   };
+  // (the scan's scratch lies where the operands go next)
   const unsigned long long mask = tile_scan<kOpRows, DK, true>(b, cp, rg, tr.nr, reinterpret_cast<float*>(gbase), s_part,
                                                                &s_mask, 0ull, la_of);
-  if (mask != 1ull) __syncthreads();          // the scan's scratch becomes operands
   {
     const uint32_t w = base + (cp >> 5) * kSlab + ((cp & 3) << 2), c16 = (uint32_t)(cp & 31) >> 2;
 #pragma unroll

@@ -180,6 +180,7 @@ __device__ __forceinline__ unsigned long long tile_scan(float2 (&v)[ROWS], int c
     for (int u = 0; u < ROWS; ++u)
       if (u == i) v[u] = acc;
   }
+  __syncthreads();                            // `la` is the caller's again, whatever the mask
   return mask;
 }
 

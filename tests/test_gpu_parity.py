@@ -950,3 +950,30 @@ def test_two_launch_prefill_bad_seqlens_reported_by_device(dk, shared, ends):
     good = torch.tensor([0] + [T] * len(ends), dtype=torch.int32, device="cuda")
     prm.cu_seqlens = good.data_ptr()
     assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
+
+
+def _rows_at_the_edge_of_a_chunk(rng, n_tiles):
+    """x, y [n_tiles, 64] of bf16 values whose 64 log decays add up to -60 to the last digits of fp32."""
+    grid = wl.round_to_bf16(np.stack(np.meshgrid(np.linspace(0.5, 1.5, 129), np.linspace(0.0, 2.0, 257)), -1)).reshape(-1, 2)
+    decay = lambda g: np.logaddexp(0.0, g[..., 0].astype(np.float64)) / (1.0 + np.exp(-g[..., 1].astype(np.float64)))
+    values = decay(grid)
+    by_value = np.argsort(values)
+    rows = grid[rng.integers(0, len(grid), (n_tiles, 64))]
+    for r in rows:
+        while not 0.9 < 60.0 - decay(r[:62]).sum() < 2.4:      # what two rows can still make up
+            r[:62] = grid[by_value[(np.clip(rng.normal(0.42, 0.25, 62), 0, 0.9999) * len(grid)).astype(int)]]
+        rest = 60.0 - decay(r[:62]).sum()
+        first = rng.integers(0, len(grid), 4000)
+        at = np.clip(np.searchsorted(values[by_value], rest - values[first]), 0, len(grid) - 1)
+        best = np.argmin(np.abs(values[first] + values[by_value[at]] - rest))
+        r[62], r[63] = grid[first[best]], grid[by_value[at[best]]]
+    return rows[..., 0], rows[..., 1]
+
+
+def test_two_launch_prefill_tiles_whose_decay_is_the_largest_of_a_chunk():
+    """64 rows that decay by e^-60 in one channel, to rounding: sums in two orders may then disagree on
+    whether the tile needs a cut."""
+    x0, y0 = _rows_at_the_edge_of_a_chunk(np.random.default_rng(7), 400)
+    p = wl.make_prefill(980, 1, 1, 400 * 64, 64, 128, "bf16")
+    p.x[0, 0, :, 0], p.y[0, 0, :, 0] = x0.reshape(-1), y0.reshape(-1)
+    _check_prefill(p)
