@@ -28,6 +28,7 @@ namespace {
 constexpr int kC = 16;          // chunk length
 constexpr int kTileV = 64;      // state columns per CTA
 constexpr int kThreads = 256;
+constexpr int kMaxDk = 256;
 
 struct SimtArgs {
   const void *q, *k, *gx, *ty, *v;
@@ -470,15 +471,17 @@ ChunkPlan chunk_plan(const rodimus_ddts_fwd_params& p) {
   return c;
 }
 
+int chunk_ops_smem_bytes(int dk) { return (int)sizeof(float) * (3 * kC * (dk + 1) + kC * kTileV); }
+int chunk_out_smem_bytes(int dk) { return (int)sizeof(float) * (dk * kTileV + kC * dk + kC * kTileV + kC * kC); }
+
+// (The kernels are opted in to the shared memory of the widest keys, once: set to each call's own need, the
+// limit could be lowered by another thread between this call's setting and its launch.)
 template <typename T>
-cudaError_t launch_chunks(const ChunkArgs& a, cudaStream_t st) {
-  const int smem_ops = (int)sizeof(float) * (3 * kC * (a.s.dk + 1) + kC * kTileV);
-  const int smem_out = (int)sizeof(float) * (a.s.dk * kTileV + kC * a.s.dk + kC * kTileV + kC * kC);
-  cudaError_t e = cudaSuccess;
-  if (smem_ops > 48 * 1024)
-    e = cudaFuncSetAttribute(ddts_chunk_ops_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_ops);
-  if (e == cudaSuccess && smem_out > 48 * 1024)
-    e = cudaFuncSetAttribute(ddts_chunk_out_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_out);
+cudaError_t launch_chunks(const ChunkArgs& a, int dev, cudaStream_t st) {
+  static std::atomic<unsigned long long> opted_ops{0}, opted_out{0};   // per instantiation
+  const int smem_ops = chunk_ops_smem_bytes(a.s.dk), smem_out = chunk_out_smem_bytes(a.s.dk);
+  cudaError_t e = opt_in_shared_memory(ddts_chunk_ops_kernel<T>, chunk_ops_smem_bytes(kMaxDk), dev, opted_ops);
+  if (e == cudaSuccess) e = opt_in_shared_memory(ddts_chunk_out_kernel<T>, chunk_out_smem_bytes(kMaxDk), dev, opted_out);
   if (e != cudaSuccess) return e;
   const long long threads = (long long)a.s.n_seq * a.s.H * a.s.dk * (a.s.dv / 4);
   ddts_chunk_ops_kernel<T><<<(unsigned)a.slots, kOpsThreads, smem_ops, st>>>(a);
@@ -515,9 +518,10 @@ cudaError_t launch_fwd_simt(const rodimus_ddts_fwd_params& p, int* n_launches) {
   const long long items = (long long)a.n_seq * p.H * a.tiles;
   if (items == 0) return cudaSuccess;
   if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
-  const size_t smem = simt_smem_bytes(p.dk);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
-  cudaError_t e;
+  int dev = 0, sms = 0;
+  cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
   const size_t chunks = fwd_simt_chunks_workspace_bytes(p);
   if (chunks > 0 && p.workspace_bytes >= chunks) {
     const ChunkPlan c = chunk_plan(p);
@@ -531,21 +535,16 @@ cudaError_t launch_fwd_simt(const rodimus_ddts_fwd_params& p, int* n_launches) {
     ca.slots_per_head = c.slots_per_head;
     ca.heads = c.heads;
     ca.slots = c.slots;
-    e = p.dtype == RODIMUS_BF16 ? launch_chunks<__nv_bfloat16>(ca, st) : launch_chunks<float>(ca, st);
+    e = p.dtype == RODIMUS_BF16 ? launch_chunks<__nv_bfloat16>(ca, dev, st) : launch_chunks<float>(ca, dev, st);
     *n_launches = 3;
     return e;
   }
-  if (p.dtype == RODIMUS_BF16) {
-    e = cudaFuncSetAttribute(ddts_fwd_simt_kernel<__nv_bfloat16>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    ddts_fwd_simt_kernel<__nv_bfloat16><<<(unsigned)items, kThreads, smem, st>>>(a);
-  } else {
-    e = cudaFuncSetAttribute(ddts_fwd_simt_kernel<float>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    ddts_fwd_simt_kernel<float><<<(unsigned)items, kThreads, smem, st>>>(a);
-  }
+  const bool bf16 = p.dtype == RODIMUS_BF16;
+  auto* const kernel = bf16 ? ddts_fwd_simt_kernel<__nv_bfloat16> : ddts_fwd_simt_kernel<float>;
+  static std::atomic<unsigned long long> opted[2];
+  e = opt_in_shared_memory(kernel, (int)simt_smem_bytes(kMaxDk), dev, opted[bf16]);
+  if (e != cudaSuccess) return e;
+  kernel<<<(unsigned)items, kThreads, simt_smem_bytes(p.dk), st>>>(a);
   *n_launches = 1;
   return cudaGetLastError();
 }

@@ -977,3 +977,30 @@ def test_two_launch_prefill_tiles_whose_decay_is_the_largest_of_a_chunk():
     p = wl.make_prefill(980, 1, 1, 400 * 64, 64, 128, "bf16")
     p.x[0, 0, :, 0], p.y[0, 0, :, 0] = x0.reshape(-1), y0.reshape(-1)
     _check_prefill(p)
+
+
+@pytest.mark.parametrize("T", [32, 16])                       # chunks side by side; one chunk
+def test_fp32_calls_of_two_threads_with_keys_of_different_width(T):
+    """Wide keys need more shared memory than narrow ones: neither thread's launches may depend on what the
+    other one last asked for."""
+    import threading
+    import torch
+    failed = []
+
+    def calls(dk):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                a = [torch.full((1, 1, T, d), 0.1, device="cuda") for d in (dk, dk, dk, dk, 64)]
+                for _ in range(3000):
+                    rd.ddts_fwd(*a)
+            stream.synchronize()
+        except Exception as e:
+            failed.append((dk, repr(e)))
+
+    threads = [threading.Thread(target=calls, args=(dk,)) for dk in (256, 144)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
