@@ -6,6 +6,7 @@
 // the package has loaded, so that there is one library in the process.
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/types.h>
 
@@ -64,13 +65,14 @@ at::Tensor bytes_like(const at::Tensor& q, size_t n) {
 }
 PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
 
-// Every function returns an int - the status - where the library refused the call.
+// Every function returns an int - the status - where the library refused the call.  PyTorch's exceptions
+// become the Python errors that its own functions raise (OutOfMemoryError among them).
 #define RODIMUS_TRY try {
-#define RODIMUS_CATCH                                         \
-  }                                                           \
-  catch (const std::exception& e) {                           \
-    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what()); \
-    return nullptr;                                           \
+#define RODIMUS_CATCH                                                  \
+  }                                                                    \
+  catch (...) {                                                        \
+    torch::translate_exception_to_python(std::current_exception());    \
+    return nullptr;                                                    \
   }
 
 // ddts_fwd(q, k, gate_x, temp_y, v, s0, cu_seqlens, cu_seqlens_host, scale, ingate, want_final_state, out,

@@ -1004,3 +1004,14 @@ def test_fp32_calls_of_two_threads_with_keys_of_different_width(T):
     for t in threads:
         t.join()
     assert not failed, failed
+
+
+def test_outputs_that_do_not_fit_raise_out_of_memory():
+    """As any allocation of PyTorch's does: a caller may catch it to retry with less."""
+    import torch
+    z = lambda *s: torch.empty(s, dtype=torch.bfloat16, device="cuda")
+    H, d = 1 << 20, 1024                                          # outputs of 2^42 bytes, inputs of none
+    with pytest.raises(torch.OutOfMemoryError):
+        rd.ddts_fwd(*(z(1, 1, 1 << 11, 64) for _ in range(4)), z(1, H, 0, d))
+    with pytest.raises(torch.OutOfMemoryError):
+        rd.ddts_step(*(z(1 << 11, 1, 64) for _ in range(4)), z(0, H, d), torch.empty(0, device="cuda"))
