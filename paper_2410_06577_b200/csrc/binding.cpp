@@ -10,6 +10,8 @@
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/types.h>
 
+#include <optional>
+
 #include "rodimus_ddts.h"
 
 namespace {
@@ -65,6 +67,15 @@ at::Tensor bytes_like(const at::Tensor& q, size_t n) {
 }
 PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
 
+// The interpreter's lock is given up while tensors are allocated (which may wait for the device) and work is
+// enqueued.
+struct NoGil {
+  PyThreadState* state = PyEval_SaveThread();
+  NoGil() = default;
+  NoGil(const NoGil&) = delete;
+  ~NoGil() { PyEval_RestoreThread(state); }
+};
+
 // Every function returns an int - the status - where the library refused the call.  PyTorch's exceptions
 // become the Python errors that its own functions raise (OutOfMemoryError among them).
 #define RODIMUS_TRY try {
@@ -102,6 +113,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   p.scale = (float)scale;
   p.N = cu.t ? (int32_t)(cu.t->numel() - 1) : 0;
   p.shared_gates = q.t->size(1) == 1 && p.H > 1;
+  std::optional<NoGil> no_gil(std::in_place);
   at::Tensor o = out.t ? *out.t : at::empty({p.B, p.H, p.T, p.dv}, q.t->options());
   at::Tensor sT;
   if (fin.t) sT = *fin.t;
@@ -118,10 +130,8 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   at::Tensor w = ws.t ? *ws.t : bytes_like(*q.t, g_fwd_ws(&p));
   p.workspace = w.data_ptr();
   p.workspace_bytes = (size_t)w.numel() * w.element_size();
-  int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = g_fwd(&p);
-  Py_END_ALLOW_THREADS
+  const int rc = g_fwd(&p);
+  no_gil.reset();
   if (rc != RODIMUS_OK) return PyLong_FromLong(rc);
   PyObject* r = PyTuple_New(2);
   if (!r) return nullptr;
@@ -154,6 +164,7 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   p.dv = (int32_t)v.t->size(2);
   p.scale = (float)scale;
   p.shared_gates = q.t->size(1) == 1 && p.H > 1;
+  std::optional<NoGil> no_gil(std::in_place);
   at::Tensor o = out.t ? *out.t : at::empty({p.Nseq, p.H, p.dv}, q.t->options());
   p.q = q.ptr(); p.k = k.ptr(); p.gate_x = x.ptr(); p.temp_y = y.ptr(); p.v = v.ptr();
   p.o = o.data_ptr();
@@ -161,10 +172,8 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   p.beta_hat = beta.ptr(); p.feed_d = (const float*)fd.ptr(); p.feed_x = fx.ptr();
   p.value_decay = vd.ptr();
   p.stream = current_stream();
-  int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = g_step(&p);
-  Py_END_ALLOW_THREADS
+  const int rc = g_step(&p);
+  no_gil.reset();
   if (rc != RODIMUS_OK) return PyLong_FromLong(rc);
   return wrap(o);
   RODIMUS_CATCH
@@ -195,6 +204,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   p.dv = (int32_t)v.t->size(3);
   p.scale = (float)scale;
   p.N = cu.t ? (int32_t)(cu.t->numel() - 1) : 0;
+  std::optional<NoGil> no_gil(std::in_place);
   at::Tensor g[5];
   for (int i = 0; i < 4; ++i) g[i] = at::empty_like(*q.t);
   g[4] = at::empty_like(*v.t);
@@ -211,10 +221,8 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   at::Tensor w = ws.t ? *ws.t : bytes_like(*q.t, g_bwd_ws(&p));
   p.workspace = w.data_ptr();
   p.workspace_bytes = (size_t)w.numel() * w.element_size();
-  int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = g_bwd(&p);
-  Py_END_ALLOW_THREADS
+  const int rc = g_bwd(&p);
+  no_gil.reset();
   if (rc != RODIMUS_OK) return PyLong_FromLong(rc);
   PyObject* r = PyTuple_New(6);
   if (!r) return nullptr;
@@ -243,14 +251,13 @@ PyObject* swska(PyObject*, PyObject* const* a, Py_ssize_t n) {
   p.window = (int32_t)PyLong_AsLong(a[3]);
   p.scale = (float)(a[4] == Py_None ? 1.0 / std::sqrt((double)p.d) : PyFloat_AsDouble(a[4]));
   if (PyErr_Occurred()) return nullptr;
+  std::optional<NoGil> no_gil(std::in_place);
   at::Tensor o = out.t ? *out.t : at::empty_like(*q.t);
   p.q = q.ptr(); p.k = k.ptr(); p.v = v.ptr();
   p.o = o.data_ptr();
   p.stream = current_stream();
-  int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = g_swska(&p);
-  Py_END_ALLOW_THREADS
+  const int rc = g_swska(&p);
+  no_gil.reset();
   if (rc != RODIMUS_OK) return PyLong_FromLong(rc);
   return wrap(o);
   RODIMUS_CATCH

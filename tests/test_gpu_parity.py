@@ -1015,3 +1015,44 @@ def test_outputs_that_do_not_fit_raise_out_of_memory():
         rd.ddts_fwd(*(z(1, 1, 1 << 11, 64) for _ in range(4)), z(1, H, 0, d))
     with pytest.raises(torch.OutOfMemoryError):
         rd.ddts_step(*(z(1 << 11, 1, 64) for _ in range(4)), z(0, H, d), torch.empty(0, device="cuda"))
+
+
+def test_other_threads_run_while_a_call_waits_for_memory():
+    """An allocation that has to give cached memory back first waits for the device."""
+    import threading
+    import time
+    import torch
+    H, T, d = 16, 8192, 128                                       # outputs of 32 MiB
+    torch.cuda.empty_cache()
+    q, v = (torch.zeros((1, H, T, d), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    k = torch.zeros((1, T, d), dtype=torch.bfloat16, device="cuda")
+    rd.swska_fwd(q, k, v, 64)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    gaps, stop = [], threading.Event()
+
+    def ticks():
+        last = time.perf_counter()
+        while not stop.is_set():
+            time.sleep(0.002)
+            now = time.perf_counter()
+            gaps.append(now - last)
+            last = now
+
+    cached = torch.empty(28 << 20, dtype=torch.uint8, device="cuda")
+    del cached
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (8 << 20)) / total)
+    ticker = threading.Thread(target=ticks)
+    try:
+        torch.cuda._sleep(1_000_000_000)                          # about half a second of the device
+        ticker.start()
+        start = time.perf_counter()
+        rd.swska_fwd(q, k, v, 64)
+        took = time.perf_counter() - start
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+        stop.set()
+        ticker.join()
+    assert took > 0.2, took                                       # the call did wait
+    assert max(gaps) < took / 2, (took, max(gaps))
