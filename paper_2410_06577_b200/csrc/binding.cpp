@@ -65,6 +65,17 @@ void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 at::Tensor bytes_like(const at::Tensor& q, size_t n) {
   return at::empty({(int64_t)(n < 256 ? 256 : n)}, q.options().dtype(at::kByte));
 }
+// The prefill's workspace: what makes it fastest or, where that does not fit into the device's memory (it may
+// be as large as the inputs), the least that every request runs with.
+at::Tensor fwd_workspace(const at::Tensor& q, size_t wanted, int32_t n_seq) {
+  const size_t least = 256 + (((size_t)(n_seq > 0 ? n_seq : 0) * 4 + 255) & ~(size_t)255);
+  try {
+    return bytes_like(q, wanted);
+  } catch (const c10::OutOfMemoryError&) {
+    if (wanted <= least) throw;
+  }
+  return bytes_like(q, least);
+}
 PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
 
 // The interpreter's lock is given up while tensors are allocated (which may wait for the device) and work is
@@ -127,7 +138,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   p.beta_hat = beta.ptr(); p.feed_d = (const float*)fd.ptr(); p.feed_x = fx.ptr();
   p.value_decay = vd.ptr();
   p.stream = current_stream();
-  at::Tensor w = ws.t ? *ws.t : bytes_like(*q.t, g_fwd_ws(&p));
+  at::Tensor w = ws.t ? *ws.t : fwd_workspace(*q.t, g_fwd_ws(&p), p.N);
   p.workspace = w.data_ptr();
   p.workspace_bytes = (size_t)w.numel() * w.element_size();
   const int rc = g_fwd(&p);

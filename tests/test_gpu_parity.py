@@ -1056,3 +1056,29 @@ def test_other_threads_run_while_a_call_waits_for_memory():
         ticker.join()
     assert took > 0.2, took                                       # the call did wait
     assert max(gaps) < took / 2, (took, max(gaps))
+
+
+@pytest.mark.parametrize("packed", [False, True])
+def test_prefill_whose_workspace_does_not_fit_runs_with_less(packed):
+    """The operands of the two-launch form take about as much memory as the inputs; a call that has room for
+    its output but not for them runs the kernel that needs none."""
+    import torch
+    H, T, dk, dv = 2, 32768, 64, 128                              # output 16 MiB, operands 28 MiB
+    torch.cuda.empty_cache()
+    q, k, x, y = (torch.empty((1, 1, T, dk), dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    v = torch.empty((1, H, T, dv), dtype=torch.bfloat16, device="cuda")
+    for t, mean, std in ((q, 0, 0.125), (k, 0, 0.125), (x, -3, 1), (y, 0, 1), (v, 0, 1)):
+        t.normal_(mean, std)
+    cu = torch.tensor([0, 1000, T], dtype=torch.int32, device="cuda") if packed else None
+    o = rd.ddts_fwd(q, k, x, y, v, cu_seqlens=cu, want_final_state=False)[0].cpu()
+    assert rd.last_launch_count() == 2 + packed
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (22 << 20)) / total)
+    try:
+        least = rd.ddts_fwd(q, k, x, y, v, cu_seqlens=cu, want_final_state=False)[0]
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert rd.last_launch_count() == 1 + packed
+    assert rel_err(host(least), host(o)) <= TOL_BF16
