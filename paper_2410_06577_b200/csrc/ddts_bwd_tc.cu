@@ -135,8 +135,11 @@ __device__ void order_tiles(const BwdTcArgs& a, int* s_nt, int* s_scan) {
       s_scan[tid] += v;
       __syncthreads();
     }
-    const int base = at + s_scan[tid] - cnt;
-    for (int j = 0; j < cnt; ++j) a.tile_order[base + j] = make_int2(a.order[j], s_nt[j] - 1 - r);
+    // a warp per rank: its sequences, the first s_scan[i] - s_scan[i - 1] of the list, lie side by side
+    for (int i = tid >> 5; i < min(kPreThreads, most - r0); i += kPreThreads / 32) {
+      const int before = i > 0 ? s_scan[i - 1] : 0, n = s_scan[i] - before;
+      for (int j = tid & 31; j < n; j += 32) a.tile_order[at + before + j] = make_int2(a.order[j], s_nt[j] - 1 - (r0 + i));
+    }
     at += s_scan[kPreThreads - 1];
     __syncthreads();
   }
@@ -147,7 +150,6 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
   __shared__ __align__(16) float s_la[kTile * DK];
   __shared__ __align__(16) float s_part[(kTile / kPreRows) * DK];
   __shared__ unsigned long long s_mask;
-  __shared__ int s_n;
   const int tid = threadIdx.x;
   if (blockIdx.x == 0 && tid == 0 && !a.cu) a.hdr->status = RODIMUS_OK;
   for (long long i = (long long)blockIdx.x * kPreThreads + tid; i < a.n_flags; i += (long long)gridDim.x * kPreThreads)
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(kPreThreads, 2) ddts_bwd_pre_kernel(const BwdT
     return;
   }
   const int head = (int)(blockIdx.x / (unsigned)a.slots_per_head), local = (int)(blockIdx.x % (unsigned)a.slots_per_head);
-  const TileRef tr = find_tile(geometry(a), head, local, &s_n);
+  const TileRef tr = find_tile<kPreThreads>(geometry(a), head, local);
   const long long slot = (long long)head * a.slots_per_head + local;
   if (tid < 4) a.tile_flag[slot * 4 + tid] = 0;
   if (tr.nr <= 0) return;

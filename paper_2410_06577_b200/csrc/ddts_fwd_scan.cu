@@ -104,14 +104,13 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
   constexpr int kOpRows = kOpRowsOf<DK>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ unsigned long long s_mask;
-  __shared__ int s_n;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
   float* s_part = reinterpret_cast<float*>(gbase + B::kBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (!a.cu && blockIdx.x == 0 && tid == 0) a.hdr->status = RODIMUS_OK;
   const int head = (int)(blockIdx.x / (unsigned)a.slots_per_head), local = (int)(blockIdx.x % (unsigned)a.slots_per_head);
-  const TileRef tr = find_tile({a.cu, a.n_seq, a.T, a.cu ? 1 : a.gate_heads}, head, local, &s_n);
+  const TileRef tr = find_tile<kOpThreads>({a.cu, a.n_seq, a.T, a.cu ? 1 : a.gate_heads}, head, local);
   let_next_kernel_start();
   if (tr.nr <= 0) return;
   const int cp = tid & (DK / 2 - 1), rg = tid / (DK / 2);

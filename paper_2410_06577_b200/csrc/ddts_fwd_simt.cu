@@ -244,29 +244,26 @@ __device__ __forceinline__ void sequence_of(const ChunkArgs& a, int n, int h, Ch
     r.slot0 = ((long long)n * a.s.H + h) * a.slots_per_head;
   }
 }
-// Block-wide.
-__device__ __forceinline__ ChunkRef chunk_of(const ChunkArgs& a, long long slot, int* s_n) {
+// Block-wide: every one of the block's THREADS threads takes part.
+template <int THREADS>
+__device__ __forceinline__ ChunkRef chunk_of(const ChunkArgs& a, long long slot) {
   ChunkRef r;
   const int head = (int)(slot / a.slots_per_head), local = (int)(slot % a.slots_per_head);
   if (!a.s.cu) {
     sequence_of(a, head / a.s.H, head % a.s.H, r);
   } else {
-    if (threadIdx.x == 0) *s_n = -1;
-    __syncthreads();
-    int best = -1;   // the last sequence whose first slot is not beyond this one
-    for (int n = threadIdx.x; n < a.s.n_seq; n += blockDim.x) {
+    // the last sequence whose first slot is not beyond this one
+    const int n = last_that_holds<THREADS>(a.s.n_seq, [&](int m) {
       ChunkRef c;
-      sequence_of(a, n, 0, c);
-      if (c.slot0 <= local) best = n;
-    }
-    if (best >= 0) atomicMax(s_n, best);
-    __syncthreads();
+      sequence_of(a, m, 0, c);
+      return c.slot0 <= local;
+    });
     r.nr = 0;
-    if (*s_n < 0) return r;
-    sequence_of(a, *s_n, head, r);
+    if (n < 0) return r;
+    sequence_of(a, n, head, r);
   }
   r.t = (int)(slot - r.slot0);
-  r.nr = min(kC, r.len - r.t * kC);
+  r.nr = r.t < 0 ? 0 : min(kC, r.len - r.t * kC);            // (negative only for a bad cu_seqlens)
   return r;
 }
 
@@ -275,7 +272,6 @@ constexpr int kOpsThreads = 1024;
 template <typename T>
 __global__ void __launch_bounds__(kOpsThreads, 1) ddts_chunk_ops_kernel(const ChunkArgs a) {
   extern __shared__ float smem[];
-  __shared__ int s_n;
   const int dk = a.s.dk, dv = a.s.dv, ld = dk + 1, tid = threadIdx.x;
   float* sQ = smem;                 // [kC][ld] q
   float* sW = sQ + kC * ld;         // [kC][ld] ahat k
@@ -284,7 +280,7 @@ __global__ void __launch_bounds__(kOpsThreads, 1) ddts_chunk_ops_kernel(const Ch
   if (!a.s.cu && blockIdx.x == 0 && tid == 0) a.s.hdr->status = RODIMUS_OK;
   const long long slot = blockIdx.x;
   let_next_kernel_start();
-  const ChunkRef r = chunk_of(a, slot, &s_n);
+  const ChunkRef r = chunk_of<kOpsThreads>(a, slot);
   if (r.nr <= 0) return;
   const long long row = r.row0 + (long long)r.t * kC;
   // rows of q,k,gx,ty: the head's own, or the sequence's single shared set
@@ -410,7 +406,6 @@ constexpr int kOutThreads = kC * kTileV;
 template <typename T>
 __global__ void __launch_bounds__(kOutThreads) ddts_chunk_out_kernel(const ChunkArgs a) {
   extern __shared__ float smem[];
-  __shared__ int s_n;
   const int dk = a.s.dk, dv = a.s.dv, tid = threadIdx.x;
   float* sS = smem;                    // [dk][kTileV]
   float* sQ = sS + dk * kTileV;        // [kC][dk]
@@ -418,7 +413,7 @@ __global__ void __launch_bounds__(kOutThreads) ddts_chunk_out_kernel(const Chunk
   float* sP = sV + kC * kTileV;        // [kC][kC]
   const long long slot = blockIdx.x / (unsigned)a.s.tiles;
   const int col0 = (int)(blockIdx.x % (unsigned)a.s.tiles) * kTileV;
-  const ChunkRef r = chunk_of(a, slot, &s_n);
+  const ChunkRef r = chunk_of<kOutThreads>(a, slot);
   if (r.nr <= 0) return;
   const long long row = r.row0 + (long long)r.t * kC;
   const int c = tid & (kTileV - 1), rr = tid / kTileV;

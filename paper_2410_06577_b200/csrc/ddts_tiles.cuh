@@ -34,8 +34,9 @@ __device__ __forceinline__ void seq_range(const int32_t* cu, int n, int T, int& 
   hi = hi < lo ? lo : (hi > T ? T : hi);
 }
 
-// Block-wide (every thread takes part; s_n is one shared int).
-__device__ __forceinline__ TileRef find_tile(const TileGeometry& a, int head, int local, int* s_n) {
+// Block-wide: every one of the block's THREADS threads takes part.
+template <int THREADS>
+__device__ __forceinline__ TileRef find_tile(const TileGeometry& a, int head, int local) {
   TileRef r;
   if (!a.cu) {
     r.n = head / a.div;
@@ -45,25 +46,20 @@ __device__ __forceinline__ TileRef find_tile(const TileGeometry& a, int head, in
     r.row0 = (long long)head * a.T + (long long)r.t * kTile;
     return r;
   }
-  if (threadIdx.x == 0) *s_n = -1;
-  __syncthreads();
-  int best = -1;   // the last sequence whose first slot is not beyond this one
-  for (int n = threadIdx.x; n < a.n_seq; n += blockDim.x) {
+  // the last sequence whose first slot is not beyond this one
+  r.n = last_that_holds<THREADS>(a.n_seq, [&](int n) {
     int lo, hi;
     seq_range(a.cu, n, a.T, lo, hi);
-    if (lo / kTile + n <= local) best = n;
-  }
-  if (best >= 0) atomicMax(s_n, best);
-  __syncthreads();
-  r.n = *s_n;
+    return lo / kTile + n <= local;
+  });
   r.nr = 0;
   if (r.n < 0) return r;
   int lo, hi;
   seq_range(a.cu, r.n, a.T, lo, hi);
   r.t = local - (lo / kTile + r.n);
   r.len = hi - lo;
-  r.nr = min(kTile, r.len - r.t * kTile);
   r.row0 = (long long)head * a.T + lo + (long long)r.t * kTile;
+  if (r.t >= 0) r.nr = min(kTile, r.len - r.t * kTile);      // (negative only for a bad cu_seqlens)
   return r;
 }
 

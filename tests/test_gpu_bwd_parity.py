@@ -230,3 +230,13 @@ def test_bwd_bad_cu_seqlens_with_overlapping_ranges_stays_in_the_workspace():
     prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
     assert rd.bwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.ERR_SEQLENS
     assert bool((ws[need:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("N", [513, 4200])                    # sorted by length; too many to sort
+def test_bwd_bf16_more_packed_sequences_than_a_block_has_threads(N):
+    lens = np.random.default_rng(N).integers(0, 3, N)
+    lens[N // 2:N // 2 + 40] = 0
+    lens[[N // 3, N // 5]] = 200, 70
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    _check(wl.make_prefill(1300 + N, 1, 1, int(cu[-1]), 128, 256, "bf16", s0_std=0.1, cu_seqlens=cu, name=f"bwd_many_{N}"),
+           1301, True)

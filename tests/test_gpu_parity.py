@@ -1082,3 +1082,14 @@ def test_prefill_whose_workspace_does_not_fit_runs_with_less(packed):
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert rd.last_launch_count() == 1 + packed
     assert rel_err(host(least), host(o)) <= TOL_BF16
+
+
+@pytest.mark.parametrize("dtype,dk,dv", [("bf16", 64, 128), ("f32", 16, 16)])
+@pytest.mark.parametrize("N", [511, 513, 1500, 4200])
+def test_more_packed_sequences_than_a_block_has_threads(dtype, dk, dv, N):
+    """A block finds the sequence of its tile in rounds; runs of empty sequences among them."""
+    lens = np.random.default_rng(N).integers(0, 4, N)
+    lens[N // 2:N // 2 + 40] = 0
+    lens[N // 3] = 200
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    _check_prefill(wl.make_prefill(990, 1, 2, int(cu[-1]), dk, dv, dtype, s0_std=0.2, cu_seqlens=cu))
