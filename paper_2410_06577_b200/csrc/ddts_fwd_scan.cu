@@ -343,10 +343,14 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   int len;
   long long slot0;
   if (a.cu) {
+    // (The plan ended before the operand kernel began.  A cu_seqlens that it has refused may leave blocks
+    // unwritten: no tile of it is looked at.  Read here the verdict costs nothing; after the wait for the
+    // operands it was 1.2 us of a small call, 24.6 us.)
+    const bool refused = *(volatile int32_t*)&hdr->status == RODIMUS_ERR_SEQLENS;
     n = a.order[n];
     int lo, hi;
     seq_range(a.cu, n, a.T, lo, hi);
-    len = hi - lo;
+    len = refused ? 0 : hi - lo;
     row0 = (long long)h * a.T + lo;
     rowq0 = (long long)hq * a.T + lo;
     slot0 = (long long)hq * a.slots_per_head + lo / kTile + n;
@@ -357,7 +361,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     slot0 = ((long long)n * a.gate_heads + hq) * a.slots_per_head;
   }
   const int col0 = slice * 128;
-  int ntiles = (len + kTile - 1) / kTile;
+  const int ntiles = (len + kTile - 1) / kTile;
   const long long state_off = ((long long)n * a.H + h) * DK * (long long)a.dv + col0;
 
   if (tid == 0) {
@@ -386,8 +390,6 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
   wait_for_previous_kernel();   // the operands are there
-  // A cu_seqlens that the plan has refused may leave blocks unwritten: no tile of it is looked at.
-  if (a.cu && *(volatile int32_t*)&hdr->status == RODIMUS_ERR_SEQLENS) ntiles = 0;
   auto wait_all = [&](int b, uint32_t parity) -> bool {   // whole warps: tensor-memory accesses need them
     return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, wc, hdr)) != 0;
   };
