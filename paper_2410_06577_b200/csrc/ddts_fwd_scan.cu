@@ -29,6 +29,7 @@
 // rows of Kt set to zero.
 #include <cuda.h>
 
+#include <cmath>
 #include <cstring>
 
 #include "ddts_common.cuh"
@@ -861,39 +862,72 @@ cudaError_t launch_scan(const ScanMaps& m, const ScanArgs& a, long long slots, l
 
 }  // namespace
 
+namespace {
+// One set of gates for all heads, against the pair kernel: microseconds of both for rows of `tiles` tiles in
+// each of n_seq sequences, `slabs` of 256 value columns that share a set, on `sms` SMs.  A pair of SMs takes
+// 3 us for the start and end of an item and 2.3 us a tile, two CTAs of the scan 5.2 and 1.1, and the operands
+// of a tile, formed once for all slabs, 2.2 us of such a pair.  (Fitted to 99 shapes of 2 to 16 slabs, 16 to
+// 2048 tokens and 8 to 4096 sequences; at none does the choice cost more than 4 %.  64 sequences of 1024
+// tokens, 4 slabs: pair 158 us, scan 115; 4096 of 1 to 16 tokens: 1629 and 1905.)
+bool scan_pays_with_shared_gates(long long n_seq, double tiles, double slabs, bool varlen, int sms) {
+  const double rounds = 2.0 * (double)n_seq * slabs / sms;
+  const double pair = 6.0 + 3.0 * rounds + 2.3 * tiles * (varlen ? rounds : std::ceil(rounds));
+  const double scan = 5.2 * rounds + tiles * rounds * (1.1 + 2.2 / slabs);
+  return scan < pair;
+}
+}  // namespace
+
 // Which requests this file's kernels compute, given room for the tiles' blocks; bytes of that room
 // (0: not this path).  All timings are one call, the other kernel against this path.
 //   dk = 64            always (B=4 H=16 T=2048, one set of gates: fp32 CUDA-core kernel 3.9 ms, here
-//                      47 us); not with block terms, whose products the fp32 kernel does not round.
-//   one set of gates   always where the pair kernel would be the other choice (same precision; layer
-//                      shape 82 -> 40 us).
+//                      47 us; 20000 sequences of 1 to 8 tokens 29 -> 12 ms); not with block terms, whose
+//                      products the fp32 kernel does not round.
+//   one set of gates   where the pair kernel would be the other choice (same precision), by the cost of both
+//                      (above); layer shape 82 -> 40 us.
 //   gates per head     the gates cost the same in both, here their operands travel through memory, and
-//                      here they are formed by all SMs however few the heads are:
+//                      here they are formed by all SMs however few the heads are; sequences of four tiles
+//                      or more on average:
 //       dv % 256 == 0  against the pair kernel, when a dense call has at most a quarter as many items of
 //                      256 columns as there are SMs (16 items x 2048 rows 77 -> 47 us, 32 items 79 ->
 //                      67, 37 x 1024 45 -> 39, but 48 x 1024 47 -> 47 and 64 x 2048 82 -> 101), a packed
-//                      one, whose longest sequence keeps the other pairs waiting, half as many (64 items
-//                      of 100..1500 rows 59 -> 47 us); sequences of four tiles or more on average.
-//       odd multiples  against the single-CTA kernel: dense calls (B=4 H=16 T=2048 dv=128 146 -> 96 us,
-//       of 128         1 x 16 x 1000 76 -> 27) and packed ones with no more items than SMs (640 items
-//                      307 -> 329 us).
+//                      one, whose longest sequence keeps the other pairs waiting, three eighths (56 items
+//                      of 64..1000 rows 45 -> 40 us, of 1..4096 135 -> 123; 72 items 45 -> 49 and 138 ->
+//                      143).  Packed sequences of one length would change sides at the dense call's line:
+//                      56 items of 300 rows 24.6 either way, of 1500 64 -> 80.
+//       odd multiples  against the single-CTA kernel, which forms the gates in every CTA and takes the
+//       of 128         same time for one item and for one on every SM.  Dense: up to three sets of gates
+//                      for four CTAs of its rounds (T=2048, dv=128: 100 items 141 -> 131 us, 148 144 ->
+//                      181, 149 274 -> 201, 256 280 -> 307; dv=384, three slices a set, always: 64 sets x
+//                      1000 150 -> 73).  Packed: one slice a set, up to seven items for eight SMs (128
+//                      items of 64..1000 rows 72 -> 60, of 650 62 -> 69, 148 of 650 62 -> 78), more slices,
+//                      up to one for every SM.
 size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
   if (p.dtype != RODIMUS_BF16 || p.value_decay || p.dv % 128 || (p.dk != 64 && p.dk != 128)) return 0;
   const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
   const bool block = p.beta_hat || p.feed_d, whole = p.dv % 256 == 0;
-  const long long n_seq = varlen ? p.N : p.B, items = n_seq * p.H * (p.dv / 128);
+  const long long n_seq = varlen ? p.N : p.B, sets = n_seq * p.H, items = sets * (p.dv / 128);
   if (p.dk == 64) {
     if (block) return 0;
-  } else if (p.shared_gates) {
-    if (!whole) return 0;
   } else {
     int dev = 0, sms = 0;
     if (current_device(&dev, &sms) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
-    if (n_seq == 0 || p.T / (varlen ? n_seq : 1) < 4 * kTile) return 0;
-    if (whole ? items > (varlen ? sms : sms / 2) : (block || (varlen && items > sms))) return 0;
+    if (items == 0) return 0;
+    if (p.shared_gates) {
+      const double tiles = varlen ? (double)p.T / ((double)n_seq * kTile) + 0.5 : (double)((p.T + kTile - 1) / kTile);
+      if (!whole || !scan_pays_with_shared_gates(n_seq, tiles, p.H * (p.dv / 256.0), varlen, sms)) return 0;
+    } else {
+      if (p.T / (varlen ? n_seq : 1) < 4 * kTile) return 0;
+      if (whole) {
+        if (varlen ? 4 * items > 3 * sms : 2 * items > sms) return 0;
+      } else if (varlen) {
+        if (block || (p.dv == 128 ? 8 * items > 7 * sms : items > sms)) return 0;
+      } else if (block || 4 * sets > 3 * sms * ((items + sms - 1) / sms)) {
+        return 0;
+      }
+    }
   }
   const ScanPlan s = scan_plan(p);
   if (s.slots > 0x7fffffffLL || items > 0x7fffffffLL) return 0;

@@ -1,6 +1,7 @@
 """GPU parity: the CUDA library, called through its C ABI, against the fp64 CPU oracle on the
 same seeded inputs.  Bar: max|err|/max|ref| <= 2e-2 (bf16 in, fp32 accumulate) and <= 1e-4
 (fp32 build), per output tensor (o and the final state separately)."""
+import ctypes
 import os
 
 import numpy as np
@@ -1093,3 +1094,28 @@ def test_more_packed_sequences_than_a_block_has_threads(dtype, dk, dv, N):
     lens[N // 3] = 200
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
     _check_prefill(wl.make_prefill(990, 1, 2, int(cu[-1]), dk, dv, dtype, s0_std=0.2, cu_seqlens=cu))
+
+
+def test_two_launch_prefill_is_chosen_where_it_is_the_faster_one():
+    """Both sides of each line of the rule, in items per SM."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+
+    def chosen(n_seq, H, T, dv, shared=0, packed=False):
+        p = rd.FwdParams()
+        p.struct_size, p.dtype, p.scale, p.shared_gates = ctypes.sizeof(rd.FwdParams), rd.BF16, 1.0, shared
+        p.B, p.H, p.T, p.dk, p.dv = 1 if packed else n_seq, H, n_seq * T if packed else T, 128, dv
+        p.N, p.cu_seqlens = (n_seq, 0x7F0000000000) if packed else (0, None)
+        return rd.fwd_workspace_bytes(p) > 256 + 4 * (n_seq + 63)
+
+    # a set of gates per head, whole pairs: a quarter of an item of 256 columns per SM, packed 3 / 8
+    assert chosen(sms // 4, 1, 256, 256) and not chosen(sms // 4 + 1, 1, 256, 256) and not chosen(4, 1, 255, 256)
+    assert chosen(3 * sms // 8, 1, 256, 256, packed=True) and not chosen(3 * sms // 8 + 1, 1, 256, 256, packed=True)
+    # odd multiples of 128: three sets of gates for four CTAs of the rounds
+    assert chosen(3 * sms // 4, 1, 512, 128) and not chosen(sms, 1, 512, 128)
+    assert chosen(sms + 1, 1, 512, 128) and not chosen(2 * sms, 1, 512, 128) and chosen(sms, 1, 512, 384)
+    assert chosen(7 * sms // 8, 1, 512, 128, packed=True) and not chosen(sms, 1, 512, 128, packed=True)
+    # one set of gates: few items, or sequences of some tiles, the fewer the more heads share a set
+    assert chosen(8, 16, 64, 256, 1) and not chosen(64, 16, 64, 256, 1) and chosen(64, 16, 65, 256, 1)
+    assert not chosen(256, 4, 128, 256, 1) and chosen(256, 4, 200, 256, 1)
+    assert not chosen(4096, 4, 16, 256, 1, packed=True) and chosen(512, 8, 128, 256, 1, packed=True)
