@@ -489,14 +489,36 @@ cudaError_t launch_chunks(const ChunkArgs& a, int dev, cudaStream_t st) {
 }  // namespace
 
 // Workspace with which this kernel's chunks are computed side by side; 0: they are not.  The states of
-// the chunks cross memory four times, which pays while they stay in L2 (126 MB): up to 64 MiB of them.
+// the chunks cross memory four times: up to 64 MiB of them, which stay in L2 (126 MB).
 // B=1 H=1 T=256 dk=dv=64 fp32: one CTA walking the 16 chunks 318 us, side by side 16.4 us a call.
+// The walk takes 4 to 45 us a chunk (dk = 16 to 256) whether it has sixteen rows or one, for several CTAs on
+// an SM at once (one with dk > 128); this form pays for every chunk and column tile, so it is not taken where
+// chunks are mostly empty and more than fill the device by themselves: 1024 items of 17 rows, dk = dv = 64,
+// 121 us in the walk and 174 side by side, of 48 rows 364 and 304; 300 items of 33 rows 101 and 82; 148 of
+// 17 31 and 31; 64 of 17, dk = dv = 256, 133 and 99.  And one block forms a chunk's whole contribution to the
+// state, one column tile after another: with dk = 256, dv = 1024 in 110 us, so that needs three chunks to pay
+// (17 rows 68 and 123 us, 33 113 and 124, 48 141 and 124), two where the walk's CTAs take several rounds (16
+// items of 17 rows 133 and 160, of 32 190 and 172).
 size_t fwd_simt_chunks_workspace_bytes(const rodimus_ddts_fwd_params& p) {
   if (p.value_decay || (long long)p.B * p.H * p.T == 0 || p.T <= kC) return 0;
-  if ((p.cu_seqlens || p.cu_seqlens_host) && p.N == 0) return 0;
+  const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
+  if (varlen && p.N == 0) return 0;
   const ChunkPlan c = chunk_plan(p);
-  if (c.slots * ((p.dv + kTileV - 1) / kTileV) > 0x7fffffffLL) return 0;
-  return c.qe - c.states <= (size_t)64 << 20 ? c.bytes : 0;
+  const long long tiles = (p.dv + kTileV - 1) / kTileV;
+  if (c.slots * tiles > 0x7fffffffLL) return 0;
+  if (c.qe - c.states > (size_t)64 << 20) return 0;
+  int dev = 0, sms = 0;
+  if (current_device(&dev, &sms) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  // chunks of a head: of a packed call about half of a chunk a sequence is left over
+  const double chunks = varlen ? (double)p.T / kC + 0.5 * p.N : (double)c.slots_per_head;
+  const double rows = p.T / chunks, work = chunks * c.heads * tiles;
+  if (rows < 12.0 && work > (rows < 10.0 ? 2.0 : 16.0) * (p.dk > 128 ? 4.0 : 1.0) * sms) return 0;
+  const long long n_seq = varlen ? p.N : p.B;
+  if (p.dk * p.dv > 65536 && p.T < (n_seq * p.H * tiles > sms ? 2 : 3) * kC * (varlen ? n_seq : 1)) return 0;
+  return c.bytes;
 }
 
 cudaError_t launch_fwd_simt(const rodimus_ddts_fwd_params& p, int* n_launches) {

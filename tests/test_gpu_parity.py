@@ -1119,3 +1119,11 @@ def test_two_launch_prefill_is_chosen_where_it_is_the_faster_one():
     assert chosen(8, 16, 64, 256, 1) and not chosen(64, 16, 64, 256, 1) and chosen(64, 16, 65, 256, 1)
     assert not chosen(256, 4, 128, 256, 1) and chosen(256, 4, 200, 256, 1)
     assert not chosen(4096, 4, 16, 256, 1, packed=True) and chosen(512, 8, 128, 256, 1, packed=True)
+
+
+@pytest.mark.parametrize("items,T,dk,dv,launches", [(4, 17, 64, 64, 3), (300, 17, 16, 16, 1), (600, 33, 16, 64, 3), (600, 33, 16, 80, 1),
+                                                    (600, 32, 16, 16, 3), (1, 47, 256, 272, 1), (1, 48, 256, 272, 3)])
+def test_fp32_chunks_side_by_side_are_chosen_where_they_are_the_faster_form(items, T, dk, dv, launches):
+    """Both sides of each line of the rule (on 148 SMs), and both forms against the oracle."""
+    _check_prefill(wl.make_prefill(995, items, 1, T, dk, dv, "f32", s0_std=0.2))
+    assert rd.last_launch_count() == launches
