@@ -70,11 +70,43 @@ struct ScanArgs {
   long long limit;
 };
 
+// Decays and their sums.  dk = 64: exact sums, so that 2^b is as exact as the rows' own decays are.  (An fp32
+// sum near -60 carries 2^-19 into every operand made of it: 1e-6 of the final state where gates decay fast,
+// 2e-7 in the fp32 kernel, which forms differences before the exponential, 1e-7 here.  It costs 0.9 % of a
+// call at the layer shape; sums in fp64, as exact, 2.7 %.)
 template <bool EXACT>
-__device__ __forceinline__ void gate_pair(float x, float y, int ingate, float& la2, float& lh2) {
-  if (EXACT) {
-    gate_logs_f32(x, y, ingate, la2, lh2);
-    la2 = fmaxf(la2 * kLog2e, -kRange2);
+struct Decay {
+  using One = float;
+  using Two = float2;
+};
+template <>
+struct Decay<true> {
+  using One = ExactSum;
+  using Two = ExactSum2;
+};
+// 2^b, and 2^(lh - b)
+__device__ __forceinline__ void exp2_of(float b, float lh, float& e, float& ek) {
+  e = ex2f(b);
+  ek = ex2f(lh - b);
+}
+__device__ __forceinline__ float scaled(float e, float rest) { return fmaf(e, rest * 0.69314718f, e); }   // e 2^rest, rest tiny
+__device__ __forceinline__ void exp2_of(ExactSum b, float lh, float& e, float& ek) {
+  const float t = b.h + b.l, r = (b.h - t) + b.l;             // b = t + r
+  e = scaled(ex2f(t), r);
+  const float u = lh - t, z = u - lh, d = (lh - (u - z)) - (t + z);   // lh - t = u + d
+  ek = scaled(ex2f(u), d - r);
+}
+
+template <bool EXACT>
+__device__ __forceinline__ void gate_pair(float x, float y, int ingate, typename Decay<EXACT>::One& la2, float& lh2) {
+  if constexpr (EXACT) {
+    float la;
+    gate_logs_f32(x, y, ingate, la, lh2);
+    const float p = fmaxf(la * kLog2e, -kRange2);
+    const float rest = p > -kRange2 ? fmaf(la, kLog2e, -p) + la * 1.925963e-8f : 0.f;   // log2 e to 48 bits
+    constexpr float kRound = 12288.f;                         // 1.5 * 2^13: adding it rounds to 2^-10
+    la2.h = (p + kRound) - kRound;
+    la2.l = (p - la2.h) + rest;
     lh2 *= kLog2e;
   } else {
     const Gate g = gate_of(x, y, ingate);
@@ -97,17 +129,19 @@ constexpr int kOpThreads = 512;
 template <int DK>
 constexpr int kOpRowsOf = DK / 16;          // 4 or 8 rows x 2 channels a thread
 template <int DK>
-constexpr int kOpSmem = Block<DK>::kBytes + (kTile / kOpRowsOf<DK>) * DK * 4 + 1024;
+constexpr int kOpSmem = Block<DK>::kBytes + (kTile / kOpRowsOf<DK>) * DK * (int)sizeof(typename Decay<Block<DK>::kExact>::One) + 1024;
 
 template <int DK>
 __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const ScanArgs a) {
   using B = Block<DK>;
+  using Sum = typename Decay<B::kExact>::One;
+  using Sums = typename Decay<B::kExact>::Two;
   constexpr int kOpRows = kOpRowsOf<DK>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ unsigned long long s_mask;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
-  float* s_part = reinterpret_cast<float*>(gbase + B::kBytes);
+  Sum* s_part = reinterpret_cast<Sum*>(gbase + B::kBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (!a.cu && blockIdx.x == 0 && tid == 0) a.hdr->status = RODIMUS_OK;
   const int head = (int)(blockIdx.x / (unsigned)a.slots_per_head), local = (int)(blockIdx.x % (unsigned)a.slots_per_head);
@@ -132,16 +166,17 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
       wk[i] = __ldg(k + i * (DK / 2));
     }
   }
-  float2 b[kOpRows], lh2[kOpRows];
+  Sums b[kOpRows];
+  float2 lh2[kOpRows];
 #pragma unroll
   for (int i = 0; i < kOpRows; ++i) {
     const float2 x = unpack_bf16(wx[i]), y = unpack_bf16(wy[i]);
     gate_pair<B::kExact>(x.x, y.x, a.ingate, b[i].x, lh2[i].x);
     gate_pair<B::kExact>(x.y, y.y, a.ingate, b[i].y, lh2[i].y);
-    if (i >= live) b[i] = make_float2(0.f, 0.f);
+    if (i >= live) b[i] = {};
   }
   auto la_of = [&](int i) {
-    float2 la = make_float2(0.f, 0.f);
+    Sums la = {};
     if (i >= live) return la;
     const float2 x = unpack_bf16(__ldg(gx + i * (DK / 2))), y = unpack_bf16(__ldg(ty + i * (DK / 2)));
     float lh;
@@ -150,7 +185,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
     return la;
   };
   // (the scan's scratch lies where the operands go next)
-  const unsigned long long mask = tile_scan<kOpRows, DK, true>(b, cp, rg, tr.nr, reinterpret_cast<float*>(gbase), s_part,
+  const unsigned long long mask = tile_scan<kOpRows, DK, true>(b, cp, rg, tr.nr, reinterpret_cast<Sum*>(gbase), s_part,
                                                                &s_mask, 0ull, la_of);
   {
     const uint32_t w = base + (cp >> 5) * kSlab + ((cp & 3) << 2), c16 = (uint32_t)(cp & 31) >> 2;
@@ -159,7 +194,9 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
       const int r = rg * kOpRows + i;
       const uint32_t at = w + r * 128 + ((c16 ^ (uint32_t)(r & 7)) << 4);
       const float2 qv = unpack_bf16(wq[i]), kv = unpack_bf16(wk[i]);
-      const float ex = ex2f(b[i].x), ey = ex2f(b[i].y);
+      float ex, ey, kex, key;
+      exp2_of(b[i].x, lh2[i].x, ex, kex);
+      exp2_of(b[i].y, lh2[i].y, ey, key);
       float qx = qv.x * a.scale * ex, qy = qv.y * a.scale * ey;
 #pragma unroll
       for (int p = 0; p < B::kQp; ++p) {
@@ -169,7 +206,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
         qx -= f.x;
         qy -= f.y;
       }
-      float kx = kv.x * ex2f(lh2[i].x - b[i].x), ky = kv.y * ex2f(lh2[i].y - b[i].y);
+      float kx = kv.x * kex, ky = kv.y * key;
 #pragma unroll
       for (int p = 0; p < B::kKp; ++p) {
         const uint32_t h = pack_bf16(kx, ky);
@@ -592,12 +629,14 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         float* dc = reinterpret_cast<float*>(gbase + C::kOffDc) + (n_cut & 7) * DK;
         for (int ch = lane; ch < DK; ch += 32) {
           const long long e = d->rowq * DK + ch;
-          float acc = 0.f, lh, la;
+          typename Decay<B::kExact>::One acc = {}, la;
+          float lh, D;
           for (int r = lo; r < hi; ++r) {
             gate_pair<B::kExact>(__bfloat162float(a.gx[e + r * DK]), __bfloat162float(a.ty[e + r * DK]), a.ingate, la, lh);
-            acc += la;
+            acc = sum1(acc, la);
           }
-          dc[ch] = ex2f(acc);
+          exp2_of(acc, 0.f, D, lh);
+          dc[ch] = D;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(FB_CUT0 + (n_cut & 7)));

@@ -108,40 +108,59 @@ __device__ __forceinline__ int chunk_end(unsigned long long mask, int r, int nr)
   return later ? __ffsll((long long)later) - 1 : nr;
 }
 
+// A sum of up to 64 decays (log2, none below -kRange2) without rounding: multiples of 2^-10, whose sums fit
+// 24 bits, and the rest, whose sums stay below 2^-5.
+struct ExactSum {
+  float h, l;
+};
+struct __align__(16) ExactSum2 {
+  ExactSum x, y;
+};
+__device__ __forceinline__ float sum1(float a, float b) { return a + b; }
+__device__ __forceinline__ ExactSum sum1(ExactSum a, ExactSum b) {
+  const float2 r = __fadd2_rn(make_float2(a.h, a.l), make_float2(b.h, b.l));
+  return {r.x, r.y};
+}
+__device__ __forceinline__ float2 sum2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ ExactSum2 sum2(ExactSum2 a, ExactSum2 b) { return {sum1(a.x, b.x), sum1(a.y, b.y)}; }
+__device__ __forceinline__ bool beyond_range(float s) { return s < -kRange2; }
+__device__ __forceinline__ bool beyond_range(ExactSum s) { return s.h + s.l < -kRange2; }
+
 // Cumulative decay (log2) since the chunk's start, in place, for ROWS rows of two of the CTA's CH
-// channels; v holds the rows' own log2 decays on entry.  `part` is a [kTile / ROWS][CH] float tile,
+// channels; v holds the rows' own log2 decays on entry.  `part` is a [kTile / ROWS][CH] tile,
 // `la` a [kTile][CH] one that is used only where a tile has several chunks; la_of(i) then gives row i's
 // own decays again.  Returns the tile's chunk mask: the given one or, when MAKE_MASK, the one it
 // determines (dyadic blocks whose decay exceeds the range in some channel are cut in the middle).
-template <int ROWS, int CH, bool MAKE_MASK, typename LaOf>
-__device__ __forceinline__ unsigned long long tile_scan(float2 (&v)[ROWS], int cp, int rg, int nr, float* la, float* part,
+// V: two channels' decays as S each, float or ExactSum.
+template <int ROWS, int CH, bool MAKE_MASK, typename V, typename S, typename LaOf>
+__device__ __forceinline__ unsigned long long tile_scan(V (&v)[ROWS], int cp, int rg, int nr, S* la, S* part,
                                                         unsigned long long* s_mask, unsigned long long mask, LaOf la_of) {
   constexpr int kGroups = kTile / ROWS;
 #pragma unroll
-  for (int i = 1; i < ROWS; ++i) v[i] = __fadd2_rn(v[i], v[i - 1]);
-  *reinterpret_cast<float2*>(part + rg * CH + 2 * cp) = v[ROWS - 1];
+  for (int i = 1; i < ROWS; ++i) v[i] = sum2(v[i], v[i - 1]);
+  *reinterpret_cast<V*>(part + rg * CH + 2 * cp) = v[ROWS - 1];
   __syncthreads();
-  float2 pre = make_float2(0.f, 0.f), all = make_float2(0.f, 0.f);
+  V pre = {}, all = {};
 #pragma unroll
   for (int w = 0; w < kGroups; ++w) {
     if (w == rg) pre = all;
-    all = __fadd2_rn(all, *reinterpret_cast<const float2*>(part + w * CH + 2 * cp));
+    all = sum2(all, *reinterpret_cast<const V*>(part + w * CH + 2 * cp));
   }
   bool whole;
   if (MAKE_MASK) {
-    whole = __syncthreads_or(all.x < -kRange2 || all.y < -kRange2) == 0;
+    whole = __syncthreads_or(beyond_range(all.x) || beyond_range(all.y)) == 0;
     mask = 1ull;
   } else {
     whole = mask == 1ull;
   }
   if (whole) {
 #pragma unroll
-    for (int i = 0; i < ROWS; ++i) v[i] = __fadd2_rn(v[i], pre);
+    for (int i = 0; i < ROWS; ++i) v[i] = sum2(v[i], pre);
     return mask;
   }
   // ---- rare: several chunks in the tile
 #pragma unroll 1
-  for (int i = 0; i < ROWS; ++i) *reinterpret_cast<float2*>(la + (rg * ROWS + i) * CH + 2 * cp) = la_of(i);
+  for (int i = 0; i < ROWS; ++i) *reinterpret_cast<V*>(la + (rg * ROWS + i) * CH + 2 * cp) = la_of(i);
   if (MAKE_MASK) {
     if (threadIdx.x == 0) *s_mask = 1ull;
     __syncthreads();
@@ -151,9 +170,9 @@ __device__ __forceinline__ unsigned long long tile_scan(float2 (&v)[ROWS], int c
       for (int len = kTile; len >= 2; len >>= 1)
 #pragma unroll 1
         for (int r0 = 0; r0 < nr; r0 += len) {
-          float s = 0.f;
-          for (int r = r0; r < min(r0 + len, nr); ++r) s += la[r * CH + d];
-          if (s < -kRange2 && r0 + len / 2 < nr) m |= 1ull << (r0 + len / 2);
+          S s = {};
+          for (int r = r0; r < min(r0 + len, nr); ++r) s = sum1(s, la[r * CH + d]);
+          if (beyond_range(s) && r0 + len / 2 < nr) m |= 1ull << (r0 + len / 2);
         }
       if (m) atomicOr(s_mask, m);
     }
@@ -165,11 +184,11 @@ __device__ __forceinline__ unsigned long long tile_scan(float2 (&v)[ROWS], int c
 #pragma unroll 1
   for (int i = 0; i < ROWS; ++i) {
     const int r = rg * ROWS + i;
-    float2 acc = make_float2(0.f, 0.f);
+    V acc = {};
     if (r < nr) {
       for (int j = chunk_start(mask, r); j <= r; ++j) {
-        acc.x += la[j * CH + 2 * cp];
-        acc.y += la[j * CH + 2 * cp + 1];
+        acc.x = sum1(acc.x, la[j * CH + 2 * cp]);
+        acc.y = sum1(acc.y, la[j * CH + 2 * cp + 1]);
       }
     }
 #pragma unroll

@@ -1127,3 +1127,15 @@ def test_fp32_chunks_side_by_side_are_chosen_where_they_are_the_faster_form(item
     """Both sides of each line of the rule (on 148 SMs), and both forms against the oracle."""
     _check_prefill(wl.make_prefill(995, items, 1, T, dk, dv, "f32", s0_std=0.2))
     assert rd.last_launch_count() == launches
+
+
+@pytest.mark.parametrize("gate_mean", [-3.0, 0.0, 2.0])
+@pytest.mark.parametrize("ingate", [rd.INGATE_POW_G, rd.INGATE_POW_SIGMOID])
+def test_two_launch_prefill_narrow_keys_keep_fp32_accuracy_however_fast_gates_decay(gate_mean, ingate):
+    """dk = 64: the final state within 5e-7 (2-norm), about eight fp32 roundings: the exponential's two units
+    in the last place, three products and the sums.  (The fp32 kernel has 1.4e-7 to 2e-7; exponents summed in
+    fp32 gave 1e-6 where gates decay fast.)"""
+    p = wl.make_prefill(996, 1, 2, 2048, 64, 128, "bf16", gate_mean=gate_mean, s0_std=0.1)
+    _, sT = _run_prefill(p, ingate, 1.0)
+    _, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0, ingate=ingate)
+    assert np.linalg.norm(sT - rs) <= 5e-7 * np.linalg.norm(rs)
