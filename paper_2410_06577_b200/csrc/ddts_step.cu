@@ -35,7 +35,9 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
   __shared__ float s_alpha[kMaxDk];
   __shared__ float s_w[kMaxDk];   // ahat * k
   __shared__ float s_q[kMaxDk];   // scale * q
-  __shared__ float4 s_red[W][LC];
+  constexpr bool kNarrow = LC < 32;
+  __shared__ float4 s_red[4][LC];
+  __shared__ float4 s_new[kNarrow ? kMaxDk : 1][LC];   // narrow: the new state of the tile
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
@@ -88,7 +90,7 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
       for (int j = 0; j < BATCH; ++j) {
         const int r = base + row0 + kStride * j;
         if (col_ok && r < dk) {
-          const float a = s_alpha[r], w = s_w[r], qq = s_q[r];
+          const float a = s_alpha[r], w = s_w[r], qq = kNarrow ? 0.f : s_q[r];
           float4 s = buf[j];
           if (VDECAY) {
             s.x = fmaf(a * bd.x, s.x, w * vv.x);
@@ -101,10 +103,14 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             s.z = fmaf(a, s.z, w * vv.z);
             s.w = fmaf(a, s.w, w * vv.w);
           }
-          acc.x = fmaf(qq, s.x, acc.x);
-          acc.y = fmaf(qq, s.y, acc.y);
-          acc.z = fmaf(qq, s.z, acc.z);
-          acc.w = fmaf(qq, s.w, acc.w);
+          if (kNarrow) {
+            s_new[r][cl] = s;
+          } else {
+            acc.x = fmaf(qq, s.x, acc.x);
+            acc.y = fmaf(qq, s.y, acc.y);
+            acc.z = fmaf(qq, s.z, acc.z);
+            acc.w = fmaf(qq, s.w, acc.w);
+          }
           st_stream(reinterpret_cast<float4*>(S + (long long)r * dv), s);
         }
       }
@@ -119,20 +125,25 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
       }
     }
 
-    // o = sum over the row subsets of the warp's lane groups, then of the warps.
-#pragma unroll
-    for (int m = LC; m < 32; m <<= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, m);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, m);
-      acc.z += __shfl_xor_sync(0xffffffffu, acc.z, m);
-      acc.w += __shfl_xor_sync(0xffffffffu, acc.w, m);
+    // o = sum over the rows of q S: rows g, g + 4, g + 8 ... in turn, then the four subsets.  One order for both
+    // tile widths, so that a sequence's output does not depend on how many others are in the call.
+    if (kNarrow) {
+      __syncthreads();
+      if (warp < 4) {                          // a subset and column a thread
+        float sum = 0.f;
+        const float* col_of = reinterpret_cast<const float*>(s_new) + lane;
+#pragma unroll 8
+        for (int r = warp; r < dk; r += 4) sum = fmaf(s_q[r], col_of[r * kTileCols], sum);
+        reinterpret_cast<float*>(s_red)[warp * kTileCols + lane] = sum;
+      }
+    } else {
+      s_red[warp][lane] = acc;
     }
-    if (lane < LC) s_red[warp][lane] = acc;
     __syncthreads();
     if (tid < LC && col_ok) {
       float4 t = s_red[0][lane];
 #pragma unroll
-      for (int w = 1; w < W; ++w) {
+      for (int w = 1; w < 4; ++w) {
         const float4 u = s_red[w][lane];
         t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
       }

@@ -1139,3 +1139,22 @@ def test_two_launch_prefill_narrow_keys_keep_fp32_accuracy_however_fast_gates_de
     _, sT = _run_prefill(p, ingate, 1.0)
     _, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0, ingate=ingate)
     assert np.linalg.norm(sT - rs) <= 5e-7 * np.linalg.norm(rs)
+
+
+@pytest.mark.parametrize("dtype,H,dk,dv", [("bf16", 16, 128, 256), ("f32", 3, 48, 80), ("bf16", 2, 256, 272)])
+@pytest.mark.parametrize("terms", [False, True])
+def test_decode_of_a_sequence_does_not_depend_on_the_batch(dtype, H, dk, dv, terms):
+    """Small calls use a narrower tile; state and output agree bit for bit with those of a large batch."""
+    import torch
+    Nseq, few = 200, 2
+    w = wl.make_decode(971, Nseq, H, dk, dv, ring=1, dtype=dtype)
+    state = torch.from_numpy(w.state).cuda()
+    args = [dev(a[0], dtype) for a in (w.q, w.k, w.x, w.y, w.v)]
+    opt = {}
+    if terms:
+        opt = dict(beta_hat=torch.sigmoid(args[4]), feed_d=torch.randn((H, dv), device="cuda"), feed_x=args[4].clone(),
+                   value_decay=torch.sigmoid(args[4]))
+    part = state[:few].clone()
+    o_part = rd.ddts_step(*(a[:few] for a in args), part, **{n: t if n == "feed_d" else t[:few] for n, t in opt.items()})
+    o = rd.ddts_step(*args, state, **opt)
+    assert torch.equal(part, state[:few]) and torch.equal(o_part, o[:few])
