@@ -96,7 +96,7 @@ constexpr int kOffTx = kOffDp + 4 * kDK * 4;              // float [2][68]: bloc
 constexpr int kOffRx = kOffTx + kRxBufs * kBlkBytes;      // float [2][68]: block received
 constexpr int kGateWarp0 = 12, kGateWarps = 16;
 constexpr int kGR = kC / kGateWarps;                       // rows per gate thread
-constexpr int kOffTot = kOffRx + kRxBufs * kBlkBytes;     // float [2][8][64]: scan partials
+constexpr int kOffTot = kOffRx + kRxBufs * kBlkBytes;     // float [2][16][64]: scan partials
 constexpr int kOffAll = kOffTot + 2 * kGateWarps * kCH * 4;   // float [2][64]: decay totals of a tile
 constexpr int kOffBar = kOffAll + 2 * kCH * 4;
 constexpr int kNumBars = 44;
@@ -106,7 +106,7 @@ constexpr int kSmemBytes = kSmemUsed + 1024;              // slack for manual 10
 static_assert(kOffTx % 16 == 0 && kOffRx % 16 == 0 && kBlkBytes % 16 == 0, "bulk copy alignment");
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 
-constexpr int kThreads = 32 * (kGateWarp0 + kGateWarps);   // 896: 28 warps (warp 24 has no role)
+constexpr int kThreads = 32 * (kGateWarp0 + kGateWarps);   // 896: 28 warps
 
 // TMEM columns (32-bit words): two state buffers S^T [lane = value column][128 channels], output
 // O^T [lane = value column][64 rows], scores P [64 rows in 16-lane groups][64], and two buffers
@@ -1435,7 +1435,7 @@ namespace {
 //   combine    S_start(k+1) = D(k) . S_start(k) + dS(k), k = 1..G-1 (elementwise, tiny)
 //   launch C   segments 1..G from their true initial states: outputs, final state
 // Segment 0 is shorter by the ratio of a state-only pass to a full pass, so that A and C0 end
-// together; the whole trades about (2G - 0.2)/(G + 0.8) of the work for G times the parallelism.
+// together; the whole trades about (2G - 0.2)/(G + 0.8) of the work (plain calls) for G times the parallelism.
 struct SplitPlan {
   int G = 0;            // segments after the head segment (0: do not split)
   int L0 = 0;           // rows of the head segment (any number: T - G * L)
@@ -1445,8 +1445,10 @@ struct SplitPlan {
 
 constexpr int kMinSegmentRows = 2048;
 constexpr int kMaxSegments = 16;
-constexpr double kStateOnlyCost = 0.8;   // head segment length relative to the others (state-only pass / full pass; of
-                                         // 0.65, 0.72, 0.78, 0.85: 422, 415, 411, 410 us for 16 x 32768 tokens)
+// Head segment's length relative to the others': a state-only pass against a full one, which is longer with the
+// block's terms.  Of 0.65, 0.72, 0.8 (heads x tokens, us): 16 x 32768 432, 426, 421, 32 x 16384 399, 389, 376,
+// 4 x 8192 126, 126, 123; with block terms 628, 643, 661, 575, 581, 585 and 168, 168, 175.
+constexpr double kStateOnlyCost = 0.8, kStateOnlyCostBlock = 0.65;
 
 SplitPlan make_split_plan(const rodimus_ddts_fwd_params& p) {
   SplitPlan sp;
@@ -1462,7 +1464,8 @@ SplitPlan make_split_plan(const rodimus_ddts_fwd_params& p) {
   if (g > p.T / kMinSegmentRows) g = p.T / kMinSegmentRows;
   if (g > kMaxSegments) g = kMaxSegments;
   if (g < 2) return sp;
-  int L = (int)((long long)(p.T / (g + kStateOnlyCost)) + kC - 1) / kC * kC;
+  const double head = p.beta_hat || p.feed_d ? kStateOnlyCostBlock : kStateOnlyCost;
+  int L = (int)((long long)(p.T / (g + head)) + kC - 1) / kC * kC;
   if ((long long)g * L >= p.T) L = (int)((p.T / (g + 1)) / kC * kC);   // keep a head segment
   const int L0 = p.T - (int)g * L;
   if (L <= 0 || L0 <= 0) return sp;
