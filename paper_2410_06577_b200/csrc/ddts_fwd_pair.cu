@@ -455,13 +455,17 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       tma_prefetch_2d(&map_k, xc, yqp);
       tma_prefetch_2d(&map_v, it.col0, yp);
       tma_prefetch_2d(&map_v, it.col0 + 64, yp);
-      if (BLOCK && a.beta_hat) {
-        tma_prefetch_2d(&map_b, it.col0, yp);
-        tma_prefetch_2d(&map_b, it.col0 + 64, yp);
+    }
+    // The block's terms are read later than the rest of the tile: asked for with its own fill they are there in
+    // time, and the first tiles of a sequence find them in L2 as well.  (Not ahead of the very first loads.)
+    if (BLOCK && j + tpos > 0) {
+      if (a.beta_hat) {
+        tma_prefetch_2d(&map_b, it.col0, y);
+        tma_prefetch_2d(&map_b, it.col0 + 64, y);
       }
-      if (BLOCK && !STATE_ONLY && a.feed_d) {
-        tma_prefetch_2d(&map_fx, it.col0, yp);
-        tma_prefetch_2d(&map_fx, it.col0 + 64, yp);
+      if (!STATE_ONLY && a.feed_d) {
+        tma_prefetch_2d(&map_fx, it.col0, y);
+        tma_prefetch_2d(&map_fx, it.col0 + 64, y);
       }
     }
   };
