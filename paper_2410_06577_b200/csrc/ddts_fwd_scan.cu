@@ -924,17 +924,21 @@ bool scan_pays_with_shared_gates(long long n_seq, double tiles, double slabs, bo
 //   one set of gates   where the pair kernel would be the other choice (same precision), by the cost of both
 //                      (above); layer shape 82 -> 40 us.
 //   gates per head     the gates cost the same in both, here their operands travel through memory, and
-//                      here they are formed by all SMs however few the heads are; sequences of four tiles
-//                      or more on average:
-//       dv % 256 == 0  against the pair kernel, when a dense call has at most a quarter as many items of
-//                      256 columns as there are SMs (16 items x 2048 rows 77 -> 47 us, 32 items 79 ->
-//                      67, 37 x 1024 45 -> 39, but 48 x 1024 47 -> 47 and 64 x 2048 82 -> 101), a packed
-//                      one, whose longest sequence keeps the other pairs waiting, three eighths (56 items
-//                      of 64..1000 rows 45 -> 40 us, of 1..4096 135 -> 123; 72 items 45 -> 49 and 138 ->
-//                      143).  Packed sequences of one length would change sides at the dense call's line:
-//                      56 items of 300 rows 24.6 either way, of 1500 64 -> 80.
-//       odd multiples  against the single-CTA kernel, which forms the gates in every CTA and takes the
-//       of 128         same time for one item and for one on every SM.  Dense: up to three sets of gates
+//                      here they are formed by all SMs however few the heads are.
+//       dv % 256 == 0  against the pair kernel.  Dense, up to one item of 256 columns for every two SMs: the
+//                      scan starts and ends sooner, and with the block's terms it takes less a tile;
+//                      without them less only up to a quarter as many items as SMs.  Items x rows, us:
+//                      16 x 2048 72 -> 47, 37 x 2048 74 -> 73, 48 x 333 22.6 -> 20.5, 48 x 777 37 -> 39, 64 x
+//                      64 11.8 -> 11.4, 64 x 192 15.8 -> 16.3, 64 x 2048 77 -> 103; with both block terms 64
+//                      x 64 12.8 -> 12.4, 48 x 333 29.6 -> 24.6, 64 x 2048 127 -> 124, 74 x 777 63.6 ->
+//                      64.2; with one 64 x 240 21.3 -> 19.2, 64 x 1000 60 -> 62.
+//                      Packed, whose longest sequence keeps the other pairs waiting, three eighths as many
+//                      as SMs, of four tiles or more on average (56 items of 64..1000 rows 45 -> 40 us, of
+//                      1..4096 135 -> 123; 72 items 45 -> 49 and 138 -> 143).  Packed sequences of one
+//                      length would change sides sooner: 56 items of 300 rows 24.6 either way, of 1500
+//                      64 -> 80.
+//       odd multiples  against the single-CTA kernel, from four tiles on; it forms the gates in every CTA and
+//       of 128         takes the same time for one item and for one on every SM.  Dense: up to three sets of gates
 //                      for four CTAs of its rounds (T=2048, dv=128: 100 items 141 -> 131 us, 148 144 ->
 //                      181, 149 274 -> 201, 256 280 -> 307; dv=384, three slices a set, always: 64 sets x
 //                      1000 150 -> 73).  Packed: one slice a set, up to seven items for eight SMs (128
@@ -958,9 +962,14 @@ size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
       const double tiles = varlen ? (double)p.T / ((double)n_seq * kTile) + 0.5 : (double)((p.T + kTile - 1) / kTile);
       if (!whole || !scan_pays_with_shared_gates(n_seq, tiles, p.H * (p.dv / 256.0), varlen, sms)) return 0;
     } else {
-      if (p.T / (varlen ? n_seq : 1) < 4 * kTile) return 0;
-      if (whole) {
-        if (varlen ? 4 * items > 3 * sms : 2 * items > sms) return 0;
+      if (whole && !varlen) {
+        const double fill = (double)items / sms, tiles = (double)((p.T + kTile - 1) / kTile);
+        const double more = !block ? 2.8 * fill - 1.47 : (p.beta_hat && p.feed_d ? 1.95 * fill - 1.65 : 2.2 * fill - 1.6);
+        if (fill > 1.0 || tiles * more > (block ? 3.0 : 3.5)) return 0;   // us of a tile more; of a call less
+      } else if (p.T / (varlen ? n_seq : 1) < 4 * kTile) {
+        return 0;
+      } else if (whole) {
+        if (4 * items > 3 * sms) return 0;
       } else if (varlen) {
         if (block || (p.dv == 128 ? 8 * items > 7 * sms : items > sms)) return 0;
       } else if (block || 4 * sets > 3 * sms * ((items + sms - 1) / sms)) {

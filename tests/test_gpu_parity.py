@@ -1101,15 +1101,22 @@ def test_two_launch_prefill_is_chosen_where_it_is_the_faster_one():
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
 
-    def chosen(n_seq, H, T, dv, shared=0, packed=False):
+    def chosen(n_seq, H, T, dv, shared=0, packed=False, terms=0):
         p = rd.FwdParams()
         p.struct_size, p.dtype, p.scale, p.shared_gates = ctypes.sizeof(rd.FwdParams), rd.BF16, 1.0, shared
         p.B, p.H, p.T, p.dk, p.dv = 1 if packed else n_seq, H, n_seq * T if packed else T, 128, dv
         p.N, p.cu_seqlens = (n_seq, 0x7F0000000000) if packed else (0, None)
+        p.beta_hat = 0x7F0000000000 if terms > 0 else None
+        p.feed_d = p.feed_x = 0x7F0000000000 if terms > 1 else None
         return rd.fwd_workspace_bytes(p) > 256 + 4 * (n_seq + 63)
 
-    # a set of gates per head, whole pairs: a quarter of an item of 256 columns per SM, packed 3 / 8
-    assert chosen(sms // 4, 1, 256, 256) and not chosen(sms // 4 + 1, 1, 256, 256) and not chosen(4, 1, 255, 256)
+    # a set of gates per head, whole pairs: a quarter of an item of 256 columns per SM, up to half of one if
+    # there are few tiles (more with the block's terms), packed 3 / 8
+    assert chosen(sms // 4, 1, 32768 // (sms // 4), 256) and chosen(sms // 4, 1, 2048, 256) and chosen(4, 1, 7, 256)
+    assert chosen(sms // 2, 1, 128, 256) and not chosen(sms // 2, 1, 193, 256) and not chosen(sms // 2 + 1, 1, 64, 256)
+    assert chosen(sms // 2, 1, 512, 256, terms=2) and not chosen(sms // 2, 1, 777, 256, terms=2)
+    assert chosen(sms // 2, 1, 256, 256, terms=1) and not chosen(sms // 2, 1, 512, 256, terms=1)
+    assert not chosen(sms // 2 + 1, 1, 64, 256, terms=2)
     assert chosen(3 * sms // 8, 1, 256, 256, packed=True) and not chosen(3 * sms // 8 + 1, 1, 256, 256, packed=True)
     # odd multiples of 128: three sets of gates for four CTAs of the rounds
     assert chosen(3 * sms // 4, 1, 512, 128) and not chosen(sms, 1, 512, 128)
@@ -1158,3 +1165,14 @@ def test_decode_of_a_sequence_does_not_depend_on_the_batch(dtype, H, dk, dv, ter
     o_part = rd.ddts_step(*(a[:few] for a in args), part, **{n: t if n == "feed_d" else t[:few] for n, t in opt.items()})
     o = rd.ddts_step(*args, state, **opt)
     assert torch.equal(part, state[:few]) and torch.equal(o_part, o[:few])
+
+
+@pytest.mark.parametrize("block", ["none", "gate", "feed", "both"])
+@pytest.mark.parametrize("T", [1, 63, 64, 65, 130])
+def test_two_launch_prefill_gates_per_head_few_tiles(block, T):
+    p = wl.make_prefill(997, 3, 2, T, 128, 256, "bf16", s0_std=0.2)
+    if block != "none":
+        assert _check_block(p, block) == 2
+    else:
+        _check_prefill(p, rd.INGATE_POW_SIGMOID, 0.5)
+        assert rd.last_launch_count() == 2
