@@ -34,7 +34,7 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
   constexpr int kThreads = 32 * W, kTileCols = 4 * LC, kSub = 32 / LC, kStride = W * kSub;
   __shared__ float s_alpha[kMaxDk];
   __shared__ float s_w[kMaxDk];   // ahat * k
-  __shared__ float s_q[kMaxDk];   // scale * q
+  __shared__ __align__(16) float s_q[kMaxDk];   // scale * q (narrow: by subset of the rows, see the sums)
   constexpr bool kNarrow = LC < 32;
   __shared__ float4 s_red[4][LC];
   __shared__ float4 s_new[kNarrow ? kMaxDk : 1][LC];   // narrow: the new state of the tile
@@ -66,7 +66,7 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
       gate_logs_f32(to_f32(gx[i]), to_f32(ty[i]), ingate, la, lh);
       s_alpha[d] = expf(la);
       s_w[d] = expf(lh) * to_f32(k[i]);
-      s_q[d] = scale * to_f32(q[i]);
+      s_q[kNarrow ? (d & 3) * (kMaxDk / 4) + (d >> 2) : d] = scale * to_f32(q[i]);
     }
     float4 vv = make_float4(0.f, 0.f, 0.f, 0.f);
     if (col_ok) {
@@ -131,9 +131,17 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
       __syncthreads();
       if (warp < 4) {                          // a subset and column a thread
         float sum = 0.f;
-        const float* col_of = reinterpret_cast<const float*>(s_new) + lane;
+        const float* col_of = reinterpret_cast<const float*>(s_new) + warp * kTileCols + lane;
+        const float4* q4 = reinterpret_cast<const float4*>(s_q + warp * (kMaxDk / 4));
 #pragma unroll 8
-        for (int r = warp; r < dk; r += 4) sum = fmaf(s_q[r], col_of[r * kTileCols], sum);
+        for (int r = 0; r < dk / 16; ++r) {
+          const float4 qq = q4[r];
+          const float* c = col_of + r * 16 * kTileCols;
+          sum = fmaf(qq.x, c[0], sum);
+          sum = fmaf(qq.y, c[4 * kTileCols], sum);
+          sum = fmaf(qq.z, c[8 * kTileCols], sum);
+          sum = fmaf(qq.w, c[12 * kTileCols], sum);
+        }
         reinterpret_cast<float*>(s_red)[warp * kTileCols + lane] = sum;
       }
     } else {
