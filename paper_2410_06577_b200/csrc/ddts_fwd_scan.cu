@@ -73,7 +73,7 @@ struct ScanArgs {
 // Decays and their sums.  dk = 64: exact sums, so that 2^b is as exact as the rows' own decays are.  (An fp32
 // sum near -60 carries 2^-19 into every operand made of it: 1e-6 of the final state where gates decay fast,
 // 2e-7 in the fp32 kernel, which forms differences before the exponential, 1e-7 here.  It costs 0.9 % of a
-// call at the layer shape; sums in fp64, as exact, 2.7 %.)
+// call at the layer shape, 3.7 % with a set of gates per head; sums in fp64, as exact, 2.7 % at the layer shape.)
 template <bool EXACT>
 struct Decay {
   using One = float;
@@ -85,16 +85,17 @@ struct Decay<true> {
   using Two = ExactSum2;
 };
 // 2^b, and 2^(lh - b)
-__device__ __forceinline__ void exp2_of(float b, float lh, float& e, float& ek) {
-  e = ex2f(b);
-  ek = ex2f(lh - b);
-}
+__device__ __forceinline__ float exp2_of(float b) { return ex2f(b); }
+__device__ __forceinline__ float exp2_of(float lh, float b) { return ex2f(lh - b); }
 __device__ __forceinline__ float scaled(float e, float rest) { return fmaf(e, rest * 0.69314718f, e); }   // e 2^rest, rest tiny
-__device__ __forceinline__ void exp2_of(ExactSum b, float lh, float& e, float& ek) {
-  const float t = b.h + b.l, r = (b.h - t) + b.l;             // b = t + r
-  e = scaled(ex2f(t), r);
+__device__ __forceinline__ float exp2_of(ExactSum b) {
+  const float t = b.h + b.l;                                  // b = t + ((b.h - t) + b.l)
+  return scaled(ex2f(t), (b.h - t) + b.l);
+}
+__device__ __forceinline__ float exp2_of(float lh, ExactSum b) {
+  const float t = b.h + b.l, r = (b.h - t) + b.l;
   const float u = lh - t, z = u - lh, d = (lh - (u - z)) - (t + z);   // lh - t = u + d
-  ek = scaled(ex2f(u), d - r);
+  return scaled(ex2f(u), d - r);
 }
 
 template <bool EXACT>
@@ -194,9 +195,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
       const int r = rg * kOpRows + i;
       const uint32_t at = w + r * 128 + ((c16 ^ (uint32_t)(r & 7)) << 4);
       const float2 qv = unpack_bf16(wq[i]), kv = unpack_bf16(wk[i]);
-      float ex, ey, kex, key;
-      exp2_of(b[i].x, lh2[i].x, ex, kex);
-      exp2_of(b[i].y, lh2[i].y, ey, key);
+      const float ex = exp2_of(b[i].x), ey = exp2_of(b[i].y);
       float qx = qv.x * a.scale * ex, qy = qv.y * a.scale * ey;
 #pragma unroll
       for (int p = 0; p < B::kQp; ++p) {
@@ -206,7 +205,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
         qx -= f.x;
         qy -= f.y;
       }
-      float kx = kv.x * kex, ky = kv.y * key;
+      float kx = kv.x * exp2_of(lh2[i].x, b[i].x), ky = kv.y * exp2_of(lh2[i].y, b[i].y);
 #pragma unroll
       for (int p = 0; p < B::kKp; ++p) {
         const uint32_t h = pack_bf16(kx, ky);
@@ -630,13 +629,12 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         for (int ch = lane; ch < DK; ch += 32) {
           const long long e = d->rowq * DK + ch;
           typename Decay<B::kExact>::One acc = {}, la;
-          float lh, D;
+          float lh;
           for (int r = lo; r < hi; ++r) {
             gate_pair<B::kExact>(__bfloat162float(a.gx[e + r * DK]), __bfloat162float(a.ty[e + r * DK]), a.ingate, la, lh);
             acc = sum1(acc, la);
           }
-          exp2_of(acc, 0.f, D, lh);
-          dc[ch] = D;
+          dc[ch] = exp2_of(acc);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(FB_CUT0 + (n_cut & 7)));

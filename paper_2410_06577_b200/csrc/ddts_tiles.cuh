@@ -52,6 +52,10 @@ __device__ __forceinline__ TileRef find_tile(const TileGeometry& a, int head, in
     seq_range(a.cu, n, a.T, lo, hi);
     return lo / kTile + n <= local;
   });
+  __shared__ int s_found;      // (through shared memory the kernels spill fewer registers)
+  if (threadIdx.x == 0) s_found = r.n;
+  __syncthreads();
+  r.n = *(volatile int*)&s_found;
   r.nr = 0;
   if (r.n < 0) return r;
   int lo, hi;
@@ -140,15 +144,24 @@ __device__ __forceinline__ unsigned long long tile_scan(V (&v)[ROWS], int cp, in
   for (int i = 1; i < ROWS; ++i) v[i] = sum2(v[i], v[i - 1]);
   *reinterpret_cast<V*>(part + rg * CH + 2 * cp) = v[ROWS - 1];
   __syncthreads();
-  V pre = {}, all = {};
+  V pre = {}, all = {};                        // of the row groups before this one, of the tile
+  bool mine = true;                            // this thread knows `all`
+  if constexpr (sizeof(V) == 8) {
 #pragma unroll
-  for (int w = 0; w < kGroups; ++w) {
-    if (w == rg) pre = all;
-    all = sum2(all, *reinterpret_cast<const V*>(part + w * CH + 2 * cp));
+    for (int w = 0; w < kGroups; ++w) {
+      if (w == rg) pre = all;
+      all = sum2(all, *reinterpret_cast<const V*>(part + w * CH + 2 * cp));
+    }
+  } else {                                     // (exact sums are twice as long: no more are read than needed)
+#pragma unroll
+    for (int w = 0; w < kGroups - 1; ++w)
+      if (w < rg) pre = sum2(pre, *reinterpret_cast<const V*>(part + w * CH + 2 * cp));
+    all = sum2(pre, v[ROWS - 1]);
+    mine = rg == kGroups - 1;
   }
   bool whole;
   if (MAKE_MASK) {
-    whole = __syncthreads_or(beyond_range(all.x) || beyond_range(all.y)) == 0;
+    whole = __syncthreads_or(mine && (beyond_range(all.x) || beyond_range(all.y))) == 0;
     mask = 1ull;
   } else {
     whole = mask == 1ull;
