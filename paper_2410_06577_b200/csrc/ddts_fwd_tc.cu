@@ -650,40 +650,6 @@ ddts_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode_fn() {
-  // looked up once (initialisation of a function-local static is thread-safe); a failed lookup
-  // leaves nullptr and the callers report an error
-  static const EncodeTiledFn fn = []() -> EncodeTiledFn {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) != cudaSuccess ||
-        qres != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-// [rows, cols] bf16 row-major, box = 64 rows x 64 columns (128 bytes), 128-byte swizzle.
-bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols) {
-  EncodeTiledFn fn = get_encode_fn();
-  if (!fn) return false;
-  const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {cols * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)kC};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 }  // namespace
 
 cudaError_t launch_fwd_tc(const rodimus_ddts_fwd_params& p, int* n_launches) {
@@ -709,9 +675,9 @@ cudaError_t launch_fwd_tc(const rodimus_ddts_fwd_params& p, int* n_launches) {
 
   CUtensorMap mq, mk, mx, my, mv;
   if (rows > 0) {
-    if (!make_map(&mq, p.q, rows, kDK) || !make_map(&mk, p.k, rows, kDK) ||
-        !make_map(&mx, p.gate_x, rows, kDK) || !make_map(&my, p.temp_y, rows, kDK) ||
-        !make_map(&mv, p.v, rows, (uint64_t)p.dv))
+    if (!encode_bf16_map(&mq, p.q, rows, kDK, kC) || !encode_bf16_map(&mk, p.k, rows, kDK, kC) ||
+        !encode_bf16_map(&mx, p.gate_x, rows, kDK, kC) || !encode_bf16_map(&my, p.temp_y, rows, kDK, kC) ||
+        !encode_bf16_map(&mv, p.v, rows, (uint64_t)p.dv, kC))
       return cudaErrorUnknown;
   } else {
     memset(&mq, 0, sizeof(mq)); mk = mq; mx = mq; my = mq; mv = mq;  // never dereferenced: no chunks

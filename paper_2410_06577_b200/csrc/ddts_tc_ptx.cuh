@@ -17,8 +17,6 @@ bool encode_bf16_slab_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64
 
 namespace {
 
-constexpr long long kWaitCycles = 4000000000LL;   // default limit of a main-loop wait: about two
-                                                  // seconds, then give up, never hang
 constexpr long long kDrainCycles = 4000000000LL;  // limit of the teardown waits (copies in flight)
 
 // What every bounded wait of a CTA shares, in shared memory: the flag a role raises when it gives
@@ -180,14 +178,6 @@ __device__ __forceinline__ void bulk_commit() {
 template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-// Waits until at most N of this thread's bulk groups are not complete (writes done).
-template <int N>
-__device__ __forceinline__ void bulk_wait() {
-  asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void sts16(uint32_t addr, uint16_t v) {
-  asm volatile("st.shared.b16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
 }
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                           uint32_t idesc, uint32_t accumulate) {
@@ -399,30 +389,6 @@ __device__ __forceinline__ void umma_bf16_atmem(uint32_t d_tmem, uint32_t a_tmem
       ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(ACC ? 1u : 0u), "r"(kDescHi)
       : "memory");
 }
-// One tcgen05.mma, bf16 x bf16 -> fp32.  Descriptors are passed whole (64 bits): stepping along K
-// is then one 64-bit add of a constant to a base the issuer keeps in registers, and the
-// accumulate flag is an immediate that the assembler folds into the predicate.
-template <bool ACC>
-__device__ __forceinline__ void umma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "n"(ACC ? 1 : 0)
-      : "memory");
-}
-// The same with the A operand in tensor memory: lane = row of A (M = 128), bf16 packed two per
-// 32-bit column, even K index in the low half (K = 16 elements = 8 columns per instruction).
-template <bool ACC>
-__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc) {
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "n"(ACC ? 1 : 0)
-      : "memory");
-}
-__device__ __forceinline__ uint64_t desc64(uint32_t lo) { return ((uint64_t)kDescHi << 32) | lo; }
 // Instruction descriptor: bf16 x bf16 -> fp32.
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N, int a_mn, int b_mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |

@@ -435,38 +435,6 @@ swska_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn sw_encode_fn() {
-  static const EncodeTiledFn fn = []() -> EncodeTiledFn {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) != cudaSuccess ||
-        qres != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-// [rows, 128] bf16 row-major; box = box_rows rows x 64 columns (128 bytes), 128-byte swizzle; rows
-// past the end of the tensor read as zeros
-bool sw_make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint32_t box_rows) {
-  EncodeTiledFn fn = sw_encode_fn();
-  if (!fn) return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)kD, rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)kD * 2};
-  const cuuint32_t box[2] = {64u, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 struct SwMapCache {     // the four maps of the last call on this host thread
   const void *q = nullptr, *k = nullptr, *v = nullptr, *o = nullptr;
   uint64_t rows_q = 0, rows_k = 0;
@@ -482,8 +450,8 @@ cudaError_t launch_swska_tc(const rodimus_swska_fwd_params& p, int* n_launches) 
   const uint64_t rows_q = (uint64_t)p.B * p.H * p.T, rows_k = (uint64_t)p.B * p.T;
   SwMapCache& c = t_sw_maps;
   if (c.q != p.q || c.k != p.k || c.v != p.v || c.o != p.o || c.rows_q != rows_q || c.rows_k != rows_k) {
-    if (!sw_make_map(&c.mq, p.q, rows_q, kBM) || !sw_make_map(&c.mk, p.k, rows_k, kBN) ||
-        !sw_make_map(&c.mv, p.v, rows_q, kBN) || !sw_make_map(&c.mo, p.o, rows_q, kBM)) {
+    if (!encode_bf16_map(&c.mq, p.q, rows_q, kD, kBM) || !encode_bf16_map(&c.mk, p.k, rows_k, kD, kBN) ||
+        !encode_bf16_map(&c.mv, p.v, rows_q, kD, kBN) || !encode_bf16_map(&c.mo, p.o, rows_q, kD, kBM)) {
       c.q = nullptr;
       return cudaErrorInvalidValue;
     }
