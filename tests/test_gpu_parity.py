@@ -1176,3 +1176,14 @@ def test_two_launch_prefill_gates_per_head_few_tiles(block, T):
     else:
         _check_prefill(p, rd.INGATE_POW_SIGMOID, 0.5)
         assert rd.last_launch_count() == 2
+
+
+@pytest.mark.parametrize("dk", [64, 128])
+def test_two_launch_prefill_dense_without_tokens(dk):
+    import torch
+    B, H, dv = 3, 2, 256
+    z = lambda h, d: torch.empty((B, h, 0, d), dtype=torch.bfloat16, device="cuda")
+    s0 = torch.randn((B, H, dk, dv), device="cuda")
+    ws = torch.full((4096,), 0xEE, dtype=torch.uint8, device="cuda")
+    o, sT = rd.ddts_fwd(*(z(H, dk) for _ in range(4)), z(H, dv), s0, workspace=ws)
+    assert o.shape == (B, H, 0, dv) and torch.equal(sT, s0) and rd.device_status(ws) == rd.OK
