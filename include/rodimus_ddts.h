@@ -33,7 +33,9 @@
  *     anything is launched.  Nothing aborts, throws or traps.
  *   - Tensors are contiguous, row-major, last index fastest; pointers are 16-byte aligned.
  *   - Inputs must be finite, with |x|, |y| <= 80.  Per-step decay factors below exp(-60) are
- *     applied as exp(-60) by the bf16 prefill kernel (difference below 2^-86 of the state).
+ *     applied as exp(-60) by the tensor-core kernels for bf16 tokens, prefill and backward
+ *     (difference below 2^-86 of the state).  Those kernels scale operands by up to exp(60) within
+ *     a chunk: products |ahat k v| from about 2^35 on may overflow in them.
  */
 #ifndef RODIMUS_DDTS_H_
 #define RODIMUS_DDTS_H_
@@ -78,8 +80,11 @@ typedef enum {
  * s0 and sT may be the same buffer.  o must not overlap any input.
  *
  * Kernels: dtype BF16 with dk == 128 and dv a multiple of 128 runs on the tcgen05 tensor
- * cores; every other supported shape (dk, dv multiples of 16, dk <= 256, dv <= 1024) and
- * dtype F32 run the fp32 CUDA-core kernel, which keeps all arithmetic in fp32.
+ * cores, and so does dk == 64 without the optional terms, given the workspace asked for (operands
+ * in parts: the final state keeps fp32 accuracy, o the 16 bits that precede its rounding); every
+ * other supported shape (dk, dv multiples of 16, dk <= 256, dv <= 1024) and dtype F32 run the fp32
+ * CUDA-core kernel, which keeps all arithmetic in fp32.  dv an odd multiple of 128 with optional
+ * terms or shared gates is such an other shape.
  */
 typedef struct {
   int32_t struct_size;       /* sizeof(rodimus_ddts_fwd_params), checked                        */
@@ -127,7 +132,8 @@ typedef struct {
  * Sec. 3.1.3, last paragraph: O(1) time and memory per token at inference).
  * q,k,gate_x,temp_y are [Nseq,H,dk]; v,o are [Nseq,H,dv]; state is fp32 [Nseq,H,dk,dv],
  * read and written in place; o reads the updated state.  dk and dv are multiples of 16 with
- * dk <= 256 and dv <= 1024.  All arithmetic is fp32.
+ * dk <= 256 and dv <= 1024.  All arithmetic is fp32; a sequence's output and state do not depend
+ * on how many others are in the call, bit for bit.
  */
 typedef struct {
   int32_t struct_size; /* sizeof(rodimus_ddts_step_params) */
@@ -157,9 +163,9 @@ typedef struct {
  * the state, so segments are joined exactly up to rounding) and part of the work is enqueued
  * on the library's own second stream, forked from and joined back into `stream` with events, so
  * the call still behaves as one piece of work on `stream`.  For bf16 requests with dk = 64, with
- * one set of gates for all heads or with few heads it includes a block of gated operands per 64
- * tokens and set of gates, and for small fp32 requests the states of 16-token chunks, so that all
- * SMs can form them ahead of the scan.  A caller that passes less (never less than 256 bytes plus
+ * one set of gates for all heads or with few heads it includes a block of gated operands (41 KiB,
+ * 57 for dk = 64) per 64 tokens and set of gates, which may be as much as the inputs take, and for
+ * small fp32 requests the states of 16-token chunks, so that all SMs can form them ahead of the scan.  A caller that passes less (never less than 256 bytes plus
  * 4 bytes per packed sequence, rounded up to 256) gets the same result, to the same accuracy, from
  * a kernel that needs no more. */
 size_t rodimus_ddts_fwd_workspace_bytes(const rodimus_ddts_fwd_params *p);
@@ -188,7 +194,10 @@ int rodimus_ddts_step(const rodimus_ddts_step_params *p);
  * the feed-through and the shared-gate layout of the forward call have no backward here.
  * dtype BF16 contracts on the tensor cores with fp32 accumulation: v, d_o and gated operands as
  * pairs of bf16 (16 bits of mantissa), the carried states as tf32; dtype F32 splits each operand
- * in two tf32 parts and keeps fp32 accuracy.  The outputs are written more than once: with BF16,
+ * in two tf32 parts and keeps fp32 accuracy.  Where a step decays by g tau of tens, its d_gate_x is
+ * a small difference of larger sums and carries, with BF16, up to 2^-11 g of the size of its first
+ * term (4 % at g = 80); among milder steps that is below the rounding of the largest gradients.
+ * The outputs are written more than once: with BF16,
  * d_q, d_k, d_gate_x and d_temp_y hold the gated operands until the last kernel stores the
  * gradients there.  The workspace holds the status word, 8 * dk bytes per token and head of
  * scratch, and 6 * dk/2 * dv * 4 bytes per (sequence, head) (a few per cent more for BF16 where

@@ -27,7 +27,7 @@
 //                          sums chained from tile to tile (fp64), dq, dk, dx, dy.
 // What this replaces for bf16 - one launch of 16-row chunks on mma.sync with the gates computed in
 // each of six CTAs per (sequence, head), bound by instruction issue - took 1.79 ms on the layer
-// shape (B=4 H=16 T=2048); this takes 0.34 ms there: 52 us (4.1 TB/s; issue slots 70 % busy) + 170 us
+// shape (B=4 H=16 T=2048); this takes 0.34 ms there (0.35 run for seconds): 52 us (4.1 TB/s; issue slots 70 % busy) + 170 us
 // (shared memory, see the sweeps) + 120 us (3.3 TB/s; issue slots 50 %, special-function units 41 %, the
 // rest latency: 18 warps on an SM on average, a third of their stalls waiting for loads).
 #include <cuda.h>

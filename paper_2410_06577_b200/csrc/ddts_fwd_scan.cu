@@ -72,7 +72,7 @@ struct ScanArgs {
 
 // Decays and their sums.  dk = 64: exact sums, so that 2^b is as exact as the rows' own decays are.  (An fp32
 // sum near -60 carries 2^-19 into every operand made of it: 1e-6 of the final state where gates decay fast,
-// 2e-7 in the fp32 kernel, which forms differences before the exponential, 1e-7 here.  It costs 0.9 % of a
+// 2e-7 in the fp32 kernel, which forms differences before the exponential, 1e-7 here.  It costs 0.6 % of a
 // call at the layer shape, 3.7 % with a set of gates per head; sums in fp64, as exact, 2.7 % at the layer shape.)
 template <bool EXACT>
 struct Decay {

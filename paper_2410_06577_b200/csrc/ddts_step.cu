@@ -7,9 +7,10 @@
 // BATCH accesses per warp with all loads of a batch in flight at once; the first batch is issued before
 // the gate math so that its latency hides the token loads and the transcendental work.
 //   W = 4, LC = 32, BATCH = 16   128 columns, every access one 512-byte row segment: the shape for
-//                                streaming many states (256 x 16 states 168 us, 0.99 of the copy rate)
+//                                streaming many states (256 x 16 states 168 us, 0.98 of the copy rate)
 //   W = 8, LC = 8,  BATCH = 8    32 columns, up to 256 rows in flight at once: calls too small to fill
 //                                the device are latency, and this spreads them over 4 times the CTAs
+//                                (device time of a step, 16 states: 4.4 us on wide tiles, 3.05 on narrow)
 #include <type_traits>
 
 #include "ddts_common.cuh"
