@@ -10,7 +10,12 @@
 //                                streaming many states (256 x 16 states 168 us, 0.98 of the copy rate)
 //   W = 8, LC = 8,  BATCH = 8    32 columns, up to 256 rows in flight at once: calls too small to fill
 //                                the device are latency, and this spreads them over 4 times the CTAs
-//                                (device time of a step, 16 states: 4.4 us on wide tiles, 3.05 on narrow)
+//                                (device time of a step, 16 states: 4.4 us on wide tiles, 2.95 on narrow)
+// Both sum q S over the rows in one order, so that a sequence's output does not depend on how many others are
+// in the call: rows g, g + 4, g + 8, g + 12 of a block of 16 in turn; the blocks' results in turn; the four g
+// in turn.  A thread of the wide tile meets its rows in that order, one of the narrow tile has a g of a block.
+// (The wide tile's plain order in the narrow one took a trip of the state through shared memory, 0.2 us; the
+// narrow one's former order in the wide one eight sums a thread, 5 to 20 % of calls of 50 to 1000 states.)
 #include <type_traits>
 
 #include "ddts_common.cuh"
@@ -32,17 +37,20 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
                  float* __restrict__ state, int n_seq_heads, int dk, int dv, float scale,
                  int ingate, const T* __restrict__ beta_hat, const float* __restrict__ feed_d,
                  const T* __restrict__ feed_x, int H, int shared, const T* __restrict__ vdecay) {
-  constexpr int kThreads = 32 * W, kTileCols = 4 * LC, kSub = 32 / LC, kStride = W * kSub;
+  constexpr int kThreads = 32 * W, kTileCols = 4 * LC, kSub = 32 / LC;
+  static_assert(W * kSub == 4 || W * kSub == 32, "a wide or a narrow tile");
+  constexpr bool kWide = W * kSub == 4;
   __shared__ float s_alpha[kMaxDk];
   __shared__ float s_w[kMaxDk];   // ahat * k
-  __shared__ __align__(16) float s_q[kMaxDk];   // scale * q (narrow: by subset of the rows, see the sums)
-  constexpr bool kNarrow = LC < 32;
-  __shared__ float4 s_red[4][LC];
-  __shared__ float4 s_new[kNarrow ? kMaxDk : 1][LC];   // narrow: the new state of the tile
+  __shared__ float s_q[kMaxDk];   // scale * q
+  __shared__ float4 s_red[kWide ? 1 : kMaxDk / 16][4][LC];   // [block of rows][g]
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
-  const int row0 = warp * kSub + lane / LC, cl = lane % LC;   // this thread's rows: row0 + kStride j
+  const int cl = lane % LC;
+  // row j of this thread's batch that begins at row `base`
+  const int row0 = kWide ? warp : warp * 16 + lane / LC;
+  auto row_of = [&](int base, int j) { return base + row0 + (kWide ? 4 * j : (j >> 2) * 128 + (j & 3) * 4); };
   const int tiles = (dv + kTileCols - 1) / kTileCols;
   const long long n_items = (long long)n_seq_heads * tiles;
 
@@ -56,7 +64,7 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     float4 buf[BATCH];
 #pragma unroll
     for (int j = 0; j < BATCH; ++j) {
-      const int r = row0 + kStride * j;
+      const int r = row_of(0, j);
       if (col_ok && r < dk) buf[j] = ld_stream(reinterpret_cast<const float4*>(S + (long long)r * dv));
     }
 
@@ -67,7 +75,7 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
       gate_logs_f32(to_f32(gx[i]), to_f32(ty[i]), ingate, la, lh);
       s_alpha[d] = expf(la);
       s_w[d] = expf(lh) * to_f32(k[i]);
-      s_q[kNarrow ? (d & 3) * (kMaxDk / 4) + (d >> 2) : d] = scale * to_f32(q[i]);
+      s_q[d] = scale * to_f32(q[i]);
     }
     float4 vv = make_float4(0.f, 0.f, 0.f, 0.f);
     if (col_ok) {
@@ -85,13 +93,13 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     }
     __syncthreads();
 
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int base = 0; base < dk; base += kStride * BATCH) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), sum = acc;
+    for (int base = 0; base < dk; base += W * kSub * BATCH) {
 #pragma unroll
       for (int j = 0; j < BATCH; ++j) {
-        const int r = base + row0 + kStride * j;
+        const int r = row_of(base, j);
         if (col_ok && r < dk) {
-          const float a = s_alpha[r], w = s_w[r], qq = kNarrow ? 0.f : s_q[r];
+          const float a = s_alpha[r], w = s_w[r], qq = s_q[r];
           float4 s = buf[j];
           if (VDECAY) {
             s.x = fmaf(a * bd.x, s.x, w * vv.x);
@@ -104,69 +112,73 @@ ddts_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             s.z = fmaf(a, s.z, w * vv.z);
             s.w = fmaf(a, s.w, w * vv.w);
           }
-          if (kNarrow) {
-            s_new[r][cl] = s;
-          } else {
-            acc.x = fmaf(qq, s.x, acc.x);
-            acc.y = fmaf(qq, s.y, acc.y);
-            acc.z = fmaf(qq, s.z, acc.z);
-            acc.w = fmaf(qq, s.w, acc.w);
+          acc.x = fmaf(qq, s.x, acc.x);
+          acc.y = fmaf(qq, s.y, acc.y);
+          acc.z = fmaf(qq, s.z, acc.z);
+          acc.w = fmaf(qq, s.w, acc.w);
+          if ((j & 3) == 3) {                   // a block's result
+            if (kWide) {
+              sum.x += acc.x; sum.y += acc.y; sum.z += acc.z; sum.w += acc.w;
+            } else {
+              s_red[r >> 4][lane / LC][cl] = acc;
+            }
+            acc = make_float4(0.f, 0.f, 0.f, 0.f);
           }
           st_stream(reinterpret_cast<float4*>(S + (long long)r * dv), s);
         }
       }
-      const int next = base + kStride * BATCH;
+      const int next = base + W * kSub * BATCH;
       if (next < dk) {
 #pragma unroll
         for (int j = 0; j < BATCH; ++j) {
-          const int r = next + row0 + kStride * j;
+          const int r = row_of(next, j);
           if (col_ok && r < dk)
             buf[j] = ld_stream(reinterpret_cast<const float4*>(S + (long long)r * dv));
         }
       }
     }
 
-    // o = sum over the rows of q S: rows g, g + 4, g + 8 ... in turn, then the four subsets.  One order for both
-    // tile widths, so that a sequence's output does not depend on how many others are in the call.
-    if (kNarrow) {
-      __syncthreads();
-      if (warp < 4) {                          // a subset and column a thread
-        float sum = 0.f;
-        const float* col_of = reinterpret_cast<const float*>(s_new) + warp * kTileCols + lane;
-        const float4* q4 = reinterpret_cast<const float4*>(s_q + warp * (kMaxDk / 4));
-#pragma unroll 8
-        for (int r = 0; r < dk / 16; ++r) {
-          const float4 qq = q4[r];
-          const float* c = col_of + r * 16 * kTileCols;
-          sum = fmaf(qq.x, c[0], sum);
-          sum = fmaf(qq.y, c[4 * kTileCols], sum);
-          sum = fmaf(qq.z, c[8 * kTileCols], sum);
-          sum = fmaf(qq.w, c[12 * kTileCols], sum);
-        }
-        reinterpret_cast<float*>(s_red)[warp * kTileCols + lane] = sum;
-      }
-    } else {
-      s_red[warp][lane] = acc;
-    }
+    // o = the blocks' results, then the four g
+    if (kWide) s_red[0][warp][lane] = sum;
     __syncthreads();
-    if (tid < LC && col_ok) {
-      float4 t = s_red[0][lane];
+    if (warp == 0) {
+      float4 t;
+      if (kWide) {
+        t = s_red[0][0][lane];
 #pragma unroll
-      for (int w = 1; w < 4; ++w) {
-        const float4 u = s_red[w][lane];
-        t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+        for (int g = 1; g < 4; ++g) {
+          const float4 u = s_red[0][g][lane];
+          t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+        }
+      } else {                                  // a g and four columns a lane
+        t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int b = 0; b < dk / 16; ++b) {
+          const float4 u = s_red[b][lane / LC][cl];
+          t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+        }
+        const float4 t0 = t;
+#pragma unroll
+        for (int g = 1; g < 4; ++g) {
+          t.x += __shfl_down_sync(0xffffffffu, t0.x, g * LC);
+          t.y += __shfl_down_sync(0xffffffffu, t0.y, g * LC);
+          t.z += __shfl_down_sync(0xffffffffu, t0.z, g * LC);
+          t.w += __shfl_down_sync(0xffffffffu, t0.w, g * LC);
+        }
       }
-      if (feed_d) {     // feed-through: o = scale q S + d . x'
-        const float* dp = feed_d + (nh % H) * dv + col;
-        const T* fp = feed_x + nh * dv + col;
-        t.x = fmaf(dp[0], to_f32(fp[0]), t.x); t.y = fmaf(dp[1], to_f32(fp[1]), t.y);
-        t.z = fmaf(dp[2], to_f32(fp[2]), t.z); t.w = fmaf(dp[3], to_f32(fp[3]), t.w);
+      if (lane < LC && col_ok) {
+        if (feed_d) {     // feed-through: o = scale q S + d . x'
+          const float* dp = feed_d + (nh % H) * dv + col;
+          const T* fp = feed_x + nh * dv + col;
+          t.x = fmaf(dp[0], to_f32(fp[0]), t.x); t.y = fmaf(dp[1], to_f32(fp[1]), t.y);
+          t.z = fmaf(dp[2], to_f32(fp[2]), t.z); t.w = fmaf(dp[3], to_f32(fp[3]), t.w);
+        }
+        T* op = o + nh * dv + col;
+        op[0] = from_f32<T>(t.x);
+        op[1] = from_f32<T>(t.y);
+        op[2] = from_f32<T>(t.z);
+        op[3] = from_f32<T>(t.w);
       }
-      T* op = o + nh * dv + col;
-      op[0] = from_f32<T>(t.x);
-      op[1] = from_f32<T>(t.y);
-      op[2] = from_f32<T>(t.z);
-      op[3] = from_f32<T>(t.w);
     }
     __syncthreads();  // s_alpha / s_red are rewritten by the next item
   }
