@@ -14,6 +14,9 @@ bool encode_bf16_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t co
 // The same matrix seen as [cols / 64][rows][64]: one box of [slabs][64][64] is `slabs` consecutive
 // 64-column tiles of 64 rows, 8 KiB each, brought by ONE copy.
 bool encode_bf16_slab_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t slabs);
+// A [heads][rows][128] array, dimensions (64, rows, 2, heads): one box is box_rows rows of one head as `slabs`
+// 64-column tiles; rows past the end of a head read as zeros and are not written.
+bool encode_bf16_heads_map(CUtensorMap* m, const void* ptr, uint64_t heads, uint64_t rows, uint32_t box_rows, uint32_t slabs);
 
 namespace {
 
@@ -141,6 +144,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+      : "memory");
+}
 // Untiled bulk copy of contiguous bytes from global memory (16-byte aligned, size a multiple of 16).
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -170,6 +180,10 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, int x, int y, int z, uint32_t ssrc) {
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
                ::"l"(map), "r"(x), "r"(y), "r"(z), "r"(ssrc) : "memory");
+}
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, int x, int y, int z, int w, uint32_t ssrc) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];"
+               ::"l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(ssrc) : "memory");
 }
 __device__ __forceinline__ void bulk_commit() {
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
