@@ -76,6 +76,7 @@ bool swska_supported(const rodimus_swska_fwd_params& p);
 cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches);
 // Workspace with which the two-launch prefill (operands, scan) takes this request; 0: it does not.
 size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p);
+bool fwd_scan_split(const rodimus_ddts_fwd_params& p);   // it would split this dense call along time
 bool fwd_tc_supported(const rodimus_ddts_fwd_params& p);
 bool fwd_pair_supported(const rodimus_ddts_fwd_params& p);
 // Workspace a dense call needs if its sequences are to be split along time (0: no split).

@@ -29,6 +29,7 @@
 // rows of Kt set to zero.
 #include <cuda.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -41,15 +42,14 @@ namespace {
 
 constexpr int kSlab = kTile * 128;          // [64 rows][128 bytes], 128-byte swizzled
 
-// The block of a tile: slabs of Kt and P, then of Qt, then D and the header.
+// The block of a tile: slabs of Kt and P, then of Qt, then D.
 template <int DK>
 struct Block {
   static constexpr bool kExact = DK == 64;
   static constexpr int kSlabs = DK / 64;                    // slabs of one part of Kt or Qt
   static constexpr int kKp = kExact ? 3 : 1, kQp = kExact ? 2 : 1;   // parts of Kt; of Qt and P
   static constexpr int kK = 0, kP = kKp * kSlabs * kSlab, kQ = kP + kQp * kSlab, kD = kQ + kQp * kSlabs * kSlab;
-  static constexpr int kHead = kD + 512;                    // chunk mask of the tile
-  static constexpr int kBytes = kD + 1024;
+  static constexpr int kBytes = kD + 1024;                  // (blocks begin at multiples of 1 KiB)
 };
 
 struct ScanArgs {
@@ -58,6 +58,7 @@ struct ScanArgs {
   float* sT;
   const float* feed_d;
   unsigned char* blocks;
+  unsigned long long* masks;   // of every tile: bit r = its row r starts a chunk
   const int32_t *cu, *order;
   WorkspaceHeader* hdr;
   int H, T, dv, n_seq;
@@ -68,6 +69,10 @@ struct ScanArgs {
   float scale;
   int ingate;
   long long limit;
+  // Calls split along time (see Segments): how the tiles are cut, which of the two launches this is, the final
+  // states of segments 0..G-1 (of 1..G-1 from a zero state) and the decays of segments 1..G-1.
+  int seg_count, seg_tiles0, seg_tiles, phase;
+  float *seg_state, *seg_decay;
 };
 
 // Decays and their sums.  dk = 64: exact sums, so that 2^b is as exact as the rows' own decays are.  (An fp32
@@ -216,7 +221,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) ddts_operands_kernel(const Scan
       }
       if (r + 1 == tr.nr) *reinterpret_cast<float2*>(gbase + B::kD + 8 * cp) = make_float2(ex, ey);
     }
-    if (tid == 0) *reinterpret_cast<unsigned long long*>(gbase + B::kHead) = mask;
+    if (tid == 0) a.masks[(long long)head * a.slots_per_head + local] = mask;
   }
   __syncthreads();
   // P = mask(Qt Kt^T): 16 x 16 blocks, those right of the diagonal are zero
@@ -350,14 +355,15 @@ struct ScanCtl {
   int n_a, n_q, n_x;   // loads issued (for the clean exit)
   int pad2;
   PassDesc desc[8];    // pass & 7: the outputs may be a few passes behind the loads
+  __align__(16) unsigned long long mask[16];   // of eight tiles, each beside a neighbour's
 };
-static_assert(sizeof(ScanCtl) <= 512, "control block");
+static_assert(sizeof(ScanCtl) <= 512 && offsetof(ScanCtl, mask) % 16 == 0, "control block");
 
 struct ScanMaps {
   CUtensorMap v, beta, fx, o, o8, o1;
 };
 
-template <int DK, bool BLOCK>
+template <int DK, bool BLOCK, bool SPLIT>
 __global__ void __launch_bounds__(Scan<DK, BLOCK>::kThreads, 1)
 ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   using B = Block<DK>;
@@ -372,8 +378,16 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q4 = warp & 3;
 
   // ---- the item
-  const int slice = (int)(blockIdx.x % (unsigned)a.cols);
-  const int sh = (int)(blockIdx.x / (unsigned)a.cols), h = sh % a.H;
+  unsigned item = blockIdx.x;
+  int seg = 0;
+  if constexpr (SPLIT) {
+    const unsigned items = gridDim.x / (unsigned)a.seg_count;
+    seg = (int)(item / items) + a.phase - 1;
+    item %= items;
+  }
+  const bool only = SPLIT && a.phase == 1 && seg > 0;      // the final state and the decay, no outputs
+  const int slice = (int)(item % (unsigned)a.cols);
+  const int sh = (int)(item / (unsigned)a.cols), h = sh % a.H;
   int n = sh / a.H;
   const int hq = a.gate_heads == 1 ? 0 : h;
   long long row0, rowq0;
@@ -396,10 +410,29 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     row0 = ((long long)n * a.H + h) * a.T;
     rowq0 = ((long long)n * a.gate_heads + hq) * a.T;
     slot0 = ((long long)n * a.gate_heads + hq) * a.slots_per_head;
+    if constexpr (SPLIT) {
+      const int t0 = seg == 0 ? 0 : a.seg_tiles0 + (seg - 1) * a.seg_tiles;
+      len = min(a.T, (a.seg_tiles0 + seg * a.seg_tiles) * kTile) - t0 * kTile;
+      row0 += (long long)t0 * kTile;
+      rowq0 += (long long)t0 * kTile;
+      slot0 += t0;
+    }
   }
   const int col0 = slice * 128;
   const int ntiles = (len + kTile - 1) / kTile;
   const long long state_off = ((long long)n * a.H + h) * DK * (long long)a.dv + col0;
+  const long long states = (long long)a.n_seq * a.H * DK * a.dv, decays = (long long)a.n_seq * a.H * DK;
+  const float* s0 = a.s0;
+  float* sT = a.sT;
+  if constexpr (SPLIT) {
+    if (a.phase == 2) {
+      s0 = a.seg_state + (seg - 1) * states;
+      if (seg != a.seg_count) sT = nullptr;
+    } else {
+      if (only) s0 = nullptr;
+      sT = a.seg_state + seg * states;
+    }
+  }
 
   if (tid == 0) {
     if (!a.cu && a.T == 0 && blockIdx.x == 0) hdr->status = RODIMUS_OK;   // (no operand kernel then)
@@ -435,16 +468,32 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     // ======================================= loads =========================================
     if (ntiles > 0 && elect_one()) {
       const unsigned char* blk = a.blocks + slot0 * B::kBytes;
-      auto mask_of = [&](int t) {
-        return __ldcg(reinterpret_cast<const unsigned long long*>(blk + (long long)t * B::kBytes + B::kHead));
+      // Split calls: the chunk masks arrive seven tiles ahead, two to a copy of 16 bytes.  Fetched one tile ahead, a
+      // mask kept this thread waiting for as long as L2 takes to answer, which was what a pass without readout took
+      // (1570 cycles; 32 x 16384 tokens 429 -> 399 us).  A full pass takes as long anyway.
+      const uint32_t masks = base + C::kOffCtl + (uint32_t)offsetof(ScanCtl, mask);
+      auto ask_mask = [&](int t) {
+        if (t < ntiles) copy_16_async(masks + 16 * (t & 7), a.masks + ((slot0 + t) & ~1ll));
+        copies_commit();
       };
-      unsigned long long next_mask = mask_of(0);
+      unsigned long long next_mask = 0ull;
+      if constexpr (SPLIT) {
+        for (int t = 0; t < 7; ++t) ask_mask(t);
+      } else {
+        next_mask = __ldcg(a.masks + slot0);
+      }
       uint32_t s = 0, ph = 1, qs = 0, qph = 1;
       int pass = 0;
       bool ok = true;
       for (int t = 0; ok && t < ntiles; ++t) {
-        const unsigned long long mask = next_mask;
-        if (t + 1 < ntiles) next_mask = mask_of(t + 1);
+        unsigned long long mask = next_mask;
+        if constexpr (SPLIT) {
+          ask_mask(t + 7);
+          copies_wait<7>();
+          mask = ctl->mask[2 * (t & 7) + (int)((slot0 + t) & 1)];
+        } else if (t + 1 < ntiles) {
+          next_mask = __ldcg(a.masks + slot0 + t + 1);
+        }
         const int nr = min(kTile, len - t * kTile);
         for (int lo = 0; lo < nr; ++pass) {
           if (!(ok = mbar_wait(bar(FB_AEMPTY0 + s), ph, wc, hdr))) break;
@@ -458,25 +507,29 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
           d->flags = (t + 1 == ntiles && hi == nr ? kLastPass : 0) | (mask != 1ull ? kCutTile : 0);
           const uint32_t st = base + s * C::kAStage, fb = bar(FB_AFULL0 + s);
           const bool beta = BLOCK && a.has_beta;
-          mbar_expect_tx(fb, C::kABytes + 2 * kSlab + (beta ? 2 * kSlab : 0));
+          const int a_bytes = only ? B::kP : C::kABytes;       // (Kt alone)
+          mbar_expect_tx(fb, a_bytes + 2 * kSlab + (beta ? 2 * kSlab : 0));
           tma_load_3d(st + C::kOffV, &maps.v, 0, (int)row, col0 >> 6, fb);
           if (beta) tma_load_3d(st + C::kOffBeta, &maps.beta, 0, (int)row, col0 >> 6, fb);
-          bulk_load(st, blk + (long long)t * B::kBytes, C::kABytes, fb);
+          bulk_load(st, blk + (long long)t * B::kBytes, a_bytes, fb);
           ctl->n_a = pass + 1;
           if (lo == 0 && t + C::kAStages < ntiles) {   // asked into L2 before its stage is free
             tma_prefetch_3d(&maps.v, 0, (int)row + C::kAStages * kTile, col0 >> 6);
             if (beta) tma_prefetch_3d(&maps.beta, 0, (int)row + C::kAStages * kTile, col0 >> 6);
-            if (BLOCK && a.feed_d) tma_prefetch_3d(&maps.fx, 0, (int)row + C::kAStages * kTile, col0 >> 6);
+            if (BLOCK && a.feed_d && !only) tma_prefetch_3d(&maps.fx, 0, (int)row + C::kAStages * kTile, col0 >> 6);
           }
           if (++s == C::kAStages) { s = 0; ph ^= 1; }
           if (!(ok = mbar_wait(bar(FB_QEMPTY0 + qs), qph, wc, hdr))) break;
-          mbar_expect_tx(bar(FB_QFULL0 + qs), C::kQBytes);
-          bulk_load(base + C::kOffQ + qs * C::kQBytes, blk + (long long)t * B::kBytes + B::kQ, C::kQBytes, bar(FB_QFULL0 + qs));
+          const int q_skip = only ? B::kD - B::kQ : 0;         // (D alone)
+          mbar_expect_tx(bar(FB_QFULL0 + qs), C::kQBytes - q_skip);
+          bulk_load(base + C::kOffQ + qs * C::kQBytes + q_skip, blk + (long long)t * B::kBytes + B::kQ + q_skip, C::kQBytes - q_skip,
+                    bar(FB_QFULL0 + qs));
           ctl->n_q = pass + 1;
           if (++qs == C::kQStages) { qs = 0; qph ^= 1; }
           lo = hi;
         }
       }
+      if constexpr (SPLIT) copies_wait<0>();
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -497,6 +550,8 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         }
         const uint32_t st = base + s * C::kAStage, sq = base + C::kOffQ + qs * C::kQBytes;
         const uint32_t dv = desc_lo_mnmajor(st + C::kOffV, kSlab);
+        // (no readout in between: the state group has taken dS of two chunks before when it reports for the last)
+        if (only && c > 0 && !mbar_wait(bar(FB_SREADY0 + ((c - 1) & 1)), ((c - 1) >> 1) & 1, wc, hdr)) break;
         tc_fence_after();
         // dS (buffer c & 1: the state group has taken dS of two chunks before, or the readout of the
         // chunk before could not have been issued)
@@ -513,6 +568,12 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
           }
         }
         umma_commit(bar(FB_SFULL0 + (c & 1)));
+        if (only) {
+          umma_commit(bar(FB_AEMPTY0 + s));
+          if (flags & kLastPass) break;
+          if (++s == C::kAStages) { s = 0; ph ^= 1; }
+          continue;
+        }
         if (!mbar_wait(bar(FB_OFREE0 + (c & 1)), ((c >> 1) & 1) ^ 1, wc, hdr)) break;
         tc_fence_after();
         const uint32_t o = tmem + C::kColO + (c & 1) * 64, sb = tmem + C::kColSb + (c & 1) * C::kSbCols;
@@ -546,16 +607,14 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
       }
     }
     __syncwarp();
-  } else if (warp == 2) {
+  } else if (warp == 2 && !only) {
     // ================================= output tiles to global ==============================
     // Feed-through: the x' tile of a pass is fetched INTO its output tile, to be combined with the
     // accumulators in place; two passes ahead, as soon as the copies have read that tile (one pass ahead
     // a fetch and a store were on the way of every pass: 2.7 us a tile instead of 1.2).
     const bool feed = BLOCK && a.feed_d != nullptr;
     int xt = 0, xlo = 0;                               // tile and first row of the next chunk to fetch for
-    auto mask_of = [&](int t) {
-      return __ldcg(reinterpret_cast<const unsigned long long*>(a.blocks + (slot0 + t) * B::kBytes + B::kHead));
-    };
+    auto mask_of = [&](int t) { return __ldcg(a.masks + slot0 + t); };
     unsigned long long xmask = feed && ntiles > 0 ? mask_of(0) : 0ull;
     auto fetch_x = [&](int c) {
       if (xt >= ntiles) return;
@@ -656,7 +715,11 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
 #pragma unroll
     for (int e = 0; e < kHalf / 2; ++e) {
       S[e] = make_float2(0.f, 0.f);
-      if (a.s0) S[e] = make_float2(__ldg(a.s0 + off + (long long)(2 * e) * a.dv), __ldg(a.s0 + off + (long long)(2 * e + 1) * a.dv));
+      if constexpr (SPLIT) {
+        if (s0) S[e] = make_float2(__ldcg(s0 + off + (long long)(2 * e) * a.dv), __ldcg(s0 + off + (long long)(2 * e + 1) * a.dv));
+      } else {
+        if (a.s0) S[e] = make_float2(__ldg(a.s0 + off + (long long)(2 * e) * a.dv), __ldg(a.s0 + off + (long long)(2 * e + 1) * a.dv));
+      }
     }
     uint32_t qs = 0, qph = 0;
     int n_cut = 0;
@@ -695,6 +758,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         const uint32_t t_sb = t_lane + C::kColSb + (c & 1) * C::kSbCols + ch0 / 2;
 #pragma unroll
         for (int piece = 0; piece < kHalf / 32; ++piece) {
+          if (only) break;
           uint32_t w[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) w[e] = pack_bf16(S[16 * piece + e].x, S[16 * piece + e].y);
@@ -720,7 +784,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
           D = reinterpret_cast<const float*>(gbase + C::kOffDc) + (n_cut & 7) * DK;
           ++n_cut;
         }
-        if ((flags & kLastPass) && !a.sT) break;
+        if ((flags & kLastPass) && !sT) break;
         if (!(ok = wait_all(FB_SFULL0 + (c & 1), (c >> 1) & 1))) break;
         tc_fence_after();
         advance(c, D);
@@ -731,14 +795,42 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         if (++qs == C::kQStages) { qs = 0; qph ^= 1; }
       }
     }
-    if (ok && a.sT) {
+    if (ok && sT) {
 #pragma unroll
       for (int e = 0; e < kHalf / 2; ++e) {
-        a.sT[off + (long long)(2 * e) * a.dv] = S[e].x;
-        a.sT[off + (long long)(2 * e + 1) * a.dv] = S[e].y;
+        sT[off + (long long)(2 * e) * a.dv] = S[e].x;
+        sT[off + (long long)(2 * e + 1) * a.dv] = S[e].y;
       }
     }
-  } else if (warp >= 12 && warp < 16) {
+  } else if (only && warp == 12) {
+    // ============================== the segment's decay ====================================
+    float prod[DK / 32];
+#pragma unroll
+    for (int i = 0; i < DK / 32; ++i) prod[i] = 1.f;
+    uint32_t qs = 0, qph = 0;
+    int n_cut = 0;
+    for (int c = 0; ntiles > 0; ++c) {
+      if (!wait_all(FB_QFULL0 + qs, qph)) break;
+      const int flags = ctl->desc[c & 7].flags;
+      const float* D = reinterpret_cast<const float*>(gbase + C::kOffQ + qs * C::kQBytes + (B::kD - B::kQ));
+      if (flags & kCutTile) {
+        if (!wait_all(FB_CUT0 + (n_cut & 7), (n_cut >> 3) & 1)) break;
+        D = reinterpret_cast<const float*>(gbase + C::kOffDc) + (n_cut & 7) * DK;
+        ++n_cut;
+      }
+#pragma unroll
+      for (int i = 0; i < DK / 32; ++i) prod[i] *= D[lane + 32 * i];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(FB_QEMPTY0 + qs));
+      if (flags & kLastPass) break;
+      if (++qs == C::kQStages) { qs = 0; qph ^= 1; }
+    }
+    if (slice == 0) {
+      float* d = a.seg_decay + (seg - 1) * decays + ((long long)n * a.H + h) * DK + lane;
+#pragma unroll
+      for (int i = 0; i < DK / 32; ++i) d[32 * i] = prod[i];
+    }
+  } else if (!only && warp >= 12 && warp < 16) {
     // ====================================== outputs ========================================
     // O^T has the value columns in the tensor-memory lanes.  The 16x256b load hands out 8x8 fragments
     // [value column][row]; stmatrix.trans writes them transposed into a tile of two swizzled 64-column
@@ -856,16 +948,95 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
+// Between the two launches of a split call: S_start(1) is state 0, S_start(k+1) = D_k . S_start(k) + dS_k takes the
+// place of dS_k.  A thread per four columns of a row; `rows` = sequences x heads x dk.
+constexpr int kJoinThreads = 256;
+__global__ void __launch_bounds__(kJoinThreads) ddts_join_kernel(float* state, const float* decay, int G, long long rows, int dv) {
+  wait_for_previous_kernel();
+  const long long i = (long long)blockIdx.x * kJoinThreads + threadIdx.x;
+  if (i >= rows * (dv / 4)) return;
+  const long long row = i / (dv / 4), states = rows * dv;
+  float4* at = reinterpret_cast<float4*>(state) + i;
+  float4 S = __ldcg(at);
+  for (int k = 1; k < G; k += 5) {          // (loads of five segments at a time)
+    float4 x[5];
+    float d[5];
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+      if (k + u >= G) continue;
+      x[u] = __ldcg(at + (k + u) * (states / 4));
+      d[u] = __ldcg(decay + (k + u - 1) * rows + row);
+    }
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+      if (k + u >= G) continue;
+      S = make_float4(fmaf(d[u], S.x, x[u].x), fmaf(d[u], S.y, x[u].y), fmaf(d[u], S.z, x[u].z), fmaf(d[u], S.w, x[u].w));
+      __stcg(at + (k + u) * (states / 4), S);
+    }
+  }
+}
+
 template <int DK>
 size_t blocks_bytes(long long slots) { return (size_t)slots * Block<DK>::kBytes; }
+
+// Few (sequence, head, 128 columns) and long sequences: split along time.  The state recurrence is linear,
+// S_end = D_seg . S_start + dS_seg, with dS_seg the segment's final state from a zero start and D_seg the product of
+// its decays.  A dense call is cut into a head segment 0 and G equal segments 1..G, and scanned in two launches with a small one between:
+//   phase 1   segment 0 as it stands; segments 1..G-1 from a zero state, without readout: dS and D
+//   join      S_start(k+1) = D_k . S_start(k) + dS_k
+//   phase 2   segments 1..G, each from its S_start
+// The operands are formed once.  A pass without readout takes kStateOnly of a full one, and the head segment is that
+// much shorter, so that phase 1 ends everywhere at once.
+struct Segments {
+  int G = 0;                  // 0: not split
+  int tiles0 = 0, tiles = 0;  // of the head segment, of each later one (the last may be shorter)
+};
+constexpr int kMaxSegments = 16, kMinSegmentTiles = 16;
+constexpr double kStateOnly = 0.4;
+
+// As many segments as there is room for on the SMs, where the scan is shorter by 20 us: two more launches, with a
+// start and an end each, cost 10 to 15 (dk = 64, one set of gates, two segments: 32 heads x 2048 tokens 43.3 us
+// whole, 45.4 split, 4 x 8 x 4096 80.8 and 75.8).  Both sides measured, whole or split by the pair kernel against
+// here (sets of gates x tokens, us):
+//   one set of gates   dk = 64, 4 heads x 32768 468 -> 98, 16 x 8192 126 -> 75; dk = 128, 16 x 16384 226 -> 111
+//   gates per head     dv = 256 8 x 8192 130 -> 74, 4 x 32768 153 -> 129, 16 x 8192 140 -> 126, 32 x 4096 129 -> 122;
+//                      while the operands stay in L2 (126 MB): 10 x 32768 273 -> 270, 16 x 32768 409 -> 411,
+//                      32 x 16384 358 -> 399.  With both block terms 16 x 32768 613 -> 541, 32 x 8192 305 -> 278;
+//                      dv = 512 8 x 32768 408 -> 301, 16 x 16384 358 -> 288; dv = 128 16 x 16384 335 -> 191, but
+//                      64 x 4096, two segments of operands from DRAM, 177 -> 183.  Below 4096 tokens the other side
+//                      is not split: 37 x 4000, two segments, 132 -> 134, with block terms 159 -> 170.
+// Small calls keep the form that they had.
+constexpr int kMinSplitPasses = 1280, kMinSplitItems = 4;   // dk = 128: items x tiles; dk = 64: items
+constexpr size_t kStaysInL2 = (size_t)136 << 20;
+
+Segments plan_segments(const rodimus_ddts_fwd_params& p, int sms) {
+  Segments s;
+  if (p.cu_seqlens || p.cu_seqlens_host) return s;
+  const long long items = (long long)p.B * p.H * (p.dv / 128), tiles = (p.T + kTile - 1) / kTile;
+  if (items <= 0 || (p.dk == 64 ? items < kMinSplitItems : items * tiles < kMinSplitPasses)) return s;
+  const int g = (int)std::min<long long>(std::min<long long>(sms / items, kMaxSegments), tiles / kMinSegmentTiles);
+  if (g < 2 || 0.8 * tiles * (1.0 - (1.0 + kStateOnly) / (g + kStateOnly)) < 20.0) return s;
+  if (p.dk == 128 && !p.shared_gates && (size_t)(p.B * (long long)p.H * tiles) * Block<128>::kBytes > kStaysInL2) {
+    if (p.dv == 256 && !p.beta_hat && !p.feed_d) return s;
+    if (p.dv % 256 && g == 2) return s;
+  }
+  if (p.dk == 128 && !p.shared_gates && p.dv % 256 == 0 && g == 2 && p.T < 4096) return s;
+  const int each = (int)std::ceil(tiles / (g + kStateOnly));
+  const long long first = tiles - (long long)g * each;
+  s.tiles0 = first > 0 ? (int)first : 1;
+  s.tiles = (int)((tiles - s.tiles0 + g - 1) / g);
+  s.G = (int)((tiles - s.tiles0 + s.tiles - 1) / s.tiles);
+  return s;
+}
 
 struct ScanPlan {
   long long slots;        // tiles, over all sets of gates
   int slots_per_head, gate_heads;
-  size_t blocks, bytes;   // workspace: offset of the blocks, total
+  Segments seg;
+  size_t blocks, masks, seg_state, seg_decay, bytes;   // workspace: offsets of the blocks, masks, segments' states and decays; total
 };
 
-ScanPlan scan_plan(const rodimus_ddts_fwd_params& p) {
+ScanPlan scan_plan(const rodimus_ddts_fwd_params& p, int sms) {
   ScanPlan s;
   const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
   s.gate_heads = p.shared_gates ? 1 : p.H;
@@ -874,25 +1045,49 @@ ScanPlan scan_plan(const rodimus_ddts_fwd_params& p) {
   size_t order = (size_t)(varlen ? p.N : 0) * sizeof(int32_t);
   s.blocks = sizeof(WorkspaceHeader) + ((order + 1023) & ~(size_t)1023);
   s.bytes = s.blocks + (p.dk == 64 ? blocks_bytes<64>(s.slots) : blocks_bytes<128>(s.slots));
+  s.masks = s.bytes;
+  s.bytes += ((size_t)s.slots * sizeof(unsigned long long) + 255) & ~(size_t)255;
+  s.seg = plan_segments(p, sms);
+  s.seg_state = s.bytes;
+  const size_t per = (size_t)p.B * p.H * p.dk * sizeof(float);
+  s.seg_decay = s.seg_state + (size_t)s.seg.G * per * p.dv;
+  if (s.seg.G > 0) s.bytes = s.seg_decay + (size_t)(s.seg.G - 1) * per;
   return s;
 }
 
 template <int DK, bool BLOCK>
-cudaError_t launch_scan(const ScanMaps& m, const ScanArgs& a, long long slots, long long items, int dev, cudaStream_t st) {
-  static std::atomic<unsigned long long> opted_ops{0}, opted{0};   // per instantiation
+cudaError_t launch_scan(const ScanMaps& m, ScanArgs& a, long long slots, long long items, int dev, cudaStream_t st, int* n_launches) {
+  static std::atomic<unsigned long long> opted_ops{0}, opted{0}, opted_split{0};   // per instantiation
   using C = Scan<DK, BLOCK>;
   cudaError_t e = opt_in_shared_memory(ddts_operands_kernel<DK>, kOpSmem<DK>, dev, opted_ops);
-  if (e == cudaSuccess) e = opt_in_shared_memory(ddts_scan_kernel<DK, BLOCK>, Scan<DK, BLOCK>::kSmem, dev, opted);
+  if (e == cudaSuccess) e = a.seg_count ? opt_in_shared_memory(ddts_scan_kernel<DK, BLOCK, true>, C::kSmem, dev, opted_split)
+                                        : opt_in_shared_memory(ddts_scan_kernel<DK, BLOCK, false>, C::kSmem, dev, opted);
   if (e != cudaSuccess) return e;
   if (slots > 0) {
     ddts_operands_kernel<DK><<<(unsigned)slots, kOpThreads, kOpSmem<DK>, st>>>(a);
+    ++*n_launches;
     // The scan may start while the operand kernel's last CTAs run: it sets up (barriers, tensor memory)
     // and waits for that kernel before it reads a block.
-    e = launch_overlapped(ddts_scan_kernel<DK, BLOCK>, (unsigned)items, C::kThreads, C::kSmem, st, m, a);
+    if (a.seg_count) {
+      const unsigned grid = (unsigned)(items * a.seg_count);
+      const long long rows = (long long)a.n_seq * a.H * DK;
+      a.phase = 1;
+      e = launch_overlapped(ddts_scan_kernel<DK, BLOCK, true>, grid, C::kThreads, C::kSmem, st, m, a);
+      if (e == cudaSuccess)
+        e = launch_overlapped(ddts_join_kernel, (unsigned)((rows * (a.dv / 4) + kJoinThreads - 1) / kJoinThreads), kJoinThreads, 0, st,
+                              a.seg_state, a.seg_decay, a.seg_count, rows, a.dv);
+      a.phase = 2;
+      if (e == cudaSuccess) e = launch_overlapped(ddts_scan_kernel<DK, BLOCK, true>, grid, C::kThreads, C::kSmem, st, m, a);
+      *n_launches += 3;
+    } else {
+      e = launch_overlapped(ddts_scan_kernel<DK, BLOCK, false>, (unsigned)items, C::kThreads, C::kSmem, st, m, a);
+      ++*n_launches;
+    }
   } else {
     // No tokens: what is in front now is the plan of the sequences, whose order the scan reads before it
     // waits for anything.  So it starts when that has ended.
-    ddts_scan_kernel<DK, BLOCK><<<(unsigned)items, C::kThreads, C::kSmem, st>>>(m, a);
+    ddts_scan_kernel<DK, BLOCK, false><<<(unsigned)items, C::kThreads, C::kSmem, st>>>(m, a);
+    ++*n_launches;
   }
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -947,15 +1142,17 @@ size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
   const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
   const bool block = p.beta_hat || p.feed_d, whole = p.dv % 256 == 0;
   const long long n_seq = varlen ? p.N : p.B, sets = n_seq * p.H, items = sets * (p.dv / 128);
+  int dev = 0, sms = 0;
+  if (current_device(&dev, &sms) != cudaSuccess) {
+    cudaGetLastError();
+    sms = 0;
+  }
   if (p.dk == 64) {
     if (block) return 0;
   } else {
-    int dev = 0, sms = 0;
-    if (current_device(&dev, &sms) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    if (items == 0) return 0;
+    if (sms == 0 || items == 0 || (!whole && (block || p.shared_gates))) return 0;
+  }
+  if (p.dk == 128 && plan_segments(p, sms).G == 0) {
     if (p.shared_gates) {
       const double tiles = varlen ? (double)p.T / ((double)n_seq * kTile) + 0.5 : (double)((p.T + kTile - 1) / kTile);
       if (!whole || !scan_pays_with_shared_gates(n_seq, tiles, p.H * (p.dv / 256.0), varlen, sms)) return 0;
@@ -975,14 +1172,26 @@ size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
       }
     }
   }
-  const ScanPlan s = scan_plan(p);
+  const ScanPlan s = scan_plan(p, sms);
   if (s.slots > 0x7fffffffLL || items > 0x7fffffffLL) return 0;
   return s.bytes;
 }
 
+bool fwd_scan_split(const rodimus_ddts_fwd_params& p) {
+  int dev = 0, sms = 0;
+  if (current_device(&dev, &sms) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return plan_segments(p, sms).G > 0;
+}
+
 cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
   *n_launches = 0;
-  const ScanPlan s = scan_plan(p);
+  int dev = 0, sms = 0;
+  cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  const ScanPlan s = scan_plan(p, sms);
   const long long n_seq = p.cu_seqlens ? p.N : p.B, items = n_seq * p.H * (p.dv / 128);
   if (items == 0) return cudaSuccess;
   char* ws = reinterpret_cast<char*>(p.workspace);
@@ -991,6 +1200,7 @@ cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
   a.gx = (const __nv_bfloat16*)p.gate_x; a.ty = (const __nv_bfloat16*)p.temp_y;
   a.s0 = p.s0; a.sT = p.sT; a.feed_d = p.feed_d;
   a.blocks = reinterpret_cast<unsigned char*>(ws + s.blocks);
+  a.masks = reinterpret_cast<unsigned long long*>(ws + s.masks);
   a.cu = p.cu_seqlens;
   a.order = reinterpret_cast<const int32_t*>(ws + sizeof(WorkspaceHeader));
   a.hdr = reinterpret_cast<WorkspaceHeader*>(ws);
@@ -1001,9 +1211,10 @@ cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
   a.has_beta = p.beta_hat != nullptr;
   a.scale = p.scale; a.ingate = p.ingate;
   a.limit = main_loop_wait_cycles();
-  int dev = 0, sms = 0;
-  cudaError_t e = current_device(&dev, &sms);
-  if (e != cudaSuccess) return e;
+  a.seg_count = s.seg.G; a.seg_tiles0 = s.seg.tiles0; a.seg_tiles = s.seg.tiles;
+  a.phase = 0;
+  a.seg_state = reinterpret_cast<float*>(ws + s.seg_state);
+  a.seg_decay = reinterpret_cast<float*>(ws + s.seg_decay);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
   ScanMaps m;
   const uint64_t rows = (uint64_t)p.B * p.H * p.T, dv = (uint64_t)p.dv;
@@ -1018,11 +1229,9 @@ cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
     memset(&m, 0, sizeof(m));   // never used: no tiles
   }
   const long long slots = rows > 0 ? s.slots : 0;
-  if (p.dk == 64) e = launch_scan<64, false>(m, a, slots, items, dev, st);
-  else if (p.beta_hat || p.feed_d) e = launch_scan<128, true>(m, a, slots, items, dev, st);
-  else e = launch_scan<128, false>(m, a, slots, items, dev, st);
-  *n_launches = slots > 0 ? 2 : 1;
-  return e;
+  if (p.dk == 64) return launch_scan<64, false>(m, a, slots, items, dev, st, n_launches);
+  if (p.beta_hat || p.feed_d) return launch_scan<128, true>(m, a, slots, items, dev, st, n_launches);
+  return launch_scan<128, false>(m, a, slots, items, dev, st, n_launches);
 }
 
 }  // namespace ddts

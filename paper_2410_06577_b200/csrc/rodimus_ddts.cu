@@ -69,11 +69,12 @@ bool fwd_pair_selected(const rodimus_ddts_fwd_params& p) { return fwd_pair_suppo
 
 bool has_block_terms(const rodimus_ddts_fwd_params& p) { return p.beta_hat || p.feed_d; }
 
-// Workspace of the two-launch prefill where it is to be used; dense calls that the pair kernel splits
-// along time stay there (their few heads fill the device only that way).
+// Workspace of the prefill that forms operands first where it is to be used; dense calls that only the pair
+// kernel splits along time stay there (their few heads fill the device only that way).
 size_t scan_path_bytes(const rodimus_ddts_fwd_params& p) {
-  if (fwd_pair_selected(p) && fwd_pair_split_workspace_bytes(p) > 0) return 0;
-  return fwd_scan_workspace_bytes(p);
+  const size_t bytes = fwd_scan_workspace_bytes(p);
+  if (bytes > 0 && fwd_pair_selected(p) && fwd_pair_split_workspace_bytes(p) > 0 && !fwd_scan_split(p)) return 0;
+  return bytes;
 }
 
 // 0: cluster-pair tensor-core kernel, 1: single-CTA tensor-core kernel (the recurrence alone),
@@ -97,8 +98,8 @@ size_t rodimus_ddts_fwd_workspace_bytes(const rodimus_ddts_fwd_params* p) {
   const size_t base = workspace_bytes_for(varlen ? p->N : 0);
   // long dense sequences with few heads run faster split along time, given room for the
   // segments' states; a caller that passes only the base size still gets the unsplit path
-  const size_t split = ddts::fwd_pair_selected(*p) ? ddts::fwd_pair_split_workspace_bytes(*p) : 0;
-  size_t more = split > 0 ? split : ddts::scan_path_bytes(*p);
+  size_t more = ddts::scan_path_bytes(*p);
+  if (more == 0 && ddts::fwd_pair_selected(*p)) more = ddts::fwd_pair_split_workspace_bytes(*p);
   if (more == 0 && ddts::fwd_kernel_choice(*p) == 2) more = ddts::fwd_simt_chunks_workspace_bytes(*p);
   return more > base ? more : base;
 }

@@ -1178,6 +1178,58 @@ def test_two_launch_prefill_gates_per_head_few_tiles(block, T):
         assert rd.last_launch_count() == 2
 
 
+@pytest.mark.parametrize("B,H,T,dk,dv,kind,gate_mean", [
+    (1, 8, 8192 - 63, 128, 256, "plain", -4.0),    # last tile of one row, long memory
+    (1, 32, 4100, 128, 256, "plain", -3.0),        # two segments
+    (2, 3, 11000, 128, 256, "plain", 1.5),         # tiles cut into chunks, a segment's decay underflows
+    (1, 16, 8250, 128, 128, "plain", -3.0),        # one slice of 128 columns a head
+    (1, 1, 32800, 128, 512, "plain", -4.0),        # the most segments, four slices
+    (1, 8, 8250, 128, 256, "both", -3.0),          # value gate and feed-through
+    (1, 8, 8250, 128, 256, "gate", -3.0),
+    (1, 4, 16500, 64, 256, "shared", -3.0),        # one set of gates for all heads
+    (1, 8, 8250, 128, 256, "shared", -3.0),
+])
+def test_prefill_that_forms_operands_first_split_along_time(B, H, T, dk, dv, kind, gate_mean):
+    if kind == "shared":
+        launches = _check_shared(1003, B, H, T, dk, dv, "bf16", ingate=rd.INGATE_POW_SIGMOID)
+    else:
+        p = wl.make_prefill(1004, B, H, T, dk, dv, "bf16", gate_mean=gate_mean, s0_std=0.3)
+        if kind == "plain":
+            _check_prefill(p, rd.INGATE_POW_G, 0.5)
+            launches = rd.last_launch_count()
+            _check_prefill(p, rd.INGATE_POW_SIGMOID, 0.5)
+        else:
+            launches = _check_block(p, kind)
+    assert launches == 4
+
+
+def test_prefill_split_along_time_narrow_keys_keep_fp32_accuracy():
+    """dk = 64, slow decay: the final state carries products over all segments (see the bound above)."""
+    p = wl.make_prefill(1005, 1, 4, 33000, 64, 128, "bf16", gate_mean=-6.0, s0_std=0.1)
+    _, sT = _run_prefill(p)
+    assert rd.last_launch_count() == 4
+    _, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0)
+    assert np.linalg.norm(sT - rs) <= 5e-7 * np.linalg.norm(rs)
+
+
+def test_prefill_split_along_time_wait_that_runs_out_is_reported():
+    import torch
+    p = wl.make_prefill(1006, 1, 8, 8250, 128, 256, "bf16", s0_std=0.3)
+    d = prefill_to_device(p)
+    o, sT = _nan_outputs(d)
+    prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT)
+    ws = torch.empty(rd.fwd_workspace_bytes(prm), dtype=torch.uint8, device="cuda")
+    prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
+    rd.test_set_wait_limit(0)
+    try:
+        assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.ERR_TIMEOUT
+    finally:
+        rd.test_set_wait_limit(-1)
+    assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
+    ro, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0)
+    assert rel_err(host(o), ro) <= TOL_BF16 and rel_err(host(sT), rs) <= TOL_BF16
+
+
 @pytest.mark.parametrize("dk", [64, 128])
 def test_two_launch_prefill_dense_without_tokens(dk):
     import torch
