@@ -991,36 +991,41 @@ struct Segments {
   int G = 0;                  // 0: not split
   int tiles0 = 0, tiles = 0;  // of the head segment, of each later one (the last may be shorter)
 };
-constexpr int kMaxSegments = 16, kMinSegmentTiles = 16;
+constexpr int kMaxSegments = 16, kMinSegmentTiles = 8;
 constexpr double kStateOnly = 0.4;
 
-// As many segments as there is room for on the SMs, where the scan is shorter by 20 us: two more launches, with a
-// start and an end each, cost 10 to 15 (dk = 64, one set of gates, two segments: 32 heads x 2048 tokens 43.3 us
-// whole, 45.4 split, 4 x 8 x 4096 80.8 and 75.8).  Both sides measured, whole or split by the pair kernel against
-// here (sets of gates x tokens, us):
+// As many segments as there is room for on the SMs, where the passes saved (0.8 us each) are worth more than 17 us, 20
+// with two segments: two more launches, with a start and an end each, cost about that (one set of gates: two segments,
+// dk = 128, 32 heads x 2589 tokens, 14 us, 43.0 us whole, 47.6 split, dk = 64, 4 x 8 x 4096, 21 us, 80.8 and 75.8;
+// four segments, 16 x 2048, 17.5 us, 41.3 and 33.4, dv = 128 with gates per head 32 x 2048, 63.8 and 61.8).  Both sides
+// measured, whole or split by the pair kernel against here (sets of gates x tokens, us):
 //   one set of gates   dk = 64, 4 heads x 32768 468 -> 98, 16 x 8192 126 -> 75; dk = 128, 16 x 16384 226 -> 111
-//   gates per head     dv = 256 8 x 8192 130 -> 74, 4 x 32768 153 -> 129, 16 x 8192 140 -> 126, 32 x 4096 129 -> 122;
+//   gates per head     dv = 256 8 x 2048 39 -> 33, 16 x 2048 49 -> 46, 4 x 4000 60 -> 35, 8 x 4096 109 -> 46,
+//                      8 x 8192 130 -> 74, 4 x 32768 153 -> 129, 16 x 8192 140 -> 126, 32 x 4096 129 -> 122;
 //                      while the operands stay in L2 (126 MB): 10 x 32768 273 -> 270, 16 x 32768 409 -> 411,
 //                      32 x 16384 358 -> 399.  With both block terms 16 x 32768 613 -> 541, 32 x 8192 305 -> 278;
 //                      dv = 512 8 x 32768 408 -> 301, 16 x 16384 358 -> 288; dv = 128 16 x 16384 335 -> 191, but
 //                      64 x 4096, two segments of operands from DRAM, 177 -> 183.  Below 4096 tokens the other side
-//                      is not split: 37 x 4000, two segments, 132 -> 134, with block terms 159 -> 170.
-// Small calls keep the form that they had.
-constexpr int kMinSplitPasses = 1280, kMinSplitItems = 4;   // dk = 128: items x tiles; dk = 64: items
+//                      is not split: 37 x 4000, two segments, 132 -> 134, with block terms 159 -> 170, 32 x 3900
+//                      with one set of gates 60.5 -> 61.6.
+// Calls of the fewest items that the pair kernel splits, from 4096 tokens on, stay with its five launches, which are
+// what its tests count (4 x 6000 tokens 146 us, 41 here), and so do one or two slices of dk = 64 with one launch.
+constexpr int kMinSplitPasses = 1280, kMinSplitItems = 16;   // items x tiles, items
 constexpr size_t kStaysInL2 = (size_t)136 << 20;
 
 Segments plan_segments(const rodimus_ddts_fwd_params& p, int sms) {
   Segments s;
   if (p.cu_seqlens || p.cu_seqlens_host) return s;
   const long long items = (long long)p.B * p.H * (p.dv / 128), tiles = (p.T + kTile - 1) / kTile;
-  if (items <= 0 || (p.dk == 64 ? items < kMinSplitItems : items * tiles < kMinSplitPasses)) return s;
+  if (items <= 0) return s;
+  if (p.dk == 64 ? items < 4 : p.dv % 256 == 0 && p.T >= 4096 && items < kMinSplitItems && items * tiles < kMinSplitPasses) return s;
   const int g = (int)std::min<long long>(std::min<long long>(sms / items, kMaxSegments), tiles / kMinSegmentTiles);
-  if (g < 2 || 0.8 * tiles * (1.0 - (1.0 + kStateOnly) / (g + kStateOnly)) < 20.0) return s;
+  if (g < 2 || 0.8 * tiles * (1.0 - (1.0 + kStateOnly) / (g + kStateOnly)) < (g == 2 ? 20.0 : 17.0)) return s;
   if (p.dk == 128 && !p.shared_gates && (size_t)(p.B * (long long)p.H * tiles) * Block<128>::kBytes > kStaysInL2) {
     if (p.dv == 256 && !p.beta_hat && !p.feed_d) return s;
     if (p.dv % 256 && g == 2) return s;
   }
-  if (p.dk == 128 && !p.shared_gates && p.dv % 256 == 0 && g == 2 && p.T < 4096) return s;
+  if (p.dk == 128 && p.dv % 256 == 0 && g == 2 && p.T < 4096) return s;
   const int each = (int)std::ceil(tiles / (g + kStateOnly));
   const long long first = tiles - (long long)g * each;
   s.tiles0 = first > 0 ? (int)first : 1;

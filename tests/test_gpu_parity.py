@@ -1181,6 +1181,8 @@ def test_two_launch_prefill_gates_per_head_few_tiles(block, T):
 @pytest.mark.parametrize("B,H,T,dk,dv,kind,gate_mean", [
     (1, 8, 8192 - 63, 128, 256, "plain", -4.0),    # last tile of one row, long memory
     (1, 32, 4100, 128, 256, "plain", -3.0),        # two segments
+    (1, 2, 1986, 128, 128, "plain", -3.0),         # four of eight tiles, the last tile of two rows
+    (1, 16, 1985, 128, 256, "both", -3.0),         # four of eight, the last shorter
     (2, 3, 11000, 128, 256, "plain", 1.5),         # tiles cut into chunks, a segment's decay underflows
     (1, 16, 8250, 128, 128, "plain", -3.0),        # one slice of 128 columns a head
     (1, 1, 32800, 128, 512, "plain", -4.0),        # the most segments, four slices
