@@ -162,7 +162,8 @@ typedef struct {
  * the sequences into time segments that run side by side (the state recurrence is linear in
  * the state, so segments are joined exactly up to rounding) and part of the work is enqueued
  * on the library's own second stream, forked from and joined back into `stream` with events, so
- * the call still behaves as one piece of work on `stream`.  For bf16 requests with dk = 64, with
+ * the call still behaves as one piece of work on `stream`.  (Calls that form gated operands first, below,
+ * need no second stream for it.)  For bf16 requests with dk = 64, with
  * one set of gates for all heads or with few heads it includes a block of gated operands (41 KiB,
  * 57 for dk = 64) per 64 tokens and set of gates, which may be as much as the inputs take, and for
  * small fp32 requests the states of 16-token chunks, so that all SMs can form them ahead of the scan.  A caller that passes less (never less than 256 bytes plus

@@ -1,5 +1,6 @@
 // Chunked DDTS prefill in two launches, for calls whose gates serve several CTAs or whose items are
-// too few to fill the device: operands first, then the scan.
+// too few to fill the device: operands first, then the scan (in two phases where it is split along time,
+// see Segments).
 //
 // Chunk algebra (appendix "Chunkwise Parallel Representation of the Rodimus Block"; chunk length 64,
 // log2 domain, decays anchored at the chunk start, b_r = sum_{j<=r} log2 alpha_j <= 0):
