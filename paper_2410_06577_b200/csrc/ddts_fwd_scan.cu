@@ -570,8 +570,8 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         }
         umma_commit(bar(FB_SFULL0 + (c & 1)));
         if (only) {
+          if (flags & kLastPass) break;        // (nobody would wait for that commit: it could arrive after the CTA's end)
           umma_commit(bar(FB_AEMPTY0 + s));
-          if (flags & kLastPass) break;
           if (++s == C::kAStages) { s = 0; ph ^= 1; }
           continue;
         }

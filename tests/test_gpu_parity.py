@@ -1232,6 +1232,29 @@ def test_prefill_split_along_time_wait_that_runs_out_is_reported():
     assert rel_err(host(o), ro) <= TOL_BF16 and rel_err(host(sT), rs) <= TOL_BF16
 
 
+def test_prefill_split_along_time_back_to_back_on_one_workspace():
+    """Calls behind one another on a user's stream, each into the blocks and states of the one before it: nothing
+    of a launch may still be on its way when the next one begins.  Head segments of one tile, segments of eight."""
+    import torch
+    ps = [wl.make_prefill(1010 + i, 1, H, T, 128, dv, "bf16", s0_std=0.3)
+          for i, (H, T, dv) in enumerate([(8, 8250, 256), (1, 2113, 128), (8, 8250, 256), (16, 1985, 256)])]
+    side = torch.cuda.Stream()
+    outs = []
+    with torch.cuda.stream(side):
+        ws = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+        for p, d in [(p, prefill_to_device(p)) for p in ps]:
+            o, sT = _nan_outputs(d)
+            prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT)
+            prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
+            assert rd.fwd_raw(prm) == rd.OK and rd.last_launch_count() == 4
+            outs.append((p, d, o, sT))
+        side.synchronize()
+    assert rd.device_status(ws) == rd.OK
+    for p, _, o, sT in outs:
+        ro, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0)
+        assert rel_err(host(o), ro) <= TOL_BF16 and rel_err(host(sT), rs) <= TOL_BF16
+
+
 @pytest.mark.parametrize("dk", [64, 128])
 def test_two_launch_prefill_dense_without_tokens(dk):
     import torch
