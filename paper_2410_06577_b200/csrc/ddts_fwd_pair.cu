@@ -1421,11 +1421,12 @@ bool encode_bf16_slab_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool encode_bf16_heads_map(CUtensorMap* m, const void* ptr, uint64_t heads, uint64_t rows, uint32_t box_rows, uint32_t slabs) {
+bool encode_bf16_heads_map(CUtensorMap* m, const void* ptr, uint64_t heads, uint64_t rows, uint64_t cols, uint32_t box_rows,
+                           uint32_t slabs) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
-  const cuuint64_t dims[4] = {64, rows, 2, heads};
-  const cuuint64_t strides[3] = {256, 128, rows * 256};
+  const cuuint64_t dims[4] = {64, rows, cols / 64, heads};
+  const cuuint64_t strides[3] = {cols * 2, 128, rows * cols * 2};
   const cuuint32_t box[4] = {64u, box_rows, slabs, 1u};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, estr,

@@ -28,6 +28,10 @@
 // (down to single rows, which always fit because a step's decay is applied as at least e^-60): P
 // then keeps pairs of the same chunk only, and the scan takes the tile once per chunk, with the other
 // rows of Kt set to zero.
+//
+// The rows of v behind a sequence's end are zeros: against the zero rows of Kt alone a NaN or an infinity of the
+// sequence or head that follows would not vanish.  Behind a head's end the tensor map sees to it, behind a packed
+// sequence's warp 3 or the warps of the value gate.
 #include <cuda.h>
 
 #include <algorithm>
@@ -338,17 +342,18 @@ enum { FB_AFULL0 = 0,                   // [3] Kt, P, v landed                  
        FB_OTFREE0, FB_OTFREE1,          // output tile's copies have read it            (1)
        FB_XFULL0, FB_XFULL1,            // feed-through tile landed in the output tile  (1 + bytes)
        FB_CUT0,                         // [8] a chunk of a cut tile is prepared        (1)
-       FB_DRAIN = FB_CUT0 + 8, FB_COUNT };
+       FB_TAIL = FB_CUT0 + 8,           // the last tile's rows of v behind the end are zeros (1; tiles of one chunk)
+       FB_DRAIN, FB_COUNT };
 static_assert(FB_COUNT <= 48, "barrier count");
 
 struct PassDesc {
   long long row;       // first row of the tile in v, o
   long long rowq;      // the same in q, k, x, y
   int lo, hi;          // rows of the chunk within the tile
-  int flags;           // kLastPass, kCutTile
-  int pad;
+  int flags;           // kLastPass, kCutTile, kTail
+  int nr;              // rows of the tile
 };
-constexpr int kLastPass = 1, kCutTile = 2;
+constexpr int kLastPass = 1, kCutTile = 2, kTail = 4;   // kTail: rows of another sequence follow
 struct ScanCtl {
   uint32_t tmem_base;
   int pad;
@@ -392,7 +397,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
   int n = sh / a.H;
   const int hq = a.gate_heads == 1 ? 0 : h;
   long long row0, rowq0;
-  int len;
+  int len, vrow0, vhead;       // (vhead, vrow0): first row as the maps of v and beta_hat count
   long long slot0;
   if (a.cu) {
     // (The plan ended before the operand kernel began.  A cu_seqlens that it has refused may leave blocks
@@ -404,17 +409,22 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     seq_range(a.cu, n, a.T, lo, hi);
     len = refused ? 0 : hi - lo;
     row0 = (long long)h * a.T + lo;
+    vhead = h;
+    vrow0 = lo;
     rowq0 = (long long)hq * a.T + lo;
     slot0 = (long long)hq * a.slots_per_head + lo / kTile + n;
   } else {
     len = a.T;
-    row0 = ((long long)n * a.H + h) * a.T;
+    vhead = sh;
+    vrow0 = 0;
+    row0 = (long long)sh * a.T;
     rowq0 = ((long long)n * a.gate_heads + hq) * a.T;
     slot0 = ((long long)n * a.gate_heads + hq) * a.slots_per_head;
     if constexpr (SPLIT) {
       const int t0 = seg == 0 ? 0 : a.seg_tiles0 + (seg - 1) * a.seg_tiles;
       len = min(a.T, (a.seg_tiles0 + seg * a.seg_tiles) * kTile) - t0 * kTile;
       row0 += (long long)t0 * kTile;
+      vrow0 = t0 * kTile;
       rowq0 += (long long)t0 * kTile;
       slot0 += t0;
     }
@@ -505,18 +515,20 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
           d->rowq = rowq0 + (long long)t * kTile;
           d->lo = lo;
           d->hi = hi;
-          d->flags = (t + 1 == ntiles && hi == nr ? kLastPass : 0) | (mask != 1ull ? kCutTile : 0);
+          d->flags = (t + 1 == ntiles && hi == nr ? kLastPass : 0) | (mask != 1ull ? kCutTile : 0) | (a.cu && nr < kTile ? kTail : 0);
+          d->nr = nr;
           const uint32_t st = base + s * C::kAStage, fb = bar(FB_AFULL0 + s);
           const bool beta = BLOCK && a.has_beta;
           const int a_bytes = only ? B::kP : C::kABytes;       // (Kt alone)
           mbar_expect_tx(fb, a_bytes + 2 * kSlab + (beta ? 2 * kSlab : 0));
-          tma_load_3d(st + C::kOffV, &maps.v, 0, (int)row, col0 >> 6, fb);
-          if (beta) tma_load_3d(st + C::kOffBeta, &maps.beta, 0, (int)row, col0 >> 6, fb);
+          const int vrow = vrow0 + t * kTile;
+          tma_load_4d(st + C::kOffV, &maps.v, 0, vrow, col0 >> 6, vhead, fb);
+          if (beta) tma_load_4d(st + C::kOffBeta, &maps.beta, 0, vrow, col0 >> 6, vhead, fb);
           bulk_load(st, blk + (long long)t * B::kBytes, a_bytes, fb);
           ctl->n_a = pass + 1;
           if (lo == 0 && t + C::kAStages < ntiles) {   // asked into L2 before its stage is free
-            tma_prefetch_3d(&maps.v, 0, (int)row + C::kAStages * kTile, col0 >> 6);
-            if (beta) tma_prefetch_3d(&maps.beta, 0, (int)row + C::kAStages * kTile, col0 >> 6);
+            tma_prefetch_4d(&maps.v, 0, vrow + C::kAStages * kTile, col0 >> 6, vhead);
+            if (beta) tma_prefetch_4d(&maps.beta, 0, vrow + C::kAStages * kTile, col0 >> 6, vhead);
             if (BLOCK && a.feed_d && !only) tma_prefetch_3d(&maps.fx, 0, (int)row + C::kAStages * kTile, col0 >> 6);
           }
           if (++s == C::kAStages) { s = 0; ph ^= 1; }
@@ -548,6 +560,8 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
         if (flags & kCutTile) {
           if (!mbar_wait(bar(FB_CUT0 + (n_cut & 7)), (n_cut >> 3) & 1, wc, hdr)) break;
           ++n_cut;
+        } else if ((flags & kTail) && !(BLOCK && a.has_beta)) {
+          if (!mbar_wait(bar(FB_TAIL), 0, wc, hdr)) break;
         }
         const uint32_t st = base + s * C::kAStage, sq = base + C::kOffQ + qs * C::kQBytes;
         const uint32_t dv = desc_lo_mnmajor(st + C::kOffV, kSlab);
@@ -667,7 +681,7 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
       if (feed) fetch_x(c + 2);
     }
   } else if (warp == 3) {
-    // ================================= chunks of cut tiles =================================
+    // ======================= chunks of cut tiles, rows behind the end ======================
     // rows of other chunks contribute nothing to a chunk's update; the chunk's decays come from the
     // same additions as its operands'
     uint32_t s = 0, ph = 0;
@@ -676,6 +690,17 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
       if (!wait_all(FB_AFULL0 + s, ph)) break;
       const volatile PassDesc* d = &ctl->desc[c & 7];
       const int lo = d->lo, hi = d->hi, flags = d->flags;
+      if ((flags & kTail) && !(BLOCK && a.has_beta)) {
+        const uint32_t v = base + s * C::kAStage + C::kOffV;
+#pragma unroll 4
+        for (int at = d->nr * 128 + lane * 16; at < kSlab; at += 512) {
+          sts128(v + at, 0u, 0u, 0u, 0u);
+          sts128(v + kSlab + at, 0u, 0u, 0u, 0u);
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0 && !(flags & kCutTile)) mbar_arrive(bar(FB_TAIL));
+      }
       if (flags & kCutTile) {
         const uint32_t k = base + s * C::kAStage + B::kK;
         for (int e = lane; e < B::kKp * B::kSlabs * kTile * 8; e += 32) {
@@ -904,13 +929,23 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     uint32_t s = 0, ph = 0;
     for (int c = 0; a.has_beta && ntiles > 0; ++c) {
       if (!wait_all(FB_AFULL0 + s, ph)) break;
-      const bool last = (ctl->desc[c & 7].flags & kLastPass) != 0;
+      const int flags = ctl->desc[c & 7].flags;
+      const bool last = (flags & kLastPass) != 0;
       const uint32_t st = base + s * C::kAStage + C::kOffV + (tid - 512) * 16;
 #pragma unroll 4
       for (int u = 0; u < 2 * kSlab / (128 * 16); ++u) {
         const uint32_t at = st + u * 128 * 16;
         const uint4 v = lds128(at), g = lds128(at + (C::kOffBeta - C::kOffV));
         sts128(at, hmul2_bf16(v.x, g.x), hmul2_bf16(v.y, g.y), hmul2_bf16(v.z, g.z), hmul2_bf16(v.w, g.w));
+      }
+      if (flags & kTail) {                               // rows behind the end, each thread those of its pieces
+        const int nr = ctl->desc[c & 7].nr;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (((tid - 512) >> 3) + 16 * u >= nr) {
+            sts128(st + u * 128 * 16, 0u, 0u, 0u, 0u);
+            sts128(st + kSlab + u * 128 * 16, 0u, 0u, 0u, 0u);
+          }
       }
       fence_proxy_async();
       __syncwarp();
@@ -1225,11 +1260,12 @@ cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
   ScanMaps m;
   const uint64_t rows = (uint64_t)p.B * p.H * p.T, dv = (uint64_t)p.dv;
   if (rows > 0) {
-    if (!encode_bf16_slab_map(&m.v, p.v, rows, dv, 2) || !encode_bf16_slab_map(&m.o, p.o, rows, dv, 2) ||
+    const uint64_t heads = (uint64_t)p.B * p.H, T = (uint64_t)p.T;
+    if (!encode_bf16_heads_map(&m.v, p.v, heads, T, dv, kTile, 2) || !encode_bf16_slab_map(&m.o, p.o, rows, dv, 2) ||
         !encode_bf16_map(&m.o8, p.o, rows, dv, 8) || !encode_bf16_map(&m.o1, p.o, rows, dv, 1))
       return cudaErrorInvalidValue;
     m.beta = m.fx = m.v;
-    if (p.beta_hat && !encode_bf16_slab_map(&m.beta, p.beta_hat, rows, dv, 2)) return cudaErrorInvalidValue;
+    if (p.beta_hat && !encode_bf16_heads_map(&m.beta, p.beta_hat, heads, T, dv, kTile, 2)) return cudaErrorInvalidValue;
     if (p.feed_x && !encode_bf16_slab_map(&m.fx, p.feed_x, rows, dv, 2)) return cudaErrorInvalidValue;
   } else {
     memset(&m, 0, sizeof(m));   // never used: no tiles

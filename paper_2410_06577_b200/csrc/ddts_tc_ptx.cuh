@@ -14,9 +14,10 @@ bool encode_bf16_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t co
 // The same matrix seen as [cols / 64][rows][64]: one box of [slabs][64][64] is `slabs` consecutive
 // 64-column tiles of 64 rows, 8 KiB each, brought by ONE copy.
 bool encode_bf16_slab_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t slabs);
-// A [heads][rows][128] array, dimensions (64, rows, 2, heads): one box is box_rows rows of one head as `slabs`
+// A [heads][rows][cols] array, dimensions (64, rows, cols / 64, heads): one box is box_rows rows of one head as `slabs`
 // 64-column tiles; rows past the end of a head read as zeros and are not written.
-bool encode_bf16_heads_map(CUtensorMap* m, const void* ptr, uint64_t heads, uint64_t rows, uint32_t box_rows, uint32_t slabs);
+bool encode_bf16_heads_map(CUtensorMap* m, const void* ptr, uint64_t heads, uint64_t rows, uint64_t cols, uint32_t box_rows,
+                           uint32_t slabs);
 
 namespace {
 
@@ -166,6 +167,10 @@ __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_grou
 __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
   asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
                ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int x, int y, int z, int w) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];"
+               ::"l"(map), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
 }
 // Ask for a 2-D tile to be brought into L2 (no shared-memory destination, nothing to wait for).
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {

@@ -505,8 +505,8 @@ cudaError_t launch_swska_tc(const rodimus_swska_fwd_params& p, int* n_launches) 
   SwMapCache& c = t_sw_maps;
   if (c.q != p.q || c.k != p.k || c.v != p.v || c.o != p.o || c.B != p.B || c.H != p.H || c.T != p.T) {
     c.q = nullptr;
-    if (!encode_bf16_heads_map(&c.mq, p.q, bh, T, kBM, 2) || !encode_bf16_heads_map(&c.mk, p.k, (uint64_t)p.B, T, kBN, 2) ||
-        !encode_bf16_heads_map(&c.mv, p.v, bh, T, kBN, 2) || !encode_bf16_heads_map(&c.mo, p.o, bh, T, 32, 1))
+    if (!encode_bf16_heads_map(&c.mq, p.q, bh, T, kD, kBM, 2) || !encode_bf16_heads_map(&c.mk, p.k, (uint64_t)p.B, T, kD, kBN, 2) ||
+        !encode_bf16_heads_map(&c.mv, p.v, bh, T, kD, kBN, 2) || !encode_bf16_heads_map(&c.mo, p.o, bh, T, kD, 32, 1))
       return cudaErrorInvalidValue;
     c.q = p.q; c.k = p.k; c.v = p.v; c.o = p.o; c.B = p.B; c.H = p.H; c.T = p.T;
   }

@@ -1255,6 +1255,62 @@ def test_prefill_split_along_time_back_to_back_on_one_workspace():
         assert rel_err(host(o), ro) <= TOL_BF16 and rel_err(host(sT), rs) <= TOL_BF16
 
 
+def _check_neighbours_stay_out(bad, B, H, T, dk, dv, terms=(), packed=None, least=False, launches=None, gate_mean=-3.0,
+                               value=float("nan")):
+    """The first rows of every head but the first (packed: of every sequence but the first) get NaN or infinities in
+    the inputs `bad`; what is computed from the rows before them stays bit for bit what it was."""
+    import torch
+    cu = None if packed is None else np.concatenate([[0], np.cumsum(packed)]).astype(np.int32)
+    p = wl.make_prefill(1030, B, H, T if cu is None else int(cu[-1]), dk, dv, "bf16", s0_std=0.2, gate_mean=gate_mean, cu_seqlens=cu)
+    d = prefill_to_device(p)
+    rng = torch.Generator(device="cuda").manual_seed(7)
+    noise = lambda like: torch.randn(like.shape, generator=rng, device="cuda").to(like.dtype)
+    kw = {}
+    if "gate" in terms: kw["beta_hat"] = torch.sigmoid(noise(d["v"]))
+    if "feed" in terms: kw.update(feed_d=noise(d["v"][0, :, 0].float()), feed_x=noise(d["v"]))
+    got = []
+    for spoilt in (False, True):
+        for name in bad if spoilt else ():
+            t = kw[name] if name in kw else d[name]
+            if cu is None: t[:, 1:, :3] = value
+            else: t[:, :, int(cu[1]):int(cu[1]) + 3] = value
+        o, sT = _nan_outputs(d)
+        prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT, d["cu"], d["cu_host"], **kw)
+        need = 256 if cu is None else 512
+        ws = torch.empty(need if least else max(need, rd.fwd_workspace_bytes(prm)), dtype=torch.uint8, device="cuda")
+        prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
+        assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
+        assert launches is None or rd.last_launch_count() == launches
+        got.append((o[:, 0], sT[:, 0]) if cu is None else (o[:, :, :int(cu[1])], sT[0]))
+    (o, sT), (o1, sT1) = got
+    assert torch.isfinite(o).all() and torch.equal(o, o1) and torch.isfinite(sT).all() and torch.equal(sT, sT1)
+
+
+@pytest.mark.parametrize("bad", [("v",), ("q", "k", "x", "y")])
+@pytest.mark.parametrize("B,H,T,dk,dv,packed,launches,gate_mean", [
+    (2, 2, 200, 128, 256, None, 2, -3.0),          # the last tile is ragged
+    (1, 3, 63, 128, 256, None, 2, -3.0),           # the only tile is
+    (1, 2, 200, 128, 256, None, 2, 1.5),           # it is cut into chunks
+    (1, 4, 0, 128, 256, (300, 250, 270), 3, -3.0),
+    (1, 4, 600, 128, 128, None, 2, -3.0),
+    (1, 3, 65, 64, 128, None, 2, -3.0),
+    (1, 3, 0, 64, 256, (1, 99, 64), 3, -3.0),
+    (1, 2, 200, 64, 128, None, 2, 2.0),
+    (1, 8, 8250, 128, 256, None, 4, -3.0),         # split along time
+])
+def test_prefill_operands_first_neighbours_nan_stays_out(bad, B, H, T, dk, dv, packed, launches, gate_mean):
+    _check_neighbours_stay_out(bad, B, H, T, dk, dv, packed=packed, launches=launches, gate_mean=gate_mean)
+
+
+@pytest.mark.parametrize("terms", [("gate",), ("feed",), ("gate", "feed")])
+@pytest.mark.parametrize("T,packed,gate_mean", [(200, None, -3.0), (200, None, 1.5), (40, None, -3.0), (0, (300, 250, 270), -3.0)])
+def test_prefill_operands_first_block_terms_neighbours_nan_stays_out(terms, T, packed, gate_mean):
+    bad = ("v",) + (("beta_hat",) if "gate" in terms else ()) + (("feed_x",) if "feed" in terms else ())
+    for value in (float("nan"), float("inf")):
+        _check_neighbours_stay_out(bad, 1, 4, T, 128, 256, terms, packed, gate_mean=gate_mean, launches=3 if packed else 2,
+                                   value=value)
+
+
 @pytest.mark.parametrize("dk", [64, 128])
 def test_two_launch_prefill_dense_without_tokens(dk):
     import torch
