@@ -288,9 +288,11 @@ __device__ __forceinline__ float2 gate_phase1(uint32_t xs, uint32_t ys, const ui
 }
 
 // Phase 2: Qt = q 2^{b}, Kt = k 2^{eh - b}, written over q and k (same swizzled offsets).
+// Rows past the pass become zero, in the two slabs of v too: they may be another sequence's, whose NaN or infinity
+// the zeros of Qt and Kt alone would not keep out.
 // STATE_ONLY: the pass only updates the state, so Qt is not needed.
 template <bool STATE_ONLY>
-__device__ __forceinline__ void gate_phase2(uint32_t qs, uint32_t ks, const uint32_t (&off)[kGR],
+__device__ __forceinline__ void gate_phase2(uint32_t qs, uint32_t ks, uint32_t vs, const uint32_t (&off)[kGR],
                                             int row0, int nr, float2 pre, const float2 (&b)[kGR],
                                             const float2 (&eh)[kGR]) {
 #pragma unroll
@@ -313,6 +315,8 @@ __device__ __forceinline__ void gate_phase2(uint32_t qs, uint32_t ks, const uint
     for (int i = 0; i < kGR; ++i) {
       if (row0 + i >= nr) {
         sts32(ks + off[i], 0u);
+        sts32(vs + off[i], 0u);
+        sts32(vs + kSlabBytes + off[i], 0u);
         if (!STATE_ONLY) sts32(qs + off[i], 0u);
       }
     }
@@ -1031,7 +1035,7 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
               }
             }
           }
-          gate_phase2<STATE_ONLY>(st + kStQ, st + kStK, off, gw * kGR, nr, pre, b, eh);
+          gate_phase2<STATE_ONLY>(st + kStQ, st + kStK, st + kStV, off, gw * kGR, nr, pre, b, eh);
         }
         // the rewritten rows are visible to the bulk-copy engine and to the tensor core; the
         // control warp sends the whole slabs to the partner once every gate warp has said so

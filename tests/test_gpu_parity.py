@@ -1311,6 +1311,22 @@ def test_prefill_operands_first_block_terms_neighbours_nan_stays_out(terms, T, p
                                    value=value)
 
 
+@pytest.mark.parametrize("bad", [("v",), ("q", "k", "x", "y")])
+@pytest.mark.parametrize("B,H,T,dv,packed,gate_mean", [(2, 2, 200, 256, None, -3.0), (1, 3, 1, 512, None, -3.0), (1, 2, 190, 256, None, 1.5),
+                                                       (1, 4, 0, 256, (100, 40, 60), -3.0), (1, 3, 0, 256, (63, 1, 64), 1.5)])
+def test_prefill_pair_kernel_neighbours_nan_stays_out(bad, B, H, T, dv, packed, gate_mean):
+    _check_neighbours_stay_out(bad, B, H, T, 128, dv, packed=packed, least=True, launches=2 if packed else 1, gate_mean=gate_mean)
+
+
+@pytest.mark.parametrize("terms", [("gate",), ("feed",), ("gate", "feed")])
+@pytest.mark.parametrize("T,packed,gate_mean", [(200, None, -3.0), (200, None, 1.5), (0, (100, 40, 60), -3.0)])
+def test_prefill_pair_kernel_block_terms_neighbours_nan_stays_out(terms, T, packed, gate_mean):
+    bad = ("v",) + (("beta_hat",) if "gate" in terms else ()) + (("feed_x",) if "feed" in terms else ())
+    for value in (float("nan"), float("inf")):
+        _check_neighbours_stay_out(bad, 1, 4, T, 128, 256, terms, packed, least=True, launches=2 if packed else 1, gate_mean=gate_mean,
+                                   value=value)
+
+
 @pytest.mark.parametrize("dk", [64, 128])
 def test_two_launch_prefill_dense_without_tokens(dk):
     import torch
