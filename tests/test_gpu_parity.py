@@ -1327,6 +1327,13 @@ def test_prefill_pair_kernel_block_terms_neighbours_nan_stays_out(terms, T, pack
                                    value=value)
 
 
+@pytest.mark.parametrize("bad", [("v",), ("q", "k", "x", "y")])
+@pytest.mark.parametrize("B,H,T,dv,packed,gate_mean", [(2, 2, 200, 128, None, -3.0), (1, 3, 1, 384, None, -3.0), (1, 2, 190, 128, None, 1.5),
+                                                       (1, 4, 0, 128, (100, 40, 60), -3.0), (1, 3, 0, 128, (63, 1, 64), 1.5)])
+def test_prefill_single_cta_kernel_neighbours_nan_stays_out(bad, B, H, T, dv, packed, gate_mean):
+    _check_neighbours_stay_out(bad, B, H, T, 128, dv, packed=packed, least=True, launches=2 if packed else 1, gate_mean=gate_mean)
+
+
 @pytest.mark.parametrize("dk", [64, 128])
 def test_two_launch_prefill_dense_without_tokens(dk):
     import torch
