@@ -942,10 +942,18 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
         tmem_st32(t_st + 32 * piece, r);
       }
       if (nr < kTile) {
-        // a short chunk: the rows past it belong to other chunks; with P's rows zero they contribute nothing
-        if (!(ok = wait_all(bar(SB_FP), c & 1))) break;
-        for (int e = rt; e < (kTile - nr) * 32; e += 256)
-          sts128(base + kOffP + (e & 3) * kSlab + (nr + (e >> 5)) * 128 + ((e >> 2) & 7) * 16, 0u, 0u, 0u, 0u);
+        // a short chunk: the rows past it belong to other chunks, or to another sequence.  With those of P and X zero
+        // they contribute nothing, whatever they hold (of P alone: a NaN or an infinity would not vanish).
+        if (!(ok = wait_all(bar(SB_FP), c & 1) && wait_all(bar(SB_FX), c & 1))) break;
+        const uint32_t at = base + ((rt >> 3) & 3) * kSlab + (rt & 7) * 16;   // (a warp's row: 8 x 16 bytes of 4 slabs)
+#pragma unroll
+        for (int u = 0; u < kTile / 8; ++u) {
+          const int r = nr + (rt >> 5) + 8 * u;
+          if (r < kTile) {
+            sts128(at + kOffP + r * 128, 0u, 0u, 0u, 0u);
+            sts128(at + kOffX + r * 128, 0u, 0u, 0u, 0u);
+          }
+        }
         fence_proxy_async();
       }
       tmem_st_wait();

@@ -240,3 +240,31 @@ def test_bwd_bf16_more_packed_sequences_than_a_block_has_threads(N):
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
     _check(wl.make_prefill(1300 + N, 1, 1, int(cu[-1]), 128, 256, "bf16", s0_std=0.1, cu_seqlens=cu, name=f"bwd_many_{N}"),
            1301, True)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("bad", [("v",), ("d_o",), ("q", "k", "x", "y")])
+@pytest.mark.parametrize("B,H,T,packed,gate_mean", [(2, 2, 200, None, -3.0), (1, 3, 63, None, -3.0), (1, 2, 200, None, 1.5),
+                                                    (1, 40, 130, None, -3.0), (1, 3, 0, (100, 40, 60), -3.0),
+                                                    (1, 2, 0, (65, 1, 64), 1.5)])
+def test_bwd_neighbours_nan_stays_out(value, bad, B, H, T, packed, gate_mean):
+    """The first rows of every head but the first (packed: of every sequence but the first) get NaN or infinities;
+    gradients of what lies before them stay bit for bit what they were.  Tiles whole and cut into chunks, sweeps
+    whole and cut in two."""
+    import torch
+    cu = None if packed is None else np.concatenate([[0], np.cumsum(packed)]).astype(np.int32)
+    p = wl.make_prefill(1400, B, H, T if cu is None else int(cu[-1]), 128, 256, "bf16", gate_mean=gate_mean, s0_std=0.2, cu_seqlens=cu)
+    g_o, g_s = wl.make_grads(1401, p, True)
+    d = prefill_to_device(p)
+    d["d_o"] = dev(g_o, p.dtype)
+    got = []
+    for spoilt in (False, True):
+        for name in bad if spoilt else ():
+            if cu is None: d[name][:, 1:, :3] = value
+            else: d[name][:, :, int(cu[1]):int(cu[1]) + 3] = value
+        g = rd.ddts_bwd(*(d[n] for n in ("q", "k", "x", "y", "v", "d_o")), d["s0"], torch.from_numpy(g_s).cuda(), cu_seqlens=d["cu"],
+                        want_d_s0=True)
+        if cu is None: got.append([t[:, 0] for t in g.values()])
+        else: got.append([g["d_s0"][0]] + [t[:, :, :int(cu[1])] for n, t in g.items() if n != "d_s0"])
+    for clean, spoilt in zip(*got):
+        assert torch.isfinite(clean).all() and torch.equal(clean, spoilt)
