@@ -60,6 +60,20 @@ def test_swska_many_items_a_cta_match_oracle(B, H, T, window):
         assert rel_err(got[b:b + 1, h:h + 1], ref) <= TOL_BF16
 
 
+@pytest.mark.parametrize("T,window", [(1, 1), (64, 64), (65, 30), (128, 200), (129, 64), (192, 70), (200, 256), (333, 64), (777, 1000)])
+def test_swska_few_items_agree_with_many(T, window):
+    """Calls whose items are all alone on their CTAs end without asking for another one and store their rows
+    without waiting for a copy; a head's output is the same bits as in a call in which CTAs take several."""
+    import torch
+    H, few = 2400 // ((T + 127) // 128) // 3, 3
+    q, k, v = (dev(a, "bf16") for a in wl.make_swska(995, 3, H, T, 128, "bf16"))
+    many = rd.swska_fwd(q, k, v, window)
+    alone = rd.swska_fwd(q[:, :few].contiguous(), k, v[:, :few].contiguous(), window)
+    assert torch.equal(many[:, :few], alone)
+    ref = sw.swska_ref(host(q[:1, :1]), host(k[:1]), host(v[:1, :1]), window, 128 ** -0.5)
+    assert rel_err(host(alone[:1, :1]), ref) <= TOL_BF16
+
+
 def test_swska_many_items_with_rising_scores():
     """Scores whose maximum rises from key tile to key tile: references move, outputs are rescaled, and start
     afresh with the next item."""
