@@ -171,6 +171,10 @@ typedef struct {
  * a kernel that needs no more. */
 size_t rodimus_ddts_fwd_workspace_bytes(const rodimus_ddts_fwd_params *p);
 
+/* The largest size under `limit` bytes that the call has a use for, down to the least it runs with
+ * (returned also where that is not under `limit`): what to ask for when more does not fit. */
+size_t rodimus_ddts_fwd_workspace_bytes_below(const rodimus_ddts_fwd_params *p, size_t limit);
+
 /* Chunked prefill; see rodimus_ddts_fwd_params. */
 int rodimus_ddts_fwd(const rodimus_ddts_fwd_params *p);
 

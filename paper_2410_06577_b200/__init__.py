@@ -26,6 +26,7 @@ EXPORTED_SYMBOLS = (
     "rodimus_ddts_fwd_kernel_name", "rodimus_status_str", "rodimus_version",
     "rodimus_ddts_fwd_noalloc", "rodimus_ddts_sfu_probe", "rodimus_ddts_test_set_wait_limit",
     "rodimus_ddts_bwd_workspace_bytes", "rodimus_ddts_bwd", "rodimus_swska_fwd",
+    "rodimus_ddts_fwd_workspace_bytes_below",
 )
 NOALLOC_MAX_SEQS = 4096
 
@@ -114,6 +115,8 @@ def load_library() -> ctypes.CDLL:
         lib = ctypes.CDLL(LIB_PATH)
         lib.rodimus_ddts_fwd_workspace_bytes.argtypes = [ctypes.POINTER(FwdParams)]
         lib.rodimus_ddts_fwd_workspace_bytes.restype = ctypes.c_size_t
+        lib.rodimus_ddts_fwd_workspace_bytes_below.argtypes = [ctypes.POINTER(FwdParams), ctypes.c_size_t]
+        lib.rodimus_ddts_fwd_workspace_bytes_below.restype = ctypes.c_size_t
         lib.rodimus_ddts_fwd.argtypes = [ctypes.POINTER(FwdParams)]
         lib.rodimus_ddts_fwd.restype = ctypes.c_int
         lib.rodimus_ddts_fwd_noalloc.argtypes = [ctypes.POINTER(FwdParams),
@@ -156,7 +159,8 @@ def _native():
         addr = lambda f: ctypes.cast(f, ctypes.c_void_p).value
         _binding.bind(addr(lib.rodimus_ddts_fwd), addr(lib.rodimus_ddts_fwd_workspace_bytes),
                       addr(lib.rodimus_ddts_step), addr(lib.rodimus_ddts_bwd),
-                      addr(lib.rodimus_ddts_bwd_workspace_bytes), addr(lib.rodimus_swska_fwd))
+                      addr(lib.rodimus_ddts_bwd_workspace_bytes), addr(lib.rodimus_swska_fwd),
+                      addr(lib.rodimus_ddts_fwd_workspace_bytes_below))
         _module, _bound = _binding, lib
     return _module
 
@@ -214,7 +218,10 @@ def fwd_params(q, k, gate_x, temp_y, v, o, s0=None, sT=None, cu_seqlens=None,
     return p
 
 
-def fwd_workspace_bytes(p: FwdParams) -> int:
+def fwd_workspace_bytes(p: FwdParams, below: Optional[int] = None) -> int:
+    """Workspace that makes the call fastest; with ``below``, the largest size under it that the call has a use for."""
+    if below is not None:
+        return int(load_library().rodimus_ddts_fwd_workspace_bytes_below(ctypes.byref(p), below))
     return int(load_library().rodimus_ddts_fwd_workspace_bytes(ctypes.byref(p)))
 
 

@@ -18,6 +18,7 @@ namespace {
 
 decltype(&rodimus_ddts_fwd) g_fwd = nullptr;
 decltype(&rodimus_ddts_fwd_workspace_bytes) g_fwd_ws = nullptr;
+decltype(&rodimus_ddts_fwd_workspace_bytes_below) g_fwd_ws_below = nullptr;
 decltype(&rodimus_ddts_step) g_step = nullptr;
 decltype(&rodimus_ddts_bwd) g_bwd = nullptr;
 decltype(&rodimus_ddts_bwd_workspace_bytes) g_bwd_ws = nullptr;
@@ -66,15 +67,17 @@ at::Tensor bytes_like(const at::Tensor& q, size_t n) {
   return at::empty({(int64_t)(n < 256 ? 256 : n)}, q.options().dtype(at::kByte));
 }
 // The prefill's workspace: what makes it fastest or, where that does not fit into the device's memory (it may
-// be as large as the inputs), the least that every request runs with.
-at::Tensor fwd_workspace(const at::Tensor& q, size_t wanted, int32_t n_seq) {
-  const size_t least = 256 + (((size_t)(n_seq > 0 ? n_seq : 0) * 4 + 255) & ~(size_t)255);
-  try {
-    return bytes_like(q, wanted);
-  } catch (const c10::OutOfMemoryError&) {
-    if (wanted <= least) throw;
+// be as large as the inputs), the next smaller size that it has a use for, down to the least it runs with.
+at::Tensor fwd_workspace(const at::Tensor& q, const rodimus_ddts_fwd_params& p) {
+  for (size_t n = g_fwd_ws(&p);;) {
+    try {
+      return bytes_like(q, n);
+    } catch (const c10::OutOfMemoryError&) {
+      const size_t less = g_fwd_ws_below(&p, n);
+      if (less >= n) throw;
+      n = less;
+    }
   }
-  return bytes_like(q, least);
 }
 PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
 
@@ -138,7 +141,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   p.beta_hat = beta.ptr(); p.feed_d = (const float*)fd.ptr(); p.feed_x = fx.ptr();
   p.value_decay = vd.ptr();
   p.stream = current_stream();
-  at::Tensor w = ws.t ? *ws.t : fwd_workspace(*q.t, g_fwd_ws(&p), p.N);
+  at::Tensor w = ws.t ? *ws.t : fwd_workspace(*q.t, p);
   p.workspace = w.data_ptr();
   p.workspace_bytes = (size_t)w.numel() * w.element_size();
   const int rc = g_fwd(&p);
@@ -274,11 +277,12 @@ PyObject* swska(PyObject*, PyObject* const* a, Py_ssize_t n) {
   RODIMUS_CATCH
 }
 
-// bind(addresses of rodimus_ddts_fwd, _fwd_workspace_bytes, _step, _bwd, _bwd_workspace_bytes, rodimus_swska_fwd)
+// bind(addresses of rodimus_ddts_fwd, _fwd_workspace_bytes, _step, _bwd, _bwd_workspace_bytes, rodimus_swska_fwd,
+//      rodimus_ddts_fwd_workspace_bytes_below)
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  if (n != 6) return PyErr_Format(PyExc_TypeError, "6 arguments expected");
-  void* f[6];
-  for (int i = 0; i < 6; ++i) {
+  if (n != 7) return PyErr_Format(PyExc_TypeError, "7 arguments expected");
+  void* f[7];
+  for (int i = 0; i < 7; ++i) {
     f[i] = PyLong_AsVoidPtr(a[i]);
     if (PyErr_Occurred()) return nullptr;
   }
@@ -288,6 +292,7 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
   g_bwd = (decltype(g_bwd))f[3];
   g_bwd_ws = (decltype(g_bwd_ws))f[4];
   g_swska = (decltype(g_swska))f[5];
+  g_fwd_ws_below = (decltype(g_fwd_ws_below))f[6];
   Py_RETURN_NONE;
 }
 

@@ -74,9 +74,10 @@ cudaError_t launch_swska(const rodimus_swska_fwd_params& p, int* n_launches);
 cudaError_t launch_swska_tc(const rodimus_swska_fwd_params& p, int* n_launches);   // bf16, tcgen05
 bool swska_supported(const rodimus_swska_fwd_params& p);
 cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches);
-// Workspace with which the two-launch prefill (operands, scan) takes this request; 0: it does not.
+// Workspace with which the prefill that forms operands first takes this request, in two launches or split along
+// time in four; 0: it does not.
 size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p);
-bool fwd_scan_split(const rodimus_ddts_fwd_params& p);   // it would split this dense call along time
+size_t fwd_scan_split_workspace_bytes(const rodimus_ddts_fwd_params& p);
 bool fwd_tc_supported(const rodimus_ddts_fwd_params& p);
 bool fwd_pair_supported(const rodimus_ddts_fwd_params& p);
 // Workspace a dense call needs if its sequences are to be split along time (0: no split).

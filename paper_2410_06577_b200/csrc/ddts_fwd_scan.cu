@@ -1077,7 +1077,7 @@ struct ScanPlan {
   size_t blocks, masks, seg_state, seg_decay, bytes;   // workspace: offsets of the blocks, masks, segments' states and decays; total
 };
 
-ScanPlan scan_plan(const rodimus_ddts_fwd_params& p, int sms) {
+ScanPlan scan_plan(const rodimus_ddts_fwd_params& p, const Segments& seg) {
   ScanPlan s;
   const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
   s.gate_heads = p.shared_gates ? 1 : p.H;
@@ -1088,7 +1088,7 @@ ScanPlan scan_plan(const rodimus_ddts_fwd_params& p, int sms) {
   s.bytes = s.blocks + (p.dk == 64 ? blocks_bytes<64>(s.slots) : blocks_bytes<128>(s.slots));
   s.masks = s.bytes;
   s.bytes += ((size_t)s.slots * sizeof(unsigned long long) + 255) & ~(size_t)255;
-  s.seg = plan_segments(p, sms);
+  s.seg = seg;
   s.seg_state = s.bytes;
   const size_t per = (size_t)p.B * p.H * p.dk * sizeof(float);
   s.seg_decay = s.seg_state + (size_t)s.seg.G * per * p.dv;
@@ -1150,7 +1150,16 @@ bool scan_pays_with_shared_gates(long long n_seq, double tiles, double slabs, bo
 }
 }  // namespace
 
-// Which requests this file's kernels compute, given room for the tiles' blocks; bytes of that room
+namespace {
+// What the kernels of this file can compute at all.
+bool scan_supported(const rodimus_ddts_fwd_params& p) {
+  if (p.dtype != RODIMUS_BF16 || p.value_decay || p.dv % 128) return false;
+  const bool block = p.beta_hat || p.feed_d;
+  return p.dk == 64 ? !block : p.dk == 128 && (p.dv % 256 == 0 || (!block && !p.shared_gates));
+}
+}  // namespace
+
+// Which requests this file's kernels compute unsplit, given room for the tiles' blocks; bytes of that room
 // (0: not this path).  All timings are one call, the other kernel against this path.
 //   dk = 64            always (B=4 H=16 T=2048, one set of gates: fp32 CUDA-core kernel 3.9 ms, here
 //                      47 us; 20000 sequences of 1 to 8 tokens 29 -> 12 ms); not with block terms, whose
@@ -1179,7 +1188,7 @@ bool scan_pays_with_shared_gates(long long n_seq, double tiles, double slabs, bo
 //                      items of 64..1000 rows 72 -> 60, of 650 62 -> 69, 148 of 650 62 -> 78), more slices,
 //                      up to one for every SM.
 size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
-  if (p.dtype != RODIMUS_BF16 || p.value_decay || p.dv % 128 || (p.dk != 64 && p.dk != 128)) return 0;
+  if (!scan_supported(p)) return 0;
   const bool varlen = p.cu_seqlens || p.cu_seqlens_host;
   const bool block = p.beta_hat || p.feed_d, whole = p.dv % 256 == 0;
   const long long n_seq = varlen ? p.N : p.B, sets = n_seq * p.H, items = sets * (p.dv / 128);
@@ -1188,15 +1197,11 @@ size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
     cudaGetLastError();
     sms = 0;
   }
-  if (p.dk == 64) {
-    if (block) return 0;
-  } else {
-    if (sms == 0 || items == 0 || (!whole && (block || p.shared_gates))) return 0;
-  }
-  if (p.dk == 128 && plan_segments(p, sms).G == 0) {
+  if (p.dk == 128) {
+    if (sms == 0 || items == 0) return 0;
     if (p.shared_gates) {
       const double tiles = varlen ? (double)p.T / ((double)n_seq * kTile) + 0.5 : (double)((p.T + kTile - 1) / kTile);
-      if (!whole || !scan_pays_with_shared_gates(n_seq, tiles, p.H * (p.dv / 256.0), varlen, sms)) return 0;
+      if (!scan_pays_with_shared_gates(n_seq, tiles, p.H * (p.dv / 256.0), varlen, sms)) return 0;
     } else {
       if (whole && !varlen) {
         const double fill = (double)items / sms, tiles = (double)((p.T + kTile - 1) / kTile);
@@ -1213,18 +1218,22 @@ size_t fwd_scan_workspace_bytes(const rodimus_ddts_fwd_params& p) {
       }
     }
   }
-  const ScanPlan s = scan_plan(p, sms);
+  const ScanPlan s = scan_plan(p, Segments{});
   if (s.slots > 0x7fffffffLL || items > 0x7fffffffLL) return 0;
   return s.bytes;
 }
 
-bool fwd_scan_split(const rodimus_ddts_fwd_params& p) {
+size_t fwd_scan_split_workspace_bytes(const rodimus_ddts_fwd_params& p) {
+  if (!scan_supported(p)) return 0;
   int dev = 0, sms = 0;
   if (current_device(&dev, &sms) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
-  return plan_segments(p, sms).G > 0;
+  const Segments seg = plan_segments(p, sms);
+  if (seg.G == 0) return 0;
+  const ScanPlan s = scan_plan(p, seg);
+  return s.slots > 0x7fffffffLL ? 0 : s.bytes;
 }
 
 cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
@@ -1232,7 +1241,8 @@ cudaError_t launch_fwd_scan(const rodimus_ddts_fwd_params& p, int* n_launches) {
   int dev = 0, sms = 0;
   cudaError_t e = current_device(&dev, &sms);
   if (e != cudaSuccess) return e;
-  const ScanPlan s = scan_plan(p, sms);
+  ScanPlan s = scan_plan(p, plan_segments(p, sms));
+  if (p.workspace_bytes < s.bytes) s = scan_plan(p, Segments{});   // room for the blocks alone
   const long long n_seq = p.cu_seqlens ? p.N : p.B, items = n_seq * p.H * (p.dv / 128);
   if (items == 0) return cudaSuccess;
   char* ws = reinterpret_cast<char*>(p.workspace);

@@ -69,22 +69,37 @@ bool fwd_pair_selected(const rodimus_ddts_fwd_params& p) { return fwd_pair_suppo
 
 bool has_block_terms(const rodimus_ddts_fwd_params& p) { return p.beta_hat || p.feed_d; }
 
-// Workspace of the prefill that forms operands first where it is to be used; dense calls that only the pair
-// kernel splits along time stay there (their few heads fill the device only that way).
-size_t scan_path_bytes(const rodimus_ddts_fwd_params& p) {
-  const size_t bytes = fwd_scan_workspace_bytes(p);
-  if (bytes > 0 && fwd_pair_selected(p) && fwd_pair_split_workspace_bytes(p) > 0 && !fwd_scan_split(p)) return 0;
-  return bytes;
+// The forms that a request can take with the workspace that each needs, the preferred one first; the last one needs
+// the least that is accepted.
+// 0: cluster-pair tensor-core kernel, 1: single-CTA tensor-core kernel (the recurrence alone),
+// 2: fp32 CUDA-core kernel, 3: operands first, then the scan
+struct FwdForms {
+  int n = 0, kernel[4];
+  size_t bytes[4];
+  void add(int k, size_t b) {
+    kernel[n] = k;
+    bytes[n++] = b;
+  }
+};
+FwdForms fwd_forms(const rodimus_ddts_fwd_params& p) {
+  FwdForms f;
+  const bool pair = fwd_pair_selected(p);
+  const size_t least = workspace_bytes_for(p.cu_seqlens || p.cu_seqlens_host ? p.N : 0);
+  const size_t pair_split = pair ? fwd_pair_split_workspace_bytes(p) : 0;
+  if (const size_t b = fwd_scan_split_workspace_bytes(p)) f.add(3, b);
+  // (few heads of a dense call fill the device only if it is split along time)
+  if (const size_t b = pair_split > 0 ? 0 : fwd_scan_workspace_bytes(p)) f.add(3, b);
+  const int k = pair ? 0 : fwd_tc_supported(p) && !has_block_terms(p) && !p.shared_gates && !p.value_decay ? 1 : 2;
+  if (const size_t b = k == 2 ? fwd_simt_chunks_workspace_bytes(p) : pair_split) f.add(k, b);
+  f.add(k, least);
+  return f;
 }
 
-// 0: cluster-pair tensor-core kernel, 1: single-CTA tensor-core kernel (the recurrence alone),
-// 2: fp32 CUDA-core kernel, 3: operands and scan in two launches (if the workspace has room for it)
 int fwd_kernel_choice(const rodimus_ddts_fwd_params& p) {
-  const size_t scan = scan_path_bytes(p);
-  if (scan > 0 && p.workspace_bytes >= scan) return 3;
-  if (fwd_pair_selected(p)) return 0;
-  if (fwd_tc_supported(p) && !has_block_terms(p) && !p.shared_gates && !p.value_decay) return 1;
-  return 2;
+  const FwdForms f = fwd_forms(p);
+  int i = 0;
+  while (i + 1 < f.n && p.workspace_bytes < f.bytes[i]) ++i;
+  return f.kernel[i];
 }
 
 }  // namespace ddts
@@ -92,16 +107,16 @@ int fwd_kernel_choice(const rodimus_ddts_fwd_params& p) {
 extern "C" {
 
 size_t rodimus_ddts_fwd_workspace_bytes(const rodimus_ddts_fwd_params* p) {
+  return rodimus_ddts_fwd_workspace_bytes_below(p, ~(size_t)0);
+}
+
+size_t rodimus_ddts_fwd_workspace_bytes_below(const rodimus_ddts_fwd_params* p, size_t limit) {
   if (!p) return 0;
-  const bool varlen = p->cu_seqlens != nullptr || p->cu_seqlens_host != nullptr;
-  if (check_fwd_sizes(p, varlen) != RODIMUS_OK) return 0;
-  const size_t base = workspace_bytes_for(varlen ? p->N : 0);
-  // long dense sequences with few heads run faster split along time, given room for the
-  // segments' states; a caller that passes only the base size still gets the unsplit path
-  size_t more = ddts::scan_path_bytes(*p);
-  if (more == 0 && ddts::fwd_pair_selected(*p)) more = ddts::fwd_pair_split_workspace_bytes(*p);
-  if (more == 0 && ddts::fwd_kernel_choice(*p) == 2) more = ddts::fwd_simt_chunks_workspace_bytes(*p);
-  return more > base ? more : base;
+  if (check_fwd_sizes(p, p->cu_seqlens != nullptr || p->cu_seqlens_host != nullptr) != RODIMUS_OK) return 0;
+  const ddts::FwdForms f = ddts::fwd_forms(*p);
+  int i = 0;
+  while (i + 1 < f.n && f.bytes[i] >= limit) ++i;
+  return f.bytes[i];
 }
 
 const char* rodimus_ddts_fwd_kernel_name(const rodimus_ddts_fwd_params* p) {

@@ -1085,6 +1085,65 @@ def test_prefill_whose_workspace_does_not_fit_runs_with_less(packed):
     assert rel_err(host(least), host(o)) <= TOL_BF16
 
 
+@pytest.mark.parametrize("H,T,dk,dv,shared,launches", [
+    (4, 8200, 64, 256, True, [4, 2, 1]),        # split, unsplit, fp32 kernel
+    (8, 4000, 128, 256, False, [4, 2, 1]),      # ..., paired CTAs
+    (4, 4000, 128, 128, False, [4, 2, 1]),      # ..., single CTA
+    (8, 8200, 128, 256, False, [4, 5, 1]),      # split, split by the pair kernel, not split
+    (40, 700, 128, 256, False, [2, 1]),
+    (72, 2048, 128, 256, False, [1]),
+])
+def test_prefill_takes_the_best_form_that_its_workspace_has_room_for(H, T, dk, dv, shared, launches):
+    import torch
+    p = wl.make_prefill(1040, 1, H, T, dk, dv, "bf16", s0_std=0.2)
+    d = prefill_to_device(p)
+    if shared:
+        d.update({n: d[n][:, :1].contiguous() for n in "qkxy"})
+    prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], d["v"], d["s0"], None)
+    size, sizes = rd.fwd_workspace_bytes(prm), []
+    while not sizes or size < sizes[-1]:
+        sizes.append(size)
+        size = rd.fwd_workspace_bytes(prm, below=size)
+    assert sizes[-1] == 256 and len(sizes) == len(launches)
+    first = None
+    for i, n in enumerate(launches):
+        for room in {sizes[i], sizes[i - 1] - 1 if i else sizes[0]}:      # just enough; all but enough for the one before
+            ws = torch.empty(room, dtype=torch.uint8, device="cuda")
+            o, sT = _nan_outputs(dict(d, q=d["v"][..., :1].expand(-1, -1, -1, dk)))
+            prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT)
+            prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
+            assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
+            assert rd.last_launch_count() == n
+            if first is None:
+                first = host(o), host(sT)
+            assert rel_err(host(o), first[0]) <= TOL_BF16 and rel_err(host(sT), first[1]) <= TOL_BF16
+
+
+def test_prefill_without_room_for_the_segments_states_keeps_its_operands():
+    """Room for the blocks of operands but not for the states of the segments as well: the call is not split, and
+    does not fall back to the fp32 kernel."""
+    import torch
+    H, T, dk, dv = 8, 32768, 64, 512                              # blocks 28.6 MiB, states 4 MiB
+    torch.cuda.empty_cache()
+    q, k, x, y = (torch.empty((1, 1, T, dk), dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    v = torch.empty((1, H, T, dv), dtype=torch.bfloat16, device="cuda")
+    for t, mean, std in ((q, 0, 0.125), (k, 0, 0.125), (x, -3, 1), (y, 0, 1), (v, 0, 1)):
+        t.normal_(mean, std)
+    out = torch.empty_like(v)
+    o = rd.ddts_fwd(q, k, x, y, v, want_final_state=False, out=out)[0].cpu()
+    assert rd.last_launch_count() == 4
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (31 << 20)) / total)
+    try:
+        rd.ddts_fwd(q, k, x, y, v, want_final_state=False, out=out)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert rd.last_launch_count() == 2
+    assert rel_err(host(out), host(o)) <= TOL_BF16
+
+
 @pytest.mark.parametrize("dtype,dk,dv", [("bf16", 64, 128), ("f32", 16, 16)])
 @pytest.mark.parametrize("N", [511, 513, 1500, 4200])
 def test_more_packed_sequences_than_a_block_has_threads(dtype, dk, dv, N):
