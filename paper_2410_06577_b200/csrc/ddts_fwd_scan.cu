@@ -35,6 +35,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstring>
 
@@ -854,7 +855,8 @@ ddts_scan_kernel(const __grid_constant__ ScanMaps maps, const ScanArgs a) {
     if (slice == 0) {
       float* d = a.seg_decay + (seg - 1) * decays + ((long long)n * a.H + h) * DK + lane;
 #pragma unroll
-      for (int i = 0; i < DK / 32; ++i) d[32 * i] = prod[i];
+      for (int i = 0; i < DK / 32; ++i) d[32 * i] = prod[i] < FLT_MIN ? FLT_MIN : prod[i];
+      // (no decay is zero: an infinite state stays infinite over any number of steps, and is no NaN behind a segment)
     }
   } else if (!only && warp >= 12 && warp < 16) {
     // ====================================== outputs ========================================

@@ -1273,6 +1273,25 @@ def test_prefill_split_along_time_narrow_keys_keep_fp32_accuracy():
     assert np.linalg.norm(sT - rs) <= 5e-7 * np.linalg.norm(rs)
 
 
+@pytest.mark.parametrize("B,H,T,dk,dv", [(2, 3, 11000, 128, 256), (1, 4, 16500, 64, 128)])
+def test_prefill_split_along_time_infinite_state_stays_infinite(B, H, T, dk, dv):
+    """Decays that multiply to less than the smallest number: an infinity of the initial state is one of the final
+    state, as in the unsplit form, and does not leave its value column."""
+    import torch
+    p = wl.make_prefill(1008, B, H, T, dk, dv, "bf16", gate_mean=1.5, s0_std=0.3)
+    o, sT = _run_prefill(p)
+    assert rd.last_launch_count() == 4
+    p.s0[0, 1, 5, 7], p.s0[-1, 0, dk - 1, 130 % dv] = np.inf, -np.inf
+    o1, sT1 = _run_prefill(p)
+    where = np.zeros(sT.shape, bool)
+    where[0, 1, 5, 7] = where[-1, 0, dk - 1, 130 % dv] = True
+    assert sT1[0, 1, 5, 7] == np.inf and sT1[-1, 0, dk - 1, 130 % dv] == -np.inf
+    assert np.array_equal(sT1[~where], sT[~where])
+    columns = np.ones(o.shape, bool)
+    columns[0, 1, :, 7] = columns[-1, 0, :, 130 % dv] = False
+    assert np.array_equal(o1[columns], o[columns]) and not np.any(np.isfinite(o1[~columns]))
+
+
 def test_prefill_split_along_time_wait_that_runs_out_is_reported():
     import torch
     p = wl.make_prefill(1006, 1, 8, 8250, 128, 256, "bf16", s0_std=0.3)
