@@ -1046,9 +1046,11 @@ constexpr double kStateOnly = 0.4;
 //                      64 x 4096, two segments of operands from DRAM, 177 -> 183.  Below 4096 tokens the other side
 //                      is not split: 37 x 4000, two segments, 132 -> 134, with block terms 159 -> 170, 32 x 3900
 //                      with one set of gates 60.5 -> 61.6.
-// Calls of the fewest items that the pair kernel splits, from 4096 tokens on, stay with its five launches, which are
-// what its tests count (4 x 6000 tokens 146 us, 41 here), and so do one or two slices of dk = 64 with one launch.
-constexpr int kMinSplitPasses = 1280, kMinSplitItems = 16;   // items x tiles, items
+// The fewest items gain the most (one call, the other form against here, us): 1 x 4096 102 -> 28.5, 1 x 32768 133 -> 73,
+// 2 x 16384 128 -> 54, 4 x 4096 103 -> 33, 4 x 6000 140 -> 40, 7 x 9000 132 -> 71, with both block terms 1 x 32768 180 ->
+// 107, 7 x 9000 182 -> 92, one set of gates 7 x 9000 129 -> 43; dk = 64, one slice of 128 columns, 1985 tokens 40 -> 31,
+// 32768 453 -> 84, three slices 547 -> 135.  (Their errors against fp64 are those of the other form: dk = 64, gates of
+// slow to fast decay, final state 2.7e-7 to 8.4e-8 in both; dk = 128 1.5e-3 to 1.8e-3 in both.)
 constexpr size_t kStaysInL2 = (size_t)136 << 20;
 
 Segments plan_segments(const rodimus_ddts_fwd_params& p, int sms) {
@@ -1056,7 +1058,6 @@ Segments plan_segments(const rodimus_ddts_fwd_params& p, int sms) {
   if (p.cu_seqlens || p.cu_seqlens_host) return s;
   const long long items = (long long)p.B * p.H * (p.dv / 128), tiles = (p.T + kTile - 1) / kTile;
   if (items <= 0) return s;
-  if (p.dk == 64 ? items < 4 : p.dv % 256 == 0 && p.T >= 4096 && items < kMinSplitItems && items * tiles < kMinSplitPasses) return s;
   const int g = (int)std::min<long long>(std::min<long long>(sms / items, kMaxSegments), tiles / kMinSegmentTiles);
   if (g < 2 || 0.8 * tiles * (1.0 - (1.0 + kStateOnly) / (g + kStateOnly)) < (g == 2 ? 20.0 : 17.0)) return s;
   if (p.dk == 128 && !p.shared_gates && (size_t)(p.B * (long long)p.H * tiles) * Block<128>::kBytes > kStaysInL2) {

@@ -414,6 +414,11 @@ def test_config2_full_size_and_split_halves():
     assert rel_err(host(torch.cat([o1, o2], dim=2)), host(o)) <= 1e-2
 
 
+def _pair_split_bytes(prm):
+    """Room for the states of the pair kernel's segments but not for the operands that are formed first with more."""
+    return rd.fwd_workspace_bytes(prm, below=rd.fwd_workspace_bytes(prm))
+
+
 @pytest.mark.gpu
 def test_time_split_with_the_alternate_input_gate_and_fast_decay():
     """The split's state-only instantiation exists per input-gate mode, and a segment's decay
@@ -426,7 +431,7 @@ def test_time_split_with_the_alternate_input_gate_and_fast_decay():
         o = torch.full((B, H, T, dv), float("nan"), dtype=torch.bfloat16, device="cuda")
         sT = torch.full((B, H, 128, dv), float("nan"), dtype=torch.float32, device="cuda")
         prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT, ingate=ingate)
-        need = rd.fwd_workspace_bytes(prm)
+        need = _pair_split_bytes(prm)
         ws = torch.empty(need, dtype=torch.uint8, device="cuda")
         prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
         assert rd.fwd_raw(prm) == rd.OK and rd.last_launch_count() == 5
@@ -456,7 +461,7 @@ def test_time_split_from_two_host_threads():
                 o = torch.full((B, H, T, dv), float("nan"), dtype=torch.bfloat16, device="cuda")
                 sT = torch.full((B, H, 128, dv), float("nan"), dtype=torch.float32, device="cuda")
                 prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT)
-                need = rd.fwd_workspace_bytes(prm)
+                need = _pair_split_bytes(prm)
                 ws = torch.empty(need, dtype=torch.uint8, device="cuda")
                 prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
                 rc = rd.fwd_raw(prm)
@@ -490,7 +495,7 @@ def test_time_split_on_a_user_stream_back_to_back():
             o = torch.full((B, H, T, dv), float("nan"), dtype=torch.bfloat16, device="cuda")
             sT = torch.full((B, H, 128, dv), float("nan"), dtype=torch.float32, device="cuda")
             prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT)
-            need = rd.fwd_workspace_bytes(prm)
+            need = _pair_split_bytes(prm)
             ws = torch.empty(need, dtype=torch.uint8, device="cuda")
             prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
             assert rd.fwd_raw(prm) == rd.OK and rd.last_launch_count() == 5
@@ -520,7 +525,7 @@ def test_long_sequences_split_along_time(B, H, T, dv, with_s0):
     o = torch.full((B, H, T, dv), float("nan"), dtype=torch.bfloat16, device="cuda")
     sT = torch.full((B, H, 128, dv), float("nan"), dtype=torch.float32, device="cuda")
     prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT, scale=0.5)
-    need = rd.fwd_workspace_bytes(prm)
+    need = _pair_split_bytes(prm)
     assert need > 4096, "this shape should ask for the segments' state workspace"
     ws = torch.empty(need, dtype=torch.uint8, device="cuda")
     prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
@@ -612,7 +617,7 @@ def _block_terms(p, seed, H):
     return beta, d, fx
 
 
-def _check_block(p, which="both", ingate=rd.INGATE_POW_G, scale=0.5, expect_kernel=None, ws_bytes=None):
+def _check_block(p, which="both", ingate=rd.INGATE_POW_G, scale=0.5, expect_kernel=None, ws_bytes=None, pair_split=False):
     import torch
     B, H, T, dk, dv = p.shape
     beta, d, fx = _block_terms(p, 5, H)
@@ -626,7 +631,7 @@ def _check_block(p, which="both", ingate=rd.INGATE_POW_G, scale=0.5, expect_kern
                         dd["cu_host"], None, scale, ingate, **kw)
     if expect_kernel:
         assert rd.fwd_kernel_name(prm) == expect_kernel
-    need = rd.fwd_workspace_bytes(prm) if ws_bytes is None else ws_bytes
+    need = _pair_split_bytes(prm) if pair_split else rd.fwd_workspace_bytes(prm) if ws_bytes is None else ws_bytes
     ws = torch.empty(max(need, 256), dtype=torch.uint8, device="cuda")
     prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
     assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
@@ -656,7 +661,7 @@ def test_block_terms_bf16_packed_sequences_many_items():
 
 def test_block_terms_with_the_time_split():
     p = wl.make_prefill(505, 1, 2, 4500, 128, 256, "bf16", s0_std=0.2)
-    assert _check_block(p, "both") == 5                                     # split: five launches
+    assert _check_block(p, "both", pair_split=True) == 5                    # split: five launches
     assert _check_block(p, "both", ws_bytes=256) == 1                       # same request, unsplit
 
 
@@ -767,7 +772,8 @@ def _shared_inputs(seed, B, H, T, dk, dv, dtype, s0_std=0.1, cu=None, gate_mean=
     return pq, pv
 
 
-def _check_shared(seed, B, H, T, dk, dv, dtype, cu=None, block=False, expect_kernel=None, ingate=rd.INGATE_POW_G):
+def _check_shared(seed, B, H, T, dk, dv, dtype, cu=None, block=False, expect_kernel=None, ingate=rd.INGATE_POW_G,
+                  pair_split=False):
     import torch
     pq, pv = _shared_inputs(seed, B, H, T, dk, dv, dtype, cu=cu)
     beta, d, fx = _block_terms(pv, 7, H)
@@ -784,7 +790,8 @@ def _check_shared(seed, B, H, T, dk, dv, dtype, cu=None, block=False, expect_ker
     assert prm.shared_gates == 1 and prm.H == H
     if expect_kernel:
         assert rd.fwd_kernel_name(prm) == expect_kernel
-    ws = torch.empty(max(rd.fwd_workspace_bytes(prm), 256), dtype=torch.uint8, device="cuda")
+    need = _pair_split_bytes(prm) if pair_split else rd.fwd_workspace_bytes(prm)
+    ws = torch.empty(max(need, 256), dtype=torch.uint8, device="cuda")
     prm.workspace, prm.workspace_bytes = ws.data_ptr(), ws.numel()
     assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
     okw = dict(beta_hat=beta, feed_d=d, feed_x=fx) if block else {}
@@ -806,7 +813,7 @@ def test_shared_gates_packed_and_time_split():
     lens = _mixed_lengths(605, 40)
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
     _check_shared(606, 1, 4, int(cu[-1]), 128, 256, "bf16", cu=cu)
-    assert _check_shared(608, 2, 2, 4500, 128, 256, "bf16") == 5     # (batch, head) units split along time
+    assert _check_shared(608, 2, 2, 4500, 128, 256, "bf16", pair_split=True) == 5     # (batch, head) units split along time
 
 
 @pytest.mark.parametrize("dtype,dk,dv,H", [("f32", 64, 64, 4), ("bf16", 64, 256, 16), ("bf16", 128, 128, 3)])
@@ -1072,7 +1079,7 @@ def test_prefill_whose_workspace_does_not_fit_runs_with_less(packed):
         t.normal_(mean, std)
     cu = torch.tensor([0, 1000, T], dtype=torch.int32, device="cuda") if packed else None
     o = rd.ddts_fwd(q, k, x, y, v, cu_seqlens=cu, want_final_state=False)[0].cpu()
-    assert rd.last_launch_count() == 2 + packed
+    assert rd.last_launch_count() == (3 if packed else 4)         # (the dense call is split along time)
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     total = torch.cuda.get_device_properties(0).total_memory
@@ -1083,6 +1090,24 @@ def test_prefill_whose_workspace_does_not_fit_runs_with_less(packed):
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert rd.last_launch_count() == 1 + packed
     assert rel_err(host(least), host(o)) <= TOL_BF16
+
+
+@pytest.mark.parametrize("H,T,dk,dv,terms", [(4, 4095, 128, 256, 0), (4, 4096, 128, 256, 0), (4, 6000, 128, 256, 0),
+                                             (1, 32768, 128, 256, 0), (2, 4096, 128, 256, 2), (1, 4096, 128, 512, 0),
+                                             (1, 4096, 64, 128, 0), (2, 4096, 64, 128, 0), (3, 32768, 64, 128, 0)])
+@pytest.mark.parametrize("shared", [0, 1])
+def test_few_heads_are_split_where_they_are_the_slower_whole(H, T, dk, dv, terms, shared):
+    """However few the heads are, and on both sides of 4096 tokens: the workspace asked for holds the blocks of operands
+    and states of segments."""
+    p = rd.FwdParams()
+    p.struct_size, p.dtype, p.scale, p.shared_gates = ctypes.sizeof(rd.FwdParams), rd.BF16, 1.0, shared and H > 1
+    p.B, p.H, p.T, p.dk, p.dv = 1, H, T, dk, dv
+    p.beta_hat = 0x7F0000000000 if terms > 0 else None
+    p.feed_d = p.feed_x = 0x7F0000000000 if terms > 1 else None
+    blocks = (T + 63) // 64 * (1 if p.shared_gates else H) * (58368 if dk == 64 else 41984)
+    sizes = [rd.fwd_workspace_bytes(p)]
+    sizes.append(rd.fwd_workspace_bytes(p, below=sizes[0]))
+    assert sizes[0] > blocks + 2 * H * dk * dv * 4 and sizes[1] < sizes[0]
 
 
 @pytest.mark.parametrize("H,T,dk,dv,shared,launches", [
@@ -1242,6 +1267,10 @@ def test_two_launch_prefill_gates_per_head_few_tiles(block, T):
     (1, 32, 4100, 128, 256, "plain", -3.0),        # two segments
     (1, 2, 1986, 128, 128, "plain", -3.0),         # four of eight tiles, the last tile of two rows
     (1, 16, 1985, 128, 256, "both", -3.0),         # four of eight, the last shorter
+    (1, 4, 4096, 128, 256, "plain", -3.0),         # few heads
+    (1, 2, 6001, 128, 256, "both", -3.0),
+    (1, 1, 4097, 64, 128, "plain", -3.0),          # one slice of 128 columns in all
+    (1, 3, 8250, 64, 128, "shared", -3.0),
     (2, 3, 11000, 128, 256, "plain", 1.5),         # tiles cut into chunks, a segment's decay underflows
     (1, 16, 8250, 128, 128, "plain", -3.0),        # one slice of 128 columns a head
     (1, 1, 32800, 128, 512, "plain", -4.0),        # the most segments, four slices
@@ -1264,12 +1293,15 @@ def test_prefill_that_forms_operands_first_split_along_time(B, H, T, dk, dv, kin
     assert launches == 4
 
 
-def test_prefill_split_along_time_narrow_keys_keep_fp32_accuracy():
-    """dk = 64, slow decay: the final state carries products over all segments (see the bound above)."""
-    p = wl.make_prefill(1005, 1, 4, 33000, 64, 128, "bf16", gate_mean=-6.0, s0_std=0.1)
-    _, sT = _run_prefill(p)
+@pytest.mark.parametrize("H,T,dv,gate_mean", [(4, 33000, 128, -6.0), (1, 32768, 128, -6.0), (1, 8200, 256, -3.0), (3, 8200, 128, 0.0),
+                                              (1, 8200, 128, 2.0)])
+@pytest.mark.parametrize("ingate", [rd.INGATE_POW_G, rd.INGATE_POW_SIGMOID])
+def test_prefill_split_along_time_narrow_keys_keep_fp32_accuracy(H, T, dv, gate_mean, ingate):
+    """dk = 64; with slow decay the final state carries products over all segments (see the bound above)."""
+    p = wl.make_prefill(1005, 1, H, T, 64, dv, "bf16", gate_mean=gate_mean, s0_std=0.1)
+    _, sT = _run_prefill(p, ingate)
     assert rd.last_launch_count() == 4
-    _, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0)
+    _, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0, ingate=ingate)
     assert np.linalg.norm(sT - rs) <= 5e-7 * np.linalg.norm(rs)
 
 
