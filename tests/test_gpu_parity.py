@@ -441,10 +441,12 @@ def test_time_split_with_the_alternate_input_gate_and_fast_decay():
 
 
 @pytest.mark.gpu
-def test_time_split_from_two_host_threads():
+@pytest.mark.parametrize("pair", [True, False])
+def test_time_split_from_two_host_threads(pair):
     """Two host threads, each on its own stream, issue split calls at the same time (the C call
     runs without the interpreter lock): the library's one extra stream per device is shared, so
-    the fork and join of one call must not pick up the other call's events."""
+    the fork and join of one call of the pair kernel must not pick up the other call's events.
+    The form with operands first keeps to the caller's stream."""
     import threading
     import torch
     B, H, T, dv = 1, 2, 4300, 256
@@ -461,10 +463,11 @@ def test_time_split_from_two_host_threads():
                 o = torch.full((B, H, T, dv), float("nan"), dtype=torch.bfloat16, device="cuda")
                 sT = torch.full((B, H, 128, dv), float("nan"), dtype=torch.float32, device="cuda")
                 prm = rd.fwd_params(d["q"], d["k"], d["x"], d["y"], d["v"], o, d["s0"], sT)
-                need = _pair_split_bytes(prm)
+                need = _pair_split_bytes(prm) if pair else rd.fwd_workspace_bytes(prm)
                 ws = torch.empty(need, dtype=torch.uint8, device="cuda")
                 prm.workspace, prm.workspace_bytes = ws.data_ptr(), need
                 rc = rd.fwd_raw(prm)
+                assert rd.last_launch_count() == (5 if pair else 4)
                 outs.append((rc, p, o, sT, ws, d))
             stream.synchronize()
         results[tag] = outs
@@ -1340,6 +1343,42 @@ def test_prefill_split_along_time_wait_that_runs_out_is_reported():
     assert rd.fwd_raw(prm) == rd.OK and rd.device_status(ws) == rd.OK
     ro, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0)
     assert rel_err(host(o), ro) <= TOL_BF16 and rel_err(host(sT), rs) <= TOL_BF16
+
+
+@pytest.mark.parametrize("H,T,dk,dv,which", [(8, 8250, 128, 256, None), (1, 1986, 128, 128, None), (4, 4500, 128, 256, "both"),
+                                             (1, 4097, 64, 128, None)])
+@pytest.mark.parametrize("s0,want", [(False, True), (True, False), (False, False)])
+def test_prefill_split_along_time_without_states(H, T, dk, dv, which, s0, want):
+    """No initial state (the head segment starts from zero), no final state (the last segment writes none)."""
+    import torch
+    p = wl.make_prefill(1020 + T, 1, H, T, dk, dv, "bf16", s0_std=0.3 if s0 else None)
+    d = prefill_to_device(p)
+    kw, okw = {}, {}
+    if which:
+        beta, fd, fx = _block_terms(p, 5, H)
+        kw = dict(beta_hat=dev(beta, p.dtype), feed_d=torch.from_numpy(fd).cuda(), feed_x=dev(fx, p.dtype))
+        okw = dict(beta_hat=beta, feed_d=fd, feed_x=fx)
+    o, sT = rd.ddts_fwd(d["q"], d["k"], d["x"], d["y"], d["v"], d["s0"], want_final_state=want, **kw)
+    assert rd.last_launch_count() == 4 and (sT is not None) == want
+    ro, rs = orc.ref_fwd(p.q, p.k, p.x, p.y, p.v, s0=p.s0, **okw)
+    assert rel_err(host(o), ro) <= TOL_BF16 and (sT is None or rel_err(host(sT), rs) <= TOL_BF16)
+
+
+def test_prefill_split_along_time_captured_in_a_graph():
+    import torch
+    p = wl.make_prefill(1025, 1, 4, 4500, 128, 256, "bf16", s0_std=0.3)
+    d = prefill_to_device(p)
+    args = [d[n] for n in ("q", "k", "x", "y", "v", "s0")]
+    o, sT = rd.ddts_fwd(*args)
+    o1, sT1 = torch.full_like(o, float("nan")), torch.full_like(sT, float("nan"))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        rd.ddts_fwd(*args, out=o1, final_state=sT1)
+    assert rd.last_launch_count() == 4
+    for _ in range(2):
+        o1.fill_(float("nan")), sT1.fill_(float("nan"))
+        graph.replay()
+        assert torch.equal(o, o1) and torch.equal(sT, sT1)
 
 
 def test_prefill_split_along_time_back_to_back_on_one_workspace():
