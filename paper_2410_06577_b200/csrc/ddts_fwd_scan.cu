@@ -17,8 +17,8 @@
 // head's own gates would be, and its blocks are read from L2 by all H dv / 128 CTAs of a sequence.
 // Figures (layer shape, B=4 H=16 T=2048 dv=256): one set of gates, dk = 64: 9.6 us + 36 us, the scan
 // bound by the issue of its contractions (1670 cycles per chunk of 28 instructions, 1216 cycles of tensor
-// work) with 11 TB/s out of L2; gates per head, dk = 128: operands 55 us (issue-bound), scan 36 us (218 MB,
-// 6 TB/s).
+// work) with 11 TB/s out of L2; gates per head, dk = 128: operands 55 us (bound by no one unit: with a
+// third fewer instructions as long), scan 36 us (218 MB, 6 TB/s).
 //
 // dk = 128: operands in bf16, the precision of the kernel with the gates inside.  dk = 64 (the paper's
 // own key width): Kt as three bf16 parts (24 bits), Qt, P and the state's copy for the readout as two
@@ -1040,7 +1040,7 @@ constexpr double kStateOnly = 0.4;
 //   one set of gates   dk = 64, 4 heads x 32768 468 -> 98, 16 x 8192 126 -> 75; dk = 128, 16 x 16384 226 -> 111
 //   gates per head     dv = 256 8 x 2048 39 -> 33, 16 x 2048 49 -> 46, 4 x 4000 60 -> 35, 8 x 4096 109 -> 46,
 //                      8 x 8192 130 -> 74, 4 x 32768 153 -> 129, 16 x 8192 140 -> 126, 32 x 4096 129 -> 122;
-//                      while the operands stay in L2 (126 MB): 10 x 32768 273 -> 270, 16 x 32768 409 -> 411,
+//                      no gain where the operands do not stay in L2: 10 x 32768 273 -> 270, 16 x 32768 409 -> 411,
 //                      32 x 16384 358 -> 399.  With both block terms 16 x 32768 613 -> 541, 32 x 8192 305 -> 278;
 //                      dv = 512 8 x 32768 408 -> 301, 16 x 16384 358 -> 288; dv = 128 16 x 16384 335 -> 191, but
 //                      64 x 4096, two segments of operands from DRAM, 177 -> 183.  Below 4096 tokens the other side
@@ -1051,6 +1051,8 @@ constexpr double kStateOnly = 0.4;
 // 107, 7 x 9000 182 -> 92, one set of gates 7 x 9000 129 -> 43; dk = 64, one slice of 128 columns, 1985 tokens 40 -> 31,
 // 32768 453 -> 84, three slices 547 -> 135.  (Their errors against fp64 are those of the other form: dk = 64, gates of
 // slow to fast decay, final state 2.7e-7 to 8.4e-8 in both; dk = 128 1.5e-3 to 1.8e-3 in both.)
+// Blocks of 86 MB (4 x 32768, 32 x 4096) are read back from L2 (126 MB) for the most part, those of 172 MB and more (16 x
+// 16384) from DRAM; the line lies between.
 constexpr size_t kStaysInL2 = (size_t)136 << 20;
 
 Segments plan_segments(const rodimus_ddts_fwd_params& p, int sms) {
