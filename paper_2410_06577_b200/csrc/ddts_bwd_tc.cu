@@ -605,8 +605,9 @@ __device__ __forceinline__ void sweep_piece(const BwdTcArgs& a, const SweepMaps&
 #pragma unroll
             for (uint32_t kk = 0; kk < 4; ++kk) umma_ss(od, pa + 128 * kk, ta + 2 * kk, kI3, 1u);
           }
-          umma_commit(bar(SB_OFULL0 + ph));
+          // (the commit that somebody waits for, also after the last chunk, comes last: none arrives after the CTA's end)
           umma_commit(bar(SB_EP));
+          umma_commit(bar(SB_OFULL0 + ph));
         }
         __syncwarp();
         if (last) break;

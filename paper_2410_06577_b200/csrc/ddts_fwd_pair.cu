@@ -621,8 +621,9 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
             umma_bf16_lo<true>(tmem + kColS + (g & 1) * 128, dv + 128 * kk, dkt + 128 * kk, kIdescS);
-          umma_commit(bar(BAR_SFULL));
+          // (the commit that somebody waits for, also after the last pass, comes last: none arrives after the CTA's end)
           if (STATE_ONLY) umma_commit(bar(BAR_EMPTY0 + s));
+          umma_commit(bar(BAR_SFULL));
           if (STATE_ONLY) { ++g; continue; }             // no scores, no outputs
           if (!(ok = mbar_wait(bar(BAR_PREADY), ph1, abort_flag, a.hdr))) break;
           if (!(ok = mbar_wait(bar(BAR_OFREE), ph1 ^ 1, abort_flag, a.hdr))) break;
@@ -637,8 +638,8 @@ ddts_fwd_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           for (int kk = 0; kk < 4; ++kk) umma_bf16_atmem<true>(tmem + kColO, t_sb + 8 * kk, dq0 + 2 * kk, kIdescOs);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) umma_bf16_atmem<true>(tmem + kColO, t_sb + 8 * (kk + 4), dq1 + 2 * kk, kIdescOs);
-          umma_commit(bar(BAR_OFULL));
           umma_commit(bar(BAR_EMPTY0 + s));   // every contraction of the pass has read its operands
+          umma_commit(bar(BAR_OFULL));
           ++g;
         }
       }

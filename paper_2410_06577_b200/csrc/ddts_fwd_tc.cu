@@ -318,8 +318,9 @@ ddts_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
               umma_bf16(tmem + kColS, desc_mnmajor(st + kOffX + kk * 2048, kSlabBytes),
                         desc_mnmajor(st + kOffV + kk * 2048, kSlabBytes), kIdescS, 1);
             }
-            umma_commit(bar(BAR_SFULL));
+            // (the commit that somebody waits for, also after the last pass, comes last: none arrives after the CTA's end)
             umma_commit(bar(BAR_EMPTY0 + s));
+            umma_commit(bar(BAR_SFULL));
           }
           __syncwarp();
           ++g;
